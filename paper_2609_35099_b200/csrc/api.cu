@@ -8,6 +8,7 @@
 #include "fast_registry.hpp"
 #include "fast/fast_common.cuh"
 #include "generic_kernels.cuh"
+#include "path_launch.hpp"
 
 namespace e3j {
 
@@ -362,6 +363,12 @@ int e3j::conv_fwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, c
         if (int s = graph_prepare(n_nodes, n_edges, senders, receivers, rp, nullptr, nullptr, st)) return s;
         rowptr = rp;
     }
+    if (path::covers(plan, 4)) {
+        path::Call<float> c{};
+        c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w;
+        c.senders = senders; c.receivers = receivers; c.rowptr = rowptr; c.out = out; c.stream = st;
+        return path::conv_fwd(plan, c, false);
+    }
     DeviceTables t;
     if (int s = get_device_tables(plan, t)) return s;
     generic::conv_fwd_kernel<false><<<grid_for(n_nodes), block_for((int64_t)plan->D * plan->nq / 4), 0, st>>>(t, dims_of(plan), n_nodes, x, sh, w,
@@ -429,6 +436,13 @@ int e3j::conv_bwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, c
         a.workspace = ws + L.scratch; a.workspace_bytes = workspace_bytes - L.scratch; a.stream = st;
         a.n_real = n_real;
         return fk->conv_bwd(a);
+    }
+    if (path::covers(plan, 4)) {
+        path::Call<float> c{};
+        c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w; c.grad_out = grad_out;
+        c.senders = senders; c.receivers = receivers; c.sender_perm = sender_perm; c.colptr = colptr; c.n_real = n_real;
+        c.grad_x = grad_x; c.grad_sh = grad_sh; c.grad_w = grad_w; c.stream = st;
+        return path::conv_bwd(plan, c, false);
     }
     DeviceTables t;
     if (int s = get_device_tables(plan, t)) return s;
@@ -590,6 +604,11 @@ int e3j_tp_fwd(const e3j_plan* plan, int64_t rows, const float* x1, const float*
     cudaStream_t st = (cudaStream_t)stream;
     const FastKernels* fk = fast_lookup(plan);
     if (fk && fk->tp_fwd) return fk->tp_fwd(rows, x1, x2, w, out, st);
+    if (rows < (1ll << 31) - 1 && path::covers(plan, 4)) {
+        path::Call<float> c{};
+        c.n_nodes = c.n_edges = rows; c.x = x1; c.sh = x2; c.w = w; c.out = out; c.stream = st;
+        return path::conv_fwd(plan, c, true);
+    }
     DeviceTables t;
     if (int s = get_device_tables(plan, t)) return s;
     generic::conv_fwd_kernel<true><<<grid_for(rows), block_for((int64_t)plan->D * plan->nq / 4), 0, st>>>(t, dims_of(plan), rows, x1, x2, w, nullptr,
@@ -609,6 +628,12 @@ int e3j_tp_bwd(const e3j_plan* plan, int64_t rows, const float* x1, const float*
     const FastKernels* fk = fast_lookup(plan);
     if (fk && fk->tp_bwd && grad_x1 && grad_x2 && grad_w)
         return fk->tp_bwd(rows, x1, x2, w, grad_out, grad_x1, grad_x2, grad_w, st);
+    if (rows < (1ll << 31) - 1 && path::covers(plan, 4)) {
+        path::Call<float> c{};
+        c.n_nodes = c.n_edges = rows; c.x = x1; c.sh = x2; c.w = w; c.grad_out = grad_out;
+        c.grad_x = grad_x1; c.grad_sh = grad_x2; c.grad_w = grad_w; c.stream = st;
+        return path::conv_bwd(plan, c, true);
+    }
     DeviceTables t;
     if (int s = get_device_tables(plan, t)) return s;
     const Dims dm = dims_of(plan);

@@ -4,7 +4,10 @@
 // defining sum in a fixed order (edges in list order, records in table order), with the coefficient values kept
 // in float64 as the plan builder computed them.  They are the float64 counterpart of generic_kernels.cuh, one
 // channel per thread; there are no signature-specialised float64 kernels.
+#include <initializer_list>
+
 #include "common.cuh"
+#include "path_launch.hpp"
 
 namespace e3j {
 
@@ -122,6 +125,14 @@ bool basic_args_ok(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     return plan && n_nodes >= 0 && n_edges >= 0 && n_nodes < (1ll << 31) - 1 && n_edges < (1ll << 31) - 1;
 }
 
+// The per-path kernels take two channels per thread with 16-byte loads; float64 arrays need not start on 16 bytes
+// here, and the channel count may be odd: those calls stay on the table-driven kernels.
+bool on_path_kernels(const e3j_plan* plan, std::initializer_list<const void*> arrays) {
+    for (const void* q : arrays)
+        if ((uintptr_t)q & 15u) return false;
+    return path::covers(plan, 2);
+}
+
 }  // namespace
 }  // namespace e3j
 
@@ -148,6 +159,12 @@ int e3j_conv_fwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         if (int s = graph_prepare(n_nodes, n_edges, senders, receivers, rp, nullptr, nullptr, st)) return s;
         rowptr = rp;
     }
+    if (on_path_kernels(plan, {x, w, out})) {
+        path::Call<double> c{};
+        c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w;
+        c.senders = senders; c.receivers = receivers; c.rowptr = rowptr; c.out = out; c.stream = st;
+        return path::conv_fwd(plan, c);
+    }
     DeviceTables t;
     if (int s = get_device_tables(plan, t)) return s;
     const Dims dm{plan->nq, plan->d, plan->dp, plan->P, plan->D, (plan->flags & E3J_PLAN_COLLAPSE_OUTPUTS) ? 1 : 0};
@@ -173,6 +190,13 @@ int e3j_conv_bwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         int32_t* pm = (int32_t*)(ws + 2 * sec);
         if (int s = graph_prepare(n_nodes, n_edges, senders, receivers, nullptr, pm, cp, st)) return s;
         sender_perm = pm; colptr = cp;
+    }
+    if (on_path_kernels(plan, {x, w, grad_out, grad_x, grad_w})) {
+        path::Call<double> c{};
+        c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w; c.grad_out = grad_out;
+        c.senders = senders; c.receivers = receivers; c.sender_perm = sender_perm; c.colptr = colptr;
+        c.grad_x = grad_x; c.grad_sh = grad_sh; c.grad_w = grad_w; c.stream = st;
+        return path::conv_bwd(plan, c);
     }
     DeviceTables t;
     if (int s = get_device_tables(plan, t)) return s;

@@ -816,6 +816,37 @@ class Sig:
         return "\n".join(o) + "\n"
 
 
+def emit_path_pairs(lmax=3):
+    """path_pairs.inc: the coupling tensor of every path (l1, l2) -> L with l <= lmax as two macros, its (row, column)
+    pairs by output row m0 and by input row m1.  P1(in, i, c): the pair's entry of A is c y[i]; P2(in, i, c, j, d):
+    c y[i] + d y[j]; B(row) and E(row) open and close a row."""
+    o = ["// GENERATED by csrc/gen_fast.py -- coupling pairs of single paths (l1, l2) -> L, see emit_path_pairs there"]
+    triples = []
+    for l1 in range(lmax + 1):
+        _, paths, recs, _ = load_records({"irreps_in": f"4x{l1}e", "sh_lmax": lmax, "out_lmax": lmax})
+        for k, p in enumerate(paths):
+            pairs = {}
+            for i0, i1, i2, i3, v in recs:
+                if i3 == k:
+                    pairs.setdefault((i0 - p["out_off"], i1), []).append((i2 - p["y_off"], v))
+            triples.append((l1, p["l2"], p["L"], pairs))
+    triples.sort(key=lambda t: t[:3])
+    o.append("#define E3J_PATH_TRIPLES(X) " + " ".join(f"X({a}, {b}, {c})" for a, b, c, _ in triples))
+    for l1, l2, L, pairs in triples:
+        for side, n_rows in ((0, 2 * L + 1), (1, 2 * l1 + 1)):
+            text = []
+            for row in range(n_rows):
+                text.append(f"B({row})")
+                for key in sorted(pairs):
+                    if key[side] == row:
+                        args = ", ".join(f"{i}, {v!r}" for i, v in pairs[key])
+                        assert len(pairs[key]) <= 2
+                        text.append(f"P{len(pairs[key])}({key[1 - side]}, {args})")
+                text.append(f"E({row})")
+            o.append(f"#define E3J_PATH_BY{side}_{l1}{l2}{L}(B, P1, P2, E) " + " ".join(text))
+    return "\n".join(o) + "\n"
+
+
 def generate(extra=None):
     """{file name: text} for the committed signatures plus, if given, the entries of an overlay list."""
     sigs = json.loads((HERE / "fast" / "signatures.json").read_text())
@@ -831,6 +862,7 @@ def generate(extra=None):
     entries = "// GENERATED by csrc/gen_fast.py -- one E3J_FAST_ENTRY(name) per specialised signature\n"
     entries += "".join(f"E3J_FAST_ENTRY(kFast_{sig['name']})\n" for sig in sigs)
     files["registry_entries.inc"] = entries
+    files["path_pairs.inc"] = emit_path_pairs()
     return files
 
 

@@ -1,0 +1,327 @@
+// Kernels for plans without generated ones, built from single coupling paths.
+//
+// A path (l1, l2) -> L with l <= 3 is one of 34 fixed tensors, so its pairs are unrolled with constant coefficients
+// (fast/path_pairs.inc) whatever signature it belongs to; the plan only says which paths there are and where their
+// rows lie.  A warp takes one path at a time (the switch below is warp-uniform) and keeps all rows of its result in
+// registers while it walks its edges, so a path's input rows and weights are loaded once per edge instead of once
+// per output row, and no coefficient record is ever fetched.
+//
+//   node sums  (forward; grad_x with the tensor transposed and the edges in sender order): one thread owns V channels
+//              of one node and one output block, 2L+1 accumulators, edges in list order;
+//   edge part  (grad_w, grad_sh): one thread owns V channels of one edge and walks all paths; grad_sh's channel sum
+//              goes through shared memory in a fixed order.
+//
+// What bounds them: the latency of the row loads at 18 to 20 warps per SM (issue slots 30-40 % busy, DRAM below 20 %),
+// not arithmetic or bandwidth.  48x(0e+1o+2e), l <= 2, 35050 edges: forward 243 -> 99 us, backward 823 -> 189 us
+// against the table-driven kernels; float64, 64x(0e+1o), l <= 2, 10176 edges, both passes: 705 -> 131 us.  Tried and
+// slower: weights and ids two steps ahead (spills, 378 against 284 us for both passes), each path's sum as a function
+// of its own, grad_out rows of the next path prefetched.
+//
+// Same sums as the table-driven kernels, in a fixed order, no atomics.  What stays on the table-driven ones: plans
+// with l > 3, more than 128 V-channel units, and (float64) odd channel counts or pointers off 16 bytes.
+#pragma once
+#include "common.cuh"
+#include "fast/path_pairs.inc"
+
+namespace e3j {
+namespace path {
+
+constexpr int kMaxDeg = 7;   // rows of the largest block, 2 * 3 + 1
+
+template <class T, int V> struct alignas(sizeof(T) * V) Pack { T v[V]; };
+
+template <class T, int V>
+__host__ __device__ __forceinline__ void load_pack(T (&dst)[V], const T* src) {
+    const Pack<T, V> p = *reinterpret_cast<const Pack<T, V>*>(src);
+#pragma unroll
+    for (int c = 0; c < V; ++c) dst[c] = p.v[c];
+}
+template <class T, int V>
+__host__ __device__ __forceinline__ void store_pack(T* dst, const T (&src)[V]) {
+    Pack<T, V> p;
+#pragma unroll
+    for (int c = 0; c < V; ++c) p.v[c] = src[c];
+    *reinterpret_cast<Pack<T, V>*>(dst) = p;
+}
+template <class T, int V>
+__host__ __device__ __forceinline__ void axpy(T (&z)[V], const T a, const T (&x)[V]) {
+#pragma unroll
+    for (int c = 0; c < V; ++c) z[c] = fma(a, x[c], z[c]);
+}
+template <class T, int V>
+__host__ __device__ __forceinline__ void axpy(T (&z)[V], const T (&a)[V], const T (&x)[V]) {
+#pragma unroll
+    for (int c = 0; c < V; ++c) z[c] = fma(a[c], x[c], z[c]);
+}
+template <class T, int V>
+__host__ __device__ __forceinline__ T dot(const T (&a)[V], const T (&b)[V]) {
+    T s = a[0] * b[0];
+#pragma unroll
+    for (int c = 1; c < V; ++c) s = fma(a[c], b[c], s);
+    return s;
+}
+
+// Tri<l1,l2,L>: sum    acc[m0] += w * (sum over the path's pairs of A(y)[m0,m1] in[m1])
+//               sum_t  acc[m1] += w * (sum of A(y)[m0,m1] in[m0])
+//               edge   dw += sum g[m0] A[m0,m1] x[m1],  dy[m2] += sum C (s x[m1]) . g[m0]
+template <int l1, int l2, int L> struct Tri;
+
+#define E3J_PB(o) { T z[V]; _Pragma("unroll") for (int c = 0; c < V; ++c) z[c] = T(0);
+#define E3J_P1(r, i, a) axpy(z, T(a) * y[i], in[r]);
+#define E3J_P2(r, i, a, j, b) axpy(z, fma(T(a), y[i], T(b) * y[j]), in[r]);
+#define E3J_PE(o) axpy(acc[o], w, z); }
+#define E3J_EB(o) { T z[V], sg[V]; _Pragma("unroll") for (int c = 0; c < V; ++c) { z[c] = T(0); sg[c] = s[c] * g[o][c]; }
+#define E3J_E1(r, i, a) { axpy(z, T(a) * y[i], x[r]); dy[i] = fma(T(a), dot(x[r], sg), dy[i]); }
+#define E3J_E2(r, i, a, j, b) { axpy(z, fma(T(a), y[i], T(b) * y[j]), x[r]); const T t_ = dot(x[r], sg); \
+                                dy[i] = fma(T(a), t_, dy[i]); dy[j] = fma(T(b), t_, dy[j]); }
+#define E3J_EE(o) axpy(dw, g[o], z); }
+#define E3J_DEFINE_TRI(l1, l2, L)                                                                                    \
+    template <> struct Tri<l1, l2, L> {                                                                              \
+        static constexpr int kL1 = l1, kL2 = l2, kL = L;                                                             \
+        template <class T, int V, int NI, int NO>                                                                    \
+        __host__ __device__ static __forceinline__ void sum(const T* y, const T (&in)[NI][V], const T (&w)[V],       \
+                                                            T (&acc)[NO][V]) {                                       \
+            E3J_PATH_BY0_##l1##l2##L(E3J_PB, E3J_P1, E3J_P2, E3J_PE)                                                 \
+        }                                                                                                            \
+        template <class T, int V, int NI, int NO>                                                                    \
+        __host__ __device__ static __forceinline__ void sum_t(const T* y, const T (&in)[NI][V], const T (&w)[V],     \
+                                                              T (&acc)[NO][V]) {                                     \
+            E3J_PATH_BY1_##l1##l2##L(E3J_PB, E3J_P1, E3J_P2, E3J_PE)                                                 \
+        }                                                                                                            \
+        template <class T, int V, int NX, int NG>                                                                    \
+        __host__ __device__ static __forceinline__ void edge(const T* y, T* dy, const T (&x)[NX][V], const T (&s)[V],\
+                                                             const T (&g)[NG][V], T (&dw)[V]) {                      \
+            E3J_PATH_BY0_##l1##l2##L(E3J_EB, E3J_E1, E3J_E2, E3J_EE)                                                 \
+        }                                                                                                            \
+    };
+E3J_PATH_TRIPLES(E3J_DEFINE_TRI)
+
+#define E3J_TRI_ID(l1, l2, L) ((l1) * 16 + (l2) * 4 + (L))
+constexpr uint8_t kNoPath = 255;   // a group of input rows that no path reads: nothing to add
+
+// One plan's paths in a processing order, passed by value (kernel parameters: constant-bank reads, nothing to upload).
+struct PathRec { uint8_t id, l1, L, k, x_off, y_off, out_off, pad; };
+struct PathTable {
+    int n_paths, n_groups;
+    uint8_t start[257];          // groups of paths that share the rows they are summed into
+    PathRec rec[255];
+};
+static_assert(sizeof(PathTable) < 3072, "the table travels in the kernel parameters");
+
+template <class T> struct Args {
+    int64_t n_nodes, n_edges;
+    const T *x, *sh, *w, *g;     // g: grad_out
+    const int32_t *senders, *receivers, *ptr, *perm, *n_real;
+    T *out, *grad_w, *grad_sh;   // out: the node sums (forward out, backward grad_x)
+    int d, dp, P, D, units;      // units: N_q / V
+    int split_log2;              // a node's edges are dealt to 2^split_log2 lanes
+    unsigned node_blocks;        // backward: blocks below this one are node sums, the others edge tiles
+};
+
+// ---------------------------------------------------------------- node sums
+// One path's share of a node's rows: summed over the lane's edges, then over the lanes that share the node, and
+// stored by the first of them (added to the rows for the group's second and later paths).
+template <class Tr, class T, int V, bool TR, bool IDENT>
+__device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, const unsigned j0, const unsigned j1,
+                                         const int step, const int row, const int q, T* dst, const bool first) {
+    constexpr int NI = TR ? 2 * Tr::kL + 1 : 2 * Tr::kL1 + 1, NO = TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1;
+    constexpr int NY = 2 * Tr::kL2 + 1;
+    constexpr int U = NI <= 3 ? 2 : 1;   // edges in flight: their input rows fill at most 28 registers
+    const T* in_base = (TR ? a.g + (size_t)rec.out_off * row : a.x + (size_t)rec.x_off * row) + q * V;
+    const T* w_base = a.w + (size_t)rec.k * row + q * V;
+    const size_t in_stride = (size_t)(TR ? a.D : a.d) * row, w_stride = (size_t)a.P * row;
+    T acc[NO][V];
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+#pragma unroll
+        for (int c = 0; c < V; ++c) acc[o][c] = T(0);
+    // the ids of an edge are fetched one step ahead of its rows; past the end: the last step's first edge again
+    int e[U], b[U];
+    auto ids = [&](unsigned j) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned jc = j + u * step < j1 ? j + u * step : j;
+            e[u] = TR && !IDENT ? a.perm[jc] : (int)jc;
+            b[u] = IDENT ? e[u] : TR ? a.receivers[e[u]] : a.senders[e[u]];
+        }
+    };
+    if (j0 < j1) ids(j0);
+#pragma unroll 1
+    for (unsigned j = j0; j < j1; j += U * step) {
+        T in[U][NI][V], y[U][NY], w[U][V];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            load_pack<T, V>(w[u], w_base + (size_t)e[u] * w_stride);
+#pragma unroll
+            for (int i = 0; i < NI; ++i) load_pack<T, V>(in[u][i], in_base + (size_t)b[u] * in_stride + i * row);
+#pragma unroll
+            for (int i = 0; i < NY; ++i) y[u][i] = a.sh[(size_t)e[u] * a.dp + rec.y_off + i];
+        }
+        if (j + U * step < j1) ids(j + U * step);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (j + u * step >= j1) break;
+            if constexpr (TR) Tr::template sum_t<T, V>(y[u], in[u], w[u], acc);
+            else Tr::template sum<T, V>(y[u], in[u], w[u], acc);
+        }
+    }
+#pragma unroll 1
+    for (int off = 32 / step; off < 32; off <<= 1) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o)
+#pragma unroll
+            for (int c = 0; c < V; ++c) acc[o][c] += __shfl_xor_sync(0xffffffffu, acc[o][c], off);
+    }
+    if (!dst) return;
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+        if (!first) {
+            T have[V];
+            load_pack<T, V>(have, dst + (size_t)o * row);
+#pragma unroll
+            for (int c = 0; c < V; ++c) acc[o][c] += have[c];
+        }
+        store_pack<T, V>(dst + (size_t)o * row, acc[o]);
+    }
+}
+
+template <class T, int V, int LM, bool TR, bool IDENT>
+__device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, const unsigned block) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int grp = (int)(block % (unsigned)t.n_groups);
+    const int per_warp = 32 >> a.split_log2, part = lane >> (5 - a.split_log2);
+    const int64_t item = ((int64_t)(block / (unsigned)t.n_groups) * warps + warp) * per_warp + (lane & (per_warp - 1));
+    const int64_t node = item / a.units;
+    const int q = (int)(item - node * a.units), row = a.units * V;
+    unsigned j0 = 0, j1 = 0;   // edge counts are below 2^31, so a step past the end does not wrap
+    T* dst = nullptr;
+    const int p0 = t.start[grp], p1 = t.start[grp + 1];
+    if (node < a.n_nodes) {
+        j0 = IDENT ? (unsigned)node : (unsigned)a.ptr[node];
+        j1 = IDENT ? (unsigned)node + 1 : (unsigned)a.ptr[node + 1];
+        if (part == 0)
+            dst = a.out + ((size_t)node * (TR ? a.d : a.D) + (TR ? t.rec[p0].x_off : t.rec[p0].out_off)) * row + q * V;
+    }
+#pragma unroll 1
+    for (int p = p0; p < p1; ++p) {
+        const PathRec rec = t.rec[p];
+        int row_p = row, step = 1 << a.split_log2;
+        asm volatile("" : "+r"(row_p), "+r"(step));   // keeps every case's address arithmetic inside the case
+        switch (rec.id) {
+#define E3J_CASE(l1, l2, L) \
+            case E3J_TRI_ID(l1, l2, L): \
+                if constexpr (l1 <= LM && l2 <= LM && L <= LM) \
+                    sum_path<Tri<l1, l2, L>, T, V, TR, IDENT>(a, rec, j0 + part, j1, step, row_p, q, dst, p == p0); \
+                break;
+            E3J_PATH_TRIPLES(E3J_CASE)
+#undef E3J_CASE
+            default: {   // kNoPath: zero rows
+                T z[V];
+#pragma unroll
+                for (int c = 0; c < V; ++c) z[c] = T(0);
+                if (dst)
+                    for (int o = 0; o < 2 * rec.l1 + 1; ++o) store_pack<T, V>(dst + (size_t)o * row, z);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------- edge part
+template <class T, int V, int LM, bool IDENT>
+__device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, const unsigned tile, T* part) {
+    const int slots = blockDim.x / a.units, slot = threadIdx.x / a.units, q = threadIdx.x - slot * a.units;
+    const int64_t e = (int64_t)tile * slots + slot;
+    const int64_t n_live = a.n_real ? min((int64_t)*a.n_real, a.n_edges) : a.n_edges;
+    const bool mine = slot < slots && e < a.n_edges, live = mine && e < n_live;
+    const int row = a.units * V;
+    constexpr int NY = (LM + 1) * (LM + 1);
+    T y[NY], dy[NY];
+#pragma unroll
+    for (int i = 0; i < NY; ++i) { dy[i] = T(0); y[i] = live && i < a.dp ? a.sh[(size_t)e * a.dp + i] : T(0); }
+    if (live) {
+        const int64_t from = IDENT ? e : (int64_t)a.senders[e], to = IDENT ? e : (int64_t)a.receivers[e];
+        const T* xe = a.x + (size_t)from * a.d * row + q * V;
+        const T* ge = a.g + (size_t)to * a.D * row + q * V;
+        const T* we = a.w + (size_t)e * a.P * row + q * V;
+        T x[2 * LM + 1][V], s1[V];   // s1: the next path's weights
+#pragma unroll
+        for (int i = 0; i < 2 * LM + 1; ++i)
+#pragma unroll
+            for (int c = 0; c < V; ++c) x[i][c] = T(0);
+        int have = -1;
+        load_pack<T, V>(s1, we + (size_t)t.rec[0].k * row);
+#pragma unroll 1
+        for (int p = 0; p < t.n_paths; ++p) {
+            const PathRec rec = t.rec[p];
+            if (rec.x_off != have) {
+                have = rec.x_off;
+#pragma unroll
+                for (int i = 0; i < 2 * LM + 1; ++i)
+                    if (i < 2 * rec.l1 + 1) load_pack<T, V>(x[i], xe + (size_t)(rec.x_off + i) * row);
+            }
+            T s[V], dw[V];
+#pragma unroll
+            for (int c = 0; c < V; ++c) { s[c] = s1[c]; dw[c] = T(0); }
+            if (p + 1 < t.n_paths) load_pack<T, V>(s1, we + (size_t)t.rec[p + 1].k * row);
+            const T* gk = ge + (size_t)rec.out_off * row;
+            int row_p = row;
+            asm volatile("" : "+r"(row_p));   // as in node_part
+            switch (rec.id) {
+#define E3J_CASE(l1, l2, L) \
+                case E3J_TRI_ID(l1, l2, L): if constexpr (l1 <= LM && l2 <= LM && L <= LM) { \
+                    T g[2 * L + 1][V]; \
+                    _Pragma("unroll") for (int i = 0; i < 2 * L + 1; ++i) load_pack<T, V>(g[i], gk + (size_t)i * row_p); \
+                    Tri<l1, l2, L>::template edge<T, V>(y + l2 * l2, dy + l2 * l2, x, s, g, dw); \
+                } break;
+                E3J_PATH_TRIPLES(E3J_CASE)
+#undef E3J_CASE
+            }
+            if (a.grad_w) store_pack<T, V>(a.grad_w + ((size_t)e * a.P + rec.k) * row + q * V, dw);
+        }
+    } else if (mine && a.grad_w) {   // a padding edge: zero rows
+        T z[V];
+#pragma unroll
+        for (int c = 0; c < V; ++c) z[c] = T(0);
+        for (int k = 0; k < a.P; ++k) store_pack<T, V>(a.grad_w + ((size_t)e * a.P + k) * row + q * V, z);
+    }
+    if (!a.grad_sh) return;
+    // channel sum: eight lanes per (edge, component) add every eighth partial, then a fixed tree over the eight
+#pragma unroll
+    for (int i = 0; i < NY; ++i)
+        if (i < a.dp) part[i * blockDim.x + threadIdx.x] = dy[i];
+    __syncthreads();
+    const int sub = threadIdx.x & 7, n_out = slots * a.dp, per_pass = blockDim.x >> 3;
+    for (int o0 = 0; o0 < n_out; o0 += per_pass) {
+        const int o = o0 + (threadIdx.x >> 3);
+        const int sl = o / a.dp, i = o - sl * a.dp;
+        T sum = T(0);
+        if (o < n_out)
+            for (int u = sub; u < a.units; u += 8) sum += part[i * blockDim.x + sl * a.units + u];
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        const int64_t eo = (int64_t)tile * slots + sl;
+        if (sub == 0 && o < n_out && eo < a.n_edges) a.grad_sh[(size_t)eo * a.dp + i] = sum;
+    }
+}
+
+// LM: the plan's largest l.  It sets the registers of a thread (an edge's input rows, harmonics and grad_out rows),
+// and with them the warps that hide the loads' latency: 4, 5 or 6 blocks of 128 threads per SM for LM = 3, 2, 1.
+constexpr int kThreads = 128;
+constexpr int blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 5 : 6; }
+
+template <class T, int V, int LM, bool IDENT>
+__global__ void __launch_bounds__(kThreads, blocks_per_sm(LM))
+fwd_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
+    node_part<T, V, LM, false, IDENT>(t, a, blockIdx.x);
+}
+
+template <class T, int V, int LM, bool IDENT>
+__global__ void __launch_bounds__(kThreads, blocks_per_sm(LM))
+bwd_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
+    __shared__ T part[(LM + 1) * (LM + 1) * kThreads];
+    if (blockIdx.x < a.node_blocks) node_part<T, V, LM, true, IDENT>(t, a, blockIdx.x);
+    else edge_part<T, V, LM, IDENT>(t, a, blockIdx.x - a.node_blocks, part);
+}
+
+}  // namespace path
+}  // namespace e3j

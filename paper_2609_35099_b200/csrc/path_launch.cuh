@@ -1,0 +1,123 @@
+// Launchers of the per-path kernels (path_kernels.cuh), one translation unit per element type.
+#pragma once
+#include "path_kernels.cuh"
+
+#include <algorithm>
+
+#include "path_launch.hpp"
+
+namespace e3j {
+namespace path {
+namespace {
+
+// Input rows that no path reads (an irrep whose products the output filter drops), cut into groups of 7, 5, 3 or 1
+// rows: f(first row, l of a block of that size).  Their grad_x is zero.
+template <class F> void for_unread_rows(const e3j_plan* plan, F f) {
+    std::vector<char> read(plan->d, 0);
+    for (const e3j_path_info_t& p : plan->paths) std::fill_n(read.begin() + p.x_off, 2 * p.l1 + 1, 1);
+    for (int row = 0; row < plan->d;) {
+        int n = 0;
+        while (n < kMaxDeg && row + n < plan->d && !read[row + n]) ++n;
+        if (n) f(row, (n - 1) / 2);
+        row += n ? 2 * ((n - 1) / 2) + 1 : 1;
+    }
+}
+
+// Paths in plan order, grouped by output block (forward), or by input block (backward).
+PathTable table_of(const e3j_plan* plan, bool by_input) {
+    PathTable t{};
+    t.n_paths = plan->P;
+    std::vector<int> order(plan->P);
+    for (int k = 0; k < plan->P; ++k) order[k] = k;
+    auto key = [&](int k) { return by_input ? plan->paths[k].x_off : plan->paths[k].out_off; };
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
+    for (int p = 0; p < plan->P; ++p) {
+        const int k = order[p];
+        const e3j_path_info_t& pi = plan->paths[k];
+        t.rec[p] = PathRec{(uint8_t)E3J_TRI_ID(pi.l1, pi.l2, pi.L), (uint8_t)pi.l1, (uint8_t)pi.L, (uint8_t)k,
+                           (uint8_t)pi.x_off, (uint8_t)pi.y_off, (uint8_t)pi.out_off, 0};
+        if (p == 0 || key(k) != key(order[p - 1])) t.start[t.n_groups++] = (uint8_t)p;
+    }
+    int n = plan->P;
+    if (by_input)
+        for_unread_rows(plan, [&](int row, int l) {
+            t.rec[n] = PathRec{kNoPath, (uint8_t)l, 0, 0, (uint8_t)row, 0, 0, 0};
+            t.start[t.n_groups++] = (uint8_t)n++;
+        });
+    t.start[t.n_groups] = (uint8_t)n;
+    return t;
+}
+
+// Lanes per (node, unit, group): the edges of a node are walked by one lane while that fills the chip (16 warps per
+// SM); smaller calls deal them to up to 8 lanes as long as each keeps about four edges.
+int split_of(int64_t n_nodes, int64_t n_edges, int units, int groups) {
+    int s = 0;
+    while (s < 3 && (n_nodes * units * groups << s) < (int64_t)sm_count() * 16 * 32 && n_edges >> (s + 3) >= n_nodes) ++s;
+    return s;
+}
+
+template <class T, int V> Args<T> args_of(const e3j_plan* plan, const Call<T>& c) {
+    Args<T> a{};
+    a.n_nodes = c.n_nodes; a.n_edges = c.n_edges; a.x = c.x; a.sh = c.sh; a.w = c.w; a.g = c.grad_out;
+    a.senders = c.senders; a.receivers = c.receivers; a.n_real = c.n_real;
+    a.d = plan->d; a.dp = plan->dp; a.P = plan->P; a.D = plan->D; a.units = plan->nq / V;
+    return a;
+}
+
+inline int64_t node_blocks(int64_t n_nodes, int units, int split, int groups, int threads) {
+    const int64_t items = n_nodes * units, per_block = threads >> split;
+    return (items + per_block - 1) / per_block * groups;
+}
+
+int largest_l(const e3j_plan* plan) {
+    int l = 1;
+    while ((l + 1) * (l + 1) < plan->dp) ++l;
+    for (const e3j_path_info_t& p : plan->paths) l = std::max({l, p.l1, p.l2, p.L});
+    return l;
+}
+
+template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, const Call<T>& c) {
+    const PathTable t = table_of(plan, false);
+    Args<T> a = args_of<T, V>(plan, c);
+    a.ptr = c.rowptr; a.out = c.out;
+    a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups);
+    const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
+    if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+    fwd_kernel<T, V, LM, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
+    return after_launch();
+}
+
+template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, const Call<T>& c) {
+    const PathTable t = table_of(plan, true);
+    Args<T> a = args_of<T, V>(plan, c);
+    a.ptr = c.colptr; a.perm = c.sender_perm; a.out = c.grad_x; a.grad_w = c.grad_w; a.grad_sh = c.grad_sh;
+    // block size: the multiple of 32 that leaves the fewest threads without an edge, the smaller of equals
+    int threads = kThreads, best = 0;
+    for (int b = 64; b <= kThreads; b += 32) {
+        const int used = 1024 * (b / a.units * a.units) / b;
+        if (used > best) { best = used; threads = b; }
+    }
+    int64_t nodes = 0, tiles = 0;
+    if (c.grad_x) {
+        a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups);
+        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
+    }
+    if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);
+    if (nodes + tiles == 0) return E3J_OK;
+    if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+    a.node_blocks = (unsigned)nodes;
+    bwd_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, 0, c.stream>>>(t, a);
+    return after_launch();
+}
+
+}  // namespace
+
+#define E3J_BY_LARGEST_L(f, T, V, IDENT)                  \
+    switch (largest_l(plan)) {                            \
+        case 1: return f<T, V, 1, IDENT>(plan, c);        \
+        case 2: return f<T, V, 2, IDENT>(plan, c);        \
+        default: return f<T, V, 3, IDENT>(plan, c);       \
+    }
+
+}  // namespace path
+}  // namespace e3j
