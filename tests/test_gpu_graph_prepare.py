@@ -1,0 +1,35 @@
+"""Graph preparation at the edges of its one-launch form (196 608 edges, 262 144 nodes), against numpy (GPU)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2609_35099_b200 as e3j
+
+pytestmark = pytest.mark.gpu
+
+
+# (nodes, edges, padding, nodes that send or receive): one edge; a list without padding and one of padding alone; runs
+# of thousands of empty rows before, between and behind; a block whose edges do not fit; the largest list and node
+# count of the form and the next
+@pytest.mark.parametrize("n,e,pad,used,hub", [
+    (1, 1, 0, 1, 0), (7, 40, 0, 7, 0), (7, 0, 5, 7, 0), (5000, 60, 13, 5000, 0), (70001, 33, 0, 3, 0),
+    (3000, 196608, 0, 3000, 0), (3000, 196609, 0, 3000, 0), (100, 20001, 3, 100, 0.5), (262144, 1000, 7, 262144, 0),
+    (262145, 1000, 7, 262145, 0)])
+def test_prepare_matches_numpy(n, e, pad, used, hub):
+    rng = np.random.default_rng(n + e)
+    ids = np.sort(rng.choice(n, used, replace=False))
+    rcv = np.sort(ids[rng.integers(0, used, e)]).astype(np.int32)
+    snd = ids[rng.integers(0, used, e)].astype(np.int32)
+    if e > 3000:
+        snd[: e // 50] = ids[1]    # a hub of some thousand edges
+    if hub:
+        snd[rng.random(e) < hub] = ids[2]    # more edges than a block collects
+    cuda = lambda a, fill: torch.from_numpy(np.concatenate([a, np.full(pad, fill, np.int32)])).cuda()
+    prepare = e3j.e3j_graph_prepare_padded if pad else e3j.e3j_graph_prepare
+    rowptr, perm, colptr = prepare(n, cuda(snd, n), cuda(rcv, n))
+    assert np.array_equal(rowptr.cpu().numpy(), np.searchsorted(rcv, np.arange(n + 1), side="left"))
+    assert np.array_equal(perm.cpu().numpy()[:e], np.argsort(snd, kind="stable"))
+    assert np.array_equal(colptr.cpu().numpy(), np.concatenate([[0], np.cumsum(np.bincount(snd, minlength=n))]))
+    only = prepare(n, cuda(snd, n), cuda(rcv, n), want_transpose=False)
+    assert torch.equal(only[0], rowptr) and only[1] is None
