@@ -1,4 +1,5 @@
 // Kernels shared by all signature-specialised entries.
+#include "../common.cuh"
 #include "fast_common.cuh"
 
 namespace e3j {
@@ -12,7 +13,7 @@ __global__ void fwd_fixup_kernel(int n_cta, int row_f4, const float4* __restrict
     if (b < 0) return;
     int last = c;
     while (last + 1 < n_cta && part_recv[2 * (last + 1)] == b) ++last;
-    for (int i = threadIdx.x; i < row_f4; i += blockDim.x) {
+    for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < row_f4; i += gridDim.y * blockDim.x) {
         float4 sum = partial[(size_t)(2 * c + 1) * row_f4 + i];
         for (int c2 = c + 1; c2 <= last; ++c2) {
             const float4 v = partial[(size_t)(2 * c2) * row_f4 + i];
@@ -35,42 +36,64 @@ __global__ void bounded_wait_selftest_kernel(uint32_t limit, int32_t* status, in
     if (threadIdx.x == 0) { result[0] = ok ? 1 : 0; result[1] = abort_flag; }
 }
 
-__global__ void bwd_zero_padding_kernel(const int32_t* __restrict__ n_real, int64_t n_edges, int w_row_f4,
-                                        int sh_row, float4* __restrict__ grad_w, float* __restrict__ grad_sh) {
-    const int64_t first = min((int64_t)*n_real, n_edges);
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t e = first + blockIdx.x; e < n_edges; e += gridDim.x) {
-        if (grad_w)
-            for (int i = threadIdx.x; i < w_row_f4; i += blockDim.x) grad_w[(size_t)e * w_row_f4 + i] = z;
-        if (grad_sh)
-            for (int i = threadIdx.x; i < sh_row; i += blockDim.x) grad_sh[(size_t)e * sh_row + i] = 0.f;
+namespace {
+__device__ __forceinline__ void zero_padding_rows(const ZeroPadding& z, int64_t block, int64_t n_blocks) {
+    const int64_t first = min((int64_t)*z.n_real, z.n_edges);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t e = first + block; e < z.n_edges; e += n_blocks) {
+        if (z.grad_w)
+            for (int i = threadIdx.x; i < z.w_row_f4; i += blockDim.x) z.grad_w[(size_t)e * z.w_row_f4 + i] = zero;
+        if (z.grad_sh)
+            for (int i = threadIdx.x; i < z.sh_row; i += blockDim.x) z.grad_sh[(size_t)e * z.sh_row + i] = 0.f;
     }
 }
+}  // namespace
+
+__global__ void bwd_zero_padding_kernel(ZeroPadding z) { zero_padding_rows(z, blockIdx.x, gridDim.x); }
 
 __global__ void bwd_dx_reduce_kernel(int64_t n_nodes, int row_f4, const float4* __restrict__ dx_edge,
                                      const int32_t* __restrict__ sender_perm, const int32_t* __restrict__ colptr,
-                                     float4* __restrict__ grad_x) {
-    grid_dependency_wait();
-    for (int64_t a = blockIdx.x; a < n_nodes; a += gridDim.x) {
-        const int j0 = colptr[a], j1 = colptr[a + 1];
-        for (int i = threadIdx.x; i < row_f4; i += blockDim.x) {
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            int j = j0;
-            // eight independent loads in flight; the additions stay in edge order
-            for (; j + 8 <= j1; j += 8) {
-                float4 v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = dx_edge[(size_t)sender_perm[j + u] * row_f4 + i];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) { acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w; }
-            }
-            for (; j < j1; ++j) {
-                const float4 v = dx_edge[(size_t)sender_perm[j] * row_f4 + i];
-                acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-            }
-            grad_x[(size_t)a * row_f4 + i] = acc;
-        }
+                                     float4* __restrict__ grad_x, ZeroPadding pad) {
+    extern __shared__ float4 part[];   // [groups - 1][row_f4]
+    if (blockIdx.x >= n_nodes) {       // padding rows: written by no other kernel, so there is nothing to wait for
+        zero_padding_rows(pad, blockIdx.x - n_nodes, gridDim.x - n_nodes);
+        return;
     }
+    const int64_t a = blockIdx.x;
+    const int groups = blockDim.x / row_f4, grp = threadIdx.x / row_f4, i = threadIdx.x - grp * row_f4;
+    const int b0 = colptr[a], n = colptr[a + 1] - b0, per = (n + groups - 1) / groups;
+    const int j0 = b0 + min(n, grp * per), j1 = b0 + min(n, (grp + 1) * per);
+    grid_dependency_wait();
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    // eight independent loads in flight; the additions stay in edge order
+    for (int j = j0; j < j1; j += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            v[u] = j + u < j1 ? dx_edge[(size_t)sender_perm[j + u] * row_f4 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w; }
+    }
+    if (grp > 0) part[(grp - 1) * row_f4 + i] = acc;
+    if (groups > 1) __syncthreads();
+    if (grp > 0) return;
+    for (int g = 0; g < groups - 1; ++g) {
+        const float4 v = part[g * row_f4 + i];
+        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+    grad_x[(size_t)a * row_f4 + i] = acc;
+}
+
+int launch_dx_reduce(int64_t n_nodes, int64_t n_edges, int row_f4, const float* dx_edge, const int32_t* sender_perm,
+                     const int32_t* colptr, float* grad_x, const ZeroPadding& pad, cudaStream_t st) {
+    int groups = 1;
+    while (groups < 8 && n_nodes * row_f4 * groups < (int64_t)sm_count() * 2048 && 2 * groups * row_f4 <= 1024 &&
+           n_edges >= n_nodes * groups * 12)
+        groups *= 2;
+    const int64_t blocks = n_nodes + (pad.n_real ? sm_count() * 4 : 0);
+    return launch_dependent(bwd_dx_reduce_kernel, dim3((unsigned)blocks), dim3(row_f4 * groups),
+                            sizeof(float4) * (groups - 1) * row_f4, st, n_nodes, row_f4,
+                            reinterpret_cast<const float4*>(dx_edge), sender_perm, colptr, reinterpret_cast<float4*>(grad_x), pad);
 }
 
 __global__ void bwd_rows_reduce_kernel(int64_t n_nodes, int row_f4, const float4* __restrict__ dx_rows,

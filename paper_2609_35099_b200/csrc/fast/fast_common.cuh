@@ -161,7 +161,7 @@ struct FwdParams {
     const float* ct_x; const float* ct_sh; const float* ct_w;
 };
 
-// Sums the pieces of every receiver row that was split between CTAs, in CTA order.
+// Sums the pieces of every receiver row that was split between CTAs, in CTA order (blockIdx.y: a part of the row).
 __global__ void fwd_fixup_kernel(int n_cta, int row_f4, const float4* __restrict__ partial,
                                  const int32_t* __restrict__ part_recv, float4* __restrict__ out);
 
@@ -181,17 +181,29 @@ __device__ __forceinline__ void cta_edge_range(const int64_t n_edges_host, const
     e_end = min(n_edges, e_begin + chunk);
 }
 
-// Backward of a padded call: zero rows of grad_w and grad_sh for the padding edges [*n_real, n_edges).
-__global__ void bwd_zero_padding_kernel(const int32_t* __restrict__ n_real, int64_t n_edges, int w_row_f4,
-                                        int sh_row, float4* __restrict__ grad_w, float* __restrict__ grad_sh);
+// Backward of a padded call: zero rows of grad_w and grad_sh for the padding edges [*n_real, n_edges).  n_real null:
+// the list has none.
+struct ZeroPadding {
+    const int32_t* n_real;
+    int64_t n_edges;
+    int w_row_f4, sh_row;
+    float4* grad_w;
+    float* grad_sh;
+};
+__global__ void bwd_zero_padding_kernel(ZeroPadding z);   // on its own where no grad_x is wanted
 
 // Self-test of the bounded wait (e3j_selftest_bounded_wait): one warp waits on a barrier that nobody arrives on.
 __global__ void bounded_wait_selftest_kernel(uint32_t limit, int32_t* status, int32_t* result);
 
-// Backward pass 2: grad_x[a] = sum of the per-edge shares of the edges sent by a, in edge order.
+// Backward pass 2: grad_x[a] = sum of the per-edge shares of the edges sent by a, in edge order.  One block per
+// sender, row_f4 * groups threads: with few senders its edges are dealt to `groups` runs whose sums are added in run
+// order (a run's loads are a chain of dependent latencies; 192 senders of 53 edges: 18 us with one run).  Further
+// blocks write the zero rows of padding edges.
 __global__ void bwd_dx_reduce_kernel(int64_t n_nodes, int row_f4, const float4* __restrict__ dx_edge,
                                      const int32_t* __restrict__ sender_perm, const int32_t* __restrict__ colptr,
-                                     float4* __restrict__ grad_x);
+                                     float4* __restrict__ grad_x, ZeroPadding pad);
+int launch_dx_reduce(int64_t n_nodes, int64_t n_edges, int row_f4, const float* dx_edge, const int32_t* sender_perm,
+                     const int32_t* colptr, float* grad_x, const ZeroPadding& pad, cudaStream_t st);
 
 }  // namespace fast
 }  // namespace e3j

@@ -52,7 +52,7 @@ int launch_fwd(const ConvArgs& a) {
     constexpr int threads = (S::FW * (S::NQ / (32 * S::V)) + 2) * 32;  // consumers + two producer warps
     fast_fwd_kernel<S><<<n_cta, threads, L::total, a.stream>>>(p);
     if (int s = after_launch()) return s;
-    return launch_dependent(fwd_fixup_kernel, dim3(n_cta), dim3(256), 0, a.stream, n_cta, S::D * S::NQ / 4, reinterpret_cast<const float4*>(p.partial),
+    return launch_dependent(fwd_fixup_kernel, dim3(n_cta, 4), dim3(256), 0, a.stream, n_cta, S::D * S::NQ / 4, reinterpret_cast<const float4*>(p.partial),
                                                  p.part_recv, reinterpret_cast<float4*>(a.out));
 }
 
@@ -153,16 +153,15 @@ int launch_bwd(const ConvArgs& a) {
         fast_bwd_kernel<S><<<n_cta, threads, L::total, a.stream>>>(p);
     }
     if (int s = after_launch()) return s;
-    if (a.n_real) {
-        bwd_zero_padding_kernel<<<sm_count() * 8, 256, 0, a.stream>>>(a.n_real, a.n_edges, S::P * S::NQ / 4, S::DSH,
-                                                              reinterpret_cast<float4*>(a.grad_w), a.grad_sh);
-        if (int s = after_launch()) return s;
+    ZeroPadding pad{};
+    if (a.n_real) pad = {a.n_real, a.n_edges, S::P * S::NQ / 4, S::DSH, reinterpret_cast<float4*>(a.grad_w), a.grad_sh};
+    if (!a.grad_x) {   // the shares stay in the scratch
+        if (!a.n_real) return E3J_OK;
+        bwd_zero_padding_kernel<<<sm_count() * 8, 256, 0, a.stream>>>(pad);
+        return after_launch();
     }
-    if (!a.grad_x) return E3J_OK;   // the shares stay in the scratch
-    // one CTA per sender: the hardware hands them out as CTAs finish, so uneven degrees do not leave a tail
-    const int64_t blocks = std::min<int64_t>(a.n_nodes, (int64_t)1 << 30);
-    return launch_dependent(bwd_dx_reduce_kernel, dim3((int)blocks), dim3(S::DIN * S::NQ / 4), 0, a.stream, a.n_nodes, S::DIN * S::NQ / 4,
-        reinterpret_cast<const float4*>(p.dx_edge), a.sender_perm, a.colptr, reinterpret_cast<float4*>(a.grad_x));
+    return launch_dx_reduce(a.n_nodes, a.n_edges, S::DIN * S::NQ / 4, p.dx_edge, a.sender_perm, a.colptr, a.grad_x, pad,
+                            a.stream);
 }
 
 // Fused double backward, edge outputs: the edge-wise sweep over (x, sh, w) and their cotangents, then the
@@ -191,9 +190,8 @@ int launch_dbl_edges(const ConvArgs& a, const float* ct_x, const float* ct_sh, c
     }
     fast_bwd1_kernel<S, false, true><<<n_cta, (L1::T * L1::CH + 1) * 32, L1::total, a.stream>>>(p);
     if (int s = after_launch()) return s;
-    const int64_t blocks = std::min<int64_t>(a.n_nodes, (int64_t)1 << 30);
-    return launch_dependent(bwd_dx_reduce_kernel, dim3((int)blocks), dim3(S::DIN * S::NQ / 4), 0, a.stream, a.n_nodes, S::DIN * S::NQ / 4,
-        reinterpret_cast<const float4*>(p.dx_edge), a.sender_perm, a.colptr, reinterpret_cast<float4*>(a.grad_x));
+    return launch_dx_reduce(a.n_nodes, a.n_edges, S::DIN * S::NQ / 4, p.dx_edge, a.sender_perm, a.colptr, a.grad_x,
+                            ZeroPadding{}, a.stream);
 }
 
 // Fused double backward, cotangent of grad_out: the forward sweep with two terms per coefficient pair, written
@@ -225,7 +223,7 @@ int launch_dbl_out(const ConvArgs& a, const float* ct_x, const float* ct_sh, con
     constexpr int threads = (L::NCONS + 2) * 32;  // consumers + two producer warps
     fast_fwd_kernel<S, true><<<n_cta, threads, L::total, a.stream>>>(p);
     if (int s = after_launch()) return s;
-    return launch_dependent(fwd_fixup_kernel, dim3(n_cta), dim3(256), 0, a.stream, n_cta, S::D * S::NQ / 4, reinterpret_cast<const float4*>(p.partial),
+    return launch_dependent(fwd_fixup_kernel, dim3(n_cta, 4), dim3(256), 0, a.stream, n_cta, S::D * S::NQ / 4, reinterpret_cast<const float4*>(p.partial),
                                                  p.part_recv, reinterpret_cast<float4*>(a.out));
 }
 
