@@ -238,34 +238,42 @@ def e3j_plan_records(plan: Plan):
 
 
 # ----------------------------------------------------------------- marshalling
+# A call's arguments are checked and converted in a few microseconds: with small graphs that is what a call costs.
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _dev_ptr(t, dtype, shape, name):
-    torch = _torch()
+    """Device address of a contiguous CUDA tensor of that type (and shape, if given); None stays None."""
     if t is None:
         return None
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype or not t.is_contiguous():
         raise TypeError(f"{name} must be contiguous {dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream):
-    torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    c = _torch()._C
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())   # torch.cuda.current_stream() without building the object
 
 
 def _workspace(nbytes: int, like, workspace):
     torch = _torch()
     if workspace is None:
-        workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=like.device)
+        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=like.device)
     if workspace.dtype != torch.uint8 or not workspace.is_cuda or workspace.numel() < nbytes:
         raise ValueError("workspace must be a CUDA uint8 tensor of sufficient size")
     return workspace
@@ -333,7 +341,7 @@ def e3j_conv_fwd(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=None
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), _entry)
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), _entry)
     return out
 
 
@@ -401,7 +409,7 @@ def e3j_conv_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr=None
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"),
         _dev_ptr(grad_sh, f32, (e, plan.d_sh), "grad_sh"),
         _dev_ptr(grad_w, f32, (e, plan.n_paths, plan.n_channels), "grad_w"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), _entry)
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), _entry)
     return grad_x, grad_sh, grad_w
 
 
@@ -444,7 +452,7 @@ def e3j_conv_bwd_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr,
         _dev_ptr(ct_x, f32, s_x, "ct_x"), _dev_ptr(ct_sh, f32, s_sh, "ct_sh"), _dev_ptr(ct_w, f32, s_w, "ct_w"),
         _dev_ptr(gg_out, f32, s_out, "gg_out"), _dev_ptr(g_x, f32, s_x, "g_x"), _dev_ptr(g_sh, f32, s_sh, "g_sh"),
         _dev_ptr(g_w, f32, s_w, "g_w"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_bwd_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_bwd_bwd")
     return gg_out, g_x, g_sh, g_w
 
 
@@ -486,7 +494,7 @@ def e3j_conv_radial_fwd(plan: Plan, x, sh, h, W, senders, receivers, rowptr=None
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_radial_fwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_fwd")
     return out
 
 
@@ -511,7 +519,7 @@ def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, r
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_radial_vec_fwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_vec_fwd")
     return out
 
 
@@ -546,7 +554,7 @@ def e3j_conv_radial_bwd(plan: Plan, x, sh, h, W, senders, receivers, grad_out, r
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"),
         _dev_ptr(grad_sh, f32, (e, plan.d_sh), "grad_sh"),
         _dev_ptr(grad_h, f32, (e, hidden), "grad_h"), _dev_ptr(grad_W, f32, s_w, "grad_W"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_radial_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_bwd")
     return grad_x, grad_sh, grad_h, grad_W
 
 
@@ -584,7 +592,7 @@ def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, g
         _dev_ptr(grad_out, f32, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"), _dev_ptr(grad_vec, f32, (e, 3), "grad_vec"),
         _dev_ptr(grad_h, f32, (e, hidden), "grad_h"), _dev_ptr(grad_W, f32, s_w, "grad_W"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_radial_vec_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_vec_bwd")
     return grad_x, grad_vec, grad_h, grad_W
 
 
@@ -664,11 +672,11 @@ def e3j_conv_bwd_scheduled(plan: Plan, x, sh, w, schedule, grad_out, grad_x=None
         raise ValueError("schedule must be the CUDA uint8 tensor returned by e3j_bwd_schedule_build")
     _check(_load().e3j_conv_bwd_scheduled(
         plan.handle, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
-        _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"), ctypes.c_void_p(schedule.data_ptr()),
+        _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"), schedule.data_ptr(),
         _dev_ptr(grad_out, f32, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"), _dev_ptr(grad_sh, f32, (e, plan.d_sh), "grad_sh"),
         _dev_ptr(grad_w, f32, (e, plan.n_paths, plan.n_channels), "grad_w"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_bwd_scheduled")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_bwd_scheduled")
     return grad_x, grad_sh, grad_w
 
 
@@ -717,7 +725,7 @@ def e3j_conv_vec_fwd(plan: Plan, x, edge_vec, w, senders, receivers, rowptr=None
         _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"), _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"), _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_vec_fwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_vec_fwd")
     return out
 
 
@@ -746,7 +754,7 @@ def e3j_conv_vec_bwd(plan: Plan, x, edge_vec, w, senders, receivers, grad_out, r
         _dev_ptr(grad_out, f32, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"), _dev_ptr(grad_vec, f32, (e, 3), "grad_vec"),
         _dev_ptr(grad_w, f32, (e, plan.n_paths, plan.n_channels), "grad_w"),
-        ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream(stream)), "e3j_conv_vec_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_vec_bwd")
     return grad_x, grad_vec, grad_w
 
 
@@ -761,7 +769,7 @@ def e3j_conv_fwd_f64(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=
         plan.handle, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f64, (e, plan.n_paths, plan.n_channels), "w"), _dev_ptr(senders, i32, (e,), "senders"),
         _dev_ptr(receivers, i32, (e,), "receivers"), _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
-        _dev_ptr(out, f64, (n, plan.d_out, plan.n_channels), "out"), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+        _dev_ptr(out, f64, (n, plan.d_out, plan.n_channels), "out"), ws.data_ptr(), ws.numel(),
         _stream(stream)), "e3j_conv_fwd_f64")
     return out
 
@@ -780,7 +788,7 @@ def e3j_conv_bwd_f64(plan: Plan, x, sh, w, senders, receivers, grad_out, sender_
         _dev_ptr(receivers, i32, (e,), "receivers"), _dev_ptr(sender_perm, i32, (e,), "sender_perm"),
         _dev_ptr(colptr, i32, (n + 1,), "colptr"), _dev_ptr(grad_out, f64, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(gx, f64, None, "grad_x"), _dev_ptr(gsh, f64, None, "grad_sh"), _dev_ptr(gw, f64, None, "grad_w"),
-        ctypes.c_void_p(ws.data_ptr()), ws.numel(), _stream(stream)), "e3j_conv_bwd_f64")
+        ws.data_ptr(), ws.numel(), _stream(stream)), "e3j_conv_bwd_f64")
     return gx, gsh, gw
 
 
@@ -799,7 +807,7 @@ def e3j_shard_prepare(n_nodes: int, node_lo: int, node_hi: int, senders, receive
     _check(_load().e3j_shard_prepare(n_nodes, e, node_lo, node_hi, _dev_ptr(senders, i32, (e,), "senders"),
                                      _dev_ptr(receivers, i32, (e,), "receivers"), _dev_ptr(ls, i32, None, "local_senders"),
                                      _dev_ptr(lr, i32, None, "local_receivers"), _dev_ptr(halo, i32, None, "halo_ids"),
-                                     _dev_ptr(count, i32, None, "n_halo"), ctypes.c_void_p(ws.data_ptr()), ws.numel(),
+                                     _dev_ptr(count, i32, None, "n_halo"), ws.data_ptr(), ws.numel(),
                                      _stream(stream)), "e3j_shard_prepare")
     return ls[:e], lr[:e], halo[:int(count.item())]
 
