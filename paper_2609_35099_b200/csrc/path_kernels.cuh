@@ -11,11 +11,11 @@
 //   edge part  (grad_w, grad_sh): one thread owns V channels of one edge and walks all paths; grad_sh's channel sum
 //              goes through shared memory in a fixed order.
 //
-// What bounds them: the latency of the row loads at 18 to 20 warps per SM (issue slots 30-40 % busy, DRAM below 20 %),
-// not arithmetic or bandwidth.  48x(0e+1o+2e), l <= 2, 35050 edges: forward 243 -> 99 us, backward 823 -> 189 us
-// against the table-driven kernels; float64, 64x(0e+1o), l <= 2, 10176 edges, both passes: 705 -> 131 us.  Tried and
-// slower: weights and ids two steps ahead (spills, 378 against 284 us for both passes), each path's sum as a function
-// of its own, grad_out rows of the next path prefetched.
+// What bounds them: the latency of the row loads at 20 to 28 warps per SM (issue slots 30-40 % busy, DRAM below 20 %),
+// not arithmetic or bandwidth.  48x(0e+1o+2e), l <= 2, 35050 edges: forward 243 -> 71 us, backward 823 -> 179 us
+// against the table-driven kernels; float64, 64x(0e+1o), l <= 2, 10176 edges, both passes: 705 -> 105 us.  Tried and
+// slower: weights and ids two steps ahead in registers (spills, 378 against 284 us for both passes), each path's sum
+// as a function of its own, grad_out rows of the next path in registers.
 //
 // Same sums as the table-driven kernels, in a fixed order, no atomics.  What stays on the table-driven ones: plans
 // with l > 3, more than 128 V-channel units, and (float64) odd channel counts or pointers off 16 bytes.
@@ -117,6 +117,24 @@ template <class T> struct Args {
     int split_log2;              // a node's edges are dealt to 2^split_log2 lanes
     unsigned node_blocks;        // backward: blocks below this one are node sums, the others edge tiles
 };
+
+// ---------------------------------------------------------------- staging
+// In the edge part every lane copies its own rows into its own columns of a ring in shared memory (cp.async) two paths
+// before it uses them: the loads in flight cost no registers, and no lane waits for another one (106 -> 89 us on the
+// workload above).  The node sums keep plain loads: their copies are scattered over rows of many nodes, which the copy
+// path takes at half the rate (99 -> 148 us).
+constexpr int kStages = 3;
+template <int BYTES> __device__ __forceinline__ void copy_async(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT> __device__ __forceinline__ void copies_wait() {
+    asm volatile("cp.async.wait_group %0;" :: "n"(LEFT) : "memory");
+}
+// A stage of one warp: up to 2 LM + 2 rows of one Pack per lane.
+template <int LM> constexpr int stage_bytes() { return (2 * LM + 2) * 512; }
+template <int LM> constexpr int ring_bytes() { return kStages * stage_bytes<LM>(); }
 
 // ---------------------------------------------------------------- node sums
 // One path's share of a node's rows: summed over the lane's edges, then over the lanes that share the node, and
@@ -228,7 +246,7 @@ __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, 
 
 // ---------------------------------------------------------------- edge part
 template <class T, int V, int LM, bool IDENT>
-__device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, const unsigned tile, T* part) {
+__device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, const unsigned tile, unsigned char* smem) {
     const int slots = blockDim.x / a.units, slot = threadIdx.x / a.units, q = threadIdx.x - slot * a.units;
     const int64_t e = (int64_t)tile * slots + slot;
     const int64_t n_live = a.n_real ? min((int64_t)*a.n_real, a.n_edges) : a.n_edges;
@@ -243,13 +261,27 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
         const T* xe = a.x + (size_t)from * a.d * row + q * V;
         const T* ge = a.g + (size_t)to * a.D * row + q * V;
         const T* we = a.w + (size_t)e * a.P * row + q * V;
-        T x[2 * LM + 1][V], s1[V];   // s1: the next path's weights
+        unsigned char* ring = smem + (threadIdx.x >> 5) * ring_bytes<LM>() + (threadIdx.x & 31) * 16;
+        auto copy = [&](int p, int stage) {   // a path's weights and grad_out rows
+            if (p < t.n_paths) {
+                const PathRec rec = t.rec[p];
+                unsigned char* at = ring + stage * stage_bytes<LM>();
+                copy_async<16>(at, we + (size_t)rec.k * row);
+                const T* gk = ge + (size_t)rec.out_off * row;
+#pragma unroll
+                for (int i = 0; i < 2 * LM + 1; ++i)
+                    if (i < 2 * rec.L + 1) copy_async<16>(at + (1 + i) * 512, gk + (size_t)i * row);
+            }
+            copies_commit();
+        };
+        T x[2 * LM + 1][V];
 #pragma unroll
         for (int i = 0; i < 2 * LM + 1; ++i)
 #pragma unroll
             for (int c = 0; c < V; ++c) x[i][c] = T(0);
-        int have = -1;
-        load_pack<T, V>(s1, we + (size_t)t.rec[0].k * row);
+        int have = -1, stage = 0;
+        copy(0, 0);
+        copy(1, 1);
 #pragma unroll 1
         for (int p = 0; p < t.n_paths; ++p) {
             const PathRec rec = t.rec[p];
@@ -259,18 +291,20 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
                 for (int i = 0; i < 2 * LM + 1; ++i)
                     if (i < 2 * rec.l1 + 1) load_pack<T, V>(x[i], xe + (size_t)(rec.x_off + i) * row);
             }
+            copies_wait<1>();
+            copy(p + 2, stage == 0 ? 2 : stage - 1);
+            const unsigned char* at = ring + stage * stage_bytes<LM>();
+            stage = stage == 2 ? 0 : stage + 1;
             T s[V], dw[V];
+            load_pack<T, V>(s, reinterpret_cast<const T*>(at));
 #pragma unroll
-            for (int c = 0; c < V; ++c) { s[c] = s1[c]; dw[c] = T(0); }
-            if (p + 1 < t.n_paths) load_pack<T, V>(s1, we + (size_t)t.rec[p + 1].k * row);
-            const T* gk = ge + (size_t)rec.out_off * row;
-            int row_p = row;
-            asm volatile("" : "+r"(row_p));   // as in node_part
+            for (int c = 0; c < V; ++c) dw[c] = T(0);
             switch (rec.id) {
 #define E3J_CASE(l1, l2, L) \
                 case E3J_TRI_ID(l1, l2, L): if constexpr (l1 <= LM && l2 <= LM && L <= LM) { \
                     T g[2 * L + 1][V]; \
-                    _Pragma("unroll") for (int i = 0; i < 2 * L + 1; ++i) load_pack<T, V>(g[i], gk + (size_t)i * row_p); \
+                    _Pragma("unroll") for (int i = 0; i < 2 * L + 1; ++i) \
+                        load_pack<T, V>(g[i], reinterpret_cast<const T*>(at + (1 + i) * 512)); \
                     Tri<l1, l2, L>::template edge<T, V>(y + l2 * l2, dy + l2 * l2, x, s, g, dw); \
                 } break;
                 E3J_PATH_TRIPLES(E3J_CASE)
@@ -285,6 +319,9 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
         for (int k = 0; k < a.P; ++k) store_pack<T, V>(a.grad_w + ((size_t)e * a.P + k) * row + q * V, z);
     }
     if (!a.grad_sh) return;
+    copies_wait<0>();
+    __syncthreads();   // the rings are free: the partials take their place
+    T* part = reinterpret_cast<T*>(smem);
     // channel sum: eight lanes per (edge, component) add every eighth partial, then a fixed tree over the eight
 #pragma unroll
     for (int i = 0; i < NY; ++i)
@@ -304,23 +341,37 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
     }
 }
 
-// LM: the plan's largest l.  It sets the registers of a thread (an edge's input rows, harmonics and grad_out rows),
-// and with them the warps that hide the loads' latency: 4, 5 or 6 blocks of 128 threads per SM for LM = 3, 2, 1.
+// LM: the plan's largest l.  It sets the registers of a thread (an edge's input rows, harmonics and grad_out rows) and
+// with them the blocks of an SM.  Measured for 4 to 7 blocks at LM = 2: the forward gains from more warps although a
+// few values spill (99 / 95 / 71 us with 5 / 6 / 7 blocks), the backward does not (179 / 186 / 214 us).
 constexpr int kThreads = 128;
-constexpr int blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 5 : 6; }
+constexpr int fwd_blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 7 : 8; }
+constexpr int bwd_blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 5 : 8; }
+template <int LM> constexpr int smem_bytes(int threads) { return threads / 32 * ring_bytes<LM>(); }
 
-template <class T, int V, int LM, bool IDENT>
-__global__ void __launch_bounds__(kThreads, blocks_per_sm(LM))
-fwd_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
-    node_part<T, V, LM, false, IDENT>(t, a, blockIdx.x);
+// TR: the forward's sums, or grad_x on its own.
+template <class T, int V, int LM, bool TR, bool IDENT>
+__global__ void __launch_bounds__(kThreads, fwd_blocks_per_sm(LM))
+node_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
+    node_part<T, V, LM, TR, IDENT>(t, a, blockIdx.x);
 }
 
+// Edge tiles, and up to l = 2 the node sums of grad_x in the same launch (48x(0e+1o+2e), l <= 2: 180 us against 205 us
+// one after the other).  With l = 3 the two parts' code together is too much for the instruction cache (16x(0e+1o+2e+3o),
+// 35050 edges: 338 to 431 us against 264 us), so grad_x has its own launch.
+constexpr bool one_launch(int lm) { return lm < 3; }
 template <class T, int V, int LM, bool IDENT>
-__global__ void __launch_bounds__(kThreads, blocks_per_sm(LM))
+__global__ void __launch_bounds__(kThreads, bwd_blocks_per_sm(LM))
 bwd_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
-    __shared__ T part[(LM + 1) * (LM + 1) * kThreads];
-    if (blockIdx.x < a.node_blocks) node_part<T, V, LM, true, IDENT>(t, a, blockIdx.x);
-    else edge_part<T, V, LM, IDENT>(t, a, blockIdx.x - a.node_blocks, part);
+    extern __shared__ __align__(16) unsigned char smem[];
+    static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");
+    if constexpr (one_launch(LM)) {
+        if (blockIdx.x < a.node_blocks) {
+            node_part<T, V, LM, true, IDENT>(t, a, blockIdx.x);
+            return;
+        }
+    }
+    edge_part<T, V, LM, IDENT>(t, a, blockIdx.x - a.node_blocks, smem);
 }
 
 }  // namespace path

@@ -48,11 +48,14 @@ PathTable table_of(const e3j_plan* plan, bool by_input) {
     return t;
 }
 
-// Lanes per (node, unit, group): the edges of a node are walked by one lane while that fills the chip (16 warps per
-// SM); smaller calls deal them to up to 8 lanes as long as each keeps about four edges.
-int split_of(int64_t n_nodes, int64_t n_edges, int units, int groups) {
+// Lanes per (node, unit, group): the edges of a node are walked by one lane while that fills the chip (`warps` per
+// SM); smaller calls deal them to up to 8 lanes as long as each keeps about four edges.  The forward wants two lanes
+// sooner (32 warps: 79 us against 99 us with 16 on the workload of path_kernels.cuh), the backward, whose node sums
+// share the SMs with the edge tiles, does not (190 against 179 us).
+constexpr int kFwdWarps = 32, kBwdWarps = 16;
+int split_of(int64_t n_nodes, int64_t n_edges, int units, int groups, int warps) {
     int s = 0;
-    while (s < 3 && (n_nodes * units * groups << s) < (int64_t)sm_count() * 16 * 32 && n_edges >> (s + 3) >= n_nodes) ++s;
+    while (s < 3 && (n_nodes * units * groups << s) < (int64_t)sm_count() * warps * 32 && n_edges >> (s + 3) >= n_nodes) ++s;
     return s;
 }
 
@@ -76,14 +79,20 @@ int largest_l(const e3j_plan* plan) {
     return l;
 }
 
+template <int LM, class K> int allow_smem(K kernel) {
+    constexpr int bytes = smem_bytes<LM>(kThreads);
+    if (bytes <= 48 * 1024) return E3J_OK;
+    return cuda_status(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+}
+
 template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, const Call<T>& c) {
     const PathTable t = table_of(plan, false);
     Args<T> a = args_of<T, V>(plan, c);
     a.ptr = c.rowptr; a.out = c.out;
-    a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups);
+    a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups, kFwdWarps);
     const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
-    fwd_kernel<T, V, LM, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
+    node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
     return after_launch();
 }
 
@@ -99,14 +108,21 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     }
     int64_t nodes = 0, tiles = 0;
     if (c.grad_x) {
-        a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups);
-        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
+        a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups, one_launch(LM) ? kBwdWarps : kFwdWarps);
+        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, one_launch(LM) ? threads : kThreads);
     }
     if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);
-    if (nodes + tiles == 0) return E3J_OK;
     if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+    if (nodes > 0 && (!one_launch(LM) || tiles == 0)) {
+        if (one_launch(LM)) nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
+        node_kernel<T, V, LM, true, IDENT><<<(unsigned)nodes, kThreads, 0, c.stream>>>(t, a);
+        if (int s = after_launch()) return s;
+        nodes = 0;
+    }
+    if (nodes + tiles == 0) return E3J_OK;
     a.node_blocks = (unsigned)nodes;
-    bwd_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, 0, c.stream>>>(t, a);
+    if (int s = allow_smem<LM>(bwd_kernel<T, V, LM, IDENT>)) return s;
+    bwd_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
     return after_launch();
 }
 
