@@ -81,13 +81,12 @@ enum {
  * that land on the same (L, p) share one output block, out[b, block(L,p) + M, q] = sum over those paths of
  * w[e, path, q] * (...), so D = sum over distinct (L, p) of (2L + 1) while the weights stay one block per
  * path.  out_off of e3j_path_info_t is then the same for the paths of a block.  Such plans use generated
- * kernels where a collapsed signature has been generated (the water-box signature), the table-driven kernels
- * otherwise. */
+ * kernels where a collapsed signature has been generated (the water-box signature), the kernels of plans without
+ * generated ones otherwise. */
 #define E3J_PLAN_COLLAPSE_OUTPUTS 2u
 /* e3j_conv_radial_fwd / e3j_conv_radial_vec_fwd take the two-step form (edge weights written to the workspace by the
- * tensor-core product, then the plain forward) even where the plan has the kernel that forms them itself: faster
- * where the [n_edges, P, N_q] array fits in memory (bench workload: 0.49 against 0.71 ms), at the price of that
- * array in the workspace. */
+ * tensor-core product, then the plain forward) whatever the size of the [n_edges, P, N_q] array; without the flag they
+ * do so up to 2 GiB (160 900 edges: 0.49 against 0.69 ms) and form the weights inside the kernel beyond. */
 #define E3J_PLAN_RADIAL_MATERIALISE 4u
 
 typedef struct e3j_plan e3j_plan; /* opaque; immutable after creation; usable from several streams */
@@ -280,7 +279,9 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
  *   hidden must be a multiple of 4; h, W, grad_h, grad_W 16-byte aligned; rowptr / sender_perm / colptr as for
  *   e3j_conv_fwd / e3j_conv_bwd; any of grad_x, grad_sh, grad_h, grad_W may be NULL.
  *   Workspace: 256-byte aligned, at least e3j_conv_radial_*_workspace_bytes(); calls that overlap on the GPU
- *   must not share it.
+ *   must not share it.  The forward forms the weight array in its workspace while the array is no larger than 2 GiB
+ *   (faster) and forms the weights inside the convolution kernel beyond that, where the plan has such a kernel; it also
+ *   does so when the workspace has no room for the array, and refuses only a workspace that holds neither form.
  *   The two gradient products fetch their operands through tensor maps (tiled bulk copies); a driver that has no
  *   encoder for them (cuTensorMapEncodeTiled, CUDA 12) makes the backward return E3J_ERR_UNSUPPORTED.
  * e3j_radial_weights writes the product itself, w_out [n_edges, P, N_q] (for callers that want the weights, and

@@ -504,8 +504,8 @@ def e3j_conv_radial_vec_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: i
 
 def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, rowptr=None, out=None, workspace=None,
                             stream=None):
-    """Forward convolution from edge vectors [E, 3] and the radial layer (h, W): neither the harmonics nor the
-    edge weights exist as arrays where the plan has the kernel for it."""
+    """Forward convolution from edge vectors [E, 3] and the radial layer (h, W): where the plan has the kernels for it
+    the harmonics never exist as an array, nor do the edge weights once they would take more than 2 GiB."""
     torch = _torch()
     n, e, hidden = x.shape[0], senders.numel(), W.shape[0]
     f32, i32 = torch.float32, torch.int32

@@ -274,3 +274,35 @@ def test_radial_calls_can_be_captured_in_a_cuda_graph():
     for a, b in zip(eager, (out, *grads)):
         assert torch.equal(a, b)
     assert e3j.e3j_plan_device_status(plan) == 0
+
+
+@pytest.mark.parametrize("n_atoms,hidden", [(192, 64), (648, 8)])
+def test_a_workspace_without_room_for_the_weights_gets_the_in_kernel_form(n_atoms, hidden):
+    """The C entry points take any workspace that holds one of the two forms: with room for the [E, P, N_q] array they
+    form it, with less they form the scalars inside the kernel, with too little for that they refuse.  Both forms give
+    the same output to rounding (1e-5 of the largest value, the bound of the other parity tests)."""
+    wl = workloads.make_graph(2, n_atoms)
+    plan = e3j.e3j_plan_create("128x0e+128x1o", 3, None, 3)
+    gen = torch.Generator(device="cuda").manual_seed(n_atoms)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda")
+    n, e, lib = wl.n_nodes, wl.n_edges, e3j._load()
+    snd, rcv = torch.from_numpy(wl.senders).cuda(), torch.from_numpy(wl.receivers).cuda()
+    rowptr = e3j.e3j_graph_prepare(n, snd, rcv)[0]
+    x, vec = draw(n, plan.d_in, 128), draw(e, 3)
+    h, W = draw(e, hidden), draw(hidden, plan.n_paths * 128) / hidden ** 0.5
+    full = e3j.e3j_conv_radial_vec_fwd_workspace_bytes(plan, n, e, hidden)
+    weights = 4 * e * plan.n_paths * 128
+
+    def call(nbytes):
+        out, ws = torch.full((n, plan.d_out, 128), float("nan"), device="cuda"), torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        status = lib.e3j_conv_radial_vec_fwd(plan.handle, n, e, hidden, *(t.data_ptr() for t in (x, vec, h, W, snd, rcv, rowptr, out, ws)),
+                                             nbytes, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        return status, out
+
+    assert full > weights
+    (s0, materialised), (s1, in_kernel), (s2, _) = call(full), call(full - weights // 2), call(256)
+    assert (s0, s1, s2) == (e3j.E3J_OK, e3j.E3J_OK, e3j.E3J_ERR_WORKSPACE)
+    assert e3j.e3j_plan_device_status(plan) == 0
+    assert not torch.equal(materialised, in_kernel)   # two kernels, not one
+    assert (materialised - in_kernel).abs().max() < 1e-5 * materialised.abs().max()
