@@ -328,9 +328,9 @@ def main():
     ap.add_argument("--config", type=int, default=2, choices=[2, 3, 4, 5],
                     help="2 = headline workload; 3 / 5 = other convolution workloads; 4 = standalone tensor product rows")
     ap.add_argument("--rows", type=int, default=1 << 20, help="rows of the tensor-product workload (--config 4)")
-    ap.add_argument("--generic", action="store_true", help="force the table-driven generic kernels")
+    ap.add_argument("--generic", action="store_true", help="force the kernels of plans without generated ones")
     ap.add_argument("--collapse", action="store_true",
-                    help="plan with collapsed output multiplicities (table-driven kernels; no CPU leg)")
+                    help="plan with collapsed output multiplicities (generated or per-path kernels; no CPU leg)")
     ap.add_argument("--pad", type=float, default=0.0,
                     help="append this fraction of padding edges and call the padded entry points (rates count real edges)")
     ap.add_argument("--double-backward", action="store_true", help="(default for configs 2 and 3; kept for old command lines)")
@@ -783,7 +783,7 @@ def main():
 
         spec = bool(plan.specialised)
         roofs = {"fwd": roof(fb, f_ms, "e3j_conv_fwd call: fast_fwd_kernel (97 %) + fwd_fixup_kernel" if spec
-                             else "e3j_conv_fwd call: generic conv_fwd_kernel", "fwd"),
+                             else "e3j_conv_fwd call: path::node_kernel", "fwd"),
                  "bwd": roof(bb, b_ms, "e3j_conv_bwd call: fast_bwd1_kernel (89 %) + bwd_dx_reduce_kernel" if spec
                              else "e3j_conv_bwd call: generic edge + node kernels", "bwd")}
         dominant = roofs["bwd"] if b_ms >= f_ms else roofs["fwd"]

@@ -759,7 +759,7 @@ def e3j_conv_vec_bwd(plan: Plan, x, edge_vec, w, senders, receivers, grad_out, r
 
 
 def e3j_conv_fwd_f64(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=None, stream=None):
-    """Float64 forward convolution (table-driven kernels)."""
+    """Float64 forward convolution (per-path kernels; odd channel counts and l > 3 on table-driven ones)."""
     torch = _torch()
     n, e, f64, i32 = x.shape[0], senders.numel(), torch.float64, torch.int32
     if out is None:

@@ -1,9 +1,9 @@
 // Float64 entry points (the paper ships float64 builds of its kernels beside the float32 ones).
 //
-// Table-driven kernels in double precision, for any plan: every output element is owned by one thread and is the
-// defining sum in a fixed order (edges in list order, records in table order), with the coefficient values kept
-// in float64 as the plan builder computed them.  They are the float64 counterpart of generic_kernels.cuh, one
-// channel per thread; there are no signature-specialised float64 kernels.
+// Plans and arrays that the per-path kernels take (path_kernels.cuh: l <= 3, an even number of channels, arrays on 16
+// bytes) run on those.  The table-driven kernels here take the rest: every output element is owned by one thread and is
+// the defining sum in a fixed order (edges in list order, records in table order), with the coefficient values kept in
+// float64 as the plan builder computed them, one channel per thread.
 #include <initializer_list>
 
 #include "common.cuh"

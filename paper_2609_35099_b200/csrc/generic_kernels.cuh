@@ -5,8 +5,8 @@
 // atomics.  This is the paper's "transposed record sets" formulation (section
 // "Differentiation": for dx the records are sorted by i1, for dy by i2): every
 // cotangent is a gather with its own sorted copy of the coefficient records.
-// They are the fallback for signatures that have no specialised kernel and the
-// on-device cross-check for the specialised ones.
+// They take the plans that neither generated kernels nor the per-path kernels
+// (path_kernels.cuh) cover: l > 3, or more than 512 channels.
 #pragma once
 #include "common.cuh"
 

@@ -313,15 +313,18 @@ prepare_one_kernel(int64_t n_nodes, int64_t n_edges, const int32_t* __restrict__
         if (s >= a0 && s < a0 + own) perm[base + m.start[s - a0] + atomicAdd(&m.of[s - a0], 1)] = (int32_t)e;
     });
     __syncthreads();
-    static_assert(2 * kOneCap >= kOneWarps * 512, "the collected edges' arrays serve as staging");
+    static_assert(4 * kOneCap == kOneWarps * kRankMax, "the collected edges' four arrays serve as staging");
     for (int i = warp; i < own; i += kOneWarps)
-        sort_bucket<512>(perm + base + m.start[i], m.start[i + 1] - m.start[i], m.edge + 512 * warp);
+        sort_bucket<kRankMax>(perm + base + m.start[i], m.start[i + 1] - m.start[i],
+                              reinterpret_cast<int32_t*>(raw) + kRankMax * warp);
 }
 
 int prepare_one(int64_t n_nodes, int64_t n_edges, const int32_t* senders, const int32_t* receivers,
                 const int32_t* pad_recv, int32_t* rowptr, int32_t* sender_perm, int32_t* colptr, cudaStream_t st) {
-    // 16 nodes a block (a thread or so per edge in the sort) until there are 128 blocks, then equal runs
-    const int64_t blocks = std::min<int64_t>(kOneBlocks, (n_nodes + 15) / 16);
+    // 16 nodes a block (a thread or so per edge in the sort), fewer where 16 would have more than about 4096 edges, up
+    // to 128 blocks, then equal runs
+    const int64_t want = std::max((n_nodes + 15) / 16, std::min(n_nodes, (n_edges + 4095) / 4096));
+    const int64_t blocks = std::min<int64_t>(kOneBlocks, want);
     const int per_block = (int)((n_nodes + blocks - 1) / blocks);
     static thread_local int attr_dev = -1;
     int dev = 0;

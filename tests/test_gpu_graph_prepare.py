@@ -10,11 +10,11 @@ pytestmark = pytest.mark.gpu
 
 
 # (nodes, edges, padding, nodes that send or receive): one edge; a list without padding and one of padding alone; runs
-# of thousands of empty rows before, between and behind; a block whose edges do not fit; the largest list and node
-# count of the form and the next
+# of thousands of empty rows before, between and behind; the largest list of the form and the next; a block whose edges
+# do not fit; a dense graph; the largest node count of the form and the next
 @pytest.mark.parametrize("n,e,pad,used,hub", [
     (1, 1, 0, 1, 0), (7, 40, 0, 7, 0), (7, 0, 5, 7, 0), (5000, 60, 13, 5000, 0), (70001, 33, 0, 3, 0),
-    (3000, 196608, 0, 3000, 0), (3000, 196609, 0, 3000, 0), (100, 20001, 3, 100, 0.5), (262144, 1000, 7, 262144, 0),
+    (3000, 196608, 0, 3000, 0), (3000, 196609, 0, 3000, 0), (100, 20001, 3, 100, 0.5), (100, 100003, 0, 100, 0), (262144, 1000, 7, 262144, 0),
     (262145, 1000, 7, 262145, 0)])
 def test_prepare_matches_numpy(n, e, pad, used, hub):
     rng = np.random.default_rng(n + e)
