@@ -8,7 +8,7 @@
 //   dx_e[i1]    = sum_k s[e,k] * u[k,i1]                       (this edge's share of grad_x[a])
 //   grad_sh[e,i2] = sum_q sum_{pairs} C[i0,i1,i2] * (s[e,k] x[a,i1]) * dm[b,i0]
 // grad_w and grad_sh are edge-local and final.  dx_e is written to a scratch array
-// [E,d,N_q]; pass 2 (bwd_dx_reduce_kernel) adds the rows of every sender in edge order, so no
+// [E,d,N_q]; pass 2 (bwd_dx_reduce_kernel) adds the rows of every sender in a fixed order, so no
 // floating-point atomics are needed and the result is bit-reproducible.
 //
 // Work split: equal contiguous edge ranges per CTA; consumer warp (g, ch) owns the paths of

@@ -195,11 +195,15 @@ __global__ void bwd_zero_padding_kernel(ZeroPadding z);   // on its own where no
 // Self-test of the bounded wait (e3j_selftest_bounded_wait): one warp waits on a barrier that nobody arrives on.
 __global__ void bounded_wait_selftest_kernel(uint32_t limit, int32_t* status, int32_t* result);
 
-// Backward pass 2: grad_x[a] = sum of the per-edge shares of the edges sent by a, in edge order.  One block per
-// sender, row_f4 * groups threads: with few senders its edges are dealt to `groups` runs whose sums are added in run
-// order (a run's loads are a chain of dependent latencies; 192 senders of 53 edges: 18 us with one run).  Further
-// blocks write the zero rows of padding edges.
-__global__ void bwd_dx_reduce_kernel(int64_t n_nodes, int row_f4, const float4* __restrict__ dx_edge,
+// Backward pass 2: grad_x[a] = sum of the per-edge shares of the edges sent by a.  One block per sender, row_f4 * groups
+// threads: with few senders a sender's edges are dealt to up to 8 runs in edge order, whose sums are added in run order
+// (a run's loads are a chain of dependent latencies; 192 senders of 53 edges: 18 us with one run).  How many runs comes
+// from the number of senders, the row and the sender's own degree, so padding entries, which lengthen the list, change
+// no bit of the result; the list's length only says how many groups of threads a block has for them (500 senders of 20
+// edges, 128x(0e+1o): with as many groups as runs at most, 8, the backward takes 48.3 us, with 4 45.0).  A hub sender's
+// runs go round its groups (10 000 edges from one sender: 939 -> 608 us).  Further blocks write the zero rows of padding
+// edges.
+__global__ void bwd_dx_reduce_kernel(int64_t n_nodes, int row_f4, int max_runs, const float4* __restrict__ dx_edge,
                                      const int32_t* __restrict__ sender_perm, const int32_t* __restrict__ colptr,
                                      float4* __restrict__ grad_x, ZeroPadding pad);
 int launch_dx_reduce(int64_t n_nodes, int64_t n_edges, int row_f4, const float* dx_edge, const int32_t* sender_perm,
