@@ -114,7 +114,7 @@ template <class T> struct Args {
     const int32_t *senders, *receivers, *ptr, *perm, *n_real;
     T *out, *grad_w, *grad_sh;   // out: the node sums (forward out, backward grad_x)
     int d, dp, P, D, units;      // units: N_q / V
-    int split_log2;              // a node's edges are dealt to 2^split_log2 lanes
+    int split_log2;              // a node has 2^split_log2 lanes; its own degree says to how many its edges are dealt
     unsigned node_blocks;        // backward: blocks below this one are node sums, the others edge tiles
 };
 
@@ -137,8 +137,8 @@ template <int LM> constexpr int stage_bytes() { return (2 * LM + 2) * 512; }
 template <int LM> constexpr int ring_bytes() { return kStages * stage_bytes<LM>(); }
 
 // ---------------------------------------------------------------- node sums
-// One path's share of a node's rows: summed over the lane's edges, then over the lanes that share the node, and
-// stored by the first of them (added to the rows for the group's second and later paths).
+// One path's share of a node's rows: summed over the lane's edges (every step-th one), then over the lanes that share
+// the node, and stored by the first of them (added to the rows for the group's second and later paths).
 template <class Tr, class T, int V, bool TR, bool IDENT>
 __device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, const unsigned j0, const unsigned j1,
                                          const int step, const int row, const int q, T* dst, const bool first) {
@@ -184,7 +184,7 @@ __device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, co
         }
     }
 #pragma unroll 1
-    for (int off = 32 / step; off < 32; off <<= 1) {
+    for (int off = 32 >> a.split_log2; off < 32; off <<= 1) {
 #pragma unroll
         for (int o = 0; o < NO; ++o)
 #pragma unroll
@@ -203,6 +203,8 @@ __device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, co
     }
 }
 
+constexpr int kLaneEdges = 4;   // a lane's edges at least, where a node's edges are dealt to several
+
 template <class T, int V, int LM, bool TR, bool IDENT>
 __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, const unsigned block) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
@@ -212,24 +214,27 @@ __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, 
     const int64_t node = item / a.units;
     const int q = (int)(item - node * a.units), row = a.units * V;
     unsigned j0 = 0, j1 = 0;   // edge counts are below 2^31, so a step past the end does not wrap
+    int step = 1;
     T* dst = nullptr;
     const int p0 = t.start[grp], p1 = t.start[grp + 1];
     if (node < a.n_nodes) {
         j0 = IDENT ? (unsigned)node : (unsigned)a.ptr[node];
         j1 = IDENT ? (unsigned)node + 1 : (unsigned)a.ptr[node + 1];
+        while (step < 1 << a.split_log2 && j1 - j0 >= 2u * kLaneEdges * step) step *= 2;
+        j0 = part < step ? j0 + part : j1;
         if (part == 0)
             dst = a.out + ((size_t)node * (TR ? a.d : a.D) + (TR ? t.rec[p0].x_off : t.rec[p0].out_off)) * row + q * V;
     }
 #pragma unroll 1
     for (int p = p0; p < p1; ++p) {
         const PathRec rec = t.rec[p];
-        int row_p = row, step = 1 << a.split_log2;
-        asm volatile("" : "+r"(row_p), "+r"(step));   // keeps every case's address arithmetic inside the case
+        int row_p = row, step_p = step;
+        asm volatile("" : "+r"(row_p), "+r"(step_p));   // keeps every case's address arithmetic inside the case
         switch (rec.id) {
 #define E3J_CASE(l1, l2, L) \
             case E3J_TRI_ID(l1, l2, L): \
                 if constexpr (l1 <= LM && l2 <= LM && L <= LM) \
-                    sum_path<Tri<l1, l2, L>, T, V, TR, IDENT>(a, rec, j0 + part, j1, step, row_p, q, dst, p == p0); \
+                    sum_path<Tri<l1, l2, L>, T, V, TR, IDENT>(a, rec, j0, j1, step_p, row_p, q, dst, p == p0); \
                 break;
             E3J_PATH_TRIPLES(E3J_CASE)
 #undef E3J_CASE

@@ -49,13 +49,14 @@ PathTable table_of(const e3j_plan* plan, bool by_input) {
 }
 
 // Lanes per (node, unit, group): the edges of a node are walked by one lane while that fills the chip (`warps` per
-// SM); smaller calls deal them to up to 8 lanes as long as each keeps about four edges.  The forward wants two lanes
+// SM); smaller calls give a node up to 8 lanes, of which the kernel uses as many as get kLaneEdges edges each.  Not a
+// function of the list's length: padding entries must not change the order of a sum.  The forward wants two lanes
 // sooner (32 warps: 79 us against 99 us with 16 on the workload of path_kernels.cuh), the backward, whose node sums
 // share the SMs with the edge tiles, does not (190 against 179 us).
 constexpr int kFwdWarps = 32, kBwdWarps = 16;
-int split_of(int64_t n_nodes, int64_t n_edges, int units, int groups, int warps) {
+int split_of(int64_t n_nodes, int units, int groups, int warps) {
     int s = 0;
-    while (s < 3 && (n_nodes * units * groups << s) < (int64_t)sm_count() * warps * 32 && n_edges >> (s + 3) >= n_nodes) ++s;
+    while (s < 3 && (n_nodes * units * groups << s) < (int64_t)sm_count() * warps * 32) ++s;
     return s;
 }
 
@@ -89,7 +90,7 @@ template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, cons
     const PathTable t = table_of(plan, false);
     Args<T> a = args_of<T, V>(plan, c);
     a.ptr = c.rowptr; a.out = c.out;
-    a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups, kFwdWarps);
+    a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kFwdWarps);
     const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
     node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
@@ -108,7 +109,7 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     }
     int64_t nodes = 0, tiles = 0;
     if (c.grad_x) {
-        a.split_log2 = split_of(c.n_nodes, c.n_edges, a.units, t.n_groups, one_launch(LM) ? kBwdWarps : kFwdWarps);
+        a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, one_launch(LM) ? kBwdWarps : kFwdWarps);
         nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, one_launch(LM) ? threads : kThreads);
     }
     if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);

@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 # 192 nodes of every degree between 0 and twice the mean: senders and receivers on both sides of each threshold of the
 # split, lists whose capacity is (1.05, 1.25, 4 times) or is not on the same side of the thresholds as the edge count
-@pytest.mark.parametrize("irreps,lmax,specialised", [("128x0e+128x1o", 3, 1), ("32x0e+32x1o", 3, 1)])
+@pytest.mark.parametrize("irreps,lmax,specialised", [("128x0e+128x1o", 3, 1), ("32x0e+32x1o", 3, 1), ("12x0e+12x1o+12x2e", 2, 0),
+                                                     ("16x0e+16x3o", 3, 0)])
 @pytest.mark.parametrize("degree", [7, 20, 47])
 def test_padded_results_do_not_depend_on_the_capacity(irreps, lmax, specialised, degree):
     n = 192
