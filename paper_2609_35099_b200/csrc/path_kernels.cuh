@@ -115,6 +115,7 @@ template <class T> struct Args {
     T *out, *grad_w, *grad_sh;   // out: the node sums (forward out, backward grad_x)
     int d, dp, P, D, units;      // units: N_q / V
     int split_log2;              // a node has 2^split_log2 lanes; its own degree says to how many its edges are dealt
+    unsigned group_blocks;
     unsigned node_blocks;        // backward: blocks below this one are node sums, the others edge tiles
 };
 
@@ -137,18 +138,17 @@ template <int LM> constexpr int stage_bytes() { return (2 * LM + 2) * 512; }
 template <int LM> constexpr int ring_bytes() { return kStages * stage_bytes<LM>(); }
 
 // ---------------------------------------------------------------- node sums
-// One path's share of a node's rows: summed over the lane's edges (every step-th one), then over the lanes that share
-// the node, and stored by the first of them (added to the rows for the group's second and later paths).
+// One path's share of a node's rows, summed over the lane's edges (every step-th one).
 template <class Tr, class T, int V, bool TR, bool IDENT>
-__device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, const unsigned j0, const unsigned j1,
-                                         const int step, const int row, const int q, T* dst, const bool first) {
+__device__ __forceinline__ void walk_path(const Args<T>& a, const PathRec rec, const unsigned j0, const unsigned j1,
+                                         const int step, const int row, const int q,
+                                         T (&acc)[TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1][V]) {
     constexpr int NI = TR ? 2 * Tr::kL + 1 : 2 * Tr::kL1 + 1, NO = TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1;
     constexpr int NY = 2 * Tr::kL2 + 1;
     constexpr int U = NI <= 3 ? 2 : 1;   // edges in flight: their input rows fill at most 28 registers
     const T* in_base = (TR ? a.g + (size_t)rec.out_off * row : a.x + (size_t)rec.x_off * row) + q * V;
     const T* w_base = a.w + (size_t)rec.k * row + q * V;
     const size_t in_stride = (size_t)(TR ? a.D : a.d) * row, w_stride = (size_t)a.P * row;
-    T acc[NO][V];
 #pragma unroll
     for (int o = 0; o < NO; ++o)
 #pragma unroll
@@ -183,8 +183,17 @@ __device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, co
             else Tr::template sum<T, V>(y[u], in[u], w[u], acc);
         }
     }
+}
+// The forward's groups: added up over the lanes that share the node and stored by the first of them (added to the rows for
+// the second and later paths of a collapsed block).
+template <class Tr, class T, int V, bool TR, bool IDENT>
+__device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, const unsigned j0, const unsigned j1,
+                                         const int step, const int used, const int row, const int q, T* dst, const bool first) {
+    constexpr int NO = TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1;
+    T acc[NO][V];
+    walk_path<Tr, T, V, TR, IDENT>(a, rec, j0, j1, step, row, q, acc);
 #pragma unroll 1
-    for (int off = 32 >> a.split_log2; off < 32; off <<= 1) {
+    for (int off = 32 >> a.split_log2; off < (32 >> a.split_log2) * used; off <<= 1) {
 #pragma unroll
         for (int o = 0; o < NO; ++o)
 #pragma unroll
@@ -203,14 +212,63 @@ __device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, co
     }
 }
 
+// The backward's groups have several paths each: their sums, each taken by itself, are added in registers, then over the
+// lanes, and stored once.
+template <int LO, class T, int V, int LM, bool IDENT>
+__device__ __forceinline__ void node_group(const PathTable& t, const Args<T>& a, const int p0, const int p1, const unsigned j0,
+                                           const unsigned j1, const int step, const int used, const int row, const int q, T* dst) {
+    constexpr int NO = 2 * LO + 1;
+    T tot[NO][V];
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+#pragma unroll
+        for (int c = 0; c < V; ++c) tot[o][c] = T(0);
+#pragma unroll 1
+    for (int p = p0; p < p1; ++p) {
+        const PathRec rec = t.rec[p];
+        int row_p = row, step_p = step;
+        asm volatile("" : "+r"(row_p), "+r"(step_p));
+        switch (rec.id) {
+#define E3J_CASE(l1, l2, L) \
+            case E3J_TRI_ID(l1, l2, L): \
+                if constexpr (l1 == LO && l2 <= LM && L <= LM) { \
+                    T acc[NO][V]; \
+                    walk_path<Tri<l1, l2, L>, T, V, true, IDENT>(a, rec, j0, j1, step_p, row_p, q, acc); \
+                    _Pragma("unroll") for (int o = 0; o < NO; ++o) \
+                        _Pragma("unroll") for (int c = 0; c < V; ++c) tot[o][c] += acc[o][c]; \
+                } \
+                break;
+            E3J_PATH_TRIPLES(E3J_CASE)
+#undef E3J_CASE
+        }
+    }
+#pragma unroll 1
+    for (int off = 32 >> a.split_log2; off < (32 >> a.split_log2) * used; off <<= 1) {
+#pragma unroll
+        for (int o = 0; o < NO; ++o)
+#pragma unroll
+            for (int c = 0; c < V; ++c) tot[o][c] += __shfl_xor_sync(0xffffffffu, tot[o][c], off);
+    }
+    if (!dst) return;
+#pragma unroll
+    for (int o = 0; o < NO; ++o) store_pack<T, V>(dst + (size_t)o * row, tot[o]);
+}
+
 constexpr int kLaneEdges = 4;   // a lane's edges at least, where a node's edges are dealt to several
 
 template <class T, int V, int LM, bool TR, bool IDENT>
 __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, const unsigned block) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    const int grp = (int)(block % (unsigned)t.n_groups);
     const int per_warp = 32 >> a.split_log2, part = lane >> (5 - a.split_log2);
-    const int64_t item = ((int64_t)(block / (unsigned)t.n_groups) * warps + warp) * per_warp + (lane & (per_warp - 1));
+    // From l = 2 on a group's blocks follow one another, so that an SM runs few different paths at a time (instruction
+    // cache; 20 000 nodes of degree 3, 16x(0e+1o+2e+3o): grad_x 589 -> 328 us), the last groups, which have the highest l,
+    // first.  With l <= 1 the few paths fit, and the groups of one node run side by side, which read the same rows
+    // (49 157 rows of a tensor product, 384x1o: 223 against 252 us).
+    unsigned turn, at;
+    if constexpr (LM >= 2) { turn = block / a.group_blocks; at = block - turn * a.group_blocks; }
+    else { at = block / (unsigned)t.n_groups; turn = block - at * (unsigned)t.n_groups; }
+    const int grp = t.n_groups - 1 - (int)turn;
+    const int64_t item = ((int64_t)at * warps + warp) * per_warp + (lane & (per_warp - 1));
     const int64_t node = item / a.units;
     const int q = (int)(item - node * a.units), row = a.units * V;
     unsigned j0 = 0, j1 = 0;   // edge counts are below 2^31, so a step past the end does not wrap
@@ -225,6 +283,24 @@ __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, 
         if (part == 0)
             dst = a.out + ((size_t)node * (TR ? a.d : a.D) + (TR ? t.rec[p0].x_off : t.rec[p0].out_off)) * row + q * V;
     }
+    const int used = IDENT ? 1 : __reduce_max_sync(0xffffffffu, step);
+    if constexpr (TR) {
+        if (t.rec[p0].id == kNoPath) {   // zero rows
+            T z[V];
+#pragma unroll
+            for (int c = 0; c < V; ++c) z[c] = T(0);
+            if (dst)
+                for (int o = 0; o < 2 * t.rec[p0].l1 + 1; ++o) store_pack<T, V>(dst + (size_t)o * row, z);
+            return;
+        }
+        switch (t.rec[p0].l1) {
+            case 0: node_group<0, T, V, LM, IDENT>(t, a, p0, p1, j0, j1, step, used, row, q, dst); break;
+            case 1: node_group<1, T, V, LM, IDENT>(t, a, p0, p1, j0, j1, step, used, row, q, dst); break;
+            case 2: if constexpr (LM >= 2) node_group<2, T, V, LM, IDENT>(t, a, p0, p1, j0, j1, step, used, row, q, dst); break;
+            case 3: if constexpr (LM >= 3) node_group<3, T, V, LM, IDENT>(t, a, p0, p1, j0, j1, step, used, row, q, dst); break;
+        }
+        return;
+    }
 #pragma unroll 1
     for (int p = p0; p < p1; ++p) {
         const PathRec rec = t.rec[p];
@@ -234,17 +310,10 @@ __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, 
 #define E3J_CASE(l1, l2, L) \
             case E3J_TRI_ID(l1, l2, L): \
                 if constexpr (l1 <= LM && l2 <= LM && L <= LM) \
-                    sum_path<Tri<l1, l2, L>, T, V, TR, IDENT>(a, rec, j0, j1, step_p, row_p, q, dst, p == p0); \
+                    sum_path<Tri<l1, l2, L>, T, V, TR, IDENT>(a, rec, j0, j1, step_p, used, row_p, q, dst, p == p0); \
                 break;
             E3J_PATH_TRIPLES(E3J_CASE)
 #undef E3J_CASE
-            default: {   // kNoPath: zero rows
-                T z[V];
-#pragma unroll
-                for (int c = 0; c < V; ++c) z[c] = T(0);
-                if (dst)
-                    for (int o = 0; o < 2 * rec.l1 + 1; ++o) store_pack<T, V>(dst + (size_t)o * row, z);
-            }
         }
     }
 }

@@ -93,6 +93,7 @@ template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, cons
     a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kFwdWarps);
     const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+    a.group_blocks = (unsigned)(blocks / t.n_groups);
     node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
     return after_launch();
 }
@@ -109,19 +110,21 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     }
     int64_t nodes = 0, tiles = 0;
     if (c.grad_x) {
-        a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, one_launch(LM) ? kBwdWarps : kFwdWarps);
+        a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kBwdWarps);
         nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, one_launch(LM) ? threads : kThreads);
     }
     if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);
     if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
     if (nodes > 0 && (!one_launch(LM) || tiles == 0)) {
         if (one_launch(LM)) nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
+        a.group_blocks = (unsigned)(nodes / t.n_groups);
         node_kernel<T, V, LM, true, IDENT><<<(unsigned)nodes, kThreads, 0, c.stream>>>(t, a);
         if (int s = after_launch()) return s;
         nodes = 0;
     }
     if (nodes + tiles == 0) return E3J_OK;
     a.node_blocks = (unsigned)nodes;
+    a.group_blocks = (unsigned)(nodes / t.n_groups);
     if (int s = allow_smem<LM>(bwd_kernel<T, V, LM, IDENT>)) return s;
     bwd_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
     return after_launch();
