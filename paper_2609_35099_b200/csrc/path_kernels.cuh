@@ -43,6 +43,13 @@ __host__ __device__ __forceinline__ void store_pack(T* dst, const T (&src)[V]) {
     for (int c = 0; c < V; ++c) p.v[c] = src[c];
     *reinterpret_cast<Pack<T, V>*>(dst) = p;
 }
+template <class T, int V, int N>
+__host__ __device__ __forceinline__ void clear(T (&z)[N][V]) {
+#pragma unroll
+    for (int o = 0; o < N; ++o)
+#pragma unroll
+        for (int c = 0; c < V; ++c) z[o][c] = T(0);
+}
 template <class T, int V>
 __host__ __device__ __forceinline__ void axpy(T (&z)[V], const T a, const T (&x)[V]) {
 #pragma unroll
@@ -138,7 +145,7 @@ template <int LM> constexpr int stage_bytes() { return (2 * LM + 2) * 512; }
 template <int LM> constexpr int ring_bytes() { return kStages * stage_bytes<LM>(); }
 
 // ---------------------------------------------------------------- node sums
-// One path's share of a node's rows, summed over the lane's edges (every step-th one).
+// One path's share of a node's rows, summed over the lane's edges (every step-th one) and added to acc.
 template <class Tr, class T, int V, bool TR, bool IDENT>
 __device__ __forceinline__ void walk_path(const Args<T>& a, const PathRec rec, const unsigned j0, const unsigned j1,
                                          const int step, const int row, const int q,
@@ -149,10 +156,6 @@ __device__ __forceinline__ void walk_path(const Args<T>& a, const PathRec rec, c
     const T* in_base = (TR ? a.g + (size_t)rec.out_off * row : a.x + (size_t)rec.x_off * row) + q * V;
     const T* w_base = a.w + (size_t)rec.k * row + q * V;
     const size_t in_stride = (size_t)(TR ? a.D : a.d) * row, w_stride = (size_t)a.P * row;
-#pragma unroll
-    for (int o = 0; o < NO; ++o)
-#pragma unroll
-        for (int c = 0; c < V; ++c) acc[o][c] = T(0);
     // the ids of an edge are fetched one step ahead of its rows; past the end: the last step's first edge again
     int e[U], b[U];
     auto ids = [&](unsigned j) {
@@ -191,6 +194,7 @@ __device__ __forceinline__ void sum_path(const Args<T>& a, const PathRec rec, co
                                          const int step, const int used, const int row, const int q, T* dst, const bool first) {
     constexpr int NO = TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1;
     T acc[NO][V];
+    clear(acc);
     walk_path<Tr, T, V, TR, IDENT>(a, rec, j0, j1, step, row, q, acc);
 #pragma unroll 1
     for (int off = 32 >> a.split_log2; off < (32 >> a.split_log2) * used; off <<= 1) {
@@ -219,10 +223,7 @@ __device__ __forceinline__ void node_group(const PathTable& t, const Args<T>& a,
                                            const unsigned j1, const int step, const int used, const int row, const int q, T* dst) {
     constexpr int NO = 2 * LO + 1;
     T tot[NO][V];
-#pragma unroll
-    for (int o = 0; o < NO; ++o)
-#pragma unroll
-        for (int c = 0; c < V; ++c) tot[o][c] = T(0);
+    clear(tot);
 #pragma unroll 1
     for (int p = p0; p < p1; ++p) {
         const PathRec rec = t.rec[p];
@@ -232,10 +233,15 @@ __device__ __forceinline__ void node_group(const PathTable& t, const Args<T>& a,
 #define E3J_CASE(l1, l2, L) \
             case E3J_TRI_ID(l1, l2, L): \
                 if constexpr (l1 == LO && l2 <= LM && L <= LM) { \
-                    T acc[NO][V]; \
-                    walk_path<Tri<l1, l2, L>, T, V, true, IDENT>(a, rec, j0, j1, step_p, row_p, q, acc); \
-                    _Pragma("unroll") for (int o = 0; o < NO; ++o) \
-                        _Pragma("unroll") for (int c = 0; c < V; ++c) tot[o][c] += acc[o][c]; \
+                    if constexpr (IDENT) {   /* one edge: nothing to sum apart */ \
+                        walk_path<Tri<l1, l2, L>, T, V, true, IDENT>(a, rec, j0, j1, step_p, row_p, q, tot); \
+                    } else { \
+                        T acc[NO][V]; \
+                        clear(acc); \
+                        walk_path<Tri<l1, l2, L>, T, V, true, IDENT>(a, rec, j0, j1, step_p, row_p, q, acc); \
+                        _Pragma("unroll") for (int o = 0; o < NO; ++o) \
+                            _Pragma("unroll") for (int c = 0; c < V; ++c) tot[o][c] += acc[o][c]; \
+                    } \
                 } \
                 break;
             E3J_PATH_TRIPLES(E3J_CASE)
@@ -396,20 +402,23 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
     copies_wait<0>();
     __syncthreads();   // the rings are free: the partials take their place
     T* part = reinterpret_cast<T*>(smem);
-    // channel sum: eight lanes per (edge, component) add every eighth partial, then a fixed tree over the eight
+    // channel sum: 2^lanes_log2 lanes per (edge, component), eight where there are as many partials, add every eighth
+    // partial each, then a fixed tree over them.  With few units there are many sums of few terms: eight lanes for each
+    // took 128 rounds with one unit (backward of a tensor product, 4x(0e+1o+2e+3o), 300 rows: 84 -> 49 us)
 #pragma unroll
     for (int i = 0; i < NY; ++i)
         if (i < a.dp) part[i * blockDim.x + threadIdx.x] = dy[i];
     __syncthreads();
-    const int sub = threadIdx.x & 7, n_out = slots * a.dp, per_pass = blockDim.x >> 3;
+    const int lanes_log2 = a.units > 4 ? 3 : a.units > 2 ? 2 : a.units - 1, lanes = 1 << lanes_log2;
+    const int sub = threadIdx.x & (lanes - 1), n_out = slots * a.dp, per_pass = blockDim.x >> lanes_log2;
     for (int o0 = 0; o0 < n_out; o0 += per_pass) {
-        const int o = o0 + (threadIdx.x >> 3);
+        const int o = o0 + (threadIdx.x >> lanes_log2);
         const int sl = o / a.dp, i = o - sl * a.dp;
         T sum = T(0);
         if (o < n_out)
-            for (int u = sub; u < a.units; u += 8) sum += part[i * blockDim.x + sl * a.units + u];
-#pragma unroll
-        for (int off = 4; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            for (int u = sub; u < a.units; u += lanes) sum += part[i * blockDim.x + sl * a.units + u];
+#pragma unroll 1
+        for (int off = lanes >> 1; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
         const int64_t eo = (int64_t)tile * slots + sl;
         if (sub == 0 && o < n_out && eo < a.n_edges) a.grad_sh[(size_t)eo * a.dp + i] = sum;
     }
