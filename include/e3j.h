@@ -281,7 +281,9 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
  *   Workspace: 256-byte aligned, at least e3j_conv_radial_*_workspace_bytes(); calls that overlap on the GPU
  *   must not share it.  The forward forms the weight array in its workspace while the array is no larger than 2 GiB
  *   (faster) and forms the weights inside the convolution kernel beyond that, where the plan has such a kernel; it also
- *   does so when the workspace has no room for the array, and refuses only a workspace that holds neither form.
+ *   does so when the workspace has no room for the array, and refuses only a workspace that holds neither form.  A
+ *   caller that wants the memory rather than the time passes e3j_conv_radial_*fwd_least_workspace_bytes(): the size
+ *   of the smaller form.
  *   The two gradient products fetch their operands through tensor maps (tiled bulk copies); a driver that has no
  *   encoder for them (cuTensorMapEncodeTiled, CUDA 12) makes the backward return E3J_ERR_UNSUPPORTED.
  * e3j_radial_weights writes the product itself, w_out [n_edges, P, N_q] (for callers that want the weights, and
@@ -289,6 +291,7 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
 int e3j_radial_weights(const e3j_plan* plan, int64_t n_edges, int hidden, const float* h, const float* W,
                        float* w_out, void* stream);
 size_t e3j_conv_radial_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden);
+size_t e3j_conv_radial_fwd_least_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden);
 int e3j_conv_radial_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden, const float* x,
                         const float* sh, const float* h, const float* W, const int32_t* senders,
                         const int32_t* receivers, const int32_t* rowptr, float* out, void* workspace,
@@ -341,11 +344,12 @@ int e3j_conv_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
                      float* grad_vec, float* grad_w, void* workspace, size_t workspace_bytes, void* stream);
 
 /* Both at once: the forward convolution from edge vectors and the radial layer, out = conv_fwd(x, Y(edge_vec), h W).
- * Where the plan has the kernel that forms the edge scalars itself (see e3j_conv_radial_fwd) that kernel forms the
- * harmonics too, and the call reads x, edge_vec, h, W and the graph only; otherwise the call is composed
- * (e3j_harmonics_fwd and e3j_radial_weights into the workspace, then e3j_conv_fwd).  Arguments as for
+ * Plans with generated kernels form the harmonics inside the convolution kernel, in both forms of e3j_conv_radial_fwd
+ * (edge scalars in the workspace, or inside the kernel: the call then reads x, edge_vec, h, W and the graph only);
+ * other plans run e3j_harmonics_fwd into the workspace first.  Arguments as for
  * e3j_conv_radial_fwd with edge_vec [n_edges, 3] in place of sh. */
 size_t e3j_conv_radial_vec_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden);
+size_t e3j_conv_radial_vec_fwd_least_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden);
 int e3j_conv_radial_vec_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden, const float* x,
                             const float* edge_vec, const float* h, const float* W, const int32_t* senders,
                             const int32_t* receivers, const int32_t* rowptr, float* out, void* workspace,

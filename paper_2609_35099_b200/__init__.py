@@ -23,8 +23,9 @@ __all__ = [
     "e3j_conv_fwd_workspace_bytes", "e3j_conv_bwd_workspace_bytes", "e3j_conv_fwd", "e3j_conv_fwd_noalloc", "e3j_noalloc_status",
     "e3j_conv_bwd", "e3j_graph_prepare_padded", "e3j_conv_fwd_padded", "e3j_conv_bwd_padded",
     "e3j_conv_bwd_bwd_workspace_bytes", "e3j_conv_bwd_bwd",
-    "e3j_radial_weights", "e3j_conv_radial_fwd_workspace_bytes", "e3j_conv_radial_bwd_workspace_bytes",
-    "e3j_conv_radial_fwd", "e3j_conv_radial_bwd", "e3j_conv_radial_vec_fwd", "e3j_conv_radial_vec_fwd_workspace_bytes", "e3j_conv_radial_vec_bwd", "e3j_conv_radial_vec_bwd_workspace_bytes",
+    "e3j_radial_weights", "e3j_conv_radial_fwd_workspace_bytes", "e3j_conv_radial_fwd_least_workspace_bytes",
+    "e3j_conv_radial_bwd_workspace_bytes",
+    "e3j_conv_radial_fwd", "e3j_conv_radial_bwd", "e3j_conv_radial_vec_fwd", "e3j_conv_radial_vec_fwd_workspace_bytes", "e3j_conv_radial_vec_fwd_least_workspace_bytes", "e3j_conv_radial_vec_bwd", "e3j_conv_radial_vec_bwd_workspace_bytes",
     "e3j_tp_fwd", "e3j_tp_bwd", "e3j_bwd_schedule_bytes", "e3j_bwd_schedule_build", "e3j_conv_bwd_scheduled", "e3j_harmonics_fwd", "e3j_harmonics_bwd", "e3j_conv_vec_fwd", "e3j_conv_vec_bwd",
     "e3j_conv_vec_fwd_workspace_bytes", "e3j_conv_vec_bwd_workspace_bytes", "e3j_conv_fwd_f64", "e3j_conv_bwd_f64", "e3j_shard_prepare", "e3j_rows_gather", "e3j_rows_add", "e3j_status_string", "e3j_selftest_bounded_wait", "e3j_launch_count", "E3J_PLAN_GENERIC_ONLY",
     "E3J_PLAN_COLLAPSE_OUTPUTS", "E3J_PLAN_RADIAL_MATERIALISE",
@@ -106,6 +107,9 @@ def _load():
     lib.e3j_radial_weights.restype = i32
     lib.e3j_conv_radial_fwd_workspace_bytes.argtypes = [vp, i64, i64, i32]
     lib.e3j_conv_radial_fwd_workspace_bytes.restype = sz
+    for name in ("e3j_conv_radial_fwd_least_workspace_bytes", "e3j_conv_radial_vec_fwd_least_workspace_bytes"):
+        getattr(lib, name).argtypes = [vp, i64, i64, i32]
+        getattr(lib, name).restype = sz
     lib.e3j_conv_radial_bwd_workspace_bytes.argtypes = [vp, i64, i64, i32]
     lib.e3j_conv_radial_bwd_workspace_bytes.restype = sz
     lib.e3j_conv_radial_fwd.argtypes = [vp, i64, i64, i32] + [vp] * 9 + [sz, vp]
@@ -270,11 +274,13 @@ def _stream(stream):
     return c._cuda_getCurrentRawStream(c._cuda_getDevice())   # torch.cuda.current_stream() without building the object
 
 
-def _workspace(nbytes: int, like, workspace):
+def _workspace(nbytes: int, like, workspace, least=None):
+    """The caller's workspace, or a new one of nbytes.  least(): the bytes a call also runs with, where that is less."""
     torch = _torch()
     if workspace is None:
         return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=like.device)
-    if workspace.dtype != torch.uint8 or not workspace.is_cuda or workspace.numel() < nbytes:
+    if workspace.dtype != torch.uint8 or not workspace.is_cuda or \
+            workspace.numel() < nbytes and (least is None or workspace.numel() < least()):
         raise ValueError("workspace must be a CUDA uint8 tensor of sufficient size")
     return workspace
 
@@ -474,6 +480,12 @@ def e3j_conv_radial_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, 
     return int(_load().e3j_conv_radial_fwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
 
 
+def e3j_conv_radial_fwd_least_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
+    """The smallest workspace e3j_conv_radial_fwd runs with: where the plan has the kernel for it, without room for the
+    edge weights, which are then formed inside the kernel (slower below 2 GiB of them)."""
+    return int(_load().e3j_conv_radial_fwd_least_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+
+
 def e3j_conv_radial_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
     return int(_load().e3j_conv_radial_bwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
 
@@ -486,7 +498,8 @@ def e3j_conv_radial_fwd(plan: Plan, x, sh, h, W, senders, receivers, rowptr=None
     f32, i32 = torch.float32, torch.int32
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
-    workspace = _workspace(e3j_conv_radial_fwd_workspace_bytes(plan, n, e, hidden), x, workspace)
+    workspace = _workspace(e3j_conv_radial_fwd_workspace_bytes(plan, n, e, hidden), x, workspace,
+                           lambda: e3j_conv_radial_fwd_least_workspace_bytes(plan, n, e, hidden))
     _check(_load().e3j_conv_radial_fwd(
         plan.handle, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
@@ -502,6 +515,11 @@ def e3j_conv_radial_vec_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: i
     return int(_load().e3j_conv_radial_vec_fwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
 
 
+def e3j_conv_radial_vec_fwd_least_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
+    """As e3j_conv_radial_fwd_least_workspace_bytes, for the call on edge vectors."""
+    return int(_load().e3j_conv_radial_vec_fwd_least_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+
+
 def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, rowptr=None, out=None, workspace=None,
                             stream=None):
     """Forward convolution from edge vectors [E, 3] and the radial layer (h, W): where the plan has the kernels for it
@@ -511,7 +529,8 @@ def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, r
     f32, i32 = torch.float32, torch.int32
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
-    workspace = _workspace(e3j_conv_radial_vec_fwd_workspace_bytes(plan, n, e, hidden), x, workspace)
+    workspace = _workspace(e3j_conv_radial_vec_fwd_workspace_bytes(plan, n, e, hidden), x, workspace,
+                           lambda: e3j_conv_radial_vec_fwd_least_workspace_bytes(plan, n, e, hidden))
     _check(_load().e3j_conv_radial_vec_fwd(
         plan.handle, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),

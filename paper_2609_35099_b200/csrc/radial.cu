@@ -192,13 +192,22 @@ RadialLayout radial_layout(const e3j_plan* plan, int64_t n_nodes, int64_t n_edge
 }
 
 // The layout a forward call runs with: the preferred one, or, where the workspace is too small for it, the one with
-// in-kernel edge scalars (if the plan has that kernel).
+// in-kernel edge scalars (if the plan has that kernel).  A workspace sized for a longer list, whose array was over the
+// limit, may lack the room a shorter list's array takes: that call runs in the kernel too.
 RadialLayout fwd_layout(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int H, size_t workspace_bytes) {
     const RadialLayout L = radial_layout(plan, n_nodes, n_edges, H, false);
     return workspace_bytes >= L.total ? L : radial_layout(plan, n_nodes, n_edges, H, false, true);
 }
+// What a forward call is best given, and the least it runs with.
 size_t fwd_workspace(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int H) {
     return std::max(radial_layout(plan, n_nodes, n_edges, H, false).total, radial_layout(plan, n_nodes, n_edges, H, false, true).total);
+}
+size_t fwd_least_workspace(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int H) {
+    return std::min(radial_layout(plan, n_nodes, n_edges, H, false).total, radial_layout(plan, n_nodes, n_edges, H, false, true).total);
+}
+// Room for harmonics, behind the convolution's workspace (calls on edge vectors)
+size_t sh_scratch_bytes(const e3j_plan* plan, int64_t n_edges) {
+    return align_up(4 * (size_t)std::max<int64_t>(n_edges, 1) * plan->dp, 256);
 }
 
 bool radial_args_ok(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int H) {
@@ -228,6 +237,11 @@ int e3j_radial_weights(const e3j_plan* plan, int64_t n_edges, int hidden, const 
 size_t e3j_conv_radial_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
     if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return 0;
     return radial::fwd_workspace(plan, n_nodes, n_edges, hidden);
+}
+
+size_t e3j_conv_radial_fwd_least_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
+    if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return 0;
+    return radial::fwd_least_workspace(plan, n_nodes, n_edges, hidden);
 }
 
 size_t e3j_conv_radial_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
@@ -310,8 +324,12 @@ int e3j_conv_radial_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, 
 
 size_t e3j_conv_radial_vec_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
     if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return 0;
-    return align_up(radial::fwd_workspace(plan, n_nodes, n_edges, hidden), 256) +
-           align_up(4 * (size_t)std::max<int64_t>(n_edges, 1) * plan->dp, 256);
+    return align_up(radial::fwd_workspace(plan, n_nodes, n_edges, hidden), 256) + radial::sh_scratch_bytes(plan, n_edges);
+}
+
+size_t e3j_conv_radial_vec_fwd_least_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
+    if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return 0;
+    return align_up(radial::fwd_least_workspace(plan, n_nodes, n_edges, hidden), 256) + radial::sh_scratch_bytes(plan, n_edges);
 }
 
 int e3j_conv_radial_vec_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden, const float* x,
@@ -321,8 +339,7 @@ int e3j_conv_radial_vec_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edg
     if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return E3J_ERR_INVALID_ARG;
     if (plan_sh_lmax(plan) < 0) return E3J_ERR_UNSUPPORTED;
     if (n_edges > 0 && !edge_vec) return E3J_ERR_INVALID_ARG;
-    // the convolution's workspace, then room for harmonics
-    const size_t sh_bytes = align_up(4 * (size_t)std::max<int64_t>(n_edges, 1) * plan->dp, 256);
+    const size_t sh_bytes = radial::sh_scratch_bytes(plan, n_edges);
     const size_t room = workspace_bytes > sh_bytes ? workspace_bytes - sh_bytes : 0;
     const size_t inner = align_up(radial::fwd_layout(plan, n_nodes, n_edges, hidden, room).total, 256);
     if (!workspace || ((uintptr_t)workspace & 255u) || workspace_bytes < inner + sh_bytes) return E3J_ERR_WORKSPACE;

@@ -306,3 +306,74 @@ def test_a_workspace_without_room_for_the_weights_gets_the_in_kernel_form(n_atom
     assert e3j.e3j_plan_device_status(plan) == 0
     assert not torch.equal(materialised, in_kernel)   # two kernels, not one
     assert (materialised - in_kernel).abs().max() < 1e-5 * materialised.abs().max()
+
+
+def _least_workspace(plan, n, e, hidden, vec=False):
+    query = e3j.e3j_conv_radial_vec_fwd_least_workspace_bytes if vec else e3j.e3j_conv_radial_fwd_least_workspace_bytes
+    return torch.empty(query(plan, n, e, hidden), dtype=torch.uint8, device=DEV)
+
+
+@pytest.mark.parametrize("n_atoms,hidden,prepared", [
+    (192, 64, True),
+    (192, 64, False),     # row pointers built in the form's own workspace
+    (648, 64, True),
+    (192, 8, True),
+    (300, 24, True),
+    (648, 32, False),
+    (None, 64, True),     # the benchmark's box, every element
+])
+def test_the_in_kernel_form_against_the_oracle(n_atoms, hidden, prepared):
+    """The forward that forms the edge weights inside the kernel, chosen by the smallest workspace: harmonics and edge
+    vectors, twice to the same bits."""
+    wl, plan, cp, x, y, h, W, _ = _radial_case(2, n_atoms, hidden)
+    n, e = wl.n_nodes, wl.n_edges
+    snd, rcv = _cuda(wl.senders), _cuda(wl.receivers)
+    dx, dy, dh, dW = _cuda(x), _cuda(y), _cuda(h), _cuda(W)
+    vec = _cuda(np.random.default_rng(3).standard_normal((e, 3)).astype(np.float32))
+    yv = e3j.e3j_harmonics_fwd(3, vec)
+    rowptr = e3j.e3j_graph_prepare(n, snd, rcv)[0] if prepared else None
+    for call, angles, oracle_y, ws in ((e3j.e3j_conv_radial_fwd, dy, y, _least_workspace(plan, n, e, hidden)),
+                                       (e3j.e3j_conv_radial_vec_fwd, vec, yv.cpu().numpy(), _least_workspace(plan, n, e, hidden, True))):
+        assert ws.numel() < 4 * e * plan.n_paths * plan.n_channels
+        out = call(plan, dx, angles, dh, dW, snd, rcv, rowptr, workspace=ws)
+        again = call(plan, dx, angles, dh, dW, snd, rcv, rowptr, workspace=ws)
+        written = call(plan, dx, angles, dh, dW, snd, rcv, rowptr)
+        torch.cuda.synchronize()
+        assert e3j.e3j_plan_device_status(plan) == 0
+        assert torch.equal(out, again) and not torch.equal(out, written)   # two kernels, not one
+        ref = oconv.conv_radial_fwd(cp, x, oracle_y, h, W, wl.senders, wl.receivers)
+        assert_blockwise_close(out.cpu().numpy(), ref, blocks_of_paths(cp.paths, "out"), what="out")
+
+
+def test_a_captured_in_kernel_form_replays_to_the_eager_bits():
+    wl, plan, cp, x, y, h, W, _ = _radial_case(2, 192, 64)
+    snd, rcv = _cuda(wl.senders), _cuda(wl.receivers)
+    dx, dy, dh, dW = _cuda(x), _cuda(y), _cuda(h), _cuda(W)
+    rowptr = e3j.e3j_graph_prepare(wl.n_nodes, snd, rcv)[0]
+    ws = _least_workspace(plan, wl.n_nodes, wl.n_edges, 64)
+    out = torch.empty((wl.n_nodes, plan.d_out, plan.n_channels), device=DEV)
+    step = lambda: e3j.e3j_conv_radial_fwd(plan, dx, dy, dh, dW, snd, rcv, rowptr, out=out, workspace=ws)
+    step()
+    torch.cuda.synchronize()
+    eager = out.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    out.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, eager)
+
+
+def test_the_binding_takes_every_workspace_that_holds_one_of_the_forms():
+    wl, plan, cp, x, y, h, W, _ = _radial_case(2, 192, 64)
+    args = plan, _cuda(x), _cuda(y), _cuda(h), _cuda(W), _cuda(wl.senders), _cuda(wl.receivers)
+    least = _least_workspace(plan, wl.n_nodes, wl.n_edges, 64)
+    full = e3j.e3j_conv_radial_fwd_workspace_bytes(plan, wl.n_nodes, wl.n_edges, 64)
+    want = e3j.e3j_conv_radial_fwd(*args)
+    for nbytes in (least.numel(), full - 1, full):
+        got = e3j.e3j_conv_radial_fwd(*args, workspace=torch.empty(nbytes, dtype=torch.uint8, device=DEV))
+        assert torch.equal(got, want) == (nbytes == full)
+        assert (got - want).abs().max() < 1e-5 * want.abs().max()
+    with pytest.raises(ValueError):
+        e3j.e3j_conv_radial_fwd(*args, workspace=least[:-256].clone())
