@@ -270,8 +270,10 @@ def _dev_ptr(t, dtype, shape, name):
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
-    c = _torch()._C
-    return c._cuda_getCurrentRawStream(c._cuda_getDevice())   # torch.cuda.current_stream() without building the object
+    torch = _torch()
+    # torch.cuda.current_stream() without building the object, where torch has the (undocumented) call for it
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
 
 
 def _workspace(nbytes: int, like, workspace, least=None):
