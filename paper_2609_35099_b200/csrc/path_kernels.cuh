@@ -441,14 +441,16 @@ node_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
 
 // Edge tiles, and up to l = 2 the node sums of grad_x in the same launch (48x(0e+1o+2e), l <= 2: 180 us against 205 us
 // one after the other).  With l = 3 the two parts' code together is too much for the instruction cache (16x(0e+1o+2e+3o),
-// 35050 edges: 338 to 431 us against 264 us), so grad_x has its own launch.
+// 35050 edges: 338 to 431 us against 264 us), so grad_x has its own launch; only where all blocks run at once do
+// the parts share one, because there each is a chain of its paths' latencies (16 nodes of degree 5, the same signature:
+// 74 -> 43 us; tensor product of 300 rows, 8x3o: 33 -> 18.5 us).
 constexpr bool one_launch(int lm) { return lm < 3; }
-template <class T, int V, int LM, bool IDENT>
+template <class T, int V, int LM, bool IDENT, bool NODES>
 __global__ void __launch_bounds__(kThreads, bwd_blocks_per_sm(LM))
 bwd_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");
-    if constexpr (one_launch(LM)) {
+    if constexpr (NODES) {
         if (blockIdx.x < a.node_blocks) {
             node_part<T, V, LM, true, IDENT>(t, a, blockIdx.x);
             return;

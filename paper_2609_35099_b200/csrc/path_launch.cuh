@@ -109,24 +109,28 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
         if (used > best) { best = used; threads = b; }
     }
     int64_t nodes = 0, tiles = 0;
+    if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);
+    bool joint = false;
     if (c.grad_x) {
         a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kBwdWarps);
-        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, one_launch(LM) ? threads : kThreads);
+        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
+        joint = tiles > 0 && (one_launch(LM) || nodes + tiles <= (int64_t)sm_count() * bwd_blocks_per_sm(LM));
+        if (!joint) nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     }
-    if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);
     if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
-    if (nodes > 0 && (!one_launch(LM) || tiles == 0)) {
-        if (one_launch(LM)) nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
-        a.group_blocks = (unsigned)(nodes / t.n_groups);
+    a.group_blocks = (unsigned)(nodes / t.n_groups);
+    if (nodes > 0 && !joint) {
         node_kernel<T, V, LM, true, IDENT><<<(unsigned)nodes, kThreads, 0, c.stream>>>(t, a);
         if (int s = after_launch()) return s;
-        nodes = 0;
     }
-    if (nodes + tiles == 0) return E3J_OK;
-    a.node_blocks = (unsigned)nodes;
-    a.group_blocks = (unsigned)(nodes / t.n_groups);
-    if (int s = allow_smem<LM>(bwd_kernel<T, V, LM, IDENT>)) return s;
-    bwd_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
+    if (tiles == 0) return E3J_OK;
+    if (int s = allow_smem<LM>(bwd_kernel<T, V, LM, IDENT, true>)) return s;
+    if (joint) {
+        a.node_blocks = (unsigned)nodes;
+        bwd_kernel<T, V, LM, IDENT, true><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
+    } else {
+        bwd_kernel<T, V, LM, IDENT, false><<<(unsigned)tiles, threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
+    }
     return after_launch();
 }
 
