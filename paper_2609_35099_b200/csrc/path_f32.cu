@@ -4,12 +4,7 @@ namespace e3j {
 namespace path {
 
 bool covers(const e3j_plan* plan, int vec) {
-    if (plan->nq % vec != 0 || plan->nq / vec > kThreads) return false;
-    for (const e3j_path_info_t& p : plan->paths)
-        if (p.l1 > 3 || p.l2 > 3 || p.L > 3) return false;
-    int extra = 0;
-    for_unread_rows(plan, [&](int, int) { ++extra; });
-    return plan->dp <= 16 && plan->P + extra <= 255;
+    return plan->path.covered && plan->nq % vec == 0 && plan->nq / vec <= kThreads;
 }
 
 int conv_fwd(const e3j_plan* plan, const Call<float>& c, bool ident) {

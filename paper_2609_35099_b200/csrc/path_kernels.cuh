@@ -22,11 +22,10 @@
 #pragma once
 #include "common.cuh"
 #include "fast/path_pairs.inc"
+#include "path_table.hpp"
 
 namespace e3j {
 namespace path {
-
-constexpr int kMaxDeg = 7;   // rows of the largest block, 2 * 3 + 1
 
 template <class T, int V> struct alignas(sizeof(T) * V) Pack { T v[V]; };
 
@@ -102,18 +101,6 @@ template <int l1, int l2, int L> struct Tri;
         }                                                                                                            \
     };
 E3J_PATH_TRIPLES(E3J_DEFINE_TRI)
-
-#define E3J_TRI_ID(l1, l2, L) ((l1) * 16 + (l2) * 4 + (L))
-constexpr uint8_t kNoPath = 255;   // a group of input rows that no path reads: nothing to add
-
-// One plan's paths in a processing order, passed by value (kernel parameters: constant-bank reads, nothing to upload).
-struct PathRec { uint8_t id, l1, L, k, x_off, y_off, out_off, pad; };
-struct PathTable {
-    int n_paths, n_groups;
-    uint8_t start[257];          // groups of paths that share the rows they are summed into
-    PathRec rec[255];
-};
-static_assert(sizeof(PathTable) < 3072, "the table travels in the kernel parameters");
 
 template <class T> struct Args {
     int64_t n_nodes, n_edges;
@@ -231,7 +218,7 @@ __device__ __forceinline__ void node_group(const PathTable& t, const Args<T>& a,
         asm volatile("" : "+r"(row_p), "+r"(step_p));
         switch (rec.id) {
 #define E3J_CASE(l1, l2, L) \
-            case E3J_TRI_ID(l1, l2, L): \
+            case tri_id(l1, l2, L): \
                 if constexpr (l1 == LO && l2 <= LM && L <= LM) { \
                     if constexpr (IDENT) {   /* one edge: nothing to sum apart */ \
                         walk_path<Tri<l1, l2, L>, T, V, true, IDENT>(a, rec, j0, j1, step_p, row_p, q, tot); \
@@ -314,7 +301,7 @@ __device__ __forceinline__ void node_part(const PathTable& t, const Args<T>& a, 
         asm volatile("" : "+r"(row_p), "+r"(step_p));   // keeps every case's address arithmetic inside the case
         switch (rec.id) {
 #define E3J_CASE(l1, l2, L) \
-            case E3J_TRI_ID(l1, l2, L): \
+            case tri_id(l1, l2, L): \
                 if constexpr (l1 <= LM && l2 <= LM && L <= LM) \
                     sum_path<Tri<l1, l2, L>, T, V, TR, IDENT>(a, rec, j0, j1, step_p, used, row_p, q, dst, p == p0); \
                 break;
@@ -381,7 +368,7 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
             for (int c = 0; c < V; ++c) dw[c] = T(0);
             switch (rec.id) {
 #define E3J_CASE(l1, l2, L) \
-                case E3J_TRI_ID(l1, l2, L): if constexpr (l1 <= LM && l2 <= LM && L <= LM) { \
+                case tri_id(l1, l2, L): if constexpr (l1 <= LM && l2 <= LM && L <= LM) { \
                     T g[2 * L + 1][V]; \
                     _Pragma("unroll") for (int i = 0; i < 2 * L + 1; ++i) \
                         load_pack<T, V>(g[i], reinterpret_cast<const T*>(at + (1 + i) * 512)); \

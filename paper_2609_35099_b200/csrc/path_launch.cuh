@@ -2,51 +2,11 @@
 #pragma once
 #include "path_kernels.cuh"
 
-#include <algorithm>
-
 #include "path_launch.hpp"
 
 namespace e3j {
 namespace path {
 namespace {
-
-// Input rows that no path reads (an irrep whose products the output filter drops), cut into groups of 7, 5, 3 or 1
-// rows: f(first row, l of a block of that size).  Their grad_x is zero.
-template <class F> void for_unread_rows(const e3j_plan* plan, F f) {
-    std::vector<char> read(plan->d, 0);
-    for (const e3j_path_info_t& p : plan->paths) std::fill_n(read.begin() + p.x_off, 2 * p.l1 + 1, 1);
-    for (int row = 0; row < plan->d;) {
-        int n = 0;
-        while (n < kMaxDeg && row + n < plan->d && !read[row + n]) ++n;
-        if (n) f(row, (n - 1) / 2);
-        row += n ? 2 * ((n - 1) / 2) + 1 : 1;
-    }
-}
-
-// Paths in plan order, grouped by output block (forward), or by input block (backward).
-PathTable table_of(const e3j_plan* plan, bool by_input) {
-    PathTable t{};
-    t.n_paths = plan->P;
-    std::vector<int> order(plan->P);
-    for (int k = 0; k < plan->P; ++k) order[k] = k;
-    auto key = [&](int k) { return by_input ? plan->paths[k].x_off : plan->paths[k].out_off; };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return key(a) < key(b); });
-    for (int p = 0; p < plan->P; ++p) {
-        const int k = order[p];
-        const e3j_path_info_t& pi = plan->paths[k];
-        t.rec[p] = PathRec{(uint8_t)E3J_TRI_ID(pi.l1, pi.l2, pi.L), (uint8_t)pi.l1, (uint8_t)pi.L, (uint8_t)k,
-                           (uint8_t)pi.x_off, (uint8_t)pi.y_off, (uint8_t)pi.out_off, 0};
-        if (p == 0 || key(k) != key(order[p - 1])) t.start[t.n_groups++] = (uint8_t)p;
-    }
-    int n = plan->P;
-    if (by_input)
-        for_unread_rows(plan, [&](int row, int l) {
-            t.rec[n] = PathRec{kNoPath, (uint8_t)l, 0, 0, (uint8_t)row, 0, 0, 0};
-            t.start[t.n_groups++] = (uint8_t)n++;
-        });
-    t.start[t.n_groups] = (uint8_t)n;
-    return t;
-}
 
 // Lanes per (node, unit, group): the edges of a node are walked by one lane while that fills the chip (`warps` per
 // SM); smaller calls give a node up to 8 lanes, of which the kernel uses as many as get kLaneEdges edges each.  Not a
@@ -73,21 +33,8 @@ inline int64_t node_blocks(int64_t n_nodes, int units, int split, int groups, in
     return (items + per_block - 1) / per_block * groups;
 }
 
-int largest_l(const e3j_plan* plan) {
-    int l = 1;
-    while ((l + 1) * (l + 1) < plan->dp) ++l;
-    for (const e3j_path_info_t& p : plan->paths) l = std::max({l, p.l1, p.l2, p.L});
-    return l;
-}
-
-template <int LM, class K> int allow_smem(K kernel) {
-    constexpr int bytes = smem_bytes<LM>(kThreads);
-    if (bytes <= 48 * 1024) return E3J_OK;
-    return cuda_status(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-}
-
 template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, const Call<T>& c) {
-    const PathTable t = table_of(plan, false);
+    const PathTable& t = plan->path.by_output;
     Args<T> a = args_of<T, V>(plan, c);
     a.ptr = c.rowptr; a.out = c.out;
     a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kFwdWarps);
@@ -99,7 +46,7 @@ template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, cons
 }
 
 template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, const Call<T>& c) {
-    const PathTable t = table_of(plan, true);
+    const PathTable& t = plan->path.by_input;
     Args<T> a = args_of<T, V>(plan, c);
     a.ptr = c.colptr; a.perm = c.sender_perm; a.out = c.grad_x; a.grad_w = c.grad_w; a.grad_sh = c.grad_sh;
     // block size: the multiple of 32 that leaves the fewest threads without an edge, the smaller of equals
@@ -124,7 +71,7 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
         if (int s = after_launch()) return s;
     }
     if (tiles == 0) return E3J_OK;
-    if (int s = allow_smem<LM>(bwd_kernel<T, V, LM, IDENT, true>)) return s;
+    static_assert(smem_bytes<LM>(kThreads) <= 48 * 1024, "more would need the kernel's attribute set");
     if (joint) {
         a.node_blocks = (unsigned)nodes;
         bwd_kernel<T, V, LM, IDENT, true><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
@@ -137,7 +84,7 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
 }  // namespace
 
 #define E3J_BY_LARGEST_L(f, T, V, IDENT)                  \
-    switch (largest_l(plan)) {                            \
+    switch (plan->path.largest_l) {                       \
         case 1: return f<T, V, 1, IDENT>(plan, c);        \
         case 2: return f<T, V, 2, IDENT>(plan, c);        \
         default: return f<T, V, 3, IDENT>(plan, c);       \

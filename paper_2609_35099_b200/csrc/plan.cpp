@@ -276,6 +276,7 @@ int build_plan(e3j_plan& plan, const char* irreps_in, int sh_lmax, const char* i
     }
     if (collapse) sig << "|collapsed";
     plan.signature = sig.str();
+    path::build_path_plan(plan, plan.path);
     return E3J_OK;
 }
 

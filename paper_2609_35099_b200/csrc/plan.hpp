@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "../../include/e3j.h"
+#include "path_table.hpp"
 
 namespace e3j {
 
@@ -53,6 +54,7 @@ struct e3j_plan {
     std::vector<e3j_path_info_t> paths;
     std::vector<e3j::Record> rec;  // sorted by (i0,i3,i1,i2)
     std::string signature;         // canonical text of (irreps_in | sh_lmax | output blocks)
+    e3j::path::PathPlan path;      // path lists of the per-path kernels
     int fast_id = -1;              // index into the specialised-kernel registry, or -1
     mutable std::mutex mu;
     mutable std::vector<e3j::DeviceTables> dev;  // one entry per device that used the plan
