@@ -243,13 +243,21 @@ def e3j_plan_records(plan: Plan):
 
 # ----------------------------------------------------------------- marshalling
 # A call's arguments are checked and converted in a few microseconds: with small graphs that is what a call costs.
-_torch_module = None
+_torch_module = _current_stream = None
+
+
+def _stream_reader(torch):
+    """A function that gives the current stream's handle: what torch.cuda.current_stream() does without building the
+    object, where torch has the (undocumented) calls for it."""
+    raw, device = (getattr(torch._C, name, None) for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    return (lambda: raw(device())) if raw and device else lambda: torch.cuda.current_stream().cuda_stream
 
 
 def _torch():
-    global _torch_module
+    global _torch_module, _current_stream
     if _torch_module is None:
         import torch
+        _current_stream = _stream_reader(torch)
         _torch_module = torch
     return _torch_module
 
@@ -270,10 +278,8 @@ def _dev_ptr(t, dtype, shape, name):
 def _stream(stream):
     if stream is not None:
         return stream.cuda_stream
-    torch = _torch()
-    # torch.cuda.current_stream() without building the object, where torch has the (undocumented) call for it
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
+    _torch()
+    return _current_stream()
 
 
 def _workspace(nbytes: int, like, workspace, least=None):
