@@ -282,11 +282,20 @@ def _stream(stream):
     return _current_stream()
 
 
-def _workspace(nbytes: int, like, workspace, least=None):
+def _as_torch_stream(stream):
+    """stream itself, or torch's view of another library's object with a cuda_stream."""
+    torch = _torch()
+    return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream)
+
+
+def _workspace(nbytes: int, like, workspace, stream, least=None):
     """The caller's workspace, or a new one of nbytes.  least(): the bytes a call also runs with, where that is less."""
     torch = _torch()
     if workspace is None:
-        return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=like.device)
+        workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=like.device)
+        if stream is not None:   # released when the call returns: not to be used again before that stream is done with it
+            workspace.record_stream(_as_torch_stream(stream))
+        return workspace
     if workspace.dtype != torch.uint8 or not workspace.is_cuda or \
             workspace.numel() < nbytes and (least is None or workspace.numel() < least()):
         raise ValueError("workspace must be a CUDA uint8 tensor of sufficient size")
@@ -321,6 +330,9 @@ def e3j_graph_prepare_padded(n_nodes: int, senders, receivers, want_transpose: b
 def e3j_graph_validate(n_nodes: int, senders, receivers, stream=None) -> int:
     """0 if the graph is usable, else the (negative) E3J_ERR_GRAPH status.  Synchronises."""
     torch = _torch()
+    if stream is not None:   # the status is cleared, written and read on that stream
+        with torch.cuda.stream(_as_torch_stream(stream)):
+            return e3j_graph_validate(n_nodes, senders, receivers)
     e = senders.numel()
     status = torch.zeros(1, dtype=torch.int32, device=senders.device)
     _check(_load().e3j_graph_validate(n_nodes, e, _dev_ptr(senders, torch.int32, (e,), "senders"),
@@ -346,7 +358,7 @@ def e3j_conv_fwd(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=None
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
     nbytes = e3j_conv_fwd_workspace_bytes(plan, n, e)
-    workspace = _workspace(nbytes, x, workspace)
+    workspace = _workspace(nbytes, x, workspace, stream)
     _check(getattr(_load(), _entry)(
         plan.handle, n, e,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
@@ -410,7 +422,7 @@ def e3j_conv_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr=None
     grad_sh = alloc(grad_sh, (e, plan.d_sh))
     grad_w = alloc(grad_w, (e, plan.n_paths, plan.n_channels))
     nbytes = e3j_conv_bwd_workspace_bytes(plan, n, e)
-    workspace = _workspace(nbytes, x, workspace)
+    workspace = _workspace(nbytes, x, workspace, stream)
     _check(getattr(_load(), _entry)(
         plan.handle, n, e,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
@@ -457,7 +469,7 @@ def e3j_conv_bwd_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr,
     s_x, s_sh = (n, plan.d_in, plan.n_channels), (e, plan.d_sh)
     s_w, s_out = (e, plan.n_paths, plan.n_channels), (n, plan.d_out, plan.n_channels)
     gg_out, g_x, g_sh, g_w = alloc(gg_out, s_out), alloc(g_x, s_x), alloc(g_sh, s_sh), alloc(g_w, s_w)
-    workspace = _workspace(e3j_conv_bwd_bwd_workspace_bytes(plan, n, e), x, workspace)
+    workspace = _workspace(e3j_conv_bwd_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
     _check(_load().e3j_conv_bwd_bwd(
         plan.handle, n, e, _dev_ptr(x, f32, s_x, "x"), _dev_ptr(sh, f32, s_sh, "sh"), _dev_ptr(w, f32, s_w, "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
@@ -506,7 +518,7 @@ def e3j_conv_radial_fwd(plan: Plan, x, sh, h, W, senders, receivers, rowptr=None
     f32, i32 = torch.float32, torch.int32
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
-    workspace = _workspace(e3j_conv_radial_fwd_workspace_bytes(plan, n, e, hidden), x, workspace,
+    workspace = _workspace(e3j_conv_radial_fwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream,
                            lambda: e3j_conv_radial_fwd_least_workspace_bytes(plan, n, e, hidden))
     _check(_load().e3j_conv_radial_fwd(
         plan.handle, n, e, hidden,
@@ -537,7 +549,7 @@ def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, r
     f32, i32 = torch.float32, torch.int32
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
-    workspace = _workspace(e3j_conv_radial_vec_fwd_workspace_bytes(plan, n, e, hidden), x, workspace,
+    workspace = _workspace(e3j_conv_radial_vec_fwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream,
                            lambda: e3j_conv_radial_vec_fwd_least_workspace_bytes(plan, n, e, hidden))
     _check(_load().e3j_conv_radial_vec_fwd(
         plan.handle, n, e, hidden,
@@ -569,7 +581,7 @@ def e3j_conv_radial_bwd(plan: Plan, x, sh, h, W, senders, receivers, grad_out, r
     grad_sh = alloc(grad_sh, (e, plan.d_sh))
     grad_h = alloc(grad_h, (e, hidden))
     grad_W = alloc(grad_W, s_w)
-    workspace = _workspace(e3j_conv_radial_bwd_workspace_bytes(plan, n, e, hidden), x, workspace)
+    workspace = _workspace(e3j_conv_radial_bwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream)
     _check(_load().e3j_conv_radial_bwd(
         plan.handle, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
@@ -608,7 +620,7 @@ def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, g
     grad_vec = alloc(grad_vec, (e, 3))
     grad_h = alloc(grad_h, (e, hidden))
     grad_W = alloc(grad_W, s_w)
-    workspace = _workspace(e3j_conv_radial_vec_bwd_workspace_bytes(plan, n, e, hidden), x, workspace)
+    workspace = _workspace(e3j_conv_radial_vec_bwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream)
     _check(_load().e3j_conv_radial_vec_bwd(
         plan.handle, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
@@ -694,7 +706,7 @@ def e3j_conv_bwd_scheduled(plan: Plan, x, sh, w, schedule, grad_out, grad_x=None
         grad_sh = torch.empty((e, plan.d_sh), dtype=f32, device=x.device)
     if grad_w is None:
         grad_w = torch.empty((e, plan.n_paths, plan.n_channels), dtype=f32, device=x.device)
-    workspace = _workspace(e3j_conv_bwd_workspace_bytes(plan, n, e), x, workspace)
+    workspace = _workspace(e3j_conv_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
     if schedule.dtype != torch.uint8 or not schedule.is_cuda:
         raise ValueError("schedule must be the CUDA uint8 tensor returned by e3j_bwd_schedule_build")
     _check(_load().e3j_conv_bwd_scheduled(
@@ -746,7 +758,7 @@ def e3j_conv_vec_fwd(plan: Plan, x, edge_vec, w, senders, receivers, rowptr=None
     f32, i32 = torch.float32, torch.int32
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
-    workspace = _workspace(e3j_conv_vec_fwd_workspace_bytes(plan, n, e), x, workspace)
+    workspace = _workspace(e3j_conv_vec_fwd_workspace_bytes(plan, n, e), x, workspace, stream)
     _check(_load().e3j_conv_vec_fwd(
         plan.handle, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"), _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
@@ -771,7 +783,7 @@ def e3j_conv_vec_bwd(plan: Plan, x, edge_vec, w, senders, receivers, grad_out, r
     grad_x = alloc(grad_x, (n, plan.d_in, plan.n_channels))
     grad_vec = alloc(grad_vec, (e, 3))
     grad_w = alloc(grad_w, (e, plan.n_paths, plan.n_channels))
-    workspace = _workspace(e3j_conv_vec_bwd_workspace_bytes(plan, n, e), x, workspace)
+    workspace = _workspace(e3j_conv_vec_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
     _check(_load().e3j_conv_vec_bwd(
         plan.handle, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"), _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
@@ -791,7 +803,7 @@ def e3j_conv_fwd_f64(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=
     n, e, f64, i32 = x.shape[0], senders.numel(), torch.float64, torch.int32
     if out is None:
         out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f64, device=x.device)
-    ws = _workspace(int(_load().e3j_conv_f64_workspace_bytes(plan.handle, n, e)), x, None)
+    ws = _workspace(int(_load().e3j_conv_f64_workspace_bytes(plan.handle, n, e)), x, None, stream)
     _check(_load().e3j_conv_fwd_f64(
         plan.handle, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f64, (e, plan.n_paths, plan.n_channels), "w"), _dev_ptr(senders, i32, (e,), "senders"),
@@ -808,7 +820,7 @@ def e3j_conv_bwd_f64(plan: Plan, x, sh, w, senders, receivers, grad_out, sender_
     gx = torch.empty((n, plan.d_in, plan.n_channels), dtype=f64, device=x.device)
     gsh = torch.empty((e, plan.d_sh), dtype=f64, device=x.device)
     gw = torch.empty((e, plan.n_paths, plan.n_channels), dtype=f64, device=x.device)
-    ws = _workspace(int(_load().e3j_conv_f64_workspace_bytes(plan.handle, n, e)), x, None)
+    ws = _workspace(int(_load().e3j_conv_f64_workspace_bytes(plan.handle, n, e)), x, None, stream)
     _check(_load().e3j_conv_bwd_f64(
         plan.handle, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f64, (e, plan.n_paths, plan.n_channels), "w"), _dev_ptr(senders, i32, (e,), "senders"),
@@ -824,6 +836,9 @@ def e3j_shard_prepare(n_nodes: int, node_lo: int, node_hi: int, senders, receive
     for its slice of the edge list (global ids in).  halo_ids (ascending global ids) is cut to its length, which
     costs one device-to-host read of the count."""
     torch = _torch()
+    if stream is not None:   # the count is cleared, written and read on that stream
+        with torch.cuda.stream(_as_torch_stream(stream)):
+            return e3j_shard_prepare(n_nodes, node_lo, node_hi, senders, receivers)
     e, i32 = senders.numel(), torch.int32
     dev = senders.device
     ls = torch.empty(max(e, 1), dtype=i32, device=dev)
