@@ -7,14 +7,15 @@
 // per output row, and no coefficient record is ever fetched.
 //
 //   node sums  (forward; grad_x with the tensor transposed and the edges in sender order): one thread owns V channels
-//              of one node and one output block, 2L+1 accumulators, edges in list order;
+//              of one node and one block of rows, edges in list order; a node of many edges has several threads where the
+//              nodes are few;
 //   edge part  (grad_w, grad_sh): one thread owns V channels of one edge and walks all paths; grad_sh's channel sum
 //              goes through shared memory in a fixed order.
 //
-// What bounds them: the latency of the row loads at 20 to 28 warps per SM (issue slots 30-40 % busy, DRAM below 20 %),
-// not arithmetic or bandwidth.  48x(0e+1o+2e), l <= 2, 35050 edges: forward 243 -> 71 us, backward 823 -> 179 us
-// against the table-driven kernels; float64, 64x(0e+1o), l <= 2, 10176 edges, both passes: 705 -> 105 us.  Tried and
-// slower: weights and ids two steps ahead in registers (spills, 378 against 284 us for both passes), each path's sum
+// What bounds them: the latency of the row loads at 17 (backward) and 24 warps per SM (issue slots 50 and 41 % busy,
+// DRAM 20 %), not arithmetic or bandwidth.  48x(0e+1o+2e), l <= 2, 35 050 edges: forward 243 -> 65 us, backward 823 ->
+// 164 us against the table-driven kernels; float64, 64x(0e+1o), l <= 2, 10 176 edges, both passes: 715 -> 106 us.  Tried
+// and slower: weights and ids two steps ahead in registers (spills, 378 against 284 us for both passes), each path's sum
 // as a function of its own, grad_out rows of the next path in registers.
 //
 // Same sums as the table-driven kernels, in a fixed order, no atomics.  What stays on the table-driven ones: plans
@@ -139,7 +140,7 @@ __device__ __forceinline__ void walk_path(const Args<T>& a, const PathRec rec, c
                                          T (&acc)[TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1][V]) {
     constexpr int NI = TR ? 2 * Tr::kL + 1 : 2 * Tr::kL1 + 1, NO = TR ? 2 * Tr::kL1 + 1 : 2 * Tr::kL + 1;
     constexpr int NY = 2 * Tr::kL2 + 1;
-    constexpr int U = NI <= 3 ? 2 : 1;   // edges in flight: their input rows fill at most 28 registers
+    constexpr int U = NI <= 3 ? 2 : 1;   // edges in flight: with three input rows or fewer two fit, with w and y of each
     const T* in_base = (TR ? a.g + (size_t)rec.out_off * row : a.x + (size_t)rec.x_off * row) + q * V;
     const T* w_base = a.w + (size_t)rec.k * row + q * V;
     const size_t in_stride = (size_t)(TR ? a.D : a.d) * row, w_stride = (size_t)a.P * row;
@@ -412,16 +413,20 @@ __device__ __forceinline__ void edge_part(const PathTable& t, const Args<T>& a, 
 }
 
 // LM: the plan's largest l.  It sets the registers of a thread (an edge's input rows, harmonics and grad_out rows) and
-// with them the blocks of an SM.  Measured for 4 to 7 blocks at LM = 2: the forward gains from more warps although a
-// few values spill (99 / 95 / 71 us with 5 / 6 / 7 blocks), the backward does not (179 / 186 / 214 us).
+// with them the blocks of an SM.  LM = 2, 48x(0e+1o+2e), 35 050 edges: the forward gains from more warps although values
+// spill (99 / 95 / 71 us with 5 / 6 / 7 blocks), the backward does not (179 / 186 / 214 us).  LM = 3, geometric mean over
+// six plans of 10 to 34 paths and 16 to 20 000 nodes: forward 1.08 / 1 / 0.93 with 3 / 4 / 5 blocks (16x(0e+1o+2e+3o), 35 000
+// edges: 136 / 127 / 101 us), backward 0.97 / 1 / 1.16.  LM = 1, 96x0e: forward 1.04 / 1 / 1.02 and backward 1.06 / 1 /
+// 1.06 with 6 / 8 / 10 blocks.
 constexpr int kThreads = 128;
-constexpr int fwd_blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 7 : 8; }
+constexpr int fwd_blocks_per_sm(int lm) { return lm == 3 ? 5 : lm == 2 ? 7 : 8; }
+constexpr int grad_x_blocks_per_sm(int lm) { return lm == 3 ? 4 : fwd_blocks_per_sm(lm); }
 constexpr int bwd_blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 5 : 8; }
 template <int LM> constexpr int smem_bytes(int threads) { return threads / 32 * ring_bytes<LM>(); }
 
 // TR: the forward's sums, or grad_x on its own.
 template <class T, int V, int LM, bool TR, bool IDENT>
-__global__ void __launch_bounds__(kThreads, fwd_blocks_per_sm(LM))
+__global__ void __launch_bounds__(kThreads, TR ? grad_x_blocks_per_sm(LM) : fwd_blocks_per_sm(LM))
 node_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
     node_part<T, V, LM, TR, IDENT>(t, a, blockIdx.x);
 }

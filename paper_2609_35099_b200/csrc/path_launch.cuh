@@ -11,8 +11,8 @@ namespace {
 // Lanes per (node, unit, group): the edges of a node are walked by one lane while that fills the chip (`warps` per
 // SM); smaller calls give a node up to 8 lanes, of which the kernel uses as many as get kLaneEdges edges each.  Not a
 // function of the list's length: padding entries must not change the order of a sum.  The forward wants two lanes
-// sooner (32 warps: 79 us against 99 us with 16 on the workload of path_kernels.cuh), the backward, whose node sums
-// share the SMs with the edge tiles, does not (190 against 179 us).
+// sooner (16x(0e+1o+2e+3o), 35 000 edges: 127 us with 32 warps, 151 with 16), the backward does not (the same signature,
+// 3000 nodes of degree 1: 181 against 110 us; 48x(0e+1o+2e), 35 050 edges: 190 against 179).
 constexpr int kFwdWarps = 32, kBwdWarps = 16;
 int split_of(int64_t n_nodes, int units, int groups, int warps) {
     int s = 0;
