@@ -60,7 +60,7 @@ def test_harmonics_of_a_zero_vector_are_finite_and_empty_input_is_fine():
 
 
 @pytest.mark.parametrize("config,n_atoms,flags", [
-    (1, None, 0),                              # table-driven kernels: harmonics through the workspace
+    (1, None, 0),                              # per-path kernels: harmonics through the workspace
     (2, 192, 0),                               # specialised kernels: harmonics formed in the table warp
     (2, 648, 0),
     (2, 192, e3j.E3J_PLAN_GENERIC_ONLY),

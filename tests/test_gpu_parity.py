@@ -512,7 +512,7 @@ def test_workspace_errors_are_reported():
 def test_specialised_and_generic_kernels_agree_on_random_graphs(seed):
     """A cross-check beside the oracle parity tests: on random graphs (sparse rows, rows of tens of edges, hubs of
     up to 2000 edges, padded lists) and for every generated signature the specialised kernels and the
-    table-driven ones give the same forward, backward, double backward and tensor products to rounding, the
+    per-path ones give the same forward, backward, double backward and tensor products to rounding, the
     specialised backward twice the same bits."""
     rng = np.random.default_rng(seed)
     sigs = [("128x0e+128x1o", 3, None, 3), ("64x0e+64x1o", 3, None, 3), ("256x0e+256x1o", 3, None, 3),

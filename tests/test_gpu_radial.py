@@ -104,11 +104,11 @@ def run_radial_parity(wl, plan, cp, x, y, h, W, g, prepared=True):
 
 
 @pytest.mark.parametrize("config,n_atoms,hidden,flags", [
-    (1, None, 16, 0),                              # table-driven kernels, 72 weight columns
+    (1, None, 16, 0),                              # per-path kernels, 72 weight columns
     (2, 192, 64, 0),
     (2, 648, 64, 0),
     (2, 192, 64, e3j.E3J_PLAN_GENERIC_ONLY),
-    (2, 648, 64, e3j.E3J_PLAN_RADIAL_MATERIALISE),   # two-step form although the plan has the in-kernel one
+    (2, 648, 64, e3j.E3J_PLAN_RADIAL_MATERIALISE),   # the same form as by the plan's own choice
     (3, 300, 64, 0),
     (5, 3000, 32, 0),
     (2, 192, 128, 0),                              # two blocks of 64 hidden units in the gradient products
@@ -173,7 +173,7 @@ def _range_boundary_receivers(rowptr, n_ranges):
 
 
 def test_conv_radial_config5_full_size_sampled():
-    """100k atoms, 4.77 M edges: the weights (31 GB as an array) exist only inside the forward kernel.  Sampled
+    """100k atoms, 4.77 M edges: the weights (31 GB as an array, over the forward's limit) exist only inside its kernel.  Sampled
     receivers, every receiver cut by a CTA range boundary included, are recomputed by the oracle; the backward is
     checked on the sampled receivers' edges (grad_sh, grad_h), on sampled senders (grad_x) and, for grad_W and the
     whole of grad_h, by the adjoint identities <grad_W, W> = <grad_h, h> = <grad_out, out>."""

@@ -183,7 +183,7 @@ def test_every_generated_signature_fits_the_allocation_free_scratch(repo_root):
 
 def test_overlay_build_generates_kernels_for_a_signature_outside_the_list(repo_root, tmp_path):
     """build.py --signatures: a signature that is not in signatures.json gets generated kernels (tile parameters
-    chosen by the generator) in a library of its own; the committed library keeps using the table-driven ones."""
+    chosen by the generator) in a library of its own; the committed library keeps using those of plans without generated ones."""
     import json
     import subprocess
     import sys
