@@ -513,8 +513,9 @@ def main():
         del ws_d, cts, gg
 
     # ---- the same convolution with the edge weights given as the radial network's last layer (h, W) instead of w:
-    # the forward that forms them inside the kernel, beside the unfused form (tensor-core product into memory, then
-    # the plain forward), and the backward (composed: product, convolution backward, two more products)
+    # the forward as called without a workspace of one's own ("fwd"), its form that makes the weights inside the kernel
+    # ("fused", chosen by the least workspace), the two steps as separate calls ("unfused": tensor-core product into
+    # memory, then the plain forward), and the backward (composed: product, convolution backward, two more products)
     radial = None
     want_radial = (args.fused_radial or args.config in (2, 3)) and not args.no_radial
     if want_radial and not args.pad and not args.collapse and not args.generic:
@@ -523,6 +524,7 @@ def main():
         hh = torch.randn((e, H), generator=gen, device=dev)
         WW = torch.randn((H, plan.n_paths * plan.n_channels), generator=gen, device=dev) / (H ** 0.5)
         ws_rf = torch.empty(max(e3j.e3j_conv_radial_fwd_workspace_bytes(plan, n, e, H), 256), dtype=torch.uint8, device=dev)
+        ws_rk = torch.empty(max(e3j.e3j_conv_radial_fwd_least_workspace_bytes(plan, n, e, H), 256), dtype=torch.uint8, device=dev)
         ws_rb = torch.empty(max(e3j.e3j_conv_radial_bwd_workspace_bytes(plan, n, e, H), 256), dtype=torch.uint8, device=dev)
         w_mat = torch.empty((e, plan.n_paths, plan.n_channels), device=dev)
         gh, gW = torch.empty_like(hh), torch.empty_like(WW)
@@ -541,8 +543,10 @@ def main():
             return a.elapsed_time(b) / k, (e3j.e3j_launch_count() - l0) // k
 
         k_r = max(3, min(args.steps, 50))
-        rf_ms, rf_launches = timed(lambda: e3j.e3j_conv_radial_fwd(plan, d["x"], d["y"], hh, WW, d["snd"], d["rcv"], rowptr,
+        rd_ms, rd_launches = timed(lambda: e3j.e3j_conv_radial_fwd(plan, d["x"], d["y"], hh, WW, d["snd"], d["rcv"], rowptr,
                                                                     out=out, workspace=ws_rf), k_r)
+        rf_ms, rf_launches = timed(lambda: e3j.e3j_conv_radial_fwd(plan, d["x"], d["y"], hh, WW, d["snd"], d["rcv"], rowptr,
+                                                                    out=out, workspace=ws_rk), k_r)
         gemm_ms, _ = timed(lambda: e3j.e3j_radial_weights(plan, hh, WW, out=w_mat), k_r)
         plain_ms, _ = timed(lambda: conv_fwd(plan, d["x"], d["y"], w_mat, d["snd"], d["rcv"], rowptr, out=out, workspace=ws_f), k_r)
         rb_ms, rb_launches = timed(lambda: e3j.e3j_conv_radial_bwd(plan, d["x"], d["y"], hh, WW, d["snd"], d["rcv"], d["g"], rowptr,
@@ -560,11 +564,12 @@ def main():
             bf16_peak = 1590.0
         fp32_peak = 148 * 128 * 1.965e9   # FMA lanes x max SM clock (nominal unit counts)
         radial = {
-            "hidden": H, "fused_fwd_ms": rf_ms, "fused_fwd_launches": rf_launches,
+            "hidden": H, "fwd_ms": rd_ms, "fwd_launches": rd_launches, "fwd_workspace_bytes": ws_rf.numel(),
+            "fused_fwd_ms": rf_ms, "fused_fwd_launches": rf_launches, "fused_fwd_workspace_bytes": ws_rk.numel(),
             "unfused_fwd_ms": gemm_ms + plain_ms, "unfused_parts_ms": {"radial_weights": gemm_ms, "conv_fwd": plain_ms},
             "bwd_ms": rb_ms, "bwd_launches": rb_launches, "bwd_form": "composed (weights and their cotangent materialised)",
-            "fwd_edges_per_s": e / (rf_ms * 1e-3),
-            "roofline_fwd": {
+            "fwd_edges_per_s": e / (rd_ms * 1e-3),
+            "roofline_fwd": {   # of the form that makes the weights inside the kernel
                 "minimal_bytes": bytes_fwd, "hbm_GBs": bytes_fwd / (rf_ms * 1e-3) / 1e9,
                 "hbm_frac_of_measured": bytes_fwd / (rf_ms * 1e-3) / 1e9 / peak_hbm,
                 "bound": "alu", "fp32_fma_per_s": fma_conv / (rf_ms * 1e-3), "fp32_peak_fma_per_s": fp32_peak,
@@ -633,7 +638,7 @@ def main():
                              "note": "e3j_conv_radial_fwd + e3j_conv_radial_bwd from pinned host buffers, copies inside "
                                      "the timed region on streams of their own, two buffer sets"}
             del sets, results, host_res
-        del ws_rf, ws_rb, w_mat, hh, WW, gh, gW
+        del ws_rf, ws_rk, ws_rb, w_mat, hh, WW, gh, gW
 
     # ---- the backward over a processing order built once per neighbour list (runs of one sender summed in registers)
     sched_block = None
@@ -785,7 +790,7 @@ def main():
         roofs = {"fwd": roof(fb, f_ms, "e3j_conv_fwd call: fast_fwd_kernel (97 %) + fwd_fixup_kernel" if spec
                              else "e3j_conv_fwd call: path::node_kernel", "fwd"),
                  "bwd": roof(bb, b_ms, "e3j_conv_bwd call: fast_bwd1_kernel (89 %) + bwd_dx_reduce_kernel" if spec
-                             else "e3j_conv_bwd call: generic edge + node kernels", "bwd")}
+                             else "e3j_conv_bwd call: path::bwd_kernel", "bwd")}
         dominant = roofs["bwd"] if b_ms >= f_ms else roofs["fwd"]
         line = {
             "metric": "conv_fwd_bwd_edges_per_s", "value": e * world / (ms_per_step * 1e-3), "unit": "edges/s",

@@ -392,9 +392,10 @@ int e3j_conv_radial_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edg
 
 /* Float64 convolution (paper, appendix on the benchmark setup: float64 builds of the kernels are shipped beside
  * the float32 ones).  Same operation, layouts, graph arguments and conventions as e3j_conv_fwd / e3j_conv_bwd with
- * every tensor in float64 and the coupling coefficients in float64 as the plan builder computed them.  Table-driven
- * kernels for every plan (there are no signature-specialised float64 kernels): each output element is one thread's
- * sum in a fixed order, bit-identical from run to run.  No alignment requirement beyond 8 bytes.  rowptr /
+ * every tensor in float64 and the coupling coefficients in float64 as the plan builder computed them.  There are no
+ * signature-specialised float64 kernels: plans with l <= 3 and an even number of up to 256 channels run on the per-path
+ * kernels where the per-channel arrays start on 16 bytes, everything else on table-driven ones; fixed summation order,
+ * bit-identical from run to run.  No alignment requirement beyond 8 bytes.  rowptr /
  * sender_perm / colptr as produced by e3j_graph_prepare, or NULL (then derived into the workspace, 256-byte
  * aligned, e3j_conv_f64_workspace_bytes()); any of grad_x, grad_sh, grad_w may be NULL. */
 size_t e3j_conv_f64_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges);

@@ -12,7 +12,7 @@ Signatures beyond the committed list: --signatures names a JSON list of entries 
 (tile parameters optional: the generator derives what is missing from shared-memory and register fits).  Their
 kernels are generated into csrc/build/overlay/ (git-ignored) with the library that the normal build produced,
 compiled, and linked with everything else into --out (default: libe3j.so itself).  A plan with such a signature
-then selects the generated kernels like any committed one; without the overlay it runs on the table-driven ones.
+then selects the generated kernels like any committed one; without the overlay it runs on the kernels of plans without generated ones.
 """
 from __future__ import annotations
 

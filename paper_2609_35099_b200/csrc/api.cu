@@ -336,7 +336,7 @@ int e3j::conv_fwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, c
     if (n_nodes == 0) return E3J_OK;
     if (!out || !x) return E3J_ERR_INVALID_ARG;
     if (n_edges > 0 && ((!sh && !edge_vec) || !w || !senders || !receivers)) return E3J_ERR_INVALID_ARG;
-    if (edge_vec && !has_fast_forward(plan)) return E3J_ERR_UNSUPPORTED;   // the table-driven kernel reads sh
+    if (edge_vec && !has_fast_forward(plan)) return E3J_ERR_UNSUPPORTED;   // the other kernels read sh
     if (!aligned16({x, w, out})) return E3J_ERR_INVALID_ARG;
     if (padded && !rowptr) return E3J_ERR_INVALID_ARG;  // rowptr[n_nodes] is where the kernels learn the edge count
     const int32_t* n_real = padded ? rowptr + n_nodes : nullptr;

@@ -3,7 +3,7 @@
 //
 //   e3j_harmonics_fwd / _bwd   sh = Y(vec / |vec|), grad_vec = (dY/dvec)^T grad_sh; one thread per edge
 //   e3j_conv_vec_fwd           the forward convolution on edge vectors: the specialised kernels form the harmonics
-//                              in their table warp (no [E, d'] array is read or written); plans on the table-driven
+//                              in their table warp (no [E, d'] array is read or written); plans without generated
 //                              kernels get them from e3j_harmonics_fwd through the workspace
 //   e3j_conv_vec_bwd           composed: harmonics into the workspace, e3j_conv_bwd with grad_sh kept as scratch,
 //                              then the chain rule into the vectors

@@ -157,10 +157,12 @@ struct RadialLayout {
     size_t rowptr, slotptr, slot_edge, group_recv, scratch, scratch_bytes;
     bool fused;
 };
-// The forward with in-kernel edge scalars saves the [E, P, N_q] array, not time: 160 900 edges, 13 paths, 128 channels,
-// 64 hidden: 0.71 ms against 0.29 + 0.20 ms for the product and the plain forward.  So the array is formed while it is
-// no larger than this (the backward forms two of them whatever their size), and the in-kernel form takes over behind it,
-// or where the caller's workspace has no room for the array.
+// The forward with in-kernel edge scalars saves the [E, P, N_q] array, not time, at any size (13 paths, 128 channels, 64
+// hidden; in-kernel against product and plain forward): 0.23 GiB of weights 0.205 / 0.139 ms, 0.99 GiB 0.70 / 0.49, 1.97
+// GiB 1.36 / 0.95, 3.94 GiB 2.69 / 1.91, 7.88 GiB 5.35 / 3.98.  So this line is one of memory: the array is formed while
+// it is no larger, which a card of 180 GB has to spare beside a model (the backward forms two of them whatever their
+// size), and the in-kernel form takes over behind it, or where the caller's workspace has no room for the array.
+// E3J_PLAN_RADIAL_MATERIALISE lifts the line, the least workspace asks for the in-kernel form below it.
 constexpr size_t kMaterialiseBytes = (size_t)2 << 30;
 
 RadialLayout radial_layout(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int H, bool bwd, bool in_kernel = false) {
@@ -301,7 +303,7 @@ static int radial_fwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edge
         if (int st = radial::radial_weights(n_edges, hidden, plan->P * plan->nq, h, W, s, t.status, (cudaStream_t)stream))
             return st;
         if (!sh && !edge_vec) return E3J_ERR_INVALID_ARG;
-        if (!sh && !has_fast_forward(plan)) {   // the table-driven kernels read harmonics: through the caller's scratch
+        if (!sh && !has_fast_forward(plan)) {   // the other kernels read harmonics: through the caller's scratch
             if (!sh_scratch) return E3J_ERR_INVALID_ARG;
             if (int st = harmonics_fwd(plan_sh_lmax(plan), n_edges, edge_vec, sh_scratch, (cudaStream_t)stream)) return st;
             sh = sh_scratch;
