@@ -172,21 +172,20 @@ int add_into(float* dst, const float* src, size_t n, cudaStream_t st) {
     return after_launch();
 }
 
-// workspace of the double backward: [forward ws | backward ws | out-sized | x-sized | sh-sized | w-sized]
+// workspace of the double backward: [forward ws | out-sized | x-sized | sh-sized | w-sized | backward ws, to the end]
 struct DoubleBwdLayout {
-    size_t fwd, bwd, t_out, t_x, t_sh, t_w, total, fwd_bytes, bwd_bytes;
+    size_t fwd, bwd, t_out, t_x, t_sh, t_w, total, fwd_bytes;
 };
 DoubleBwdLayout dbl_layout(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     DoubleBwdLayout L{};
     L.fwd_bytes = layout(plan, n_nodes, n_edges, false).total;
-    L.bwd_bytes = layout(plan, n_nodes, n_edges, true).total;
     size_t off = 0;
     L.fwd = off; off = align_up(off + L.fwd_bytes, 256);
-    L.bwd = off; off = align_up(off + L.bwd_bytes, 256);
     L.t_out = off; off = align_up(off + 4 * (size_t)n_nodes * plan->D * plan->nq, 256);
     L.t_x = off; off = align_up(off + 4 * (size_t)n_nodes * plan->d * plan->nq, 256);
     L.t_sh = off; off = align_up(off + 4 * (size_t)n_edges * ((plan->dp + 3) / 4 * 4), 256);
     L.t_w = off; off = align_up(off + 4 * (size_t)n_edges * plan->P * plan->nq, 256);
+    L.bwd = off; off = align_up(off + layout(plan, n_nodes, n_edges, true).total, 256);
     L.total = off;
     return L;
 }
@@ -206,6 +205,12 @@ int check_workspace(const void* ws, size_t have, size_t need) {
 }
 
 }  // namespace
+
+size_t bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges) {
+    if (fast_lookup(plan) || !path::covers(plan, 4) || !path::uses_shares(plan)) return 0;
+    return align_up(4 * (size_t)n_edges * plan->d * plan->nq, 256);
+}
+
 }  // namespace e3j
 
 using namespace e3j;
@@ -316,7 +321,7 @@ size_t e3j_conv_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64
 
 size_t e3j_conv_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     if (!plan || n_nodes < 0 || n_edges < 0) return 0;
-    return layout(plan, n_nodes, n_edges, true).total;
+    return layout(plan, n_nodes, n_edges, true).total + bwd_shares_bytes(plan, n_edges);
 }
 
 }  // extern "C"
@@ -442,6 +447,8 @@ int e3j::conv_bwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, c
         c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w; c.grad_out = grad_out;
         c.senders = senders; c.receivers = receivers; c.sender_perm = sender_perm; c.colptr = colptr; c.n_real = n_real;
         c.grad_x = grad_x; c.grad_sh = grad_sh; c.grad_w = grad_w; c.stream = st;
+        const size_t room = bwd_shares_bytes(plan, n_edges);
+        if (room > 0 && workspace_bytes >= L.total + room) c.shares = (float*)(ws + L.total);
         return path::conv_bwd(plan, c, false);
     }
     DeviceTables t;
@@ -482,7 +489,7 @@ int e3j_conv_bwd_padded(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges_p
 
 size_t e3j_conv_bwd_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     if (!plan || n_nodes < 0 || n_edges < 0) return 0;
-    return dbl_layout(plan, n_nodes, n_edges).total;
+    return dbl_layout(plan, n_nodes, n_edges).total + bwd_shares_bytes(plan, n_edges);
 }
 
 int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const float* x,
@@ -502,6 +509,7 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
     cudaStream_t st = (cudaStream_t)stream;
     const DoubleBwdLayout L = dbl_layout(plan, n_nodes, n_edges);
     if (int s = check_workspace(workspace, workspace_bytes, L.total)) return s;
+    const size_t bwd_bytes = workspace_bytes - L.bwd;
     char* ws = (char*)workspace;
     float* t_out = (float*)(ws + L.t_out);
     float* t_x = (float*)(ws + L.t_x);
@@ -554,7 +562,7 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         a.senders = senders; a.receivers = receivers; a.rowptr = rowptr;
         a.sender_perm = sender_perm; a.colptr = colptr; a.grad_out = grad_out;
         a.grad_x = g_x; a.grad_sh = g_sh; a.grad_w = g_w;
-        a.workspace = ws + L.bwd + W.scratch; a.workspace_bytes = L.bwd_bytes - W.scratch; a.stream = st;
+        a.workspace = ws + L.bwd + W.scratch; a.workspace_bytes = bwd_bytes - W.scratch; a.stream = st;
         return fk->dbl_edges(a, ct_x, ct_sh, ct_w);
     }
     bool have_x = false, have_sh = false, have_w = false;
@@ -569,14 +577,14 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         float* o_sh = g_sh ? g_sh : t_sh;
         float* o_w = g_w ? g_w : t_w;
         if (int s = conv_bwd_impl(plan, n_nodes, n_edges, ct_x, sh, w, senders, receivers, rowptr, sender_perm, colptr,
-                                  grad_out, t_x, o_sh, o_w, ws + L.bwd, L.bwd_bytes, stream, false)) return s;
+                                  grad_out, t_x, o_sh, o_w, ws + L.bwd, bwd_bytes, stream, false)) return s;
         have_sh = g_sh != nullptr; have_w = g_w != nullptr;
     }
     if ((g_x || g_w) && ct_sh) {   // sh <- ct_sh: contributes to x and w
         float* o_x = g_x ? g_x : t_x;
         float* o_w = (g_w && !have_w) ? g_w : t_w;
         if (int s = conv_bwd_impl(plan, n_nodes, n_edges, x, ct_sh, w, senders, receivers, rowptr, sender_perm, colptr,
-                                  grad_out, o_x, t_sh, o_w, ws + L.bwd, L.bwd_bytes, stream, false)) return s;
+                                  grad_out, o_x, t_sh, o_w, ws + L.bwd, bwd_bytes, stream, false)) return s;
         have_x = g_x != nullptr;
         if (int s = put(g_w, t_w, have_w, n_w)) return s;
     }
@@ -584,7 +592,7 @@ int e3j_conv_bwd_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         float* o_x = (g_x && !have_x) ? g_x : t_x;
         float* o_sh = (g_sh && !have_sh) ? g_sh : t_sh;
         if (int s = conv_bwd_impl(plan, n_nodes, n_edges, x, sh, ct_w, senders, receivers, rowptr, sender_perm, colptr,
-                                  grad_out, o_x, o_sh, t_w, ws + L.bwd, L.bwd_bytes, stream, false)) return s;
+                                  grad_out, o_x, o_sh, t_w, ws + L.bwd, bwd_bytes, stream, false)) return s;
         if (int s = put(g_x, t_x, have_x, n_x)) return s;
         if (int s = put(g_sh, t_sh, have_sh, n_sh)) return s;
     }

@@ -140,9 +140,17 @@ using namespace e3j;
 
 extern "C" {
 
+// [rowptr | colptr | sender_perm | shares of grad_x (backward on the per-path kernels; used where there is room)]
+static size_t graph_bytes(int64_t n_nodes, int64_t n_edges) {
+    return 2 * align_up(4 * (size_t)(n_nodes + 1), 256) + align_up(4 * (size_t)std::max<int64_t>(n_edges, 1), 256);
+}
+static size_t shares_bytes(const e3j_plan* plan, int64_t n_edges) {
+    return path::covers(plan, 2) && path::uses_shares(plan) ? align_up(8 * (size_t)n_edges * plan->d * plan->nq, 256) : 0;
+}
+
 size_t e3j_conv_f64_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     if (!plan || n_nodes < 0 || n_edges < 0) return 0;
-    return 2 * align_up(4 * (size_t)(n_nodes + 1), 256) + align_up(4 * (size_t)std::max<int64_t>(n_edges, 1), 256);
+    return graph_bytes(n_nodes, n_edges) + shares_bytes(plan, n_edges);
 }
 
 int e3j_conv_fwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const double* x, const double* sh,
@@ -153,7 +161,7 @@ int e3j_conv_fwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
     if (!x || !out || (n_edges > 0 && (!sh || !w || !senders || !receivers))) return E3J_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     if (!rowptr) {
-        if (!workspace || ((uintptr_t)workspace & 255u) || workspace_bytes < e3j_conv_f64_workspace_bytes(plan, n_nodes, n_edges))
+        if (!workspace || ((uintptr_t)workspace & 255u) || workspace_bytes < graph_bytes(n_nodes, n_edges))
             return E3J_ERR_WORKSPACE;
         int32_t* rp = (int32_t*)workspace;
         if (int s = graph_prepare(n_nodes, n_edges, senders, receivers, rp, nullptr, nullptr, st)) return s;
@@ -182,7 +190,7 @@ int e3j_conv_bwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
     if ((sender_perm == nullptr) != (colptr == nullptr)) return E3J_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     if (grad_x && !sender_perm) {
-        if (!workspace || ((uintptr_t)workspace & 255u) || workspace_bytes < e3j_conv_f64_workspace_bytes(plan, n_nodes, n_edges))
+        if (!workspace || ((uintptr_t)workspace & 255u) || workspace_bytes < graph_bytes(n_nodes, n_edges))
             return E3J_ERR_WORKSPACE;
         char* ws = (char*)workspace;
         const size_t sec = align_up(4 * (size_t)(n_nodes + 1), 256);
@@ -196,6 +204,9 @@ int e3j_conv_bwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w; c.grad_out = grad_out;
         c.senders = senders; c.receivers = receivers; c.sender_perm = sender_perm; c.colptr = colptr;
         c.grad_x = grad_x; c.grad_sh = grad_sh; c.grad_w = grad_w; c.stream = st;
+        const size_t graph = graph_bytes(n_nodes, n_edges), room = shares_bytes(plan, n_edges);
+        if (room > 0 && workspace && ((uintptr_t)workspace & 255u) == 0 && workspace_bytes >= graph + room)
+            c.shares = (double*)((char*)workspace + graph);
         return path::conv_bwd(plan, c);
     }
     DeviceTables t;

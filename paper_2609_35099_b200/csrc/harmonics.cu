@@ -95,16 +95,17 @@ int plan_sh_lmax(const e3j_plan* plan) {
 
 namespace {
 
-// workspace of the calls on edge vectors: [convolution workspace | sh | grad_sh]
-struct VecLayout { size_t conv, conv_bytes, sh, gsh, total; };
+// workspace of the calls on edge vectors: [sh | grad_sh | convolution workspace, to the end]
+struct VecLayout { size_t sh, gsh, conv, total; };
 VecLayout vec_layout(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, bool bwd) {
     VecLayout L{};
-    L.conv_bytes = bwd ? e3j_conv_bwd_workspace_bytes(plan, n_nodes, n_edges)
-                       : e3j_conv_fwd_workspace_bytes(plan, n_nodes, n_edges);
+    const size_t conv_bytes = bwd ? e3j_conv_bwd_workspace_bytes(plan, n_nodes, n_edges) - bwd_shares_bytes(plan, n_edges)
+                                  : e3j_conv_fwd_workspace_bytes(plan, n_nodes, n_edges);
     const size_t sh_bytes = align_up(4 * (size_t)std::max<int64_t>(n_edges, 1) * plan->dp, 256);
-    size_t off = align_up(L.conv_bytes, 256);
+    size_t off = 0;
     L.sh = off; if (bwd || !has_fast_forward(plan)) off += sh_bytes;
     L.gsh = off; if (bwd) off += sh_bytes;
+    L.conv = off; off += align_up(conv_bytes, 256);
     L.total = off;
     return L;
 }
@@ -142,7 +143,7 @@ size_t e3j_conv_vec_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, i
 
 size_t e3j_conv_vec_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     if (!args_ok(plan, n_nodes, n_edges)) return 0;
-    return vec_layout(plan, n_nodes, n_edges, true).total;
+    return vec_layout(plan, n_nodes, n_edges, true).total + bwd_shares_bytes(plan, n_edges);
 }
 
 int e3j_conv_vec_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const float* x, const float* edge_vec,
@@ -157,11 +158,11 @@ int e3j_conv_vec_fwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
     char* ws = (char*)workspace;
     if (has_fast_forward(plan))
         return conv_fwd_impl(plan, n_nodes, n_edges, x, nullptr, w, senders, receivers, rowptr, out, ws + L.conv,
-                             L.conv_bytes, stream, false, edge_vec);
+                             workspace_bytes - L.conv, stream, false, edge_vec);
     float* sh = (float*)(ws + L.sh);
     if (int rc = harmonics_fwd(lmax, n_edges, edge_vec, sh, (cudaStream_t)stream)) return rc;
-    return conv_fwd_impl(plan, n_nodes, n_edges, x, sh, w, senders, receivers, rowptr, out, ws + L.conv, L.conv_bytes,
-                         stream, false);
+    return conv_fwd_impl(plan, n_nodes, n_edges, x, sh, w, senders, receivers, rowptr, out, ws + L.conv,
+                         workspace_bytes - L.conv, stream, false);
 }
 
 int e3j_conv_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const float* x, const float* edge_vec,
@@ -180,8 +181,8 @@ int e3j_conv_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
     float* gsh = (float*)(ws + L.gsh);
     if (int rc = harmonics_fwd(lmax, n_edges, edge_vec, sh, st)) return rc;
     if (int rc = conv_bwd_impl(plan, n_nodes, n_edges, x, sh, w, senders, receivers, rowptr, sender_perm, colptr,
-                               grad_out, grad_x, grad_vec ? gsh : nullptr, grad_w, ws + L.conv, L.conv_bytes, stream,
-                               false)) return rc;
+                               grad_out, grad_x, grad_vec ? gsh : nullptr, grad_w, ws + L.conv,
+                               workspace_bytes - L.conv, stream, false)) return rc;
     if (grad_vec && n_nodes > 0)
         if (int rc = harmonics_bwd(lmax, n_edges, edge_vec, gsh, grad_vec, st)) return rc;
     return E3J_OK;

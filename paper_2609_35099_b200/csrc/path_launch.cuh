@@ -13,7 +13,8 @@ namespace {
 // function of the list's length: padding entries must not change the order of a sum.  The forward wants two lanes
 // sooner (16x(0e+1o+2e+3o), 35 000 edges: 127 us with 32 warps, 151 with 16), the backward does not (the same signature,
 // 3000 nodes of degree 1: 181 against 110 us; 48x(0e+1o+2e), 35 050 edges: 190 against 179).
-constexpr int kFwdWarps = 32, kBwdWarps = 16;
+// The sum of the shares is nothing but loads: two lanes until every SM has its 64 warps.
+constexpr int kFwdWarps = 32, kBwdWarps = 16, kShareWarps = 64;
 int split_of(int64_t n_nodes, int units, int groups, int warps) {
     int s = 0;
     while (s < 3 && (n_nodes * units * groups << s) < (int64_t)sm_count() * warps * 32) ++s;
@@ -34,14 +35,16 @@ inline int64_t node_blocks(int64_t n_nodes, int units, int split, int groups, in
 }
 
 template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, const Call<T>& c) {
-    const PathTable& t = plan->path.by_output;
+    const bool pairs = !plan->path.shared_rows;
+    const PathTable& t = pairs ? plan->path.by_pair : plan->path.by_output;
     Args<T> a = args_of<T, V>(plan, c);
     a.ptr = c.rowptr; a.out = c.out;
     a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kFwdWarps);
     const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
     a.group_blocks = (unsigned)(blocks / t.n_groups);
-    node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
+    if (pairs) pair_kernel<T, V, LM, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
+    else node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
     return after_launch();
 }
 
@@ -49,36 +52,45 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     const PathTable& t = plan->path.by_input;
     Args<T> a = args_of<T, V>(plan, c);
     a.ptr = c.colptr; a.perm = c.sender_perm; a.out = c.grad_x; a.grad_w = c.grad_w; a.grad_sh = c.grad_sh;
+    const EdgeTable& et = sizeof(T) == 8 ? plan->path.edges_f64 : plan->path.edges_f32;
+    const bool edges = (c.grad_w || c.grad_sh) && c.n_edges > 0;
+    const bool from_shares = c.grad_x && edges && (IDENT || c.shares);
     // block size: the multiple of 32 that leaves the fewest threads without an edge, the smaller of equals
     int threads = kThreads, best = 0;
     for (int b = 64; b <= kThreads; b += 32) {
         const int used = 1024 * (b / a.units * a.units) / b;
         if (used > best) { best = used; threads = b; }
     }
-    int64_t nodes = 0, tiles = 0;
-    if (c.grad_w || c.grad_sh) tiles = (c.n_edges + threads / a.units - 1) / (threads / a.units);
-    bool joint = false;
-    if (c.grad_x) {
+    const int64_t tiles = edges ? (c.n_edges + threads / a.units - 1) / (threads / a.units) : 0;
+    static_assert(smem_bytes<LM>(kThreads) <= 48 * 1024, "more would need the kernel's attribute set");
+    if (c.grad_x && !from_shares) {
         a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kBwdWarps);
-        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
-        joint = tiles > 0 && (one_launch(LM) || nodes + tiles <= (int64_t)sm_count() * bwd_blocks_per_sm(LM));
-        if (!joint) nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
-    }
-    if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
-    a.group_blocks = (unsigned)(nodes / t.n_groups);
-    if (nodes > 0 && !joint) {
+        int64_t nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
+        if (tiles > 0 && (one_launch(LM) || nodes + tiles <= (int64_t)sm_count() * joint_blocks_per_sm(LM))) {
+            if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+            a.group_blocks = (unsigned)(nodes / t.n_groups);
+            a.node_blocks = (unsigned)nodes;
+            joint_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, et, a);
+            return after_launch();
+        }
+        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
+        if (nodes >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+        a.group_blocks = (unsigned)(nodes / t.n_groups);
         node_kernel<T, V, LM, true, IDENT><<<(unsigned)nodes, kThreads, 0, c.stream>>>(t, a);
         if (int s = after_launch()) return s;
     }
-    if (tiles == 0) return E3J_OK;
-    static_assert(smem_bytes<LM>(kThreads) <= 48 * 1024, "more would need the kernel's attribute set");
-    if (joint) {
-        a.node_blocks = (unsigned)nodes;
-        bwd_kernel<T, V, LM, IDENT, true><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
-    } else {
-        bwd_kernel<T, V, LM, IDENT, false><<<(unsigned)tiles, threads, smem_bytes<LM>(threads), c.stream>>>(t, a);
+    if (tiles > 0) {
+        if (tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+        a.dx = !from_shares ? nullptr : IDENT ? c.grad_x : c.shares;
+        edge_kernel<T, V, LM, IDENT><<<(unsigned)tiles, threads, smem_bytes<LM>(threads), c.stream>>>(et, a);
+        if (int s = after_launch()) return s;
     }
-    return after_launch();
+    if (!from_shares || IDENT) return E3J_OK;
+    a.dx = c.shares;
+    a.split_log2 = split_of(c.n_nodes, a.d * a.units, 1, kShareWarps);
+    const int64_t blocks = node_blocks(c.n_nodes, a.d * a.units, a.split_log2, 1, kThreads);
+    if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+    return launch_dependent(share_sum_kernel<T, V>, dim3((unsigned)blocks), dim3(kThreads), 0, c.stream, a);
 }
 
 }  // namespace

@@ -150,10 +150,10 @@ const FastKernels* fused_forward(const e3j_plan* plan, int H) {
     return (fk && fk->radial_fwd && fk->fwd_scratch_bytes && H % 8 == 0 && H <= fast::kMaxHidden) ? fk : nullptr;
 }
 
-// workspace of the composed calls: [conv workspace | s | grad_s | layer partials]; of the forward with in-kernel
+// workspace of the composed calls: [s | grad_s | layer partials | conv workspace, to the end]; of the forward with in-kernel
 // edge scalars: [rowptr | slotptr | slot_edge | group_recv | boundary-row scratch]
 struct RadialLayout {
-    size_t conv, s, gs, partial, total, conv_bytes;
+    size_t conv, s, gs, partial, total;
     size_t rowptr, slotptr, slot_edge, group_recv, scratch, scratch_bytes;
     bool fused;
 };
@@ -183,12 +183,12 @@ RadialLayout radial_layout(const e3j_plan* plan, int64_t n_nodes, int64_t n_edge
         L.total = off;
         return L;
     }
-    L.conv_bytes = bwd ? e3j_conv_bwd_workspace_bytes(plan, n_nodes, n_edges)
-                       : e3j_conv_fwd_workspace_bytes(plan, n_nodes, n_edges);
-    L.conv = off; off = align_up(off + L.conv_bytes, 256);
     L.s = off; off = align_up(off + 4 * (size_t)std::max<int64_t>(n_edges, 1) * C, 256);
     L.gs = off; if (bwd) off = align_up(off + 4 * (size_t)std::max<int64_t>(n_edges, 1) * C, 256);
     L.partial = off; if (bwd) off = align_up(off + 4 * (size_t)(fast::kMaxSms) * H * C, 256);
+    const size_t conv_bytes = bwd ? e3j_conv_bwd_workspace_bytes(plan, n_nodes, n_edges) - bwd_shares_bytes(plan, n_edges)
+                                  : e3j_conv_fwd_workspace_bytes(plan, n_nodes, n_edges);
+    L.conv = off; off = align_up(off + conv_bytes, 256);
     L.total = off;
     return L;
 }
@@ -248,7 +248,7 @@ size_t e3j_conv_radial_fwd_least_workspace_bytes(const e3j_plan* plan, int64_t n
 
 size_t e3j_conv_radial_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
     if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return 0;
-    return radial::radial_layout(plan, n_nodes, n_edges, hidden, true).total;
+    return radial::radial_layout(plan, n_nodes, n_edges, hidden, true).total + bwd_shares_bytes(plan, n_edges);
 }
 
 }  // extern "C"
@@ -309,8 +309,8 @@ static int radial_fwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edge
             sh = sh_scratch;
         }
     }
-    return conv_fwd_impl(plan, n_nodes, n_edges, x, sh, s, senders, receivers, rowptr, out, ws + L.conv, L.conv_bytes,
-                         stream, false, sh ? nullptr : edge_vec);
+    return conv_fwd_impl(plan, n_nodes, n_edges, x, sh, s, senders, receivers, rowptr, out, ws + L.conv,
+                         workspace_bytes - L.conv, stream, false, sh ? nullptr : edge_vec);
 }
 
 extern "C" {
@@ -372,8 +372,8 @@ int e3j_conv_radial_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, 
     // the convolution's own backward, with the edge-scalar cotangent kept as scratch
     const bool want_gs = grad_h || grad_W;
     if (int rc = conv_bwd_impl(plan, n_nodes, n_edges, x, sh, s, senders, receivers, rowptr, sender_perm, colptr,
-                               grad_out, grad_x, grad_sh, want_gs ? gs : nullptr, ws + L.conv, L.conv_bytes, stream,
-                               false)) return rc;
+                               grad_out, grad_x, grad_sh, want_gs ? gs : nullptr, ws + L.conv, workspace_bytes - L.conv,
+                               stream, false)) return rc;
     // chain rule through s = h W
     if (grad_h)
         if (int rc = radial::grad_hidden(n_edges, hidden, C, gs, W, grad_h, t.status, st)) return rc;
@@ -384,8 +384,7 @@ int e3j_conv_radial_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, 
 
 size_t e3j_conv_radial_vec_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden) {
     if (!radial::radial_args_ok(plan, n_nodes, n_edges, hidden)) return 0;
-    return align_up(radial::radial_layout(plan, n_nodes, n_edges, hidden, true).total, 256) +
-           2 * align_up(4 * (size_t)std::max<int64_t>(n_edges, 1) * plan->dp, 256);
+    return 2 * radial::sh_scratch_bytes(plan, n_edges) + e3j_conv_radial_bwd_workspace_bytes(plan, n_nodes, n_edges, hidden);
 }
 
 int e3j_conv_radial_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, int hidden, const float* x,
@@ -397,16 +396,16 @@ int e3j_conv_radial_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edg
     const int lmax = plan_sh_lmax(plan);
     if (lmax < 0) return E3J_ERR_UNSUPPORTED;
     if (n_edges > 0 && !edge_vec) return E3J_ERR_INVALID_ARG;
-    const size_t inner = align_up(radial::radial_layout(plan, n_nodes, n_edges, hidden, true).total, 256);
-    const size_t sh_bytes = align_up(4 * (size_t)std::max<int64_t>(n_edges, 1) * plan->dp, 256);
-    if (!workspace || ((uintptr_t)workspace & 255u) || workspace_bytes < inner + 2 * sh_bytes) return E3J_ERR_WORKSPACE;
-    float* sh = (float*)((char*)workspace + inner);
-    float* gsh = (float*)((char*)workspace + inner + sh_bytes);
+    const size_t sh_bytes = radial::sh_scratch_bytes(plan, n_edges), inner = 2 * sh_bytes;   // [sh | grad_sh | inner call, to the end]
+    if (!workspace || ((uintptr_t)workspace & 255u) ||
+        workspace_bytes < inner + radial::radial_layout(plan, n_nodes, n_edges, hidden, true).total) return E3J_ERR_WORKSPACE;
+    float* sh = (float*)workspace;
+    float* gsh = (float*)((char*)workspace + sh_bytes);
     cudaStream_t st = (cudaStream_t)stream;
     if (int rc = harmonics_fwd(lmax, n_edges, edge_vec, sh, st)) return rc;
     if (int rc = e3j_conv_radial_bwd(plan, n_nodes, n_edges, hidden, x, sh, h, W, senders, receivers, rowptr, sender_perm,
-                                     colptr, grad_out, grad_x, grad_vec ? gsh : nullptr, grad_h, grad_W, workspace, inner,
-                                     stream)) return rc;
+                                     colptr, grad_out, grad_x, grad_vec ? gsh : nullptr, grad_h, grad_W,
+                                     (char*)workspace + inner, workspace_bytes - inner, stream)) return rc;
     if (grad_vec && n_nodes > 0)
         if (int rc = harmonics_bwd(lmax, n_edges, edge_vec, gsh, grad_vec, st)) return rc;
     return E3J_OK;
