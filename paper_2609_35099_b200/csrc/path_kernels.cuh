@@ -12,8 +12,7 @@
 //              (its channel sum goes through shared memory in a fixed order) and the edge's share of grad_x, which a second
 //              kernel adds up over the sender-sorted list;
 //   node sums by single output blocks: the forward of plans whose paths share output rows, and grad_x (tensor transposed,
-//              edges in sender order) where the workspace has no room for the shares, where it is all that is asked for, or
-//              where every input is scalar.
+//              edges in sender order) where the workspace has no room for the shares or where every input is scalar.
 //
 // What bounds them, 48x(0e+1o+2e), l <= 2, 35 050 edges: the edge part its instructions (90 us, 55 % of the issue slots, half
 // of them multiply-adds), the forward the latency of its row loads at 24 warps per SM (53 us, 40 % of the issue slots), the
@@ -423,7 +422,8 @@ __device__ __forceinline__ void pair_part(const PathTable& t, const Args<T>& a, 
 }
 
 // ---------------------------------------------------------------- edge part
-template <class T, int V, int LM, bool IDENT>
+// ONLY_X: the shares of grad_x and nothing else, to the same bits.
+template <class T, int V, int LM, bool IDENT, bool ONLY_X = false>
 __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, const unsigned tile, unsigned char* smem) {
     const int slots = blockDim.x / a.units, slot = threadIdx.x / a.units, q = threadIdx.x - slot * a.units;
     const int64_t e = (int64_t)tile * slots + slot;
@@ -484,7 +484,7 @@ __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, 
                 const char* at = xe + rec.x;
 #pragma unroll
                 for (int i = 0; i < ROWS; ++i) {
-                    if (i < x_rows) load_pack<T, V>(x[i], reinterpret_cast<const T*>(at));
+                    if (!ONLY_X && i < x_rows) load_pack<T, V>(x[i], reinterpret_cast<const T*>(at));
                     at += row_bytes;
                 }
             }
@@ -502,12 +502,13 @@ __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, 
                     T g[2 * L + 1][V]; \
                     _Pragma("unroll") for (int i = 0; i < 2 * L + 1; ++i) \
                         load_pack<T, V>(g[i], reinterpret_cast<const T*>(at + (1 + i) * 512)); \
-                    Tri<l1, l2, L>::template edge<T, V>(y + l2 * l2, dy + l2 * l2, x, s, g, dw, dx); \
+                    if constexpr (ONLY_X) Tri<l1, l2, L>::template sum_t<0, T, V>(y + l2 * l2, g, s, dx); \
+                    else Tri<l1, l2, L>::template edge<T, V>(y + l2 * l2, dy + l2 * l2, x, s, g, dw, dx); \
                 } break;
                 E3J_PATH_TRIPLES(E3J_CASE)
 #undef E3J_CASE
             }
-            if (a.grad_w) store_pack<T, V>(reinterpret_cast<T*>(gw + rec.w), dw);
+            if (!ONLY_X && a.grad_w) store_pack<T, V>(reinterpret_cast<T*>(gw + rec.w), dw);
         }
         put_dx();
         if (a.dx) {
@@ -523,7 +524,7 @@ __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, 
         for (int c = 0; c < V; ++c) z[c] = T(0);
         for (int k = 0; k < a.P; ++k) store_pack<T, V>(a.grad_w + ((size_t)e * a.P + k) * row + q * V, z);
     }
-    if (!a.grad_sh) return;
+    if (ONLY_X || !a.grad_sh) return;
     copies_wait<0>();
     __syncthreads();   // the rings are free: the partials take their place
     T* part = reinterpret_cast<T*>(smem);
@@ -578,12 +579,12 @@ pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
     pair_part<T, V, LM, IDENT>(t, a, blockIdx.x);
 }
 
-template <class T, int V, int LM, bool IDENT>
+template <class T, int V, int LM, bool IDENT, bool ONLY_X>
 __global__ void __launch_bounds__(kThreads, edge_blocks_per_sm<T>(LM))
 edge_kernel(const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");
-    edge_part<T, V, LM, IDENT>(et, a, blockIdx.x, smem);
+    edge_part<T, V, LM, IDENT, ONLY_X>(et, a, blockIdx.x, smem);
 }
 
 // Edge tiles, and up to l = 2 the node sums of grad_x in the same launch.  With l = 3 the two parts' code together is too

@@ -54,14 +54,14 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     a.ptr = c.colptr; a.perm = c.sender_perm; a.out = c.grad_x; a.grad_w = c.grad_w; a.grad_sh = c.grad_sh;
     const EdgeTable& et = sizeof(T) == 8 ? plan->path.edges_f64 : plan->path.edges_f32;
     const bool edges = (c.grad_w || c.grad_sh) && c.n_edges > 0;
-    const bool from_shares = c.grad_x && edges && (IDENT || c.shares);
+    const bool from_shares = c.grad_x && (IDENT ? edges : c.shares && c.n_edges > 0);
     // block size: the multiple of 32 that leaves the fewest threads without an edge, the smaller of equals
     int threads = kThreads, best = 0;
     for (int b = 64; b <= kThreads; b += 32) {
         const int used = 1024 * (b / a.units * a.units) / b;
         if (used > best) { best = used; threads = b; }
     }
-    const int64_t tiles = edges ? (c.n_edges + threads / a.units - 1) / (threads / a.units) : 0;
+    const int64_t tiles = edges || from_shares ? (c.n_edges + threads / a.units - 1) / (threads / a.units) : 0;
     static_assert(smem_bytes<LM>(kThreads) <= 48 * 1024, "more would need the kernel's attribute set");
     if (c.grad_x && !from_shares) {
         a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kBwdWarps);
@@ -82,7 +82,8 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     if (tiles > 0) {
         if (tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
         a.dx = !from_shares ? nullptr : IDENT ? c.grad_x : c.shares;
-        edge_kernel<T, V, LM, IDENT><<<(unsigned)tiles, threads, smem_bytes<LM>(threads), c.stream>>>(et, a);
+        const auto kernel = edges || IDENT ? edge_kernel<T, V, LM, IDENT, false> : edge_kernel<T, V, LM, false, true>;
+        kernel<<<(unsigned)tiles, threads, smem_bytes<LM>(threads), c.stream>>>(et, a);
         if (int s = after_launch()) return s;
     }
     if (!from_shares || IDENT) return E3J_OK;
