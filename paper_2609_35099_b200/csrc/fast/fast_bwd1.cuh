@@ -59,12 +59,19 @@ struct Bwd1Smem {
     static constexpr int X_EDGE = S::DIN * S::NQ;
     static constexpr int DM_ROW = S::D * S::NQ;     // grad_out[receiver]
     static constexpr int WIN = 32;                  // edges per metadata window; the ring holds two windows
+    // XG: the sender rows are not staged, the warp that needs one reads it from global memory (L2).  For signatures that the
+    // room lets have longer tiles, up to where the next warp would take registers away (backward, 78 000 edges of 1500 atoms):
+    // 64x(0e+1o+2e+3o) six edges instead of four, with packed arithmetic 857 -> 712 us; 64x(0e+1o) fifteen instead of ten, 154
+    // -> 140; 32x(0e+1o) fifteen instead of sixteen, 117 -> 91; 96x(0e+1o) seven instead of six, 256 -> 249.  128 and 256
+    // channels: no gain (128x(0e+1o) 252 -> 259 with eight, 128x(0e+1o+2e) 714 -> 712 with four instead of three).
+    static constexpr bool XG = !ROWS && !DBL && S::EXG;
     static constexpr size_t up(size_t v, size_t a) { return (v + a - 1) / a * a; }
     static constexpr size_t off_bar = 0;                                   // full[NS], empty[NS]
     static constexpr size_t off_join = off_bar + 16 * NS;                  // join[NS][T]: the CH warps of an edge
     static constexpr size_t off_abort = off_join + 8 * NS * T;
     static constexpr size_t off_meta = up(off_abort + 4, 16);              // int[NS][4]: first edge, n_e | last << 8, block a | block b << 8 | edges of a << 16
-    static constexpr size_t off_rcv = off_meta + 16 * NS;                  // int[2 * WIN]
+    static constexpr size_t off_tsnd = off_meta + 16 * NS;                 // int[NS][T]: senders of a tile's edges (XG)
+    static constexpr size_t off_rcv = up(off_tsnd + (XG ? 4 * NS * T : 0), 16);   // int[2 * WIN]
     static constexpr size_t off_snd = off_rcv + 4 * 2 * WIN;               // int[2 * WIN]
     static constexpr size_t off_y = off_snd + 4 * 2 * WIN;                 // float[2 * WIN][DSH]
     static constexpr size_t off_uy = off_y + 4 * 2 * WIN * S::DSH;         // float[2 * WIN][DSH] (DBL)
@@ -74,7 +81,7 @@ struct Bwd1Smem {
     static constexpr size_t st_us = st_s + 4 * (size_t)T * S_EDGE;               // (DBL)
     static constexpr size_t st_x = st_s + 4 * (size_t)NIN * T * S_EDGE;
     static constexpr size_t st_ux = st_x + 4 * (size_t)T * X_EDGE;               // (DBL)
-    static constexpr size_t st_A = st_x + 4 * (size_t)NIN * T * X_EDGE;
+    static constexpr size_t st_A = st_x + (XG ? 0 : 4 * (size_t)NIN * T * X_EDGE);
     static constexpr size_t st_B = st_A + 4 * (size_t)T * S::B_APAD;             // (DBL)
     static constexpr size_t st_dy = st_A + 4 * (size_t)NIN * T * S::B_APAD;      // float[T][CH][16] (CH > 1)
     static constexpr size_t st_dm = up(st_dy + (CH > 1 ? 4 * (size_t)T * CH * 16 : 0), 128);   // float[T][D][NQ] (ROWS)
@@ -118,7 +125,13 @@ __device__ __forceinline__ void bwd1_consumer(const BwdParams& p, unsigned char*
         if (j < n_e) {
             const unsigned char* st = smem + L::off_stage + stage * (int)L::stage_bytes;
             const int64_t e = e_begin + first + j;
-            const Vec* xs = reinterpret_cast<const Vec*>(st + L::st_x) + j * (L::X_EDGE / VW) + vlane;
+            const Vec* xs;
+            if constexpr (L::XG) {
+                const int* tsnd = reinterpret_cast<const int*>(smem + L::off_tsnd) + stage * L::T;
+                xs = reinterpret_cast<const Vec*>(p.x + (size_t)tsnd[j] * L::X_EDGE) + vlane;
+            } else {
+                xs = reinterpret_cast<const Vec*>(st + L::st_x) + j * (L::X_EDGE / VW) + vlane;
+            }
             const Vec* ss = reinterpret_cast<const Vec*>(st + L::st_s) + j * (L::S_EDGE / VW) + vlane;
             const float* As = reinterpret_cast<const float*>(st + L::st_A) + j * S::B_APAD;
             const Vec* dms = (ROWS ? reinterpret_cast<const Vec*>(st + L::st_dm) + j * (L::DM_ROW / VW)
@@ -281,7 +294,7 @@ __device__ __forceinline__ void bwd1_producer(const BwdParams& p, unsigned char*
             int* meta = reinterpret_cast<int*>(smem + L::off_meta) + 4 * stage;
             meta[0] = done; meta[1] = n_e | (last << 8); meta[2] = block_a | (block << 8) | (n_a << 16);
             // arrival and byte count in one step: the phase cannot complete before the bytes are expected
-            mbar_arrive_expect_tx(&full[stage], (uint32_t)n_e * 4u * (L::NIN * (L::S_EDGE + L::X_EDGE) + (ROWS ? L::DM_ROW : 0)) +
+            mbar_arrive_expect_tx(&full[stage], (uint32_t)n_e * 4u * (L::NIN * (L::S_EDGE + (L::XG ? 0 : L::X_EDGE)) + (ROWS ? L::DM_ROW : 0)) +
                                                     ((new_block ? 4u : 0u) + (second ? 4u : 0u)) * L::DM_ROW);
             if (n_e > 0)
                 bulk_g2s(st + L::st_s, p.w + (size_t)(e_begin + done) * L::S_EDGE, (uint32_t)n_e * 4u * L::S_EDGE,
@@ -297,7 +310,8 @@ __device__ __forceinline__ void bwd1_producer(const BwdParams& p, unsigned char*
         } else {
             if (lane < n_e) {
                 const size_t snd = (size_t)snd_ring[i & (2 * WIN - 1)];
-                bulk_g2s(st + L::st_x + (size_t)lane * 4 * L::X_EDGE, p.x + snd * L::X_EDGE, 4u * L::X_EDGE, &full[stage]);
+                if constexpr (L::XG) reinterpret_cast<int*>(smem + L::off_tsnd)[stage * T + lane] = (int)snd;
+                else bulk_g2s(st + L::st_x + (size_t)lane * 4 * L::X_EDGE, p.x + snd * L::X_EDGE, 4u * L::X_EDGE, &full[stage]);
                 if (DBL)
                     bulk_g2s(st + L::st_ux + (size_t)lane * 4 * L::X_EDGE, p.ct_x + snd * L::X_EDGE, 4u * L::X_EDGE,
                              &full[stage]);

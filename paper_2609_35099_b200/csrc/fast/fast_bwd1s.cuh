@@ -35,7 +35,7 @@ __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src_gmem)
 
 template <class S>
 struct Bwd1sSmem {
-    static constexpr int T = S::ET, NS = kSchedStages, NSLOT = kSchedSlots;
+    static constexpr int T = S::ST, NS = kSchedStages, NSLOT = kSchedSlots;
     static constexpr int VW = S::EV;
     using Vec = typename VecOf<VW>::type;
     static_assert(S::NQ == 32 * VW, "one warp per edge");
@@ -234,7 +234,7 @@ __device__ __forceinline__ void bwd1s_producer(const SchedParams& p, unsigned ch
 }
 
 template <class S>
-__global__ void __launch_bounds__((S::ET + 1) * 32, 1) fast_bwd1s_kernel(const SchedParams p) {
+__global__ void __launch_bounds__((S::ST + 1) * 32, 1) fast_bwd1s_kernel(const SchedParams p) {
     using L = Bwd1sSmem<S>;
     constexpr int T = L::T, NS = L::NS;
     static_assert(S::B_NREC <= 2, "an A slot holds at most two records");

@@ -228,7 +228,8 @@ struct Sig_s128_l3 {
     using BVec = float4;
     static constexpr int BW = 4, BT = 8, BS = 2, BC = 3, B_RMAX = 7, B_APAD = 24, B_NREC = 1;
     // edge-wise backward (one warp per edge, grad_out rows read from shared memory): edges per tile (0 = not generated), ring stages
-    static constexpr int ET = 16, ES = 2, EV = 4;
+    static constexpr int ET = 16, ES = 2, EV = 4, EXG = 0;   // EXG: sender rows not staged
+    static constexpr int ST = 16;   // columns of the scheduled backward
     // the same for the standalone tensor product: rows per ring slot (0 = not generated), ring slots
     static constexpr int ETR = 0, ESR = 3;
     // fused double backward (edge outputs): edges per tile (0 = not generated), ring stages

@@ -598,7 +598,8 @@ struct Sig_w128_l3_natural {
     using BVec = float4;
     static constexpr int BW = 4, BT = 5, BS = 2, BC = 2, B_RMAX = 12, B_APAD = 84, B_NREC = 2;
     // edge-wise backward (one warp per edge, grad_out rows read from shared memory): edges per tile (0 = not generated), ring stages
-    static constexpr int ET = 11, ES = 2, EV = 4;
+    static constexpr int ET = 11, ES = 2, EV = 4, EXG = 0;   // EXG: sender rows not staged
+    static constexpr int ST = 11;   // columns of the scheduled backward
     // the same for the standalone tensor product: rows per ring slot (0 = not generated), ring slots
     static constexpr int ETR = 0, ESR = 3;
     // fused double backward (edge outputs): edges per tile (0 = not generated), ring stages

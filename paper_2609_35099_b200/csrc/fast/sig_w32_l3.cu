@@ -355,7 +355,8 @@ struct Sig_w32_l3 {
     using BVec = float;
     static constexpr int BW = 4, BT = 8, BS = 2, BC = 2, B_RMAX = 15, B_APAD = 124, B_NREC = 2;
     // edge-wise backward (one warp per edge, grad_out rows read from shared memory): edges per tile (0 = not generated), ring stages
-    static constexpr int ET = 16, ES = 2, EV = 1;
+    static constexpr int ET = 15, ES = 2, EV = 1, EXG = 1;   // EXG: sender rows not staged
+    static constexpr int ST = 15;   // columns of the scheduled backward
     // the same for the standalone tensor product: rows per ring slot (0 = not generated), ring slots
     static constexpr int ETR = 0, ESR = 3;
     // fused double backward (edge outputs): edges per tile (0 = not generated), ring stages

@@ -784,7 +784,8 @@ struct Sig_w64_l3 {
     using BVec = float2;
     static constexpr int BW = 4, BT = 8, BS = 2, BC = 2, B_RMAX = 15, B_APAD = 124, B_NREC = 2;
     // edge-wise backward (one warp per edge, grad_out rows read from shared memory): edges per tile (0 = not generated), ring stages
-    static constexpr int ET = 10, ES = 2, EV = 2;
+    static constexpr int ET = 15, ES = 2, EV = 2, EXG = 1;   // EXG: sender rows not staged
+    static constexpr int ST = 10;   // columns of the scheduled backward
     // the same for the standalone tensor product: rows per ring slot (0 = not generated), ring slots
     static constexpr int ETR = 0, ESR = 3;
     // fused double backward (edge outputs): edges per tile (0 = not generated), ring stages
@@ -1533,724 +1534,757 @@ struct Sig_w64_l3 {
         const EVec x1 = xs[1 * NQV];
         const EVec x2 = xs[2 * NQV];
         const EVec x3 = xs[3 * NQV];
+        float2 dyv[16];
         const EVec s0 = ss[0 * NQV];  // path 0: l1=0 l2=0 -> L=0
-        const EVec sx0_0 = vmul(s0, x0);
+        const EVec sx0_0 = pmul(s0, x0);
         EVec u0_0; vzero(u0_0);
         const EVec d0_0 = dms[0 * NQV];
         const float4 a0 = *reinterpret_cast<const float4*>(As + 0);
-        vfma(u0_0, a0.x, d0_0);
-        { const float t = vdot(sx0_0, d0_0);
-          dyl[0] = 1.0f * t;
+        pfma(u0_0, a0.x, d0_0);
+        { const float2 t = pmul(sx0_0, d0_0);
+          vzero(dyv[0]);
+          pfma(dyv[0], 1.0f, t);
         }
-        EVec ds0 = vmul(x0, u0_0);
+        EVec ds0 = pmul(x0, u0_0);
         if (gw) gw[0 * NQV] = ds0;
-        dxp[0] = vmul(s0, u0_0);
+        dxp[0] = pmul(s0, u0_0);
         const EVec s1 = ss[1 * NQV];  // path 1: l1=1 l2=1 -> L=0
-        const EVec sx1_1 = vmul(s1, x1);
+        const EVec sx1_1 = pmul(s1, x1);
         EVec u1_1; vzero(u1_1);
-        const EVec sx1_2 = vmul(s1, x2);
+        const EVec sx1_2 = pmul(s1, x2);
         EVec u1_2; vzero(u1_2);
-        const EVec sx1_3 = vmul(s1, x3);
+        const EVec sx1_3 = pmul(s1, x3);
         EVec u1_3; vzero(u1_3);
         const EVec d1_1 = dms[1 * NQV];
         const float4 a8 = *reinterpret_cast<const float4*>(As + 32);
-        vfma(u1_1, a8.x, d1_1);
-        { const float t = vdot(sx1_1, d1_1);
-          dyl[1] = 0.577350259f * t;
+        pfma(u1_1, a8.x, d1_1);
+        { const float2 t = pmul(sx1_1, d1_1);
+          vzero(dyv[1]);
+          pfma(dyv[1], 0.577350259f, t);
         }
-        vfma(u1_2, a8.y, d1_1);
-        { const float t = vdot(sx1_2, d1_1);
-          dyl[2] = 0.577350259f * t;
+        pfma(u1_2, a8.y, d1_1);
+        { const float2 t = pmul(sx1_2, d1_1);
+          vzero(dyv[2]);
+          pfma(dyv[2], 0.577350259f, t);
         }
-        vfma(u1_3, a8.z, d1_1);
-        { const float t = vdot(sx1_3, d1_1);
-          dyl[3] = 0.577350259f * t;
+        pfma(u1_3, a8.z, d1_1);
+        { const float2 t = pmul(sx1_3, d1_1);
+          vzero(dyv[3]);
+          pfma(dyv[3], 0.577350259f, t);
         }
-        EVec ds1 = vmul(x1, u1_1);
-        vfma(ds1, x2, u1_2);
-        vfma(ds1, x3, u1_3);
+        EVec ds1 = pmul(x1, u1_1);
+        pfma(ds1, x2, u1_2);
+        pfma(ds1, x3, u1_3);
         if (gw) gw[1 * NQV] = ds1;
-        dxp[1] = vmul(s1, u1_1);
-        dxp[2] = vmul(s1, u1_2);
-        dxp[3] = vmul(s1, u1_3);
+        dxp[1] = pmul(s1, u1_1);
+        dxp[2] = pmul(s1, u1_2);
+        dxp[3] = pmul(s1, u1_3);
         const EVec s2 = ss[2 * NQV];  // path 2: l1=0 l2=1 -> L=1
-        const EVec sx2_0 = vmul(s2, x0);
+        const EVec sx2_0 = pmul(s2, x0);
         EVec u2_0; vzero(u2_0);
         const EVec d2_2 = dms[2 * NQV];
-        vfma(u2_0, a0.y, d2_2);
-        { const float t = vdot(sx2_0, d2_2);
-          dyl[1] = fmaf(1.0f, t, dyl[1]);
+        pfma(u2_0, a0.y, d2_2);
+        { const float2 t = pmul(sx2_0, d2_2);
+          pfma(dyv[1], 1.0f, t);
         }
         const EVec d2_3 = dms[3 * NQV];
-        vfma(u2_0, a0.z, d2_3);
-        { const float t = vdot(sx2_0, d2_3);
-          dyl[2] = fmaf(1.0f, t, dyl[2]);
+        pfma(u2_0, a0.z, d2_3);
+        { const float2 t = pmul(sx2_0, d2_3);
+          pfma(dyv[2], 1.0f, t);
         }
         const EVec d2_4 = dms[4 * NQV];
-        vfma(u2_0, a0.w, d2_4);
-        { const float t = vdot(sx2_0, d2_4);
-          dyl[3] = fmaf(1.0f, t, dyl[3]);
+        pfma(u2_0, a0.w, d2_4);
+        { const float2 t = pmul(sx2_0, d2_4);
+          pfma(dyv[3], 1.0f, t);
         }
-        EVec ds2 = vmul(x0, u2_0);
+        EVec ds2 = pmul(x0, u2_0);
         if (gw) gw[2 * NQV] = ds2;
-        vfma(dxp[0], s2, u2_0);
+        pfma(dxp[0], s2, u2_0);
         const EVec s3 = ss[3 * NQV];  // path 3: l1=1 l2=0 -> L=1
-        const EVec sx3_1 = vmul(s3, x1);
+        const EVec sx3_1 = pmul(s3, x1);
         EVec u3_1; vzero(u3_1);
-        const EVec sx3_2 = vmul(s3, x2);
+        const EVec sx3_2 = pmul(s3, x2);
         EVec u3_2; vzero(u3_2);
-        const EVec sx3_3 = vmul(s3, x3);
+        const EVec sx3_3 = pmul(s3, x3);
         EVec u3_3; vzero(u3_3);
         const EVec d3_5 = dms[5 * NQV];
         const float4 a16 = *reinterpret_cast<const float4*>(As + 64);
-        vfma(u3_1, a16.x, d3_5);
-        { const float t = vdot(sx3_1, d3_5);
-          dyl[0] = fmaf(1.0f, t, dyl[0]);
+        pfma(u3_1, a16.x, d3_5);
+        { const float2 t = pmul(sx3_1, d3_5);
+          pfma(dyv[0], 1.0f, t);
         }
         const EVec d3_6 = dms[6 * NQV];
-        vfma(u3_2, a16.y, d3_6);
-        { const float t = vdot(sx3_2, d3_6);
-          dyl[0] = fmaf(1.0f, t, dyl[0]);
+        pfma(u3_2, a16.y, d3_6);
+        { const float2 t = pmul(sx3_2, d3_6);
+          pfma(dyv[0], 1.0f, t);
         }
         const EVec d3_7 = dms[7 * NQV];
-        vfma(u3_3, a16.z, d3_7);
-        { const float t = vdot(sx3_3, d3_7);
-          dyl[0] = fmaf(1.0f, t, dyl[0]);
+        pfma(u3_3, a16.z, d3_7);
+        { const float2 t = pmul(sx3_3, d3_7);
+          pfma(dyv[0], 1.0f, t);
         }
-        EVec ds3 = vmul(x1, u3_1);
-        vfma(ds3, x2, u3_2);
-        vfma(ds3, x3, u3_3);
+        EVec ds3 = pmul(x1, u3_1);
+        pfma(ds3, x2, u3_2);
+        pfma(ds3, x3, u3_3);
         if (gw) gw[3 * NQV] = ds3;
-        vfma(dxp[1], s3, u3_1);
-        vfma(dxp[2], s3, u3_2);
-        vfma(dxp[3], s3, u3_3);
+        pfma(dxp[1], s3, u3_1);
+        pfma(dxp[2], s3, u3_2);
+        pfma(dxp[3], s3, u3_3);
         const EVec s4 = ss[4 * NQV];  // path 4: l1=1 l2=2 -> L=1
-        const EVec sx4_1 = vmul(s4, x1);
+        const EVec sx4_1 = pmul(s4, x1);
         EVec u4_1; vzero(u4_1);
-        const EVec sx4_2 = vmul(s4, x2);
+        const EVec sx4_2 = pmul(s4, x2);
         EVec u4_2; vzero(u4_2);
-        const EVec sx4_3 = vmul(s4, x3);
+        const EVec sx4_3 = pmul(s4, x3);
         EVec u4_3; vzero(u4_3);
         const EVec d4_8 = dms[8 * NQV];
         const float4 a23 = *reinterpret_cast<const float4*>(As + 92);
-        vfma(u4_1, a23.x, d4_8);
-        { const float t = vdot(sx4_1, d4_8);
-          dyl[6] = 0.316227764f * t;
-          dyl[8] = 0.547722578f * t;
+        pfma(u4_1, a23.x, d4_8);
+        { const float2 t = pmul(sx4_1, d4_8);
+          vzero(dyv[6]);
+          pfma(dyv[6], 0.316227764f, t);
+          vzero(dyv[8]);
+          pfma(dyv[8], 0.547722578f, t);
         }
         const EVec d4_9 = dms[9 * NQV];
-        vfma(u4_1, a23.w, d4_9);
-        { const float t = vdot(sx4_1, d4_9);
-          dyl[5] = -0.547722578f * t;
+        pfma(u4_1, a23.w, d4_9);
+        { const float2 t = pmul(sx4_1, d4_9);
+          vzero(dyv[5]);
+          pfma(dyv[5], -0.547722578f, t);
         }
         const EVec d4_10 = dms[10 * NQV];
         const float4 a24 = *reinterpret_cast<const float4*>(As + 96);
-        vfma(u4_1, a24.z, d4_10);
-        { const float t = vdot(sx4_1, d4_10);
-          dyl[4] = -0.547722578f * t;
+        pfma(u4_1, a24.z, d4_10);
+        { const float2 t = pmul(sx4_1, d4_10);
+          vzero(dyv[4]);
+          pfma(dyv[4], -0.547722578f, t);
         }
-        vfma(u4_2, a23.y, d4_8);
-        { const float t = vdot(sx4_2, d4_8);
-          dyl[5] = fmaf(-0.547722578f, t, dyl[5]);
+        pfma(u4_2, a23.y, d4_8);
+        { const float2 t = pmul(sx4_2, d4_8);
+          pfma(dyv[5], -0.547722578f, t);
         }
-        vfma(u4_2, a24.x, d4_9);
-        { const float t = vdot(sx4_2, d4_9);
-          dyl[6] = fmaf(-0.632455528f, t, dyl[6]);
+        pfma(u4_2, a24.x, d4_9);
+        { const float2 t = pmul(sx4_2, d4_9);
+          pfma(dyv[6], -0.632455528f, t);
         }
-        vfma(u4_2, a24.w, d4_10);
-        { const float t = vdot(sx4_2, d4_10);
-          dyl[7] = -0.547722578f * t;
+        pfma(u4_2, a24.w, d4_10);
+        { const float2 t = pmul(sx4_2, d4_10);
+          vzero(dyv[7]);
+          pfma(dyv[7], -0.547722578f, t);
         }
-        vfma(u4_3, a23.z, d4_8);
-        { const float t = vdot(sx4_3, d4_8);
-          dyl[4] = fmaf(-0.547722578f, t, dyl[4]);
+        pfma(u4_3, a23.z, d4_8);
+        { const float2 t = pmul(sx4_3, d4_8);
+          pfma(dyv[4], -0.547722578f, t);
         }
-        vfma(u4_3, a24.y, d4_9);
-        { const float t = vdot(sx4_3, d4_9);
-          dyl[7] = fmaf(-0.547722578f, t, dyl[7]);
+        pfma(u4_3, a24.y, d4_9);
+        { const float2 t = pmul(sx4_3, d4_9);
+          pfma(dyv[7], -0.547722578f, t);
         }
         const float4 a25 = *reinterpret_cast<const float4*>(As + 100);
-        vfma(u4_3, a25.x, d4_10);
-        { const float t = vdot(sx4_3, d4_10);
-          dyl[6] = fmaf(0.316227764f, t, dyl[6]);
-          dyl[8] = fmaf(-0.547722578f, t, dyl[8]);
+        pfma(u4_3, a25.x, d4_10);
+        { const float2 t = pmul(sx4_3, d4_10);
+          pfma(dyv[6], 0.316227764f, t);
+          pfma(dyv[8], -0.547722578f, t);
         }
-        EVec ds4 = vmul(x1, u4_1);
-        vfma(ds4, x2, u4_2);
-        vfma(ds4, x3, u4_3);
+        EVec ds4 = pmul(x1, u4_1);
+        pfma(ds4, x2, u4_2);
+        pfma(ds4, x3, u4_3);
         if (gw) gw[4 * NQV] = ds4;
-        vfma(dxp[1], s4, u4_1);
-        vfma(dxp[2], s4, u4_2);
-        vfma(dxp[3], s4, u4_3);
+        pfma(dxp[1], s4, u4_1);
+        pfma(dxp[2], s4, u4_2);
+        pfma(dxp[3], s4, u4_3);
         const EVec s5 = ss[5 * NQV];  // path 5: l1=1 l2=1 -> L=1
-        const EVec sx5_1 = vmul(s5, x1);
+        const EVec sx5_1 = pmul(s5, x1);
         EVec u5_1; vzero(u5_1);
-        const EVec sx5_2 = vmul(s5, x2);
+        const EVec sx5_2 = pmul(s5, x2);
         EVec u5_2; vzero(u5_2);
-        const EVec sx5_3 = vmul(s5, x3);
+        const EVec sx5_3 = pmul(s5, x3);
         EVec u5_3; vzero(u5_3);
         const EVec d5_11 = dms[11 * NQV];
-        vfma(u5_2, a16.w, d5_11);
-        { const float t = vdot(sx5_2, d5_11);
-          dyl[3] = fmaf(0.707106769f, t, dyl[3]);
+        pfma(u5_2, a16.w, d5_11);
+        { const float2 t = pmul(sx5_2, d5_11);
+          pfma(dyv[3], 0.707106769f, t);
         }
         const EVec d5_12 = dms[12 * NQV];
         const float4 a17 = *reinterpret_cast<const float4*>(As + 68);
-        vfma(u5_1, a17.y, d5_12);
-        { const float t = vdot(sx5_1, d5_12);
-          dyl[3] = fmaf(-0.707106769f, t, dyl[3]);
+        pfma(u5_1, a17.y, d5_12);
+        { const float2 t = pmul(sx5_1, d5_12);
+          pfma(dyv[3], -0.707106769f, t);
         }
         const EVec d5_13 = dms[13 * NQV];
-        vfma(u5_1, a17.w, d5_13);
-        { const float t = vdot(sx5_1, d5_13);
-          dyl[2] = fmaf(0.707106769f, t, dyl[2]);
+        pfma(u5_1, a17.w, d5_13);
+        { const float2 t = pmul(sx5_1, d5_13);
+          pfma(dyv[2], 0.707106769f, t);
         }
-        vfma(u5_3, a17.x, d5_11);
-        { const float t = vdot(sx5_3, d5_11);
-          dyl[2] = fmaf(-0.707106769f, t, dyl[2]);
+        pfma(u5_3, a17.x, d5_11);
+        { const float2 t = pmul(sx5_3, d5_11);
+          pfma(dyv[2], -0.707106769f, t);
         }
-        vfma(u5_3, a17.z, d5_12);
-        { const float t = vdot(sx5_3, d5_12);
-          dyl[1] = fmaf(0.707106769f, t, dyl[1]);
+        pfma(u5_3, a17.z, d5_12);
+        { const float2 t = pmul(sx5_3, d5_12);
+          pfma(dyv[1], 0.707106769f, t);
         }
         const float4 a18 = *reinterpret_cast<const float4*>(As + 72);
-        vfma(u5_2, a18.x, d5_13);
-        { const float t = vdot(sx5_2, d5_13);
-          dyl[1] = fmaf(-0.707106769f, t, dyl[1]);
+        pfma(u5_2, a18.x, d5_13);
+        { const float2 t = pmul(sx5_2, d5_13);
+          pfma(dyv[1], -0.707106769f, t);
         }
-        EVec ds5 = vmul(x1, u5_1);
-        vfma(ds5, x2, u5_2);
-        vfma(ds5, x3, u5_3);
+        EVec ds5 = pmul(x1, u5_1);
+        pfma(ds5, x2, u5_2);
+        pfma(ds5, x3, u5_3);
         if (gw) gw[5 * NQV] = ds5;
-        vfma(dxp[1], s5, u5_1);
-        vfma(dxp[2], s5, u5_2);
-        vfma(dxp[3], s5, u5_3);
+        pfma(dxp[1], s5, u5_1);
+        pfma(dxp[2], s5, u5_2);
+        pfma(dxp[3], s5, u5_3);
         const EVec s6 = ss[6 * NQV];  // path 6: l1=0 l2=2 -> L=2
-        const EVec sx6_0 = vmul(s6, x0);
+        const EVec sx6_0 = pmul(s6, x0);
         EVec u6_0; vzero(u6_0);
         const EVec d6_14 = dms[14 * NQV];
-        vfma(u6_0, a25.y, d6_14);
-        { const float t = vdot(sx6_0, d6_14);
-          dyl[4] = fmaf(1.0f, t, dyl[4]);
+        pfma(u6_0, a25.y, d6_14);
+        { const float2 t = pmul(sx6_0, d6_14);
+          pfma(dyv[4], 1.0f, t);
         }
         const EVec d6_15 = dms[15 * NQV];
-        vfma(u6_0, a25.z, d6_15);
-        { const float t = vdot(sx6_0, d6_15);
-          dyl[5] = fmaf(1.0f, t, dyl[5]);
+        pfma(u6_0, a25.z, d6_15);
+        { const float2 t = pmul(sx6_0, d6_15);
+          pfma(dyv[5], 1.0f, t);
         }
         const EVec d6_16 = dms[16 * NQV];
-        vfma(u6_0, a25.w, d6_16);
-        { const float t = vdot(sx6_0, d6_16);
-          dyl[6] = fmaf(1.0f, t, dyl[6]);
+        pfma(u6_0, a25.w, d6_16);
+        { const float2 t = pmul(sx6_0, d6_16);
+          pfma(dyv[6], 1.0f, t);
         }
         const EVec d6_17 = dms[17 * NQV];
         const float4 a26 = *reinterpret_cast<const float4*>(As + 104);
-        vfma(u6_0, a26.x, d6_17);
-        { const float t = vdot(sx6_0, d6_17);
-          dyl[7] = fmaf(1.0f, t, dyl[7]);
+        pfma(u6_0, a26.x, d6_17);
+        { const float2 t = pmul(sx6_0, d6_17);
+          pfma(dyv[7], 1.0f, t);
         }
         const EVec d6_18 = dms[18 * NQV];
-        vfma(u6_0, a26.y, d6_18);
-        { const float t = vdot(sx6_0, d6_18);
-          dyl[8] = fmaf(1.0f, t, dyl[8]);
+        pfma(u6_0, a26.y, d6_18);
+        { const float2 t = pmul(sx6_0, d6_18);
+          pfma(dyv[8], 1.0f, t);
         }
-        EVec ds6 = vmul(x0, u6_0);
+        EVec ds6 = pmul(x0, u6_0);
         if (gw) gw[6 * NQV] = ds6;
-        vfma(dxp[0], s6, u6_0);
+        pfma(dxp[0], s6, u6_0);
         const EVec s7 = ss[7 * NQV];  // path 7: l1=1 l2=1 -> L=2
-        const EVec sx7_1 = vmul(s7, x1);
+        const EVec sx7_1 = pmul(s7, x1);
         EVec u7_1; vzero(u7_1);
-        const EVec sx7_2 = vmul(s7, x2);
+        const EVec sx7_2 = pmul(s7, x2);
         EVec u7_2; vzero(u7_2);
-        const EVec sx7_3 = vmul(s7, x3);
+        const EVec sx7_3 = pmul(s7, x3);
         EVec u7_3; vzero(u7_3);
         const EVec d7_19 = dms[19 * NQV];
         const float4 a1 = *reinterpret_cast<const float4*>(As + 4);
-        vfma(u7_1, a1.x, d7_19);
-        { const float t = vdot(sx7_1, d7_19);
-          dyl[3] = fmaf(0.707106769f, t, dyl[3]);
+        pfma(u7_1, a1.x, d7_19);
+        { const float2 t = pmul(sx7_1, d7_19);
+          pfma(dyv[3], 0.707106769f, t);
         }
         const EVec d7_20 = dms[20 * NQV];
-        vfma(u7_1, a1.z, d7_20);
-        { const float t = vdot(sx7_1, d7_20);
-          dyl[2] = fmaf(0.707106769f, t, dyl[2]);
+        pfma(u7_1, a1.z, d7_20);
+        { const float2 t = pmul(sx7_1, d7_20);
+          pfma(dyv[2], 0.707106769f, t);
         }
         const EVec d7_21 = dms[21 * NQV];
         const float4 a2 = *reinterpret_cast<const float4*>(As + 8);
-        vfma(u7_1, a2.x, d7_21);
-        { const float t = vdot(sx7_1, d7_21);
-          dyl[1] = fmaf(-0.408248305f, t, dyl[1]);
+        pfma(u7_1, a2.x, d7_21);
+        { const float2 t = pmul(sx7_1, d7_21);
+          pfma(dyv[1], -0.408248305f, t);
         }
         const EVec d7_22 = dms[22 * NQV];
-        vfma(u7_2, a2.w, d7_22);
-        { const float t = vdot(sx7_2, d7_22);
-          dyl[3] = fmaf(0.707106769f, t, dyl[3]);
+        pfma(u7_2, a2.w, d7_22);
+        { const float2 t = pmul(sx7_2, d7_22);
+          pfma(dyv[3], 0.707106769f, t);
         }
         const EVec d7_23 = dms[23 * NQV];
         const float4 a3 = *reinterpret_cast<const float4*>(As + 12);
-        vfma(u7_1, a3.y, d7_23);
-        { const float t = vdot(sx7_1, d7_23);
-          dyl[1] = fmaf(-0.707106769f, t, dyl[1]);
+        pfma(u7_1, a3.y, d7_23);
+        { const float2 t = pmul(sx7_1, d7_23);
+          pfma(dyv[1], -0.707106769f, t);
         }
-        vfma(u7_3, a1.y, d7_19);
-        { const float t = vdot(sx7_3, d7_19);
-          dyl[1] = fmaf(0.707106769f, t, dyl[1]);
+        pfma(u7_3, a1.y, d7_19);
+        { const float2 t = pmul(sx7_3, d7_19);
+          pfma(dyv[1], 0.707106769f, t);
         }
-        vfma(u7_2, a1.w, d7_20);
-        { const float t = vdot(sx7_2, d7_20);
-          dyl[1] = fmaf(0.707106769f, t, dyl[1]);
+        pfma(u7_2, a1.w, d7_20);
+        { const float2 t = pmul(sx7_2, d7_20);
+          pfma(dyv[1], 0.707106769f, t);
         }
-        vfma(u7_2, a2.y, d7_21);
-        { const float t = vdot(sx7_2, d7_21);
-          dyl[2] = fmaf(0.816496611f, t, dyl[2]);
+        pfma(u7_2, a2.y, d7_21);
+        { const float2 t = pmul(sx7_2, d7_21);
+          pfma(dyv[2], 0.816496611f, t);
         }
-        vfma(u7_3, a3.x, d7_22);
-        { const float t = vdot(sx7_3, d7_22);
-          dyl[2] = fmaf(0.707106769f, t, dyl[2]);
+        pfma(u7_3, a3.x, d7_22);
+        { const float2 t = pmul(sx7_3, d7_22);
+          pfma(dyv[2], 0.707106769f, t);
         }
-        vfma(u7_3, a3.z, d7_23);
-        { const float t = vdot(sx7_3, d7_23);
-          dyl[3] = fmaf(0.707106769f, t, dyl[3]);
+        pfma(u7_3, a3.z, d7_23);
+        { const float2 t = pmul(sx7_3, d7_23);
+          pfma(dyv[3], 0.707106769f, t);
         }
-        vfma(u7_3, a2.z, d7_21);
-        { const float t = vdot(sx7_3, d7_21);
-          dyl[3] = fmaf(-0.408248305f, t, dyl[3]);
+        pfma(u7_3, a2.z, d7_21);
+        { const float2 t = pmul(sx7_3, d7_21);
+          pfma(dyv[3], -0.408248305f, t);
         }
-        EVec ds7 = vmul(x1, u7_1);
-        vfma(ds7, x2, u7_2);
-        vfma(ds7, x3, u7_3);
+        EVec ds7 = pmul(x1, u7_1);
+        pfma(ds7, x2, u7_2);
+        pfma(ds7, x3, u7_3);
         if (gw) gw[7 * NQV] = ds7;
-        vfma(dxp[1], s7, u7_1);
-        vfma(dxp[2], s7, u7_2);
-        vfma(dxp[3], s7, u7_3);
+        pfma(dxp[1], s7, u7_1);
+        pfma(dxp[2], s7, u7_2);
+        pfma(dxp[3], s7, u7_3);
         const EVec s8 = ss[8 * NQV];  // path 8: l1=1 l2=3 -> L=2
-        const EVec sx8_1 = vmul(s8, x1);
+        const EVec sx8_1 = pmul(s8, x1);
         EVec u8_1; vzero(u8_1);
-        const EVec sx8_2 = vmul(s8, x2);
+        const EVec sx8_2 = pmul(s8, x2);
         EVec u8_2; vzero(u8_2);
-        const EVec sx8_3 = vmul(s8, x3);
+        const EVec sx8_3 = pmul(s8, x3);
         EVec u8_3; vzero(u8_3);
         const EVec d8_24 = dms[24 * NQV];
-        vfma(u8_1, a26.z, d8_24);
-        { const float t = vdot(sx8_1, d8_24);
-          dyl[13] = 0.154303357f * t;
-          dyl[15] = 0.597614288f * t;
+        pfma(u8_1, a26.z, d8_24);
+        { const float2 t = pmul(sx8_1, d8_24);
+          vzero(dyv[13]);
+          pfma(dyv[13], 0.154303357f, t);
+          vzero(dyv[15]);
+          pfma(dyv[15], 0.597614288f, t);
         }
         const EVec d8_25 = dms[25 * NQV];
         const float4 a27 = *reinterpret_cast<const float4*>(As + 108);
-        vfma(u8_1, a27.y, d8_25);
-        { const float t = vdot(sx8_1, d8_25);
-          dyl[12] = 0.377964467f * t;
-          dyl[14] = 0.487950027f * t;
+        pfma(u8_1, a27.y, d8_25);
+        { const float2 t = pmul(sx8_1, d8_25);
+          vzero(dyv[12]);
+          pfma(dyv[12], 0.377964467f, t);
+          vzero(dyv[14]);
+          pfma(dyv[14], 0.487950027f, t);
         }
         const EVec d8_26 = dms[26 * NQV];
         const float4 a28 = *reinterpret_cast<const float4*>(As + 112);
-        vfma(u8_1, a28.x, d8_26);
-        { const float t = vdot(sx8_1, d8_26);
-          dyl[11] = -0.534522474f * t;
+        pfma(u8_1, a28.x, d8_26);
+        { const float2 t = pmul(sx8_1, d8_26);
+          vzero(dyv[11]);
+          pfma(dyv[11], -0.534522474f, t);
         }
         const EVec d8_27 = dms[27 * NQV];
-        vfma(u8_1, a28.w, d8_27);
-        { const float t = vdot(sx8_1, d8_27);
-          dyl[10] = -0.487950027f * t;
+        pfma(u8_1, a28.w, d8_27);
+        { const float2 t = pmul(sx8_1, d8_27);
+          vzero(dyv[10]);
+          pfma(dyv[10], -0.487950027f, t);
         }
         const EVec d8_28 = dms[28 * NQV];
         const float4 a29 = *reinterpret_cast<const float4*>(As + 116);
-        vfma(u8_1, a29.z, d8_28);
-        { const float t = vdot(sx8_1, d8_28);
-          dyl[9] = -0.597614288f * t;
-          dyl[11] = fmaf(-0.154303357f, t, dyl[11]);
+        pfma(u8_1, a29.z, d8_28);
+        { const float2 t = pmul(sx8_1, d8_28);
+          vzero(dyv[9]);
+          pfma(dyv[9], -0.597614288f, t);
+          pfma(dyv[11], -0.154303357f, t);
         }
-        vfma(u8_2, a26.w, d8_24);
-        { const float t = vdot(sx8_2, d8_24);
-          dyl[10] = fmaf(-0.487950027f, t, dyl[10]);
+        pfma(u8_2, a26.w, d8_24);
+        { const float2 t = pmul(sx8_2, d8_24);
+          pfma(dyv[10], -0.487950027f, t);
         }
-        vfma(u8_2, a27.z, d8_25);
-        { const float t = vdot(sx8_2, d8_25);
-          dyl[11] = fmaf(-0.617213428f, t, dyl[11]);
+        pfma(u8_2, a27.z, d8_25);
+        { const float2 t = pmul(sx8_2, d8_25);
+          pfma(dyv[11], -0.617213428f, t);
         }
-        vfma(u8_2, a28.y, d8_26);
-        { const float t = vdot(sx8_2, d8_26);
-          dyl[12] = fmaf(-0.654653668f, t, dyl[12]);
+        pfma(u8_2, a28.y, d8_26);
+        { const float2 t = pmul(sx8_2, d8_26);
+          pfma(dyv[12], -0.654653668f, t);
         }
-        vfma(u8_2, a29.x, d8_27);
-        { const float t = vdot(sx8_2, d8_27);
-          dyl[13] = fmaf(-0.617213428f, t, dyl[13]);
+        pfma(u8_2, a29.x, d8_27);
+        { const float2 t = pmul(sx8_2, d8_27);
+          pfma(dyv[13], -0.617213428f, t);
         }
-        vfma(u8_2, a29.w, d8_28);
-        { const float t = vdot(sx8_2, d8_28);
-          dyl[14] = fmaf(-0.487950027f, t, dyl[14]);
+        pfma(u8_2, a29.w, d8_28);
+        { const float2 t = pmul(sx8_2, d8_28);
+          pfma(dyv[14], -0.487950027f, t);
         }
-        vfma(u8_3, a27.x, d8_24);
-        { const float t = vdot(sx8_3, d8_24);
-          dyl[9] = fmaf(-0.597614288f, t, dyl[9]);
-          dyl[11] = fmaf(0.154303357f, t, dyl[11]);
+        pfma(u8_3, a27.x, d8_24);
+        { const float2 t = pmul(sx8_3, d8_24);
+          pfma(dyv[9], -0.597614288f, t);
+          pfma(dyv[11], 0.154303357f, t);
         }
-        vfma(u8_3, a27.w, d8_25);
-        { const float t = vdot(sx8_3, d8_25);
-          dyl[10] = fmaf(-0.487950027f, t, dyl[10]);
+        pfma(u8_3, a27.w, d8_25);
+        { const float2 t = pmul(sx8_3, d8_25);
+          pfma(dyv[10], -0.487950027f, t);
         }
-        vfma(u8_3, a28.z, d8_26);
-        { const float t = vdot(sx8_3, d8_26);
-          dyl[13] = fmaf(-0.534522474f, t, dyl[13]);
+        pfma(u8_3, a28.z, d8_26);
+        { const float2 t = pmul(sx8_3, d8_26);
+          pfma(dyv[13], -0.534522474f, t);
         }
-        vfma(u8_3, a29.y, d8_27);
-        { const float t = vdot(sx8_3, d8_27);
-          dyl[12] = fmaf(0.377964467f, t, dyl[12]);
-          dyl[14] = fmaf(-0.487950027f, t, dyl[14]);
+        pfma(u8_3, a29.y, d8_27);
+        { const float2 t = pmul(sx8_3, d8_27);
+          pfma(dyv[12], 0.377964467f, t);
+          pfma(dyv[14], -0.487950027f, t);
         }
         const float4 a30 = *reinterpret_cast<const float4*>(As + 120);
-        vfma(u8_3, a30.x, d8_28);
-        { const float t = vdot(sx8_3, d8_28);
-          dyl[13] = fmaf(0.154303357f, t, dyl[13]);
-          dyl[15] = fmaf(-0.597614288f, t, dyl[15]);
+        pfma(u8_3, a30.x, d8_28);
+        { const float2 t = pmul(sx8_3, d8_28);
+          pfma(dyv[13], 0.154303357f, t);
+          pfma(dyv[15], -0.597614288f, t);
         }
-        EVec ds8 = vmul(x1, u8_1);
-        vfma(ds8, x2, u8_2);
-        vfma(ds8, x3, u8_3);
+        EVec ds8 = pmul(x1, u8_1);
+        pfma(ds8, x2, u8_2);
+        pfma(ds8, x3, u8_3);
         if (gw) gw[8 * NQV] = ds8;
-        vfma(dxp[1], s8, u8_1);
-        vfma(dxp[2], s8, u8_2);
-        vfma(dxp[3], s8, u8_3);
+        pfma(dxp[1], s8, u8_1);
+        pfma(dxp[2], s8, u8_2);
+        pfma(dxp[3], s8, u8_3);
         const EVec s9 = ss[9 * NQV];  // path 9: l1=1 l2=2 -> L=2
-        const EVec sx9_1 = vmul(s9, x1);
+        const EVec sx9_1 = pmul(s9, x1);
         EVec u9_1; vzero(u9_1);
-        const EVec sx9_2 = vmul(s9, x2);
+        const EVec sx9_2 = pmul(s9, x2);
         EVec u9_2; vzero(u9_2);
-        const EVec sx9_3 = vmul(s9, x3);
+        const EVec sx9_3 = pmul(s9, x3);
         EVec u9_3; vzero(u9_3);
         const EVec d9_29 = dms[29 * NQV];
-        vfma(u9_1, a3.w, d9_29);
-        { const float t = vdot(sx9_1, d9_29);
-          dyl[5] = fmaf(0.408248305f, t, dyl[5]);
+        pfma(u9_1, a3.w, d9_29);
+        { const float2 t = pmul(sx9_1, d9_29);
+          pfma(dyv[5], 0.408248305f, t);
         }
         const EVec d9_30 = dms[30 * NQV];
         const float4 a4 = *reinterpret_cast<const float4*>(As + 16);
-        vfma(u9_1, a4.z, d9_30);
-        { const float t = vdot(sx9_1, d9_30);
-          dyl[4] = fmaf(-0.408248305f, t, dyl[4]);
+        pfma(u9_1, a4.z, d9_30);
+        { const float2 t = pmul(sx9_1, d9_30);
+          pfma(dyv[4], -0.408248305f, t);
         }
         const EVec d9_31 = dms[31 * NQV];
         const float4 a5 = *reinterpret_cast<const float4*>(As + 20);
-        vfma(u9_1, a5.y, d9_31);
-        { const float t = vdot(sx9_1, d9_31);
-          dyl[7] = fmaf(-0.707106769f, t, dyl[7]);
+        pfma(u9_1, a5.y, d9_31);
+        { const float2 t = pmul(sx9_1, d9_31);
+          pfma(dyv[7], -0.707106769f, t);
         }
         const EVec d9_32 = dms[32 * NQV];
-        vfma(u9_1, a5.w, d9_32);
-        { const float t = vdot(sx9_1, d9_32);
-          dyl[6] = fmaf(0.707106769f, t, dyl[6]);
-          dyl[8] = fmaf(-0.408248305f, t, dyl[8]);
+        pfma(u9_1, a5.w, d9_32);
+        { const float2 t = pmul(sx9_1, d9_32);
+          pfma(dyv[6], 0.707106769f, t);
+          pfma(dyv[8], -0.408248305f, t);
         }
         const EVec d9_33 = dms[33 * NQV];
         const float4 a6 = *reinterpret_cast<const float4*>(As + 24);
-        vfma(u9_1, a6.z, d9_33);
-        { const float t = vdot(sx9_1, d9_33);
-          dyl[7] = fmaf(0.408248305f, t, dyl[7]);
+        pfma(u9_1, a6.z, d9_33);
+        { const float2 t = pmul(sx9_1, d9_33);
+          pfma(dyv[7], 0.408248305f, t);
         }
-        vfma(u9_2, a4.x, d9_29);
-        { const float t = vdot(sx9_2, d9_29);
-          dyl[8] = fmaf(0.816496611f, t, dyl[8]);
+        pfma(u9_2, a4.x, d9_29);
+        { const float2 t = pmul(sx9_2, d9_29);
+          pfma(dyv[8], 0.816496611f, t);
         }
-        vfma(u9_2, a4.w, d9_30);
-        { const float t = vdot(sx9_2, d9_30);
-          dyl[7] = fmaf(0.408248305f, t, dyl[7]);
+        pfma(u9_2, a4.w, d9_30);
+        { const float2 t = pmul(sx9_2, d9_30);
+          pfma(dyv[7], 0.408248305f, t);
         }
-        vfma(u9_3, a5.z, d9_31);
-        { const float t = vdot(sx9_3, d9_31);
-          dyl[5] = fmaf(0.707106769f, t, dyl[5]);
+        pfma(u9_3, a5.z, d9_31);
+        { const float2 t = pmul(sx9_3, d9_31);
+          pfma(dyv[5], 0.707106769f, t);
         }
-        vfma(u9_2, a6.x, d9_32);
-        { const float t = vdot(sx9_2, d9_32);
-          dyl[5] = fmaf(-0.408248305f, t, dyl[5]);
+        pfma(u9_2, a6.x, d9_32);
+        { const float2 t = pmul(sx9_2, d9_32);
+          pfma(dyv[5], -0.408248305f, t);
         }
-        vfma(u9_2, a6.w, d9_33);
-        { const float t = vdot(sx9_2, d9_33);
-          dyl[4] = fmaf(-0.816496611f, t, dyl[4]);
+        pfma(u9_2, a6.w, d9_33);
+        { const float2 t = pmul(sx9_2, d9_33);
+          pfma(dyv[4], -0.816496611f, t);
         }
-        vfma(u9_3, a4.y, d9_29);
-        { const float t = vdot(sx9_3, d9_29);
-          dyl[7] = fmaf(-0.408248305f, t, dyl[7]);
+        pfma(u9_3, a4.y, d9_29);
+        { const float2 t = pmul(sx9_3, d9_29);
+          pfma(dyv[7], -0.408248305f, t);
         }
-        vfma(u9_3, a5.x, d9_30);
-        { const float t = vdot(sx9_3, d9_30);
-          dyl[6] = fmaf(-0.707106769f, t, dyl[6]);
-          dyl[8] = fmaf(-0.408248305f, t, dyl[8]);
+        pfma(u9_3, a5.x, d9_30);
+        { const float2 t = pmul(sx9_3, d9_30);
+          pfma(dyv[6], -0.707106769f, t);
+          pfma(dyv[8], -0.408248305f, t);
         }
-        vfma(u9_3, a6.y, d9_32);
-        { const float t = vdot(sx9_3, d9_32);
-          dyl[4] = fmaf(0.408248305f, t, dyl[4]);
+        pfma(u9_3, a6.y, d9_32);
+        { const float2 t = pmul(sx9_3, d9_32);
+          pfma(dyv[4], 0.408248305f, t);
         }
         const float4 a7 = *reinterpret_cast<const float4*>(As + 28);
-        vfma(u9_3, a7.x, d9_33);
-        { const float t = vdot(sx9_3, d9_33);
-          dyl[5] = fmaf(0.408248305f, t, dyl[5]);
+        pfma(u9_3, a7.x, d9_33);
+        { const float2 t = pmul(sx9_3, d9_33);
+          pfma(dyv[5], 0.408248305f, t);
         }
-        EVec ds9 = vmul(x1, u9_1);
-        vfma(ds9, x2, u9_2);
-        vfma(ds9, x3, u9_3);
+        EVec ds9 = pmul(x1, u9_1);
+        pfma(ds9, x2, u9_2);
+        pfma(ds9, x3, u9_3);
         if (gw) gw[9 * NQV] = ds9;
-        vfma(dxp[1], s9, u9_1);
-        vfma(dxp[2], s9, u9_2);
-        vfma(dxp[3], s9, u9_3);
+        pfma(dxp[1], s9, u9_1);
+        pfma(dxp[2], s9, u9_2);
+        pfma(dxp[3], s9, u9_3);
         const EVec s10 = ss[10 * NQV];  // path 10: l1=0 l2=3 -> L=3
-        const EVec sx10_0 = vmul(s10, x0);
+        const EVec sx10_0 = pmul(s10, x0);
         EVec u10_0; vzero(u10_0);
         const EVec d10_34 = dms[34 * NQV];
-        vfma(u10_0, a8.w, d10_34);
-        { const float t = vdot(sx10_0, d10_34);
-          dyl[9] = fmaf(1.0f, t, dyl[9]);
+        pfma(u10_0, a8.w, d10_34);
+        { const float2 t = pmul(sx10_0, d10_34);
+          pfma(dyv[9], 1.0f, t);
         }
         const EVec d10_35 = dms[35 * NQV];
         const float4 a9 = *reinterpret_cast<const float4*>(As + 36);
-        vfma(u10_0, a9.x, d10_35);
-        { const float t = vdot(sx10_0, d10_35);
-          dyl[10] = fmaf(1.0f, t, dyl[10]);
+        pfma(u10_0, a9.x, d10_35);
+        { const float2 t = pmul(sx10_0, d10_35);
+          pfma(dyv[10], 1.0f, t);
         }
         const EVec d10_36 = dms[36 * NQV];
-        vfma(u10_0, a9.y, d10_36);
-        { const float t = vdot(sx10_0, d10_36);
-          dyl[11] = fmaf(1.0f, t, dyl[11]);
+        pfma(u10_0, a9.y, d10_36);
+        { const float2 t = pmul(sx10_0, d10_36);
+          pfma(dyv[11], 1.0f, t);
         }
         const EVec d10_37 = dms[37 * NQV];
-        vfma(u10_0, a9.z, d10_37);
-        { const float t = vdot(sx10_0, d10_37);
-          dyl[12] = fmaf(1.0f, t, dyl[12]);
+        pfma(u10_0, a9.z, d10_37);
+        { const float2 t = pmul(sx10_0, d10_37);
+          pfma(dyv[12], 1.0f, t);
         }
         const EVec d10_38 = dms[38 * NQV];
-        vfma(u10_0, a9.w, d10_38);
-        { const float t = vdot(sx10_0, d10_38);
-          dyl[13] = fmaf(1.0f, t, dyl[13]);
+        pfma(u10_0, a9.w, d10_38);
+        { const float2 t = pmul(sx10_0, d10_38);
+          pfma(dyv[13], 1.0f, t);
         }
         const EVec d10_39 = dms[39 * NQV];
         const float4 a10 = *reinterpret_cast<const float4*>(As + 40);
-        vfma(u10_0, a10.x, d10_39);
-        { const float t = vdot(sx10_0, d10_39);
-          dyl[14] = fmaf(1.0f, t, dyl[14]);
+        pfma(u10_0, a10.x, d10_39);
+        { const float2 t = pmul(sx10_0, d10_39);
+          pfma(dyv[14], 1.0f, t);
         }
         const EVec d10_40 = dms[40 * NQV];
-        vfma(u10_0, a10.y, d10_40);
-        { const float t = vdot(sx10_0, d10_40);
-          dyl[15] = fmaf(1.0f, t, dyl[15]);
+        pfma(u10_0, a10.y, d10_40);
+        { const float2 t = pmul(sx10_0, d10_40);
+          pfma(dyv[15], 1.0f, t);
         }
-        EVec ds10 = vmul(x0, u10_0);
+        EVec ds10 = pmul(x0, u10_0);
         if (gw) gw[10 * NQV] = ds10;
-        vfma(dxp[0], s10, u10_0);
+        pfma(dxp[0], s10, u10_0);
         const EVec s11 = ss[11 * NQV];  // path 11: l1=1 l2=2 -> L=3
-        const EVec sx11_1 = vmul(s11, x1);
+        const EVec sx11_1 = pmul(s11, x1);
         EVec u11_1; vzero(u11_1);
-        const EVec sx11_2 = vmul(s11, x2);
+        const EVec sx11_2 = pmul(s11, x2);
         EVec u11_2; vzero(u11_2);
-        const EVec sx11_3 = vmul(s11, x3);
+        const EVec sx11_3 = pmul(s11, x3);
         EVec u11_3; vzero(u11_3);
         const EVec d11_41 = dms[41 * NQV];
-        vfma(u11_1, a18.y, d11_41);
-        { const float t = vdot(sx11_1, d11_41);
-          dyl[8] = fmaf(0.707106769f, t, dyl[8]);
+        pfma(u11_1, a18.y, d11_41);
+        { const float2 t = pmul(sx11_1, d11_41);
+          pfma(dyv[8], 0.707106769f, t);
         }
         const EVec d11_42 = dms[42 * NQV];
-        vfma(u11_1, a18.w, d11_42);
-        { const float t = vdot(sx11_1, d11_42);
-          dyl[7] = fmaf(0.577350259f, t, dyl[7]);
+        pfma(u11_1, a18.w, d11_42);
+        { const float2 t = pmul(sx11_1, d11_42);
+          pfma(dyv[7], 0.577350259f, t);
         }
         const EVec d11_43 = dms[43 * NQV];
         const float4 a19 = *reinterpret_cast<const float4*>(As + 76);
-        vfma(u11_1, a19.z, d11_43);
-        { const float t = vdot(sx11_1, d11_43);
-          dyl[6] = fmaf(0.632455528f, t, dyl[6]);
-          dyl[8] = fmaf(0.182574183f, t, dyl[8]);
+        pfma(u11_1, a19.z, d11_43);
+        { const float2 t = pmul(sx11_1, d11_43);
+          pfma(dyv[6], 0.632455528f, t);
+          pfma(dyv[8], 0.182574183f, t);
         }
         const EVec d11_44 = dms[44 * NQV];
         const float4 a20 = *reinterpret_cast<const float4*>(As + 80);
-        vfma(u11_1, a20.y, d11_44);
-        { const float t = vdot(sx11_1, d11_44);
-          dyl[5] = fmaf(-0.44721359f, t, dyl[5]);
+        pfma(u11_1, a20.y, d11_44);
+        { const float2 t = pmul(sx11_1, d11_44);
+          pfma(dyv[5], -0.44721359f, t);
         }
         const EVec d11_45 = dms[45 * NQV];
         const float4 a21 = *reinterpret_cast<const float4*>(As + 84);
-        vfma(u11_1, a21.x, d11_45);
-        { const float t = vdot(sx11_1, d11_45);
-          dyl[4] = fmaf(-0.182574183f, t, dyl[4]);
+        pfma(u11_1, a21.x, d11_45);
+        { const float2 t = pmul(sx11_1, d11_45);
+          pfma(dyv[4], -0.182574183f, t);
         }
         const EVec d11_46 = dms[46 * NQV];
-        vfma(u11_1, a21.w, d11_46);
-        { const float t = vdot(sx11_1, d11_46);
-          dyl[5] = fmaf(-0.577350259f, t, dyl[5]);
+        pfma(u11_1, a21.w, d11_46);
+        { const float2 t = pmul(sx11_1, d11_46);
+          pfma(dyv[5], -0.577350259f, t);
         }
         const EVec d11_47 = dms[47 * NQV];
         const float4 a22 = *reinterpret_cast<const float4*>(As + 88);
-        vfma(u11_1, a22.z, d11_47);
-        { const float t = vdot(sx11_1, d11_47);
-          dyl[4] = fmaf(-0.707106769f, t, dyl[4]);
+        pfma(u11_1, a22.z, d11_47);
+        { const float2 t = pmul(sx11_1, d11_47);
+          pfma(dyv[4], -0.707106769f, t);
         }
-        vfma(u11_3, a18.z, d11_41);
-        { const float t = vdot(sx11_3, d11_41);
-          dyl[4] = fmaf(0.707106769f, t, dyl[4]);
+        pfma(u11_3, a18.z, d11_41);
+        { const float2 t = pmul(sx11_3, d11_41);
+          pfma(dyv[4], 0.707106769f, t);
         }
-        vfma(u11_2, a19.x, d11_42);
-        { const float t = vdot(sx11_2, d11_42);
-          dyl[4] = fmaf(0.577350259f, t, dyl[4]);
+        pfma(u11_2, a19.x, d11_42);
+        { const float2 t = pmul(sx11_2, d11_42);
+          pfma(dyv[4], 0.577350259f, t);
         }
-        vfma(u11_2, a19.w, d11_43);
-        { const float t = vdot(sx11_2, d11_43);
-          dyl[5] = fmaf(0.730296731f, t, dyl[5]);
+        pfma(u11_2, a19.w, d11_43);
+        { const float2 t = pmul(sx11_2, d11_43);
+          pfma(dyv[5], 0.730296731f, t);
         }
-        vfma(u11_2, a20.z, d11_44);
-        { const float t = vdot(sx11_2, d11_44);
-          dyl[6] = fmaf(0.774596691f, t, dyl[6]);
+        pfma(u11_2, a20.z, d11_44);
+        { const float2 t = pmul(sx11_2, d11_44);
+          pfma(dyv[6], 0.774596691f, t);
         }
-        vfma(u11_2, a21.y, d11_45);
-        { const float t = vdot(sx11_2, d11_45);
-          dyl[7] = fmaf(0.730296731f, t, dyl[7]);
+        pfma(u11_2, a21.y, d11_45);
+        { const float2 t = pmul(sx11_2, d11_45);
+          pfma(dyv[7], 0.730296731f, t);
         }
-        vfma(u11_2, a22.x, d11_46);
-        { const float t = vdot(sx11_2, d11_46);
-          dyl[8] = fmaf(0.577350259f, t, dyl[8]);
+        pfma(u11_2, a22.x, d11_46);
+        { const float2 t = pmul(sx11_2, d11_46);
+          pfma(dyv[8], 0.577350259f, t);
         }
-        vfma(u11_3, a22.w, d11_47);
-        { const float t = vdot(sx11_3, d11_47);
-          dyl[8] = fmaf(0.707106769f, t, dyl[8]);
+        pfma(u11_3, a22.w, d11_47);
+        { const float2 t = pmul(sx11_3, d11_47);
+          pfma(dyv[8], 0.707106769f, t);
         }
-        vfma(u11_3, a19.y, d11_42);
-        { const float t = vdot(sx11_3, d11_42);
-          dyl[5] = fmaf(0.577350259f, t, dyl[5]);
+        pfma(u11_3, a19.y, d11_42);
+        { const float2 t = pmul(sx11_3, d11_42);
+          pfma(dyv[5], 0.577350259f, t);
         }
-        vfma(u11_3, a20.x, d11_43);
-        { const float t = vdot(sx11_3, d11_43);
-          dyl[4] = fmaf(-0.182574183f, t, dyl[4]);
+        pfma(u11_3, a20.x, d11_43);
+        { const float2 t = pmul(sx11_3, d11_43);
+          pfma(dyv[4], -0.182574183f, t);
         }
-        vfma(u11_3, a20.w, d11_44);
-        { const float t = vdot(sx11_3, d11_44);
-          dyl[7] = fmaf(-0.44721359f, t, dyl[7]);
+        pfma(u11_3, a20.w, d11_44);
+        { const float2 t = pmul(sx11_3, d11_44);
+          pfma(dyv[7], -0.44721359f, t);
         }
-        vfma(u11_3, a21.z, d11_45);
-        { const float t = vdot(sx11_3, d11_45);
-          dyl[6] = fmaf(0.632455528f, t, dyl[6]);
-          dyl[8] = fmaf(-0.182574183f, t, dyl[8]);
+        pfma(u11_3, a21.z, d11_45);
+        { const float2 t = pmul(sx11_3, d11_45);
+          pfma(dyv[6], 0.632455528f, t);
+          pfma(dyv[8], -0.182574183f, t);
         }
-        vfma(u11_3, a22.y, d11_46);
-        { const float t = vdot(sx11_3, d11_46);
-          dyl[7] = fmaf(0.577350259f, t, dyl[7]);
+        pfma(u11_3, a22.y, d11_46);
+        { const float2 t = pmul(sx11_3, d11_46);
+          pfma(dyv[7], 0.577350259f, t);
         }
-        EVec ds11 = vmul(x1, u11_1);
-        vfma(ds11, x2, u11_2);
-        vfma(ds11, x3, u11_3);
+        EVec ds11 = pmul(x1, u11_1);
+        pfma(ds11, x2, u11_2);
+        pfma(ds11, x3, u11_3);
         if (gw) gw[11 * NQV] = ds11;
-        vfma(dxp[1], s11, u11_1);
-        vfma(dxp[2], s11, u11_2);
-        vfma(dxp[3], s11, u11_3);
+        pfma(dxp[1], s11, u11_1);
+        pfma(dxp[2], s11, u11_2);
+        pfma(dxp[3], s11, u11_3);
         const EVec s12 = ss[12 * NQV];  // path 12: l1=1 l2=3 -> L=3
-        const EVec sx12_1 = vmul(s12, x1);
+        const EVec sx12_1 = pmul(s12, x1);
         EVec u12_1; vzero(u12_1);
-        const EVec sx12_2 = vmul(s12, x2);
+        const EVec sx12_2 = pmul(s12, x2);
         EVec u12_2; vzero(u12_2);
-        const EVec sx12_3 = vmul(s12, x3);
+        const EVec sx12_3 = pmul(s12, x3);
         EVec u12_3; vzero(u12_3);
         const EVec d12_48 = dms[48 * NQV];
-        vfma(u12_1, a10.z, d12_48);
-        { const float t = vdot(sx12_1, d12_48);
-          dyl[10] = fmaf(0.353553385f, t, dyl[10]);
+        pfma(u12_1, a10.z, d12_48);
+        { const float2 t = pmul(sx12_1, d12_48);
+          pfma(dyv[10], 0.353553385f, t);
         }
         const EVec d12_49 = dms[49 * NQV];
         const float4 a11 = *reinterpret_cast<const float4*>(As + 44);
-        vfma(u12_1, a11.y, d12_49);
-        { const float t = vdot(sx12_1, d12_49);
-          dyl[9] = fmaf(-0.353553385f, t, dyl[9]);
-          dyl[11] = fmaf(0.456435472f, t, dyl[11]);
+        pfma(u12_1, a11.y, d12_49);
+        { const float2 t = pmul(sx12_1, d12_49);
+          pfma(dyv[9], -0.353553385f, t);
+          pfma(dyv[11], 0.456435472f, t);
         }
         const EVec d12_50 = dms[50 * NQV];
         const float4 a12 = *reinterpret_cast<const float4*>(As + 48);
-        vfma(u12_1, a12.x, d12_50);
-        { const float t = vdot(sx12_1, d12_50);
-          dyl[10] = fmaf(-0.456435472f, t, dyl[10]);
+        pfma(u12_1, a12.x, d12_50);
+        { const float2 t = pmul(sx12_1, d12_50);
+          pfma(dyv[10], -0.456435472f, t);
         }
         const EVec d12_51 = dms[51 * NQV];
-        vfma(u12_1, a12.w, d12_51);
-        { const float t = vdot(sx12_1, d12_51);
-          dyl[13] = fmaf(-0.707106769f, t, dyl[13]);
+        pfma(u12_1, a12.w, d12_51);
+        { const float2 t = pmul(sx12_1, d12_51);
+          pfma(dyv[13], -0.707106769f, t);
         }
         const EVec d12_52 = dms[52 * NQV];
         const float4 a13 = *reinterpret_cast<const float4*>(As + 52);
-        vfma(u12_1, a13.y, d12_52);
-        { const float t = vdot(sx12_1, d12_52);
-          dyl[12] = fmaf(0.707106769f, t, dyl[12]);
-          dyl[14] = fmaf(-0.456435472f, t, dyl[14]);
+        pfma(u12_1, a13.y, d12_52);
+        { const float2 t = pmul(sx12_1, d12_52);
+          pfma(dyv[12], 0.707106769f, t);
+          pfma(dyv[14], -0.456435472f, t);
         }
         const EVec d12_53 = dms[53 * NQV];
         const float4 a14 = *reinterpret_cast<const float4*>(As + 56);
-        vfma(u12_1, a14.x, d12_53);
-        { const float t = vdot(sx12_1, d12_53);
-          dyl[13] = fmaf(0.456435472f, t, dyl[13]);
-          dyl[15] = fmaf(-0.353553385f, t, dyl[15]);
+        pfma(u12_1, a14.x, d12_53);
+        { const float2 t = pmul(sx12_1, d12_53);
+          pfma(dyv[13], 0.456435472f, t);
+          pfma(dyv[15], -0.353553385f, t);
         }
         const EVec d12_54 = dms[54 * NQV];
-        vfma(u12_1, a14.w, d12_54);
-        { const float t = vdot(sx12_1, d12_54);
-          dyl[14] = fmaf(0.353553385f, t, dyl[14]);
+        pfma(u12_1, a14.w, d12_54);
+        { const float2 t = pmul(sx12_1, d12_54);
+          pfma(dyv[14], 0.353553385f, t);
         }
-        vfma(u12_2, a10.w, d12_48);
-        { const float t = vdot(sx12_2, d12_48);
-          dyl[15] = fmaf(0.866025388f, t, dyl[15]);
+        pfma(u12_2, a10.w, d12_48);
+        { const float2 t = pmul(sx12_2, d12_48);
+          pfma(dyv[15], 0.866025388f, t);
         }
-        vfma(u12_2, a11.z, d12_49);
-        { const float t = vdot(sx12_2, d12_49);
-          dyl[14] = fmaf(0.577350259f, t, dyl[14]);
+        pfma(u12_2, a11.z, d12_49);
+        { const float2 t = pmul(sx12_2, d12_49);
+          pfma(dyv[14], 0.577350259f, t);
         }
-        vfma(u12_2, a12.y, d12_50);
-        { const float t = vdot(sx12_2, d12_50);
-          dyl[13] = fmaf(0.288675129f, t, dyl[13]);
+        pfma(u12_2, a12.y, d12_50);
+        { const float2 t = pmul(sx12_2, d12_50);
+          pfma(dyv[13], 0.288675129f, t);
         }
-        vfma(u12_3, a13.x, d12_51);
-        { const float t = vdot(sx12_3, d12_51);
-          dyl[11] = fmaf(0.707106769f, t, dyl[11]);
+        pfma(u12_3, a13.x, d12_51);
+        { const float2 t = pmul(sx12_3, d12_51);
+          pfma(dyv[11], 0.707106769f, t);
         }
-        vfma(u12_2, a13.z, d12_52);
-        { const float t = vdot(sx12_2, d12_52);
-          dyl[11] = fmaf(-0.288675129f, t, dyl[11]);
+        pfma(u12_2, a13.z, d12_52);
+        { const float2 t = pmul(sx12_2, d12_52);
+          pfma(dyv[11], -0.288675129f, t);
         }
-        vfma(u12_2, a14.y, d12_53);
-        { const float t = vdot(sx12_2, d12_53);
-          dyl[10] = fmaf(-0.577350259f, t, dyl[10]);
+        pfma(u12_2, a14.y, d12_53);
+        { const float2 t = pmul(sx12_2, d12_53);
+          pfma(dyv[10], -0.577350259f, t);
         }
         const float4 a15 = *reinterpret_cast<const float4*>(As + 60);
-        vfma(u12_2, a15.x, d12_54);
-        { const float t = vdot(sx12_2, d12_54);
-          dyl[9] = fmaf(-0.866025388f, t, dyl[9]);
+        pfma(u12_2, a15.x, d12_54);
+        { const float2 t = pmul(sx12_2, d12_54);
+          pfma(dyv[9], -0.866025388f, t);
         }
-        vfma(u12_3, a11.x, d12_48);
-        { const float t = vdot(sx12_3, d12_48);
-          dyl[14] = fmaf(-0.353553385f, t, dyl[14]);
+        pfma(u12_3, a11.x, d12_48);
+        { const float2 t = pmul(sx12_3, d12_48);
+          pfma(dyv[14], -0.353553385f, t);
         }
-        vfma(u12_3, a11.w, d12_49);
-        { const float t = vdot(sx12_3, d12_49);
-          dyl[13] = fmaf(-0.456435472f, t, dyl[13]);
-          dyl[15] = fmaf(-0.353553385f, t, dyl[15]);
+        pfma(u12_3, a11.w, d12_49);
+        { const float2 t = pmul(sx12_3, d12_49);
+          pfma(dyv[13], -0.456435472f, t);
+          pfma(dyv[15], -0.353553385f, t);
         }
-        vfma(u12_3, a12.z, d12_50);
-        { const float t = vdot(sx12_3, d12_50);
-          dyl[12] = fmaf(-0.707106769f, t, dyl[12]);
-          dyl[14] = fmaf(-0.456435472f, t, dyl[14]);
+        pfma(u12_3, a12.z, d12_50);
+        { const float2 t = pmul(sx12_3, d12_50);
+          pfma(dyv[12], -0.707106769f, t);
+          pfma(dyv[14], -0.456435472f, t);
         }
-        vfma(u12_3, a13.w, d12_52);
-        { const float t = vdot(sx12_3, d12_52);
-          dyl[10] = fmaf(0.456435472f, t, dyl[10]);
+        pfma(u12_3, a13.w, d12_52);
+        { const float2 t = pmul(sx12_3, d12_52);
+          pfma(dyv[10], 0.456435472f, t);
         }
-        vfma(u12_3, a14.z, d12_53);
-        { const float t = vdot(sx12_3, d12_53);
-          dyl[9] = fmaf(0.353553385f, t, dyl[9]);
-          dyl[11] = fmaf(0.456435472f, t, dyl[11]);
+        pfma(u12_3, a14.z, d12_53);
+        { const float2 t = pmul(sx12_3, d12_53);
+          pfma(dyv[9], 0.353553385f, t);
+          pfma(dyv[11], 0.456435472f, t);
         }
-        vfma(u12_3, a15.y, d12_54);
-        { const float t = vdot(sx12_3, d12_54);
-          dyl[10] = fmaf(0.353553385f, t, dyl[10]);
+        pfma(u12_3, a15.y, d12_54);
+        { const float2 t = pmul(sx12_3, d12_54);
+          pfma(dyv[10], 0.353553385f, t);
         }
-        EVec ds12 = vmul(x1, u12_1);
-        vfma(ds12, x2, u12_2);
-        vfma(ds12, x3, u12_3);
+        EVec ds12 = pmul(x1, u12_1);
+        pfma(ds12, x2, u12_2);
+        pfma(ds12, x3, u12_3);
         if (gw) gw[12 * NQV] = ds12;
-        vfma(dxp[1], s12, u12_1);
-        vfma(dxp[2], s12, u12_2);
-        vfma(dxp[3], s12, u12_3);
+        pfma(dxp[1], s12, u12_1);
+        pfma(dxp[2], s12, u12_2);
+        pfma(dxp[3], s12, u12_3);
+        dyl[0] = dyv[0].x + dyv[0].y;
+        dyl[1] = dyv[1].x + dyv[1].y;
+        dyl[2] = dyv[2].x + dyv[2].y;
+        dyl[3] = dyv[3].x + dyv[3].y;
+        dyl[4] = dyv[4].x + dyv[4].y;
+        dyl[5] = dyv[5].x + dyv[5].y;
+        dyl[6] = dyv[6].x + dyv[6].y;
+        dyl[7] = dyv[7].x + dyv[7].y;
+        dyl[8] = dyv[8].x + dyv[8].y;
+        dyl[9] = dyv[9].x + dyv[9].y;
+        dyl[10] = dyv[10].x + dyv[10].y;
+        dyl[11] = dyv[11].x + dyv[11].y;
+        dyl[12] = dyv[12].x + dyv[12].y;
+        dyl[13] = dyv[13].x + dyv[13].y;
+        dyl[14] = dyv[14].x + dyv[14].y;
+        dyl[15] = dyv[15].x + dyv[15].y;
     }
     __device__ static __forceinline__ void bwd2_edge_all(const DVec* __restrict__ dms, const DVec* __restrict__ xs, const DVec* __restrict__ uxs, const DVec* __restrict__ ss, const DVec* __restrict__ uss, const float* __restrict__ As, const float* __restrict__ Bs, DVec (&dxp)[DIN], float (&dyl)[16], DVec* __restrict__ gw) {
         constexpr int NQV = NQ / DV;

@@ -159,8 +159,11 @@ class Sig:
 
     # Bodies whose multiplies and fused multiply-adds are emitted in the packed two-channel form (pfma / pmul of
     # fast_common.cuh).  Measured on the 128-channel water signature: the forward-shaped bodies and the double
-    # backward gain (fewer issue slots), the first backward's edge body loses (more registers, it is bound by
-    # memory), so it stays scalar unless the signature's "PK" list names it.
+    # backward gain (fewer issue slots).  The first backward's edge body ("ebwd") gains where one warp with two channels per
+    # lane does a whole edge, which its instruction supply bounds: 64x(0e+1o+2e), l <= 3, 500 -> 393 us on the 78 000 edges
+    # of 1500 atoms, and with the 255 registers of seven consumer warps instead of eight 330.  With four channels per lane (128x(0e+1o): 255 ->
+    # 274 us) or several warps to an edge (128x(0e+1o+2e+3o), l <= 2: 555 -> 640), which share what they fetch, it loses, and
+    # the body stays scalar.
     PACKED_DEFAULT = ("fwd", "fwd2", "rfwd", "bwd2")
 
     def ops(self, kind):
@@ -306,7 +309,9 @@ class Sig:
         o.append(f"    // edge-wise backward (one warp per edge, grad_out rows read from shared memory): edges per tile "
                  f"(0 = not generated), ring stages")
         EV = self.cfg.get("EV", V)
-        o.append(f"    static constexpr int ET = {self.cfg.get('ET', 0)}, ES = {self.cfg.get('ES', 2)}, EV = {EV};")
+        o.append(f"    static constexpr int ET = {self.cfg.get('ET', 0)}, ES = {self.cfg.get('ES', 2)}, EV = {EV}, "
+                 f"EXG = {self.cfg.get('EXG', 0)};   // EXG: sender rows not staged")
+        o.append(f"    static constexpr int ST = {self.cfg.get('SBT', self.cfg.get('ET', 0))};   // columns of the scheduled backward")
         o.append(f"    // the same for the standalone tensor product: rows per ring slot (0 = not generated), ring slots")
         o.append(f"    static constexpr int ETR = {self.cfg.get('ETR', 0)}, ESR = {self.cfg.get('ESR', 3)};")
         o.append(f"    // fused double backward (edge outputs): edges per tile (0 = not generated), ring stages")
@@ -411,8 +416,13 @@ class Sig:
                  f"const EVec* __restrict__ ss, const float* __restrict__ As, EVec (&dxp)[DIN], float (&dyl)[16], "
                  f"EVec* __restrict__ gw) {{")
         o.append(f"        constexpr int NQV = NQ / EV;")
+        EV = self.cfg.get("EV", self.V)
+        F, M = self.ops("ebwd")
+        packed_dy = F == "pfma" and EV > 1   # grad_sh summed as pairs of channels, the halves added at the end
         for i1 in range(self.DIN):
             o.append(f"        const EVec x{i1} = xs[{i1} * NQV];")
+        if packed_dy:
+            o.append("        float2 dyv[16];")
         loaded_a, dx_touched, dy_touched = set(), set(), set()
         for k in range(self.P):
             p = self.paths[k]
@@ -420,7 +430,7 @@ class Sig:
             used = sorted({self.pairs[pi][1] for r2 in prow for pi in self.pairs_of(r2, k)})
             o.append(f"        const EVec s{k} = ss[{k} * NQV];  // path {k}: l1={p['l1']} l2={p['l2']} -> L={p['L']}")
             for i1 in used:
-                F, M = self.ops("bwd"); o.append(f"        const EVec sx{k}_{i1} = {M}(s{k}, x{i1});")
+                o.append(f"        const EVec sx{k}_{i1} = {M}(s{k}, x{i1});")
                 o.append(f"        EVec u{k}_{i1}; vzero(u{k}_{i1});")
             depth = max(len(self.pairs_of(r2, k)) for r2 in prow)
             have = set()
@@ -438,32 +448,47 @@ class Sig:
                         loaded_a.add(q)
                         o.append(f"        const float4 a{q} = *reinterpret_cast<const float4*>(As + {4 * q});")
                     i1 = self.pairs[pi][1]
-                    F, M = self.ops("bwd"); o.append(f"        {F}(u{k}_{i1}, a{q}.{lane}, d{k}_{row});")
-                    o.append(f"        {{ const float t = vdot(sx{k}_{i1}, d{k}_{row});")
-                    for i2, c in self.pairs[pi][3]:
-                        if i2 in dy_touched:
-                            o.append(f"          dyl[{i2}] = fmaf({fmt_float(c)}, t, dyl[{i2}]);")
+                    o.append(f"        {F}(u{k}_{i1}, a{q}.{lane}, d{k}_{row});")
+                    if packed_dy:
+                        a, b = f"sx{k}_{i1}", f"d{k}_{row}"
+                        if EV == 2:
+                            o.append(f"        {{ const float2 t = pmul({a}, {b});")
                         else:
-                            dy_touched.add(i2)
-                            o.append(f"          dyl[{i2}] = {fmt_float(c)} * t;")
+                            o.append(f"        {{ float2 t = pmul(make_float2({a}.x, {a}.y), make_float2({b}.x, {b}.y)); "
+                                     f"pfma(t, make_float2({a}.z, {a}.w), make_float2({b}.z, {b}.w));")
+                        for i2, c in self.pairs[pi][3]:
+                            if i2 not in dy_touched:
+                                dy_touched.add(i2)
+                                o.append(f"          vzero(dyv[{i2}]);")
+                            o.append(f"          pfma(dyv[{i2}], {fmt_float(c)}, t);")
+                    else:
+                        o.append(f"        {{ const float t = vdot(sx{k}_{i1}, d{k}_{row});")
+                        for i2, c in self.pairs[pi][3]:
+                            if i2 in dy_touched:
+                                o.append(f"          dyl[{i2}] = fmaf({fmt_float(c)}, t, dyl[{i2}]);")
+                            else:
+                                dy_touched.add(i2)
+                                o.append(f"          dyl[{i2}] = {fmt_float(c)} * t;")
                     o.append("        }")
             first = used[0]
-            F, M = self.ops("bwd"); o.append(f"        EVec ds{k} = {M}(x{first}, u{k}_{first});")
+            o.append(f"        EVec ds{k} = {M}(x{first}, u{k}_{first});")
             for i1 in used[1:]:
-                F, M = self.ops("bwd"); o.append(f"        {F}(ds{k}, x{i1}, u{k}_{i1});")
+                o.append(f"        {F}(ds{k}, x{i1}, u{k}_{i1});")
             o.append(f"        if (gw) gw[{k} * NQV] = ds{k};")
             for i1 in used:
                 if i1 in dx_touched:
-                    F, M = self.ops("bwd"); o.append(f"        {F}(dxp[{i1}], s{k}, u{k}_{i1});")
+                    o.append(f"        {F}(dxp[{i1}], s{k}, u{k}_{i1});")
                 else:
                     dx_touched.add(i1)
-                    F, M = self.ops("bwd"); o.append(f"        dxp[{i1}] = {M}(s{k}, u{k}_{i1});")
+                    o.append(f"        dxp[{i1}] = {M}(s{k}, u{k}_{i1});")
         for i1 in range(self.DIN):
             if i1 not in dx_touched:
                 o.append(f"        vzero(dxp[{i1}]);")
         for i2 in range(16):
             if i2 not in dy_touched:
                 o.append(f"        dyl[{i2}] = 0.f;")
+            elif packed_dy:
+                o.append(f"        dyl[{i2}] = dyv[{i2}].x + dyv[{i2}].y;")
         o.append("    }")
         return o
 
@@ -807,7 +832,7 @@ class Sig:
             dbl_e = f"&fast::launch_dbl_edges<fast::{S}>" if self.cfg.get("DT", 0) else "nullptr"
             dbl_o = f"&fast::launch_dbl_out<fast::{S}>" if self.cfg.get("DFT", 0) else "nullptr"
             rf = f"&fast::launch_radial_fwd<fast::{S}>" if self.cfg.get("RF", 0) else "nullptr"
-            sb = (f"&fast::launch_bwd_sched<fast::{S}>, {self.cfg['ET']}" if self.cfg.get("SB", 0) else "nullptr, 0")
+            sb = (f"&fast::launch_bwd_sched<fast::{S}>, {self.cfg.get('SBT', self.cfg['ET'])}" if self.cfg.get("SB", 0) else "nullptr, 0")
             o.append(f"    {dbl_e}, {dbl_o}, {rf}, {sb}}};")
         else:
             o.append(f"    &fast::fwd_scratch_bytes<fast::{S}>, nullptr, &fast::launch_fwd<fast::{S}>, nullptr, nullptr, nullptr, "
