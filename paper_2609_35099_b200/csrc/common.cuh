@@ -32,9 +32,10 @@ inline int after_launch() {
 
 // Launch of a kernel that follows another one on the same stream and starts with fast::grid_dependency_wait(): the
 // launch itself (and the scheduling of its first CTAs) overlaps the tail of its predecessor; the wait inside the
-// kernel holds it until the predecessor has finished and its writes are visible (programmatic dependent launch).
+// kernel holds it until the predecessor has finished and its writes are visible (programmatic dependent launch).  128x(0e+1o),
+// 9600 edges: forward 22.6 -> 20.1 us, backward 41.1 -> 38.7; 78 000 edges: 106 -> 104, 278 -> 277.
 template <class... KArgs, class... Args>
-inline int launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+inline int launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -375,9 +375,6 @@ fast_bwd1_kernel(const BwdParams p) {
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::off_abort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int64_t n_edges, chunk, e_begin, e_end;   // n_edges: the real edges (a padded call learns their number here)
-    cta_edge_range(p.n_edges, p.chunk, p.n_real, n_edges, chunk, e_begin, e_end);
-
     if (threadIdx.x == 0) {
         // full: the producer's arrival with the copies' byte count and its arrival after the tables;
         // empty: the T warps that work on the slot
@@ -386,6 +383,9 @@ fast_bwd1_kernel(const BwdParams p) {
         *abort_flag = 0;
         mbar_fence_init();
     }
+    grid_dependency_wait();
+    int64_t n_edges, chunk, e_begin, e_end;   // n_edges: the real edges (a padded call learns their number here)
+    cta_edge_range(p.n_edges, p.chunk, p.n_real, n_edges, chunk, e_begin, e_end);
     __syncthreads();
     if (warp == NCONS) bwd1_producer<S, ROWS, DBL>(p, smem, lane, e_begin, e_end);
     else bwd1_consumer<S, ROWS, DBL>(p, smem, warp, lane, e_begin, e_end);

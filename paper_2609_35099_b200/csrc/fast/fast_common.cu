@@ -8,6 +8,7 @@ namespace fast {
 __global__ void fwd_fixup_kernel(int n_cta, int row_f4, const float4* __restrict__ partial,
                                  const int32_t* __restrict__ part_recv, float4* __restrict__ out) {
     grid_dependency_wait();
+    grid_dependency_trigger();
     const int c = blockIdx.x;
     const int b = part_recv[2 * c + 1];  // a row whose first piece is this CTA's tail
     if (b < 0) return;
@@ -66,7 +67,7 @@ bwd_dx_reduce_kernel(int64_t n_nodes, int row_f4, int max_runs, const float4* __
                                      const int32_t* __restrict__ sender_perm, const int32_t* __restrict__ colptr,
                                      float4* __restrict__ grad_x, ZeroPadding pad) {
     extern __shared__ float4 part[];   // [max_runs][row_f4] where max_runs > 1
-    if (blockIdx.x >= n_nodes) {       // padding rows: written by no other kernel, so there is nothing to wait for
+    if (blockIdx.x >= n_nodes) {   // padding rows: not the sweep's, which itself started after all that came before it
         zero_padding_rows(pad, blockIdx.x - n_nodes, gridDim.x - n_nodes);
         return;
     }
@@ -77,6 +78,7 @@ bwd_dx_reduce_kernel(int64_t n_nodes, int row_f4, int max_runs, const float4* __
     while (runs < max_runs && n > kRunEdges * runs) runs *= 2;
     const int per = (n + runs - 1) / runs;
     grid_dependency_wait();
+    grid_dependency_trigger();
     float4 acc;
     for (int r = grp; r < runs; r += groups) {
         const int j1 = b0 + min(n, (r + 1) * per);

@@ -203,16 +203,16 @@ fast_fwd_kernel(const FwdParams p) {
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::off_abort);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int64_t n_edges, chunk, e_begin, e_end;   // n_edges: the real edges (a padded call learns their number here)
-    cta_edge_range(p.n_edges, p.chunk, p.n_real, n_edges, chunk, e_begin, e_end);
-    const int n_tiles = (int)((e_end - e_begin + T - 1) / T);
-
     if (threadIdx.x == 0) {
         // full: the copy warp's arrival (with the byte count) and the table warp's arrival
         for (int s = 0; s < NS; ++s) { mbar_init(&full[s], 2); mbar_init(&empty[s], NCONS); }
         *abort_flag = 0;
         mbar_fence_init();
     }
+    grid_dependency_wait();
+    int64_t n_edges, chunk, e_begin, e_end;   // n_edges: the real edges (a padded call learns their number here)
+    cta_edge_range(p.n_edges, p.chunk, p.n_real, n_edges, chunk, e_begin, e_end);
+    const int n_tiles = (int)((e_end - e_begin + T - 1) / T);
     __syncthreads();
     if (warp == NCONS) producer_loop<L, FwdTab<S>, 0>(p, smem, lane, e_begin, e_end, n_tiles);
     else if (warp == NCONS + 1) producer_loop<L, FwdTab<S>, 1>(p, smem, lane, e_begin, e_end, n_tiles);

@@ -50,8 +50,7 @@ int launch_fwd(const ConvArgs& a) {
     p.status = a.status;
     p.n_real = a.n_real;
     constexpr int threads = (S::FW * (S::NQ / (32 * S::V)) + 2) * 32;  // consumers + two producer warps
-    fast_fwd_kernel<S><<<n_cta, threads, L::total, a.stream>>>(p);
-    if (int s = after_launch()) return s;
+    if (int s = launch_dependent(fast_fwd_kernel<S>, dim3(n_cta), dim3(threads), L::total, a.stream, p)) return s;
     return launch_dependent(fwd_fixup_kernel, dim3(n_cta, 4), dim3(256), 0, a.stream, n_cta, S::D * S::NQ / 4, reinterpret_cast<const float4*>(p.partial),
                                                  p.part_recv, reinterpret_cast<float4*>(a.out));
 }
@@ -74,8 +73,7 @@ int launch_tp_fwd(int64_t rows, const float* x1, const float* x2, const float* w
     const int64_t per = (rows + n_cta - 1) / n_cta;
     p.chunk = (per + 3) / 4 * 4;
     constexpr int threads = (S::FW * (S::NQ / (32 * S::V)) + 2) * 32;
-    fast_fwd_kernel<S><<<n_cta, threads, L::total, st>>>(p);
-    return after_launch();
+    return launch_dependent(fast_fwd_kernel<S>, dim3(n_cta), dim3(threads), L::total, st, p);
 }
 
 template <class S>
@@ -100,7 +98,7 @@ int launch_tp_bwd(int64_t rows, const float* x1, const float* x2, const float* w
             E3J_CUDA_TRY(cudaFuncSetAttribute(fast_bwd1_kernel<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L1::total));
             attr_dev = dev;
         }
-        fast_bwd1_kernel<S, true><<<n_cta, (L1::T * L1::CH * L1::NG + 1) * 32, L1::total, st>>>(p);
+        return launch_dependent(fast_bwd1_kernel<S, true>, dim3(n_cta), dim3((L1::T * L1::CH * L1::NG + 1) * 32), L1::total, st, p);
     } else {
         if (attr_dev != dev) {
             E3J_CUDA_TRY(cudaFuncSetAttribute(fast_bwd_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total));
@@ -108,8 +106,8 @@ int launch_tp_bwd(int64_t rows, const float* x1, const float* x2, const float* w
         }
         constexpr int threads = (S::BW * (S::NQ / (32 * S::BV)) + 1) * 32;  // consumers + one producer warp
         fast_bwd_kernel<S><<<n_cta, threads, L::total, st>>>(p);
+        return after_launch();
     }
-    return after_launch();
 }
 
 // scratch of the backward: this edge's share of grad_x, [E][d][N_q]
@@ -143,7 +141,8 @@ int launch_bwd(const ConvArgs& a) {
             E3J_CUDA_TRY(cudaFuncSetAttribute(fast_bwd1_kernel<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L1::total));
             attr_dev = dev;
         }
-        fast_bwd1_kernel<S, false><<<n_cta, (L1::T * L1::CH + 1) * 32, L1::total, a.stream>>>(p);  // consumers + one producer warp
+        const dim3 threads((L1::T * L1::CH + 1) * 32);   // consumers + one producer warp
+        if (int s = launch_dependent(fast_bwd1_kernel<S, false>, dim3(n_cta), threads, L1::total, a.stream, p)) return s;
     } else {
         if (attr_dev != dev) {
             E3J_CUDA_TRY(cudaFuncSetAttribute(fast_bwd_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::total));
@@ -151,8 +150,8 @@ int launch_bwd(const ConvArgs& a) {
         }
         constexpr int threads = (S::BW * (S::NQ / (32 * S::BV)) + 1) * 32;  // consumers + one producer warp
         fast_bwd_kernel<S><<<n_cta, threads, L::total, a.stream>>>(p);
+        if (int s = after_launch()) return s;
     }
-    if (int s = after_launch()) return s;
     ZeroPadding pad{};
     if (a.n_real) pad = {a.n_real, a.n_edges, S::P * S::NQ / 4, S::DSH, reinterpret_cast<float4*>(a.grad_w), a.grad_sh};
     if (!a.grad_x) {   // the shares stay in the scratch
@@ -188,8 +187,8 @@ int launch_dbl_edges(const ConvArgs& a, const float* ct_x, const float* ct_sh, c
         E3J_CUDA_TRY(cudaFuncSetAttribute(fast_bwd1_kernel<S, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L1::total));
         attr_dev = dev;
     }
-    fast_bwd1_kernel<S, false, true><<<n_cta, (L1::T * L1::CH + 1) * 32, L1::total, a.stream>>>(p);
-    if (int s = after_launch()) return s;
+    if (int s = launch_dependent(fast_bwd1_kernel<S, false, true>, dim3(n_cta), dim3((L1::T * L1::CH + 1) * 32), L1::total,
+                                 a.stream, p)) return s;
     return launch_dx_reduce(a.n_nodes, a.n_edges, S::DIN * S::NQ / 4, p.dx_edge, a.sender_perm, a.colptr, a.grad_x,
                             ZeroPadding{}, a.stream);
 }
@@ -221,8 +220,7 @@ int launch_dbl_out(const ConvArgs& a, const float* ct_x, const float* ct_sh, con
     p.partial = reinterpret_cast<float*>(reinterpret_cast<char*>(a.workspace) + kPartRecvBytes);
     p.status = a.status;
     constexpr int threads = (L::NCONS + 2) * 32;  // consumers + two producer warps
-    fast_fwd_kernel<S, true><<<n_cta, threads, L::total, a.stream>>>(p);
-    if (int s = after_launch()) return s;
+    if (int s = launch_dependent(fast_fwd_kernel<S, true>, dim3(n_cta), dim3(threads), L::total, a.stream, p)) return s;
     return launch_dependent(fwd_fixup_kernel, dim3(n_cta, 4), dim3(256), 0, a.stream, n_cta, S::D * S::NQ / 4, reinterpret_cast<const float4*>(p.partial),
                                                  p.part_recv, reinterpret_cast<float4*>(a.out));
 }

@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fast/fast_common.cuh"
 
 namespace e3j {
 namespace {
@@ -256,6 +257,8 @@ prepare_one_kernel(int64_t n_nodes, int64_t n_edges, const int32_t* __restrict__
     for (int i = threadIdx.x; i <= own; i += kOneThreads) m.start[i] = 0;
     if (threadIdx.x == 0) m.collected = m.before = 0;
     __syncthreads();
+    fast::grid_dependency_wait();
+    fast::grid_dependency_trigger();
     int32_t smaller = 0;
     for_senders(n_nodes, n_edges, senders, pad_recv, [&](int64_t e, int32_t s) {
         smaller += s < a0;
@@ -350,9 +353,8 @@ int prepare_one(int64_t n_nodes, int64_t n_edges, const int32_t* senders, const 
         E3J_CUDA_TRY(cudaFuncSetAttribute(prepare_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OneSmem)));
         attr_dev = dev;
     }
-    prepare_one_kernel<<<(int)blocks, kOneThreads, sizeof(OneSmem), st>>>(n_nodes, n_edges, senders, receivers, pad_recv,
-                                                                        rowptr, colptr, sender_perm, per_block);
-    return after_launch();
+    return launch_dependent(prepare_one_kernel, dim3((int)blocks), dim3(kOneThreads), sizeof(OneSmem), st, n_nodes, n_edges, senders,
+                            receivers, pad_recv, rowptr, colptr, sender_perm, per_block);
 }
 
 inline int blocks_for(int64_t n, int threads) {

@@ -8,6 +8,7 @@
 //   e3j_conv_vec_bwd           composed: harmonics into the workspace, e3j_conv_bwd with grad_sh kept as scratch,
 //                              then the chain rule into the vectors
 #include "common.cuh"
+#include "fast/fast_common.cuh"
 #include "fast/harmonics.cuh"
 
 namespace e3j {
@@ -16,6 +17,8 @@ namespace {
 template <int DSH>
 __global__ void __launch_bounds__(256)
 harmonics_fwd_kernel(int64_t n, const float* __restrict__ vec, float* __restrict__ sh) {
+    fast::grid_dependency_wait();
+    fast::grid_dependency_trigger();
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         float x, y, z, inv_r, Y[DSH];
         fast::unit_vector(vec[3 * e], vec[3 * e + 1], vec[3 * e + 2], x, y, z, inv_r);
@@ -36,6 +39,8 @@ template <int DSH>
 __global__ void __launch_bounds__(256)
 harmonics_bwd_kernel(int64_t n, const float* __restrict__ vec, const float* __restrict__ grad_sh,
                      float* __restrict__ grad_vec) {
+    fast::grid_dependency_wait();
+    fast::grid_dependency_trigger();
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         float x, y, z, inv_r, g[DSH], gx, gy, gz;
         fast::unit_vector(vec[3 * e], vec[3 * e + 1], vec[3 * e + 2], x, y, z, inv_r);
@@ -65,25 +70,23 @@ inline int grid_for(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 
 int harmonics_fwd(int lmax, int64_t n, const float* vec, float* sh, cudaStream_t st) {
     if (n == 0) return E3J_OK;
     switch (lmax) {
-        case 0: harmonics_fwd_kernel<1><<<grid_for(n), 256, 0, st>>>(n, vec, sh); break;
-        case 1: harmonics_fwd_kernel<4><<<grid_for(n), 256, 0, st>>>(n, vec, sh); break;
-        case 2: harmonics_fwd_kernel<9><<<grid_for(n), 256, 0, st>>>(n, vec, sh); break;
-        case 3: harmonics_fwd_kernel<16><<<grid_for(n), 256, 0, st>>>(n, vec, sh); break;
-        default: return E3J_ERR_UNSUPPORTED;
+        case 0: return launch_dependent(harmonics_fwd_kernel<1>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, sh);
+        case 1: return launch_dependent(harmonics_fwd_kernel<4>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, sh);
+        case 2: return launch_dependent(harmonics_fwd_kernel<9>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, sh);
+        case 3: return launch_dependent(harmonics_fwd_kernel<16>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, sh);
     }
-    return after_launch();
+    return E3J_ERR_UNSUPPORTED;
 }
 
 int harmonics_bwd(int lmax, int64_t n, const float* vec, const float* grad_sh, float* grad_vec, cudaStream_t st) {
     if (n == 0) return E3J_OK;
     switch (lmax) {
-        case 0: harmonics_bwd_kernel<1><<<grid_for(n), 256, 0, st>>>(n, vec, grad_sh, grad_vec); break;
-        case 1: harmonics_bwd_kernel<4><<<grid_for(n), 256, 0, st>>>(n, vec, grad_sh, grad_vec); break;
-        case 2: harmonics_bwd_kernel<9><<<grid_for(n), 256, 0, st>>>(n, vec, grad_sh, grad_vec); break;
-        case 3: harmonics_bwd_kernel<16><<<grid_for(n), 256, 0, st>>>(n, vec, grad_sh, grad_vec); break;
-        default: return E3J_ERR_UNSUPPORTED;
+        case 0: return launch_dependent(harmonics_bwd_kernel<1>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, grad_sh, grad_vec);
+        case 1: return launch_dependent(harmonics_bwd_kernel<4>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, grad_sh, grad_vec);
+        case 2: return launch_dependent(harmonics_bwd_kernel<9>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, grad_sh, grad_vec);
+        case 3: return launch_dependent(harmonics_bwd_kernel<16>, dim3(grid_for(n)), dim3(256), 0, st, n, vec, grad_sh, grad_vec);
     }
-    return after_launch();
+    return E3J_ERR_UNSUPPORTED;
 }
 
 // lmax of the plan's harmonics, or -1 if d' is not (lmax + 1)^2 with lmax <= 3

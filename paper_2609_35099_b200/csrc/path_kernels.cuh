@@ -576,6 +576,7 @@ node_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
 template <class T, int V, int LM, bool IDENT>
 __global__ void __launch_bounds__(kThreads, pair_blocks_per_sm(LM))
 pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
+    fast::grid_dependency_wait();
     pair_part<T, V, LM, IDENT>(t, a, blockIdx.x);
 }
 
@@ -584,6 +585,7 @@ __global__ void __launch_bounds__(kThreads, edge_blocks_per_sm<T>(LM))
 edge_kernel(const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");
+    fast::grid_dependency_wait();
     edge_part<T, V, LM, IDENT, ONLY_X>(et, a, blockIdx.x, smem);
 }
 
@@ -624,6 +626,7 @@ share_sum_kernel(const __grid_constant__ Args<T> a) {
     }
     const int used = __reduce_max_sync(0xffffffffu, step);
     fast::grid_dependency_wait();
+    fast::grid_dependency_trigger();
     T acc[V];
 #pragma unroll
     for (int c = 0; c < V; ++c) acc[c] = T(0);

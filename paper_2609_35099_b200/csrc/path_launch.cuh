@@ -43,8 +43,8 @@ template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, cons
     const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
     a.group_blocks = (unsigned)(blocks / t.n_groups);
-    if (pairs) pair_kernel<T, V, LM, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
-    else node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
+    if (pairs) return launch_dependent(pair_kernel<T, V, LM, IDENT>, dim3((unsigned)blocks), dim3(kThreads), 0, c.stream, t, a);
+    node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
     return after_launch();
 }
 
@@ -83,8 +83,7 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
         if (tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
         a.dx = !from_shares ? nullptr : IDENT ? c.grad_x : c.shares;
         const auto kernel = edges || IDENT ? edge_kernel<T, V, LM, IDENT, false> : edge_kernel<T, V, LM, false, true>;
-        kernel<<<(unsigned)tiles, threads, smem_bytes<LM>(threads), c.stream>>>(et, a);
-        if (int s = after_launch()) return s;
+        if (int s = launch_dependent(kernel, dim3((unsigned)tiles), dim3(threads), smem_bytes<LM>(threads), c.stream, et, a)) return s;
     }
     if (!from_shares || IDENT) return E3J_OK;
     a.dx = c.shares;
