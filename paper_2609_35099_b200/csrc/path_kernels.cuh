@@ -86,7 +86,7 @@ template <int l1, int l2, int L> struct Tri;
 #define E3J_E1(r, i, a) { axpy(u, T(a) * y[i], g[r]); dy[i] = fma(T(a), dot(sx, g[r]), dy[i]); }
 #define E3J_E2(r, i, a, j, b) { axpy(u, fma(T(a), y[i], T(b) * y[j]), g[r]); const T t_ = dot(sx, g[r]); \
                                 dy[i] = fma(T(a), t_, dy[i]); dy[j] = fma(T(b), t_, dy[j]); }
-#define E3J_EE(o) axpy(dw, x[o], u); axpy(dx[o], s, u); }
+#define E3J_EE(o) axpy(dw, x[o], u); if constexpr (DX) axpy(dx[o], s, u); }
 #define E3J_DEFINE_TRI(l1, l2, L)                                                                                    \
     template <> struct Tri<l1, l2, L> {                                                                              \
         static constexpr int kL1 = l1, kL2 = l2, kL = L;                                                             \
@@ -100,7 +100,7 @@ template <int l1, int l2, int L> struct Tri;
                                                               T (&acc)[NO][V]) {                                     \
             E3J_PATH_BY1_##l1##l2##L(E3J_PB, E3J_P1, E3J_P2, E3J_PE)                                                 \
         }                                                                                                            \
-        template <class T, int V, int NX, int NG>                                                                    \
+        template <bool DX, class T, int V, int NX, int NG>                                                           \
         __host__ __device__ static __forceinline__ void edge(const T* y, T* dy, const T (&x)[NX][V], const T (&s)[V],\
                                                              const T (&g)[NG][V], T (&dw)[V], T (&dx)[NX][V]) {      \
             E3J_PATH_BY1_##l1##l2##L(E3J_EB, E3J_E1, E3J_E2, E3J_EE)                                                 \
@@ -422,14 +422,17 @@ __device__ __forceinline__ void pair_part(const PathTable& t, const Args<T>& a, 
 }
 
 // ---------------------------------------------------------------- edge part
-// ONLY_X: the shares of grad_x and nothing else, to the same bits.
-template <class T, int V, int LM, bool IDENT, bool ONLY_X = false>
+// All three gradients, the shares of grad_x alone (to the same bits), or grad_w and grad_sh alone (16x(0e+1o+2e+3o), 35 050
+// edges: grad_w 100 us with the shares formed all the same, 85 without; 48x(0e+1o+2e), l <= 2: 74 and 64 us).
+enum class Want { kAll, kX, kEdges };
+template <class T, int V, int LM, bool IDENT, Want WANT>
 __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, const unsigned tile, unsigned char* smem) {
     const int slots = blockDim.x / a.units, slot = threadIdx.x / a.units, q = threadIdx.x - slot * a.units;
     const int64_t e = (int64_t)tile * slots + slot;
     const int64_t n_live = a.n_real ? min((int64_t)*a.n_real, a.n_edges) : a.n_edges;
     const bool mine = slot < slots && e < a.n_edges, live = mine && e < n_live;
     constexpr int NY = (LM + 1) * (LM + 1), ROWS = 2 * LM + 1;
+    constexpr bool ONLY_X = WANT == Want::kX, DX = WANT != Want::kEdges;
     const int row = a.units * V;
     const uint32_t row_bytes = (uint32_t)(row * sizeof(T)), unit = (uint32_t)(q * V * sizeof(T));
     T y[NY], dy[NY];
@@ -463,7 +466,7 @@ __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, 
         int x_rows = 0, stage = 0;
         uint32_t x_at = 0;
         auto put_dx = [&] {
-            if (!a.dx) return;
+            if (!DX || !a.dx) return;
             char* at = gx + x_at;
 #pragma unroll
             for (int i = 0; i < ROWS; ++i) {
@@ -503,7 +506,7 @@ __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, 
                     _Pragma("unroll") for (int i = 0; i < 2 * L + 1; ++i) \
                         load_pack<T, V>(g[i], reinterpret_cast<const T*>(at + (1 + i) * 512)); \
                     if constexpr (ONLY_X) Tri<l1, l2, L>::template sum_t<0, T, V>(y + l2 * l2, g, s, dx); \
-                    else Tri<l1, l2, L>::template edge<T, V>(y + l2 * l2, dy + l2 * l2, x, s, g, dw, dx); \
+                    else Tri<l1, l2, L>::template edge<DX, T, V>(y + l2 * l2, dy + l2 * l2, x, s, g, dw, dx); \
                 } break;
                 E3J_PATH_TRIPLES(E3J_CASE)
 #undef E3J_CASE
@@ -511,7 +514,7 @@ __device__ __forceinline__ void edge_part(const EdgeTable& t, const Args<T>& a, 
             if (!ONLY_X && a.grad_w) store_pack<T, V>(reinterpret_cast<T*>(gw + rec.w), dw);
         }
         put_dx();
-        if (a.dx) {
+        if (DX && a.dx) {
             T z[V];
 #pragma unroll
             for (int c = 0; c < V; ++c) z[c] = T(0);
@@ -580,13 +583,13 @@ pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
     pair_part<T, V, LM, IDENT>(t, a, blockIdx.x);
 }
 
-template <class T, int V, int LM, bool IDENT, bool ONLY_X>
-__global__ void __launch_bounds__(kThreads, edge_blocks_per_sm<T>(LM))
+template <class T, int V, int LM, bool IDENT, Want WANT>
+__global__ void __launch_bounds__(kThreads, WANT == Want::kEdges ? joint_blocks_per_sm(LM) : edge_blocks_per_sm<T>(LM))
 edge_kernel(const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");
     fast::grid_dependency_wait();
-    edge_part<T, V, LM, IDENT, ONLY_X>(et, a, blockIdx.x, smem);
+    edge_part<T, V, LM, IDENT, WANT>(et, a, blockIdx.x, smem);
 }
 
 // Edge tiles, and up to l = 2 the node sums of grad_x in the same launch.  With l = 3 the two parts' code together is too
@@ -601,7 +604,7 @@ joint_kernel(const __grid_constant__ PathTable t, const __grid_constant__ EdgeTa
         node_part<T, V, LM, true, IDENT>(t, a, blockIdx.x);
         return;
     }
-    edge_part<T, V, LM, IDENT>(et, a, blockIdx.x - a.node_blocks, smem);
+    edge_part<T, V, LM, IDENT, Want::kEdges>(et, a, blockIdx.x - a.node_blocks, smem);
 }
 
 // grad_x from the edges' shares: one 16-byte unit of a node's row to 2^split_log2 lanes, which take every so manieth

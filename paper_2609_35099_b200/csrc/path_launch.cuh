@@ -82,7 +82,8 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     if (tiles > 0) {
         if (tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
         a.dx = !from_shares ? nullptr : IDENT ? c.grad_x : c.shares;
-        const auto kernel = edges || IDENT ? edge_kernel<T, V, LM, IDENT, false> : edge_kernel<T, V, LM, false, true>;
+        const auto kernel = !from_shares ? edge_kernel<T, V, LM, IDENT, Want::kEdges>
+                            : edges || IDENT ? edge_kernel<T, V, LM, IDENT, Want::kAll> : edge_kernel<T, V, LM, false, Want::kX>;
         if (int s = launch_dependent(kernel, dim3((unsigned)tiles), dim3(threads), smem_bytes<LM>(threads), c.stream, et, a)) return s;
     }
     if (!from_shares || IDENT) return E3J_OK;
