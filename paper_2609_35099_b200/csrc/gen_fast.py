@@ -74,7 +74,8 @@ def fmt_float(v: float) -> str:
 
 def auto_params(sig, info):
     """Tile parameters for a signature that gives none ("auto": 1, or an overlay entry): channels per lane from the
-    channel count, row groups from the number of coefficient pairs, tile sizes from what fits in shared memory
+    channel count, four row groups (64x(0e+1o+2e), l <= 3, 303 pairs, 160 000 edges: two 346 us, three 264, four
+    255; more and longer bodies than that, 64x(0e+1o+2e+3o), likewise), tile sizes from what fits in shared memory
     (the formulas of FwdSmem / BwdSmem / Bwd1Smem) and CTAs per SM from the registers the bodies need.  The
     hand-tuned entries of signatures.json were found by measurement; these are the starting point such a search
     would begin from."""
@@ -87,7 +88,7 @@ def auto_params(sig, info):
     smem = 227 * 1024
     up = lambda v, a: (v + a - 1) // a * a
     need = {4: 168, 2: 104, 1: 72}[V]
-    out = {"V": V, "FW": 4 if info["n_pairs"] <= 300 else 2, "FS": 2, "BV": V, "BW": 4, "BS": 2, "EV": V, "ES": 2}
+    out = {"V": V, "FW": 4, "FS": 2, "BV": V, "BW": 4, "BS": 2, "EV": V, "ES": 2}
     # forward: CTAs per SM by registers, then the largest tile that fits
     threads = (out["FW"] * CH + 2) * 32
     FC = 2 if 65536 // (2 * threads) >= need else 1
