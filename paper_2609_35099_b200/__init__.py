@@ -177,6 +177,32 @@ def _check(status: int, where: str) -> int:
     return status
 
 
+_native = None      # the marshalling in native code (csrc/host/marshal.cpp), where it has been built
+_addresses = {}     # of the entry points it has called
+
+
+def _address(entry: str) -> int:
+    address = _addresses[entry] = ctypes.cast(getattr(_load(), entry), ctypes.c_void_p).value
+    return address
+
+
+def _run(entry: str, *args) -> None:
+    """Calls an entry point with integers and addresses (None: NULL); raises on a negative status."""
+    if _native is None:
+        status = getattr(_load(), entry)(*args)
+    else:
+        status = _native.call(_addresses.get(entry) or _address(entry), *args)
+    if status < 0:
+        raise E3JError(status, entry)
+
+
+def _bytes(entry: str, *args) -> int:
+    """The same for the functions that return a size."""
+    if _native is None:
+        return int(getattr(_load(), entry)(*args))
+    return _native.call_size(_addresses.get(entry) or _address(entry), *args)
+
+
 class Plan:
     """Owner of one e3j_plan handle (released when the object is collected)."""
 
@@ -254,10 +280,16 @@ def _stream_reader(torch):
 
 
 def _torch():
-    global _torch_module, _current_stream
+    global _torch_module, _current_stream, _native, _dev_ptr, _empty
     if _torch_module is None:
         import torch
         _current_stream = _stream_reader(torch)
+        try:
+            from . import _marshal as native   # (linked against torch's libraries)
+            native.set_slow(_dev_ptr, _empty)
+            _native, _dev_ptr, _empty = native, native.dev_ptr, native.empty
+        except ImportError:
+            pass
         _torch_module = torch
     return _torch_module
 
@@ -273,6 +305,11 @@ def _dev_ptr(t, dtype, shape, name):
     if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t.data_ptr()
+
+
+def _empty(shape, dtype, like):
+    """An uninitialised tensor on the device of `like`."""
+    return _torch().empty(shape, dtype=dtype, device=like.device)
 
 
 def _stream(stream):
@@ -292,7 +329,7 @@ def _workspace(nbytes: int, like, workspace, stream, least=None):
     """The caller's workspace, or a new one of nbytes.  least(): the bytes a call also runs with, where that is less."""
     torch = _torch()
     if workspace is None:
-        workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=like.device)
+        workspace = _empty((max(nbytes, 256),), torch.uint8, like)
         if stream is not None:   # released when the call returns: not to be used again before that stream is done with it
             workspace.record_stream(_as_torch_stream(stream))
         return workspace
@@ -307,15 +344,14 @@ def e3j_graph_prepare(n_nodes: int, senders, receivers, want_transpose: bool = T
     """(rowptr, sender_perm, colptr) int32 CUDA tensors; the last two are None unless want_transpose."""
     torch = _torch()
     e = senders.numel()
-    rowptr = torch.empty(n_nodes + 1, dtype=torch.int32, device=senders.device)
-    perm = torch.empty(max(e, 1), dtype=torch.int32, device=senders.device) if want_transpose else None
-    colptr = torch.empty(n_nodes + 1, dtype=torch.int32, device=senders.device) if want_transpose else None
-    _check(getattr(_load(), _entry)(n_nodes, e, _dev_ptr(senders, torch.int32, (e,), "senders"),
+    rowptr = _empty((n_nodes + 1,), torch.int32, senders)
+    perm = _empty((max(e, 1),), torch.int32, senders) if want_transpose else None
+    colptr = _empty((n_nodes + 1,), torch.int32, senders) if want_transpose else None
+    _run(_entry, n_nodes, e, _dev_ptr(senders, torch.int32, (e,), "senders"),
                                     _dev_ptr(receivers, torch.int32, (e,), "receivers"),
                                     _dev_ptr(rowptr, torch.int32, None, "rowptr"),
                                     _dev_ptr(perm, torch.int32, None, "sender_perm"),
-                                    _dev_ptr(colptr, torch.int32, None, "colptr"), _stream(stream)),
-           _entry)
+                                    _dev_ptr(colptr, torch.int32, None, "colptr"), _stream(stream))
     if perm is not None:
         perm = perm[:e]
     return rowptr, perm, colptr
@@ -343,11 +379,11 @@ def e3j_graph_validate(n_nodes: int, senders, receivers, stream=None) -> int:
 
 
 def e3j_conv_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
-    return int(_load().e3j_conv_fwd_workspace_bytes(plan.handle, n_nodes, n_edges))
+    return _bytes("e3j_conv_fwd_workspace_bytes", plan.handle.value, n_nodes, n_edges)
 
 
 def e3j_conv_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
-    return int(_load().e3j_conv_bwd_workspace_bytes(plan.handle, n_nodes, n_edges))
+    return _bytes("e3j_conv_bwd_workspace_bytes", plan.handle.value, n_nodes, n_edges)
 
 
 def e3j_conv_fwd(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=None, workspace=None,
@@ -356,18 +392,17 @@ def e3j_conv_fwd(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=None
     n, e = x.shape[0], senders.numel()
     f32, i32 = torch.float32, torch.int32
     if out is None:
-        out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
+        out = _empty((n, plan.d_out, plan.n_channels), f32, x)
     nbytes = e3j_conv_fwd_workspace_bytes(plan, n, e)
     workspace = _workspace(nbytes, x, workspace, stream)
-    _check(getattr(_load(), _entry)(
-        plan.handle, n, e,
+    _run(_entry, plan.handle.value, n, e,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), _entry)
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return out
 
 
@@ -386,13 +421,12 @@ def e3j_conv_fwd_noalloc(plan: Plan, x, sh, w, senders, receivers, out, stream=N
     torch = _torch()
     n, e = x.shape[0], senders.numel()
     f32, i32 = torch.float32, torch.int32
-    _check(_load().e3j_conv_fwd_noalloc(
-        plan.handle, n, e,
+    _run("e3j_conv_fwd_noalloc", plan.handle.value, n, e,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
-        _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"), _stream(stream)), "e3j_conv_fwd_noalloc")
+        _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"), _stream(stream))
     return out
 
 
@@ -415,7 +449,7 @@ def e3j_conv_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr=None
 
     def alloc(flag, shape):
         if flag is True:
-            return torch.empty(shape, dtype=f32, device=x.device)
+            return _empty(shape, f32, x)
         return flag if isinstance(flag, torch.Tensor) else None
 
     grad_x = alloc(grad_x, (n, plan.d_in, plan.n_channels))
@@ -423,8 +457,7 @@ def e3j_conv_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr=None
     grad_w = alloc(grad_w, (e, plan.n_paths, plan.n_channels))
     nbytes = e3j_conv_bwd_workspace_bytes(plan, n, e)
     workspace = _workspace(nbytes, x, workspace, stream)
-    _check(getattr(_load(), _entry)(
-        plan.handle, n, e,
+    _run(_entry, plan.handle.value, n, e,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
@@ -435,7 +468,7 @@ def e3j_conv_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr=None
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"),
         _dev_ptr(grad_sh, f32, (e, plan.d_sh), "grad_sh"),
         _dev_ptr(grad_w, f32, (e, plan.n_paths, plan.n_channels), "grad_w"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), _entry)
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return grad_x, grad_sh, grad_w
 
 
@@ -448,7 +481,7 @@ def e3j_conv_bwd_padded(plan: Plan, x, sh, w, senders, receivers, grad_out, rowp
 
 
 def e3j_conv_bwd_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
-    return int(_load().e3j_conv_bwd_bwd_workspace_bytes(plan.handle, n_nodes, n_edges))
+    return _bytes("e3j_conv_bwd_bwd_workspace_bytes", plan.handle.value, n_nodes, n_edges)
 
 
 def e3j_conv_bwd_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr, sender_perm, colptr,
@@ -463,22 +496,21 @@ def e3j_conv_bwd_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr,
 
     def alloc(flag, shape):
         if flag is True:
-            return torch.empty(shape, dtype=f32, device=x.device)
+            return _empty(shape, f32, x)
         return flag if isinstance(flag, torch.Tensor) else None
 
     s_x, s_sh = (n, plan.d_in, plan.n_channels), (e, plan.d_sh)
     s_w, s_out = (e, plan.n_paths, plan.n_channels), (n, plan.d_out, plan.n_channels)
     gg_out, g_x, g_sh, g_w = alloc(gg_out, s_out), alloc(g_x, s_x), alloc(g_sh, s_sh), alloc(g_w, s_w)
     workspace = _workspace(e3j_conv_bwd_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
-    _check(_load().e3j_conv_bwd_bwd(
-        plan.handle, n, e, _dev_ptr(x, f32, s_x, "x"), _dev_ptr(sh, f32, s_sh, "sh"), _dev_ptr(w, f32, s_w, "w"),
+    _run("e3j_conv_bwd_bwd", plan.handle.value, n, e, _dev_ptr(x, f32, s_x, "x"), _dev_ptr(sh, f32, s_sh, "sh"), _dev_ptr(w, f32, s_w, "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"), _dev_ptr(sender_perm, i32, (e,), "sender_perm"),
         _dev_ptr(colptr, i32, (n + 1,), "colptr"), _dev_ptr(grad_out, f32, s_out, "grad_out"),
         _dev_ptr(ct_x, f32, s_x, "ct_x"), _dev_ptr(ct_sh, f32, s_sh, "ct_sh"), _dev_ptr(ct_w, f32, s_w, "ct_w"),
         _dev_ptr(gg_out, f32, s_out, "gg_out"), _dev_ptr(g_x, f32, s_x, "g_x"), _dev_ptr(g_sh, f32, s_sh, "g_sh"),
         _dev_ptr(g_w, f32, s_w, "g_w"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_bwd_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return gg_out, g_x, g_sh, g_w
 
 
@@ -488,26 +520,25 @@ def e3j_radial_weights(plan: Plan, h, W, out=None, stream=None):
     e, hidden = h.shape
     f32 = torch.float32
     if out is None:
-        out = torch.empty((e, plan.n_paths, plan.n_channels), dtype=f32, device=h.device)
-    _check(_load().e3j_radial_weights(
-        plan.handle, e, hidden, _dev_ptr(h, f32, (e, hidden), "h"),
+        out = _empty((e, plan.n_paths, plan.n_channels), f32, h)
+    _run("e3j_radial_weights", plan.handle.value, e, hidden, _dev_ptr(h, f32, (e, hidden), "h"),
         _dev_ptr(W, f32, (hidden, plan.n_paths * plan.n_channels), "W"),
-        _dev_ptr(out, f32, (e, plan.n_paths, plan.n_channels), "out"), _stream(stream)), "e3j_radial_weights")
+        _dev_ptr(out, f32, (e, plan.n_paths, plan.n_channels), "out"), _stream(stream))
     return out
 
 
 def e3j_conv_radial_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
-    return int(_load().e3j_conv_radial_fwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+    return _bytes("e3j_conv_radial_fwd_workspace_bytes", plan.handle.value, n_nodes, n_edges, hidden)
 
 
 def e3j_conv_radial_fwd_least_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
     """The smallest workspace e3j_conv_radial_fwd runs with: where the plan has the kernel for it, without room for the
     edge weights, which are then formed inside the kernel (slower below 2 GiB of them)."""
-    return int(_load().e3j_conv_radial_fwd_least_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+    return _bytes("e3j_conv_radial_fwd_least_workspace_bytes", plan.handle.value, n_nodes, n_edges, hidden)
 
 
 def e3j_conv_radial_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
-    return int(_load().e3j_conv_radial_bwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+    return _bytes("e3j_conv_radial_bwd_workspace_bytes", plan.handle.value, n_nodes, n_edges, hidden)
 
 
 def e3j_conv_radial_fwd(plan: Plan, x, sh, h, W, senders, receivers, rowptr=None, out=None, workspace=None,
@@ -517,27 +548,26 @@ def e3j_conv_radial_fwd(plan: Plan, x, sh, h, W, senders, receivers, rowptr=None
     n, e, hidden = x.shape[0], senders.numel(), W.shape[0]
     f32, i32 = torch.float32, torch.int32
     if out is None:
-        out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
+        out = _empty((n, plan.d_out, plan.n_channels), f32, x)
     workspace = _workspace(e3j_conv_radial_fwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream,
                            lambda: e3j_conv_radial_fwd_least_workspace_bytes(plan, n, e, hidden))
-    _check(_load().e3j_conv_radial_fwd(
-        plan.handle, n, e, hidden,
+    _run("e3j_conv_radial_fwd", plan.handle.value, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(h, f32, (e, hidden), "h"), _dev_ptr(W, f32, (hidden, plan.n_paths * plan.n_channels), "W"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_fwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return out
 
 
 def e3j_conv_radial_vec_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
-    return int(_load().e3j_conv_radial_vec_fwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+    return _bytes("e3j_conv_radial_vec_fwd_workspace_bytes", plan.handle.value, n_nodes, n_edges, hidden)
 
 
 def e3j_conv_radial_vec_fwd_least_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
     """As e3j_conv_radial_fwd_least_workspace_bytes, for the call on edge vectors."""
-    return int(_load().e3j_conv_radial_vec_fwd_least_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+    return _bytes("e3j_conv_radial_vec_fwd_least_workspace_bytes", plan.handle.value, n_nodes, n_edges, hidden)
 
 
 def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, rowptr=None, out=None, workspace=None,
@@ -548,17 +578,16 @@ def e3j_conv_radial_vec_fwd(plan: Plan, x, edge_vec, h, W, senders, receivers, r
     n, e, hidden = x.shape[0], senders.numel(), W.shape[0]
     f32, i32 = torch.float32, torch.int32
     if out is None:
-        out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
+        out = _empty((n, plan.d_out, plan.n_channels), f32, x)
     workspace = _workspace(e3j_conv_radial_vec_fwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream,
                            lambda: e3j_conv_radial_vec_fwd_least_workspace_bytes(plan, n, e, hidden))
-    _check(_load().e3j_conv_radial_vec_fwd(
-        plan.handle, n, e, hidden,
+    _run("e3j_conv_radial_vec_fwd", plan.handle.value, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
         _dev_ptr(h, f32, (e, hidden), "h"), _dev_ptr(W, f32, (hidden, plan.n_paths * plan.n_channels), "W"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_vec_fwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return out
 
 
@@ -573,7 +602,7 @@ def e3j_conv_radial_bwd(plan: Plan, x, sh, h, W, senders, receivers, grad_out, r
 
     def alloc(flag, shape):
         if flag is True:
-            return torch.empty(shape, dtype=f32, device=x.device)
+            return _empty(shape, f32, x)
         return flag if isinstance(flag, torch.Tensor) else None
 
     s_w = (hidden, plan.n_paths * plan.n_channels)
@@ -582,8 +611,7 @@ def e3j_conv_radial_bwd(plan: Plan, x, sh, h, W, senders, receivers, grad_out, r
     grad_h = alloc(grad_h, (e, hidden))
     grad_W = alloc(grad_W, s_w)
     workspace = _workspace(e3j_conv_radial_bwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream)
-    _check(_load().e3j_conv_radial_bwd(
-        plan.handle, n, e, hidden,
+    _run("e3j_conv_radial_bwd", plan.handle.value, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(h, f32, (e, hidden), "h"), _dev_ptr(W, f32, s_w, "W"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
@@ -593,12 +621,12 @@ def e3j_conv_radial_bwd(plan: Plan, x, sh, h, W, senders, receivers, grad_out, r
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"),
         _dev_ptr(grad_sh, f32, (e, plan.d_sh), "grad_sh"),
         _dev_ptr(grad_h, f32, (e, hidden), "grad_h"), _dev_ptr(grad_W, f32, s_w, "grad_W"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return grad_x, grad_sh, grad_h, grad_W
 
 
 def e3j_conv_radial_vec_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int, hidden: int) -> int:
-    return int(_load().e3j_conv_radial_vec_bwd_workspace_bytes(plan.handle, n_nodes, n_edges, hidden))
+    return _bytes("e3j_conv_radial_vec_bwd_workspace_bytes", plan.handle.value, n_nodes, n_edges, hidden)
 
 
 def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, grad_out, rowptr=None, sender_perm=None,
@@ -612,7 +640,7 @@ def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, g
 
     def alloc(flag, shape):
         if flag is True:
-            return torch.empty(shape, dtype=f32, device=x.device)
+            return _empty(shape, f32, x)
         return flag if isinstance(flag, torch.Tensor) else None
 
     s_w = (hidden, plan.n_paths * plan.n_channels)
@@ -621,8 +649,7 @@ def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, g
     grad_h = alloc(grad_h, (e, hidden))
     grad_W = alloc(grad_W, s_w)
     workspace = _workspace(e3j_conv_radial_vec_bwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream)
-    _check(_load().e3j_conv_radial_vec_bwd(
-        plan.handle, n, e, hidden,
+    _run("e3j_conv_radial_vec_bwd", plan.handle.value, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
         _dev_ptr(h, f32, (e, hidden), "h"), _dev_ptr(W, f32, s_w, "W"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
@@ -631,7 +658,7 @@ def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, g
         _dev_ptr(grad_out, f32, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"), _dev_ptr(grad_vec, f32, (e, 3), "grad_vec"),
         _dev_ptr(grad_h, f32, (e, hidden), "grad_h"), _dev_ptr(grad_W, f32, s_w, "grad_W"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_radial_vec_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return grad_x, grad_vec, grad_h, grad_W
 
 
@@ -639,12 +666,11 @@ def e3j_tp_fwd(plan: Plan, x1, x2, w, out=None, stream=None):
     torch = _torch()
     rows, f32 = x1.shape[0], torch.float32
     if out is None:
-        out = torch.empty((rows, plan.d_out, plan.n_channels), dtype=f32, device=x1.device)
-    _check(_load().e3j_tp_fwd(
-        plan.handle, rows, _dev_ptr(x1, f32, (rows, plan.d_in, plan.n_channels), "x1"),
+        out = _empty((rows, plan.d_out, plan.n_channels), f32, x1)
+    _run("e3j_tp_fwd", plan.handle.value, rows, _dev_ptr(x1, f32, (rows, plan.d_in, plan.n_channels), "x1"),
         _dev_ptr(x2, f32, (rows, plan.d_sh), "x2"),
         _dev_ptr(w, f32, (rows, plan.n_paths, plan.n_channels), "w"),
-        _dev_ptr(out, f32, (rows, plan.d_out, plan.n_channels), "out"), _stream(stream)), "e3j_tp_fwd")
+        _dev_ptr(out, f32, (rows, plan.d_out, plan.n_channels), "out"), _stream(stream))
     return out
 
 
@@ -654,19 +680,18 @@ def e3j_tp_bwd(plan: Plan, x1, x2, w, grad_out, grad_x1=True, grad_x2=True, grad
 
     def alloc(flag, shape):
         if flag is True:
-            return torch.empty(shape, dtype=f32, device=x1.device)
+            return _empty(shape, f32, x1)
         return flag if isinstance(flag, torch.Tensor) else None
 
     grad_x1 = alloc(grad_x1, (rows, plan.d_in, plan.n_channels))
     grad_x2 = alloc(grad_x2, (rows, plan.d_sh))
     grad_w = alloc(grad_w, (rows, plan.n_paths, plan.n_channels))
-    _check(_load().e3j_tp_bwd(
-        plan.handle, rows, _dev_ptr(x1, f32, (rows, plan.d_in, plan.n_channels), "x1"),
+    _run("e3j_tp_bwd", plan.handle.value, rows, _dev_ptr(x1, f32, (rows, plan.d_in, plan.n_channels), "x1"),
         _dev_ptr(x2, f32, (rows, plan.d_sh), "x2"),
         _dev_ptr(w, f32, (rows, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(grad_out, f32, (rows, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x1, f32, None, "grad_x1"), _dev_ptr(grad_x2, f32, None, "grad_x2"),
-        _dev_ptr(grad_w, f32, None, "grad_w"), _stream(stream)), "e3j_tp_bwd")
+        _dev_ptr(grad_w, f32, None, "grad_w"), _stream(stream))
     return grad_x1, grad_x2, grad_w
 
 
@@ -701,21 +726,20 @@ def e3j_conv_bwd_scheduled(plan: Plan, x, sh, w, schedule, grad_out, grad_x=None
     n, e = x.shape[0], w.shape[0]
     f32 = torch.float32
     if grad_x is None:
-        grad_x = torch.empty((n, plan.d_in, plan.n_channels), dtype=f32, device=x.device)
+        grad_x = _empty((n, plan.d_in, plan.n_channels), f32, x)
     if grad_sh is None:
-        grad_sh = torch.empty((e, plan.d_sh), dtype=f32, device=x.device)
+        grad_sh = _empty((e, plan.d_sh), f32, x)
     if grad_w is None:
-        grad_w = torch.empty((e, plan.n_paths, plan.n_channels), dtype=f32, device=x.device)
+        grad_w = _empty((e, plan.n_paths, plan.n_channels), f32, x)
     workspace = _workspace(e3j_conv_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
     if schedule.dtype != torch.uint8 or not schedule.is_cuda:
         raise ValueError("schedule must be the CUDA uint8 tensor returned by e3j_bwd_schedule_build")
-    _check(_load().e3j_conv_bwd_scheduled(
-        plan.handle, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
+    _run("e3j_conv_bwd_scheduled", plan.handle.value, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"), schedule.data_ptr(),
         _dev_ptr(grad_out, f32, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"), _dev_ptr(grad_sh, f32, (e, plan.d_sh), "grad_sh"),
         _dev_ptr(grad_w, f32, (e, plan.n_paths, plan.n_channels), "grad_w"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_bwd_scheduled")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return grad_x, grad_sh, grad_w
 
 
@@ -724,9 +748,9 @@ def e3j_harmonics_fwd(lmax: int, edge_vec, out=None, stream=None):
     torch = _torch()
     e, f32 = edge_vec.shape[0], torch.float32
     if out is None:
-        out = torch.empty((e, (lmax + 1) ** 2), dtype=f32, device=edge_vec.device)
-    _check(_load().e3j_harmonics_fwd(lmax, e, _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
-                                     _dev_ptr(out, f32, (e, (lmax + 1) ** 2), "sh"), _stream(stream)), "e3j_harmonics_fwd")
+        out = _empty((e, (lmax + 1) ** 2), f32, edge_vec)
+    _run("e3j_harmonics_fwd", lmax, e, _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
+                                     _dev_ptr(out, f32, (e, (lmax + 1) ** 2), "sh"), _stream(stream))
     return out
 
 
@@ -735,19 +759,19 @@ def e3j_harmonics_bwd(lmax: int, edge_vec, grad_sh, out=None, stream=None):
     torch = _torch()
     e, f32 = edge_vec.shape[0], torch.float32
     if out is None:
-        out = torch.empty((e, 3), dtype=f32, device=edge_vec.device)
-    _check(_load().e3j_harmonics_bwd(lmax, e, _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
+        out = _empty((e, 3), f32, edge_vec)
+    _run("e3j_harmonics_bwd", lmax, e, _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
                                      _dev_ptr(grad_sh, f32, (e, (lmax + 1) ** 2), "grad_sh"),
-                                     _dev_ptr(out, f32, (e, 3), "grad_vec"), _stream(stream)), "e3j_harmonics_bwd")
+                                     _dev_ptr(out, f32, (e, 3), "grad_vec"), _stream(stream))
     return out
 
 
 def e3j_conv_vec_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
-    return int(_load().e3j_conv_vec_fwd_workspace_bytes(plan.handle, n_nodes, n_edges))
+    return _bytes("e3j_conv_vec_fwd_workspace_bytes", plan.handle.value, n_nodes, n_edges)
 
 
 def e3j_conv_vec_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
-    return int(_load().e3j_conv_vec_bwd_workspace_bytes(plan.handle, n_nodes, n_edges))
+    return _bytes("e3j_conv_vec_bwd_workspace_bytes", plan.handle.value, n_nodes, n_edges)
 
 
 def e3j_conv_vec_fwd(plan: Plan, x, edge_vec, w, senders, receivers, rowptr=None, out=None, workspace=None,
@@ -757,14 +781,13 @@ def e3j_conv_vec_fwd(plan: Plan, x, edge_vec, w, senders, receivers, rowptr=None
     n, e = x.shape[0], senders.numel()
     f32, i32 = torch.float32, torch.int32
     if out is None:
-        out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f32, device=x.device)
+        out = _empty((n, plan.d_out, plan.n_channels), f32, x)
     workspace = _workspace(e3j_conv_vec_fwd_workspace_bytes(plan, n, e), x, workspace, stream)
-    _check(_load().e3j_conv_vec_fwd(
-        plan.handle, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
+    _run("e3j_conv_vec_fwd", plan.handle.value, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"), _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"), _dev_ptr(out, f32, (n, plan.d_out, plan.n_channels), "out"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_vec_fwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return out
 
 
@@ -777,15 +800,14 @@ def e3j_conv_vec_bwd(plan: Plan, x, edge_vec, w, senders, receivers, grad_out, r
 
     def alloc(flag, shape):
         if flag is True:
-            return torch.empty(shape, dtype=f32, device=x.device)
+            return _empty(shape, f32, x)
         return flag if isinstance(flag, torch.Tensor) else None
 
     grad_x = alloc(grad_x, (n, plan.d_in, plan.n_channels))
     grad_vec = alloc(grad_vec, (e, 3))
     grad_w = alloc(grad_w, (e, plan.n_paths, plan.n_channels))
     workspace = _workspace(e3j_conv_vec_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
-    _check(_load().e3j_conv_vec_bwd(
-        plan.handle, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
+    _run("e3j_conv_vec_bwd", plan.handle.value, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"), _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"), _dev_ptr(sender_perm, i32, (e,), "sender_perm"),
@@ -793,7 +815,7 @@ def e3j_conv_vec_bwd(plan: Plan, x, edge_vec, w, senders, receivers, grad_out, r
         _dev_ptr(grad_out, f32, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(grad_x, f32, (n, plan.d_in, plan.n_channels), "grad_x"), _dev_ptr(grad_vec, f32, (e, 3), "grad_vec"),
         _dev_ptr(grad_w, f32, (e, plan.n_paths, plan.n_channels), "grad_w"),
-        workspace.data_ptr(), workspace.numel(), _stream(stream)), "e3j_conv_vec_bwd")
+        workspace.data_ptr(), workspace.numel(), _stream(stream))
     return grad_x, grad_vec, grad_w
 
 
@@ -802,14 +824,13 @@ def e3j_conv_fwd_f64(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=
     torch = _torch()
     n, e, f64, i32 = x.shape[0], senders.numel(), torch.float64, torch.int32
     if out is None:
-        out = torch.empty((n, plan.d_out, plan.n_channels), dtype=f64, device=x.device)
-    ws = _workspace(int(_load().e3j_conv_f64_workspace_bytes(plan.handle, n, e)), x, None, stream)
-    _check(_load().e3j_conv_fwd_f64(
-        plan.handle, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
+        out = _empty((n, plan.d_out, plan.n_channels), f64, x)
+    ws = _workspace(_bytes("e3j_conv_f64_workspace_bytes", plan.handle.value, n, e), x, None, stream)
+    _run("e3j_conv_fwd_f64", plan.handle.value, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f64, (e, plan.n_paths, plan.n_channels), "w"), _dev_ptr(senders, i32, (e,), "senders"),
         _dev_ptr(receivers, i32, (e,), "receivers"), _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),
         _dev_ptr(out, f64, (n, plan.d_out, plan.n_channels), "out"), ws.data_ptr(), ws.numel(),
-        _stream(stream)), "e3j_conv_fwd_f64")
+        _stream(stream))
     return out
 
 
@@ -817,17 +838,16 @@ def e3j_conv_bwd_f64(plan: Plan, x, sh, w, senders, receivers, grad_out, sender_
     """Float64 backward convolution: (grad_x, grad_sh, grad_w)."""
     torch = _torch()
     n, e, f64, i32 = x.shape[0], senders.numel(), torch.float64, torch.int32
-    gx = torch.empty((n, plan.d_in, plan.n_channels), dtype=f64, device=x.device)
-    gsh = torch.empty((e, plan.d_sh), dtype=f64, device=x.device)
-    gw = torch.empty((e, plan.n_paths, plan.n_channels), dtype=f64, device=x.device)
-    ws = _workspace(int(_load().e3j_conv_f64_workspace_bytes(plan.handle, n, e)), x, None, stream)
-    _check(_load().e3j_conv_bwd_f64(
-        plan.handle, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
+    gx = _empty((n, plan.d_in, plan.n_channels), f64, x)
+    gsh = _empty((e, plan.d_sh), f64, x)
+    gw = _empty((e, plan.n_paths, plan.n_channels), f64, x)
+    ws = _workspace(_bytes("e3j_conv_f64_workspace_bytes", plan.handle.value, n, e), x, None, stream)
+    _run("e3j_conv_bwd_f64", plan.handle.value, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f64, (e, plan.n_paths, plan.n_channels), "w"), _dev_ptr(senders, i32, (e,), "senders"),
         _dev_ptr(receivers, i32, (e,), "receivers"), _dev_ptr(sender_perm, i32, (e,), "sender_perm"),
         _dev_ptr(colptr, i32, (n + 1,), "colptr"), _dev_ptr(grad_out, f64, (n, plan.d_out, plan.n_channels), "grad_out"),
         _dev_ptr(gx, f64, None, "grad_x"), _dev_ptr(gsh, f64, None, "grad_sh"), _dev_ptr(gw, f64, None, "grad_w"),
-        ws.data_ptr(), ws.numel(), _stream(stream)), "e3j_conv_bwd_f64")
+        ws.data_ptr(), ws.numel(), _stream(stream))
     return gx, gsh, gw
 
 

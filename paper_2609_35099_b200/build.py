@@ -4,7 +4,8 @@
 
 Every translation unit under csrc/ (and the generated ones under csrc/fast/) is
 compiled with nvcc for compute_100a / sm_100a and linked into
-paper_2609_35099_b200/libe3j.so.  nvcc cross-compiles without a GPU.  Object files
+paper_2609_35099_b200/libe3j.so, and the Python binding's marshalling
+(csrc/host/) with g++ into _marshal.so.  nvcc cross-compiles without a GPU.  Object files
 and the ptxas resource report (registers, spills, shared memory) go to csrc/build/.
 
 Signatures beyond the committed list: --signatures names a JSON list of entries like
@@ -75,12 +76,39 @@ def _link(objs, out: Path) -> None:
     os.replace(tmp, out)
 
 
+def _build_marshal(force: bool) -> None:
+    """The binding's native marshalling, against the installed torch.  Without torch's headers the binding does the same in
+    Python."""
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    src, out, stamp = CSRC / "host" / "marshal.cpp", PKG / "_marshal.so", BUILD / "marshal.stamp"
+    key = hashlib.sha256(src.read_bytes()).hexdigest()[:16] + torch.__version__ + sys.version
+    if not force and out.exists() and stamp.exists() and stamp.read_text() == key:
+        return
+    lib = Path(torch.__file__).parent / "lib"
+    tmp = out.with_suffix(f".tmp{os.getpid()}.so")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *(f"-I{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], "/usr/local/cuda/include"]),
+           str(src), "-o", str(tmp), f"-L{lib}", "-ltorch_python", "-ltorch_cpu", "-lc10"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(f"_marshal not built, the binding converts its arguments in Python:\n{res.stderr[-2000:]}")
+        out.unlink(missing_ok=True)
+        return
+    os.replace(tmp, out)
+    stamp.write_text(key)
+
+
 def build(force: bool = False, verbose: bool = False) -> Path:
     BUILD.mkdir(parents=True, exist_ok=True)
     digest = _deps_digest()
     srcs = sources()
     with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as ex:
+        marshal = ex.submit(_build_marshal, force)
         objs = list(ex.map(lambda s: _compile(s, digest, force, verbose), srcs))
+        marshal.result()
     newest = max(o.stat().st_mtime for o in objs)
     if force or not OUT.exists() or OUT.stat().st_mtime < newest:
         _link(objs, OUT)
