@@ -41,10 +41,12 @@ def test_with_and_without_room_for_the_shares(irreps, lmax, nodes, degree, real)
     full = query(plan.handle, nodes, e)
     least = full - (size * e * plan.d_in * plan.n_channels + 255) // 256 * 256
 
-    def call(nbytes):
+    def call(nbytes, want_x=True):
         grads = [torch.full_like(t, float("nan")) for t in (x, sh, w)]
         ws = torch.full((max(nbytes, 256),), 255, dtype=torch.uint8, device="cuda")
         p = [t.data_ptr() for t in (x, sh, w, s, r, rowptr, perm, colptr, g, *grads, ws)]
+        if not want_x:
+            p[9] = None
         if f64:
             del p[5]
         status = (lib.e3j_conv_bwd_f64 if f64 else lib.e3j_conv_bwd)(plan.handle, nodes, e, *p, nbytes,
@@ -60,6 +62,8 @@ def test_with_and_without_room_for_the_shares(irreps, lmax, nodes, degree, real)
     for res in (shares, inputs):
         for have, ref, kind in zip(res, want, ("x", "sh", "w")):
             assert_blockwise_close(have.cpu().numpy(), ref, blocks_of_paths(cp.paths, kind), tol=1e-12 if f64 else 1e-5, what=kind)
+    _, edges = call(full, want_x=False)
+    assert edges[0].isnan().all() and all(torch.equal(a, b) for a, b in zip(shares[1:], edges[1:]))
     if not f64:
         assert call(least - 256)[0] == e3j.E3J_ERR_WORKSPACE
 
