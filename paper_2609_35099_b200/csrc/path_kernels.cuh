@@ -14,11 +14,11 @@
 //   node sums by single output blocks: the forward of plans whose paths share output rows, and grad_x (tensor transposed,
 //              edges in sender order) where the workspace has no room for the shares or where every input is scalar.
 //
-// What bounds them, 48x(0e+1o+2e), l <= 2, 35 050 edges: the edge part its instructions (90 us, 55 % of the issue slots, half
-// of them multiply-adds), the forward the latency of its row loads at 24 warps per SM (53 us, 40 % of the issue slots), the
-// sum of the shares its loads (16 us).  Both passes 218 -> 161 us against one thread per output block with grad_x from the
+// What bounds them, 48x(0e+1o+2e), l <= 2, 35 050 edges: the edge part its instructions (90 us, 60 % of the issue slots, half
+// of them multiply-adds), the forward the latency of its row loads at 24 warps per SM (50 us, 45 % of the issue slots), the
+// sum of the shares its loads (16 us).  Both passes 218 -> 157 us against one thread per output block with grad_x from the
 // edges' inputs (every path's input rows and harmonics loaded again, the weights read twice in the backward); float64,
-// 64x(0e+1o), l <= 2, 10 176 edges: 106 -> 80 us.  Tried and slower: a block's tiles one after the other with the copies
+// 64x(0e+1o), l <= 2, 10 176 edges: 106 -> 77 us.  Tried and slower: a block's tiles one after the other with the copies
 // running on from tile to tile and the input rows among them (fewer warps fit: backward 106 -> 145 us); weights and ids two
 // steps ahead in registers (spills), each path's sum as a function of its own, grad_out rows of the next path in registers.
 //
