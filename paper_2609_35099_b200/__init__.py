@@ -284,9 +284,9 @@ def _torch():
     if _torch_module is None:
         import torch
         _current_stream = _stream_reader(torch)
-        try:
+        try:   # several threads may come here together: each leaves the same behind, and no name changes that is read here
             from . import _marshal as native   # (linked against torch's libraries)
-            native.set_slow(_dev_ptr, _empty)
+            native.set_slow(_dev_ptr_in_python, _empty_in_python)
             _native, _dev_ptr, _empty = native, native.dev_ptr, native.empty
         except ImportError:
             pass
@@ -294,7 +294,7 @@ def _torch():
     return _torch_module
 
 
-def _dev_ptr(t, dtype, shape, name):
+def _dev_ptr_in_python(t, dtype, shape, name):
     """Device address of a contiguous CUDA tensor of that type (and shape, if given); None stays None."""
     if t is None:
         return None
@@ -307,9 +307,12 @@ def _dev_ptr(t, dtype, shape, name):
     return t.data_ptr()
 
 
-def _empty(shape, dtype, like):
+def _empty_in_python(shape, dtype, like):
     """An uninitialised tensor on the device of `like`."""
     return _torch().empty(shape, dtype=dtype, device=like.device)
+
+
+_dev_ptr, _empty = _dev_ptr_in_python, _empty_in_python   # replaced by the native functions where there are any
 
 
 def _stream(stream):
