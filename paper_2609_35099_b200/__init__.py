@@ -15,6 +15,9 @@ an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import importlib
+import sysconfig
+import warnings
 from pathlib import Path
 
 __all__ = [
@@ -279,17 +282,37 @@ def _stream_reader(torch):
     return (lambda: raw(device())) if raw and device else lambda: torch.cuda.current_stream().cuda_stream
 
 
+def _marshal_abi(torch) -> str:
+    """What the native marshalling is compiled against: it reads the objects of this torch and this interpreter directly."""
+    return f"torch {torch.__version__} ({torch.version.git_version}), {sysconfig.get_config_var('EXT_SUFFIX')}"
+
+
+def _native_marshalling(torch):
+    """The module built from csrc/host/marshal.cpp, or None where there is none for this torch and interpreter."""
+    try:
+        native = importlib.import_module("._marshal", __package__)   # (linked against torch's libraries)
+        built_for = getattr(native, "built_for", "unknown")
+        if built_for == _marshal_abi(torch):
+            return native
+        reason = f"built for {built_for}, this is {_marshal_abi(torch)}"
+    except ModuleNotFoundError:
+        return None
+    except ImportError as error:
+        reason = str(error)
+    warnings.warn(f"native marshalling not used, calls convert their arguments in Python until the next build: {reason}",
+                  RuntimeWarning, stacklevel=4)
+    return None
+
+
 def _torch():
     global _torch_module, _current_stream, _native, _dev_ptr, _empty
     if _torch_module is None:
         import torch
         _current_stream = _stream_reader(torch)
-        try:   # several threads may come here together: each leaves the same behind, and no name changes that is read here
-            from . import _marshal as native   # (linked against torch's libraries)
+        native = _native_marshalling(torch)
+        if native is not None:   # several threads may come here together: each leaves the same behind, and no name changes that is read here
             native.set_slow(_dev_ptr_in_python, _empty_in_python)
             _native, _dev_ptr, _empty = native, native.dev_ptr, native.empty
-        except ImportError:
-            pass
         _torch_module = torch
     return _torch_module
 

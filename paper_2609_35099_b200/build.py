@@ -5,7 +5,7 @@
 Every translation unit under csrc/ (and the generated ones under csrc/fast/) is
 compiled with nvcc for compute_100a / sm_100a and linked into
 paper_2609_35099_b200/libe3j.so, and the Python binding's marshalling
-(csrc/host/) with g++ into _marshal.so.  nvcc cross-compiles without a GPU.  Object files
+(csrc/host/) with g++ into _marshal (with the interpreter's suffix).  nvcc cross-compiles without a GPU.  Object files
 and the ptxas resource report (registers, spills, shared memory) go to csrc/build/.
 
 Signatures beyond the committed list: --signatures names a JSON list of entries like
@@ -23,6 +23,7 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -79,17 +80,21 @@ def _link(objs, out: Path) -> None:
 def _build_marshal(force: bool) -> None:
     """The binding's native marshalling, against the installed torch.  Without torch's headers the binding does the same in
     Python."""
-    import sysconfig
-
     import torch
     from torch.utils import cpp_extension
-    src, out, stamp = CSRC / "host" / "marshal.cpp", PKG / "_marshal.so", BUILD / "marshal.stamp"
-    key = hashlib.sha256(src.read_bytes()).hexdigest()[:16] + torch.__version__ + sys.version
+
+    from . import _marshal_abi
+    abi = _marshal_abi(torch)
+    src, out, stamp = CSRC / "host" / "marshal.cpp", PKG / f"_marshal{sysconfig.get_config_var('EXT_SUFFIX')}", BUILD / "marshal.stamp"
+    for old in PKG.glob("_marshal*.so"):   # another interpreter's, or one without a suffix, which any interpreter would load
+        if old != out and ".tmp" not in old.name:
+            old.unlink()
+    key = hashlib.sha256(src.read_bytes()).hexdigest()[:16] + abi
     if not force and out.exists() and stamp.exists() and stamp.read_text() == key:
         return
     lib = Path(torch.__file__).parent / "lib"
     tmp = out.with_suffix(f".tmp{os.getpid()}.so")
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f'-DE3J_BUILT_FOR="{abi}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            *(f"-I{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], "/usr/local/cuda/include"]),
            str(src), "-o", str(tmp), f"-L{lib}", "-ltorch_python", "-ltorch_cpu", "-lc10"]
     res = subprocess.run(cmd, capture_output=True, text=True)

@@ -141,4 +141,10 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&module); }
+// built_for: the torch and the interpreter whose object layouts are compiled in here; the binding uses the module with
+// these alone.
+PyMODINIT_FUNC PyInit__marshal() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", E3J_BUILT_FOR) != 0) Py_CLEAR(m);
+    return m;
+}

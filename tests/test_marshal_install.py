@@ -1,10 +1,12 @@
 """How the binding takes up its native marshalling (csrc/host/marshal.cpp): no device."""
+import pathlib
+import shutil
 import subprocess
 import sys
 
 import pytest
 
-pytest.importorskip("torch")
+torch = pytest.importorskip("torch")
 
 
 def _run(code, cwd):
@@ -33,3 +35,27 @@ for _ in range(2):   # (again with everything in place: the order that a preempt
     e3j._torch()
 """, repo_root)
     assert done.stdout.splitlines() == ["x must be a CUDA tensor"] * 2, done.stderr[-2000:]
+
+
+def test_a_module_built_for_another_torch_is_not_used(repo_root):
+    """Its functions would read tensors with the wrong layouts."""
+    done = _run("""
+import sys, types, warnings
+import paper_2609_35099_b200 as e3j
+def never(*args): raise SystemExit("called")
+other = types.SimpleNamespace(set_slow=never, dev_ptr=never, empty=never, call=never, call_size=never, built_for="torch 1.0")
+sys.modules[e3j.__name__ + "._marshal"] = other
+with warnings.catch_warnings(record=True) as seen:
+    warnings.simplefilter("always")
+    e3j._torch()
+print(e3j._native, "torch 1.0" in str(seen[0].message))
+""", repo_root)
+    assert done.stdout.split() == ["None", "True"], done.stderr[-2000:]
+
+
+def test_it_is_there_where_it_can_be_built(repo_root):
+    from torch.utils import cpp_extension
+    if not shutil.which("g++") or not any((pathlib.Path(d) / "torch" / "csrc" / "Dtype.h").exists() for d in cpp_extension.include_paths()):
+        pytest.skip("no g++, or no headers of torch")
+    done = _run("import paper_2609_35099_b200 as e3j; t = e3j._torch(); print(e3j._native.built_for == e3j._marshal_abi(t))", repo_root)
+    assert done.stdout.split() == ["True"], done.stderr[-2000:]
