@@ -78,32 +78,33 @@ def _link(objs, out: Path) -> None:
 
 
 def _build_marshal(force: bool) -> None:
-    """The binding's native marshalling, against the installed torch.  Without torch's headers the binding does the same in
-    Python."""
-    import torch
-    from torch.utils import cpp_extension
-
-    from . import _marshal_abi
-    abi = _marshal_abi(torch)
-    src, out, stamp = CSRC / "host" / "marshal.cpp", PKG / f"_marshal{sysconfig.get_config_var('EXT_SUFFIX')}", BUILD / "marshal.stamp"
+    """The binding's native marshalling, against the installed torch.  Where that cannot be done (no torch, no compiler) the
+    binding does the same in Python; the library does not depend on it."""
+    out, stamp = PKG / f"_marshal{sysconfig.get_config_var('EXT_SUFFIX')}", BUILD / "marshal.stamp"
+    tmp = out.with_suffix(f".tmp{os.getpid()}.so")
     for old in PKG.glob("_marshal*.so"):   # another interpreter's, or one without a suffix, which any interpreter would load
         if old != out and ".tmp" not in old.name:
             old.unlink()
-    key = hashlib.sha256(src.read_bytes()).hexdigest()[:16] + abi
-    if not force and out.exists() and stamp.exists() and stamp.read_text() == key:
-        return
-    lib = Path(torch.__file__).parent / "lib"
-    tmp = out.with_suffix(f".tmp{os.getpid()}.so")
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f'-DE3J_BUILT_FOR="{abi}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           *(f"-I{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], "/usr/local/cuda/include"]),
-           str(src), "-o", str(tmp), f"-L{lib}", "-ltorch_python", "-ltorch_cpu", "-lc10"]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        sys.stderr.write(f"_marshal not built, the binding converts its arguments in Python:\n{res.stderr[-2000:]}")
+    try:
+        import torch
+        from torch.utils import cpp_extension
+
+        from . import _marshal_abi
+        abi, src, lib = _marshal_abi(torch), CSRC / "host" / "marshal.cpp", Path(torch.__file__).parent / "lib"
+        key = hashlib.sha256(src.read_bytes()).hexdigest()[:16] + abi
+        if not force and out.exists() and stamp.exists() and stamp.read_text() == key:
+            return
+        cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f'-DE3J_BUILT_FOR="{abi}"',
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               *(f"-I{d}" for d in [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], "/usr/local/cuda/include"]),
+               str(src), "-o", str(tmp), f"-L{lib}", "-ltorch_python", "-ltorch_cpu", "-lc10"]
+        subprocess.run(cmd, capture_output=True, text=True, check=True)
+        os.replace(tmp, out)
+        stamp.write_text(key)
+    except Exception as error:
+        sys.stderr.write(f"_marshal not built, the binding converts its arguments in Python: {error}\n"
+                         f"{(getattr(error, 'stderr', None) or '')[-2000:]}")
         out.unlink(missing_ok=True)
-        return
-    os.replace(tmp, out)
-    stamp.write_text(key)
 
 
 def build(force: bool = False, verbose: bool = False) -> Path:

@@ -3,6 +3,7 @@ import pathlib
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 import pytest
 
@@ -59,3 +60,22 @@ def test_it_is_there_where_it_can_be_built(repo_root):
         pytest.skip("no g++, or no headers of torch")
     done = _run("import paper_2609_35099_b200 as e3j; t = e3j._torch(); print(e3j._native.built_for == e3j._marshal_abi(t))", repo_root)
     assert done.stdout.split() == ["True"], done.stderr[-2000:]
+
+
+@pytest.mark.parametrize("missing", ["torch", "g++"])
+def test_the_library_is_linked_without_it(missing, tmp_path, monkeypatch, capsys):
+    """The C library needs neither torch nor a host compiler of that name; what an earlier build left is taken away."""
+    from paper_2609_35099_b200 import build
+    stale = tmp_path / f"_marshal{sysconfig.get_config_var('EXT_SUFFIX')}"
+    stale.write_bytes(b"")
+    obj = tmp_path / "one.o"
+    obj.write_bytes(b"")
+    for name, value in dict(PKG=tmp_path, BUILD=tmp_path, OUT=tmp_path / "libe3j.so", sources=lambda: ["one.cu"],
+                            _deps_digest=lambda: "", _compile=lambda *args: obj, _link=lambda objs, out: out.write_text("linked")).items():
+        monkeypatch.setattr(build, name, value)
+    if missing == "torch":
+        monkeypatch.setitem(sys.modules, "torch", None)
+    else:
+        monkeypatch.setenv("PATH", str(tmp_path))
+    assert build.build().read_text() == "linked"
+    assert not stale.exists() and "the binding converts its arguments in Python" in capsys.readouterr().err
