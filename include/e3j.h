@@ -203,8 +203,13 @@ int e3j_noalloc_status(int32_t* status);
  * stores of grad_sh / grad_w and the sender sum of grad_x).  rowptr, sender_perm, colptr as produced by e3j_graph_prepare, or NULL
  * (then derived into the workspace on every call).  A node that sends nothing gets
  * a zero grad_x row. */
-size_t e3j_conv_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges);   /* plans without generated kernels:
- * with room for [n_edges, d, N_q] floats that only make the call faster; it and the calls that contain it run without it */
+size_t e3j_conv_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges);
+/* Plans without generated kernels sum grad_x from the edges' shares of it where the workspace has room for them,
+ * [n_edges, d, N_q] elements: faster than from the edges' inputs, and in another order, so grad_x has other last bits
+ * (each of the two is the same from run to run; grad_sh and grad_w do not depend on it).  This is what the workspace
+ * queries of e3j_conv_bwd, _bwd_padded, _bwd_bwd, _vec_bwd, _radial_bwd and _radial_vec_bwd (element_bytes 4) and
+ * e3j_conv_f64_workspace_bytes (8) hold for it: those calls also run with that much less.  0 for other plans. */
+size_t e3j_conv_bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges, int element_bytes);
 int e3j_conv_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const float* x,
                  const float* sh, const float* w, const int32_t* senders,
                  const int32_t* receivers, const int32_t* rowptr, const int32_t* sender_perm,
@@ -398,8 +403,9 @@ int e3j_conv_radial_vec_bwd(const e3j_plan* plan, int64_t n_nodes, int64_t n_edg
  * kernels where the per-channel arrays start on 16 bytes, everything else on table-driven ones; fixed summation order,
  * bit-identical from run to run.  No alignment requirement beyond 8 bytes.  rowptr /
  * sender_perm / colptr as produced by e3j_graph_prepare, or NULL (then derived into the workspace, 256-byte
- * aligned, e3j_conv_f64_workspace_bytes()); with that many bytes the backward is faster, also where the
- * graph's arrays are given; any of grad_x, grad_sh, grad_w may be NULL. */
+ * aligned, e3j_conv_f64_workspace_bytes()); of these the forward and a backward without grad_x have no use for
+ * e3j_conv_bwd_shares_bytes(), any other backward takes them also where the graph's arrays are given; any of grad_x,
+ * grad_sh, grad_w may be NULL. */
 size_t e3j_conv_f64_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges);
 int e3j_conv_fwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const double* x, const double* sh,
                      const double* w, const int32_t* senders, const int32_t* receivers, const int32_t* rowptr,

@@ -23,7 +23,7 @@ from pathlib import Path
 __all__ = [
     "E3JError", "Plan", "library_path", "e3j_plan_create", "e3j_plan_destroy", "e3j_plan_info",
     "e3j_plan_paths", "e3j_plan_records", "e3j_plan_signature", "e3j_plan_device_status", "e3j_graph_prepare", "e3j_graph_validate",
-    "e3j_conv_fwd_workspace_bytes", "e3j_conv_bwd_workspace_bytes", "e3j_conv_fwd", "e3j_conv_fwd_noalloc", "e3j_noalloc_status",
+    "e3j_conv_fwd_workspace_bytes", "e3j_conv_bwd_workspace_bytes", "e3j_conv_bwd_shares_bytes", "e3j_conv_fwd", "e3j_conv_fwd_noalloc", "e3j_noalloc_status",
     "e3j_conv_bwd", "e3j_graph_prepare_padded", "e3j_conv_fwd_padded", "e3j_conv_bwd_padded",
     "e3j_conv_bwd_bwd_workspace_bytes", "e3j_conv_bwd_bwd",
     "e3j_radial_weights", "e3j_conv_radial_fwd_workspace_bytes", "e3j_conv_radial_fwd_least_workspace_bytes",
@@ -95,6 +95,8 @@ def _load():
     lib.e3j_conv_fwd_workspace_bytes.restype = sz
     lib.e3j_conv_bwd_workspace_bytes.argtypes = [vp, i64, i64]
     lib.e3j_conv_bwd_workspace_bytes.restype = sz
+    lib.e3j_conv_bwd_shares_bytes.argtypes = [vp, i64, i32]
+    lib.e3j_conv_bwd_shares_bytes.restype = sz
     lib.e3j_conv_fwd.argtypes = [vp, i64, i64] + [vp] * 8 + [sz, vp]
     lib.e3j_conv_bwd.argtypes = [vp, i64, i64] + [vp] * 13 + [sz, vp]
     lib.e3j_conv_fwd_padded.argtypes = [vp, i64, i64] + [vp] * 8 + [sz, vp]
@@ -410,6 +412,12 @@ def e3j_conv_fwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
 
 def e3j_conv_bwd_workspace_bytes(plan: Plan, n_nodes: int, n_edges: int) -> int:
     return _bytes("e3j_conv_bwd_workspace_bytes", plan.handle.value, n_nodes, n_edges)
+
+
+def e3j_conv_bwd_shares_bytes(plan: Plan, n_edges: int, element_bytes: int = 4) -> int:
+    """The part of the workspace queries of calls with a backward (element_bytes 8: in float64) that these also run
+    without: slower, and with grad_x summed in another order."""
+    return _bytes("e3j_conv_bwd_shares_bytes", plan.handle.value, n_edges, element_bytes)
 
 
 def e3j_conv_fwd(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=None, workspace=None,
@@ -851,7 +859,8 @@ def e3j_conv_fwd_f64(plan: Plan, x, sh, w, senders, receivers, rowptr=None, out=
     n, e, f64, i32 = x.shape[0], senders.numel(), torch.float64, torch.int32
     if out is None:
         out = _empty((n, plan.d_out, plan.n_channels), f64, x)
-    ws = _workspace(_bytes("e3j_conv_f64_workspace_bytes", plan.handle.value, n, e), x, None, stream)
+    ws = _workspace(_bytes("e3j_conv_f64_workspace_bytes", plan.handle.value, n, e) - e3j_conv_bwd_shares_bytes(plan, e, 8),
+                    x, None, stream)
     _run("e3j_conv_fwd_f64", plan.handle.value, n, e, _dev_ptr(x, f64, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f64, (e, plan.d_sh), "sh"),
         _dev_ptr(w, f64, (e, plan.n_paths, plan.n_channels), "w"), _dev_ptr(senders, i32, (e,), "senders"),
         _dev_ptr(receivers, i32, (e,), "receivers"), _dev_ptr(rowptr, i32, (n + 1,), "rowptr"),

@@ -206,9 +206,10 @@ int check_workspace(const void* ws, size_t have, size_t need) {
 
 }  // namespace
 
-size_t bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges) {
-    if (fast_lookup(plan) || !path::covers(plan, 4) || !path::uses_shares(plan)) return 0;
-    return align_up(4 * (size_t)n_edges * plan->d * plan->nq, 256);
+size_t bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges, int element_bytes) {
+    const bool f64 = element_bytes == 8;
+    if ((!f64 && fast_lookup(plan)) || !path::covers(plan, f64 ? 2 : 4) || !path::uses_shares(plan)) return 0;
+    return align_up((size_t)element_bytes * n_edges * plan->d * plan->nq, 256);
 }
 
 }  // namespace e3j
@@ -322,6 +323,11 @@ size_t e3j_conv_fwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64
 size_t e3j_conv_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     if (!plan || n_nodes < 0 || n_edges < 0) return 0;
     return layout(plan, n_nodes, n_edges, true).total + bwd_shares_bytes(plan, n_edges);
+}
+
+size_t e3j_conv_bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges, int element_bytes) {
+    if (!plan || n_edges < 0 || (element_bytes != 4 && element_bytes != 8)) return 0;
+    return bwd_shares_bytes(plan, n_edges, element_bytes);
 }
 
 }  // extern "C"

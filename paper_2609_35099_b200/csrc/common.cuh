@@ -95,7 +95,7 @@ int conv_fwd_impl(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const 
 // Room that the backward of a plan without generated kernels has use for behind the rest of its workspace: each edge's
 // share of grad_x.  Part of e3j_conv_bwd_workspace_bytes(); a call that has everything but this room sums grad_x from
 // the edges' inputs instead, so calls that compose the backward put its workspace last.
-size_t bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges);
+size_t bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges, int element_bytes = 4);
 // Harmonics of edge vectors (harmonics.cu): sh [n, (lmax+1)^2] from vec [n, 3] and the gradient back; lmax <= 3.
 int harmonics_fwd(int lmax, int64_t n, const float* vec, float* sh, cudaStream_t st);
 int harmonics_bwd(int lmax, int64_t n, const float* vec, const float* grad_sh, float* grad_vec, cudaStream_t st);

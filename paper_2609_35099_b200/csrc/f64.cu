@@ -144,13 +144,10 @@ extern "C" {
 static size_t graph_bytes(int64_t n_nodes, int64_t n_edges) {
     return 2 * align_up(4 * (size_t)(n_nodes + 1), 256) + align_up(4 * (size_t)std::max<int64_t>(n_edges, 1), 256);
 }
-static size_t shares_bytes(const e3j_plan* plan, int64_t n_edges) {
-    return path::covers(plan, 2) && path::uses_shares(plan) ? align_up(8 * (size_t)n_edges * plan->d * plan->nq, 256) : 0;
-}
 
 size_t e3j_conv_f64_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges) {
     if (!plan || n_nodes < 0 || n_edges < 0) return 0;
-    return graph_bytes(n_nodes, n_edges) + shares_bytes(plan, n_edges);
+    return graph_bytes(n_nodes, n_edges) + bwd_shares_bytes(plan, n_edges, 8);
 }
 
 int e3j_conv_fwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, const double* x, const double* sh,
@@ -204,7 +201,7 @@ int e3j_conv_bwd_f64(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges, con
         c.n_nodes = n_nodes; c.n_edges = n_edges; c.x = x; c.sh = sh; c.w = w; c.grad_out = grad_out;
         c.senders = senders; c.receivers = receivers; c.sender_perm = sender_perm; c.colptr = colptr;
         c.grad_x = grad_x; c.grad_sh = grad_sh; c.grad_w = grad_w; c.stream = st;
-        const size_t graph = graph_bytes(n_nodes, n_edges), room = shares_bytes(plan, n_edges);
+        const size_t graph = graph_bytes(n_nodes, n_edges), room = bwd_shares_bytes(plan, n_edges, 8);
         if (room > 0 && workspace && ((uintptr_t)workspace & 255u) == 0 && workspace_bytes >= graph + room)
             c.shares = (double*)((char*)workspace + graph);
         return path::conv_bwd(plan, c);
