@@ -367,6 +367,13 @@ def _workspace(nbytes: int, like, workspace, stream, least=None):
     return workspace
 
 
+def _bwd_workspace(nbytes: int, plan, n_edges: int, like, workspace, stream, want_x: bool):
+    """_workspace of a call with a backward: nbytes less the room for shares of grad_x where that gradient is not wanted, and a
+    caller's workspace may be without that room."""
+    least = lambda: nbytes - e3j_conv_bwd_shares_bytes(plan, n_edges)
+    return _workspace(nbytes if want_x else least(), like, workspace, stream, least)
+
+
 def e3j_graph_prepare(n_nodes: int, senders, receivers, want_transpose: bool = True, stream=None,
                       _entry: str = "e3j_graph_prepare"):
     """(rowptr, sender_perm, colptr) int32 CUDA tensors; the last two are None unless want_transpose."""
@@ -489,8 +496,7 @@ def e3j_conv_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr=None
     grad_x = alloc(grad_x, (n, plan.d_in, plan.n_channels))
     grad_sh = alloc(grad_sh, (e, plan.d_sh))
     grad_w = alloc(grad_w, (e, plan.n_paths, plan.n_channels))
-    nbytes = e3j_conv_bwd_workspace_bytes(plan, n, e)
-    workspace = _workspace(nbytes, x, workspace, stream)
+    workspace = _bwd_workspace(e3j_conv_bwd_workspace_bytes(plan, n, e), plan, e, x, workspace, stream, grad_x is not None)
     _run(_entry, plan.handle.value, n, e,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
@@ -536,7 +542,7 @@ def e3j_conv_bwd_bwd(plan: Plan, x, sh, w, senders, receivers, grad_out, rowptr,
     s_x, s_sh = (n, plan.d_in, plan.n_channels), (e, plan.d_sh)
     s_w, s_out = (e, plan.n_paths, plan.n_channels), (n, plan.d_out, plan.n_channels)
     gg_out, g_x, g_sh, g_w = alloc(gg_out, s_out), alloc(g_x, s_x), alloc(g_sh, s_sh), alloc(g_w, s_w)
-    workspace = _workspace(e3j_conv_bwd_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
+    workspace = _bwd_workspace(e3j_conv_bwd_bwd_workspace_bytes(plan, n, e), plan, e, x, workspace, stream, True)
     _run("e3j_conv_bwd_bwd", plan.handle.value, n, e, _dev_ptr(x, f32, s_x, "x"), _dev_ptr(sh, f32, s_sh, "sh"), _dev_ptr(w, f32, s_w, "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),
         _dev_ptr(rowptr, i32, (n + 1,), "rowptr"), _dev_ptr(sender_perm, i32, (e,), "sender_perm"),
@@ -644,7 +650,7 @@ def e3j_conv_radial_bwd(plan: Plan, x, sh, h, W, senders, receivers, grad_out, r
     grad_sh = alloc(grad_sh, (e, plan.d_sh))
     grad_h = alloc(grad_h, (e, hidden))
     grad_W = alloc(grad_W, s_w)
-    workspace = _workspace(e3j_conv_radial_bwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream)
+    workspace = _bwd_workspace(e3j_conv_radial_bwd_workspace_bytes(plan, n, e, hidden), plan, e, x, workspace, stream, grad_x is not None)
     _run("e3j_conv_radial_bwd", plan.handle.value, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(sh, f32, (e, plan.d_sh), "sh"),
         _dev_ptr(h, f32, (e, hidden), "h"), _dev_ptr(W, f32, s_w, "W"),
@@ -682,7 +688,7 @@ def e3j_conv_radial_vec_bwd(plan: Plan, x, edge_vec, h, W, senders, receivers, g
     grad_vec = alloc(grad_vec, (e, 3))
     grad_h = alloc(grad_h, (e, hidden))
     grad_W = alloc(grad_W, s_w)
-    workspace = _workspace(e3j_conv_radial_vec_bwd_workspace_bytes(plan, n, e, hidden), x, workspace, stream)
+    workspace = _bwd_workspace(e3j_conv_radial_vec_bwd_workspace_bytes(plan, n, e, hidden), plan, e, x, workspace, stream, grad_x is not None)
     _run("e3j_conv_radial_vec_bwd", plan.handle.value, n, e, hidden,
         _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"), _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"),
         _dev_ptr(h, f32, (e, hidden), "h"), _dev_ptr(W, f32, s_w, "W"),
@@ -840,7 +846,7 @@ def e3j_conv_vec_bwd(plan: Plan, x, edge_vec, w, senders, receivers, grad_out, r
     grad_x = alloc(grad_x, (n, plan.d_in, plan.n_channels))
     grad_vec = alloc(grad_vec, (e, 3))
     grad_w = alloc(grad_w, (e, plan.n_paths, plan.n_channels))
-    workspace = _workspace(e3j_conv_vec_bwd_workspace_bytes(plan, n, e), x, workspace, stream)
+    workspace = _bwd_workspace(e3j_conv_vec_bwd_workspace_bytes(plan, n, e), plan, e, x, workspace, stream, grad_x is not None)
     _run("e3j_conv_vec_bwd", plan.handle.value, n, e, _dev_ptr(x, f32, (n, plan.d_in, plan.n_channels), "x"),
         _dev_ptr(edge_vec, f32, (e, 3), "edge_vec"), _dev_ptr(w, f32, (e, plan.n_paths, plan.n_channels), "w"),
         _dev_ptr(senders, i32, (e,), "senders"), _dev_ptr(receivers, i32, (e,), "receivers"),

@@ -13,13 +13,14 @@ class _Asked(Exception):
 
 
 def _asked_for(monkeypatch, call, *args, **kwargs):
-    """The workspace size that a call asks for (tensors on the host: it gets no further)."""
-    def workspace(nbytes, *rest):
-        raise _Asked(nbytes)
+    """The workspace size that a call asks for, and the smallest it takes from its caller (tensors on the host: it gets no
+    further)."""
+    def workspace(nbytes, like, given, stream, least=None):
+        raise _Asked(nbytes, least() if least else nbytes)
     monkeypatch.setattr(e3j, "_workspace", workspace)
     with pytest.raises(_Asked) as asked:
         call(*args, **kwargs)
-    return asked.value.args[0]
+    return asked.value.args
 
 
 def _inputs(plan, real=torch.float32):
@@ -34,7 +35,42 @@ def test_the_float64_forward_takes_the_graph_arrays_only(irreps, monkeypatch):
     plan = e3j.e3j_plan_create(irreps, 2, None, 2)
     x, sh, w, snd, rcv, g = _inputs(plan, torch.float64)
     graph = 2 * ((4 * (N + 1) + 255) // 256 * 256) + (4 * E + 255) // 256 * 256
-    assert _asked_for(monkeypatch, e3j.e3j_conv_fwd_f64, plan, x, sh, w, snd, rcv) == graph
+    assert _asked_for(monkeypatch, e3j.e3j_conv_fwd_f64, plan, x, sh, w, snd, rcv)[0] == graph
     shares = 0 if irreps == "8x0e" else (8 * E * plan.d_in * plan.n_channels + 255) // 256 * 256
     assert e3j.e3j_conv_bwd_shares_bytes(plan, E, 8) == shares
-    assert _asked_for(monkeypatch, e3j.e3j_conv_bwd_f64, plan, x, sh, w, snd, rcv, g) == graph + shares
+    assert _asked_for(monkeypatch, e3j.e3j_conv_bwd_f64, plan, x, sh, w, snd, rcv, g)[0] == graph + shares
+
+
+def _backwards(plan):
+    """(call, its workspace query) of everything that contains a backward."""
+    x, sh, w, snd, rcv, g = _inputs(plan)
+    vec, h = torch.zeros(E, 3), torch.zeros(E, HIDDEN)
+    W = torch.zeros(HIDDEN, plan.n_paths * plan.n_channels)
+    return {
+        "conv": (lambda **k: e3j.e3j_conv_bwd(plan, x, sh, w, snd, rcv, g, **k), e3j.e3j_conv_bwd_workspace_bytes(plan, N, E)),
+        "padded": (lambda **k: e3j.e3j_conv_bwd_padded(plan, x, sh, w, snd, rcv, g, snd, snd, snd, **k), e3j.e3j_conv_bwd_workspace_bytes(plan, N, E)),
+        "vec": (lambda **k: e3j.e3j_conv_vec_bwd(plan, x, vec, w, snd, rcv, g, **k), e3j.e3j_conv_vec_bwd_workspace_bytes(plan, N, E)),
+        "radial": (lambda **k: e3j.e3j_conv_radial_bwd(plan, x, sh, h, W, snd, rcv, g, **k),
+                   e3j.e3j_conv_radial_bwd_workspace_bytes(plan, N, E, HIDDEN)),
+        "radial_vec": (lambda **k: e3j.e3j_conv_radial_vec_bwd(plan, x, vec, h, W, snd, rcv, g, **k),
+                       e3j.e3j_conv_radial_vec_bwd_workspace_bytes(plan, N, E, HIDDEN)),
+    }
+
+
+@pytest.mark.parametrize("call", ["conv", "padded", "vec", "radial", "radial_vec"])
+@pytest.mark.parametrize("irreps", ["48x0e+48x1o+48x2e", "128x0e+128x1o"])
+def test_no_room_for_shares_of_a_gradient_that_is_not_wanted(irreps, call, monkeypatch):
+    plan = e3j.e3j_plan_create(irreps, 2, None, 2)
+    shares = e3j.e3j_conv_bwd_shares_bytes(plan, E)
+    assert (shares > 0) == (not plan.specialised)
+    run, full = _backwards(plan)[call]
+    assert _asked_for(monkeypatch, run) == (full, full - shares)
+    assert _asked_for(monkeypatch, run, grad_x=False) == (full - shares, full - shares)
+
+
+def test_the_double_backward_takes_a_workspace_without_the_room(monkeypatch):
+    plan = e3j.e3j_plan_create("48x0e+48x1o+48x2e", 2, None, 2)
+    x, sh, w, snd, rcv, g = _inputs(plan)
+    full = e3j.e3j_conv_bwd_bwd_workspace_bytes(plan, N, E)
+    asked = _asked_for(monkeypatch, e3j.e3j_conv_bwd_bwd, plan, x, sh, w, snd, rcv, g, None, None, None, x, sh, w)
+    assert asked == (full, full - e3j.e3j_conv_bwd_shares_bytes(plan, E)) and asked[1] < asked[0]

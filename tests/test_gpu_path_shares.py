@@ -79,3 +79,34 @@ def test_output_filters(irreps, lmax, out):
     want = (oconv.conv_fwd(cp, *host[:3], snd, rcv), *oconv.conv_bwd(cp, *host[:3], snd, rcv, host[3]))
     for have, ref, kind in zip(got, want, ("out", "x", "sh", "w")):
         assert_blockwise_close(have.cpu().numpy(), ref, blocks_of_paths(cp.paths, kind), what=kind)
+
+
+def test_calls_with_a_backward_run_on_a_workspace_without_the_room():
+    """Through the binding: the same edge gradients to the bit, the same grad_x up to the order of its sums."""
+    plan, cp, snd, rcv, host, (x, sh, w, g) = _case("12x0e+12x1o+12x2e", 2, None, 40, 12, torch.float32)
+    n, e, hidden = 40, len(rcv), 8
+    s, r = torch.from_numpy(snd).cuda(), torch.from_numpy(rcv).cuda()
+    graph = e3j.e3j_graph_prepare(n, s, r)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    vec = torch.randn(e, 3, generator=gen, device="cuda")
+    h, W = torch.randn(e, hidden, generator=gen, device="cuda"), torch.randn(hidden, plan.n_paths * plan.n_channels, generator=gen, device="cuda")
+    calls = [
+        (e3j.e3j_conv_bwd_workspace_bytes(plan, n, e), lambda **k: e3j.e3j_conv_bwd(plan, x, sh, w, s, r, g, *graph, **k)),
+        (e3j.e3j_conv_bwd_workspace_bytes(plan, n, e), lambda **k: e3j.e3j_conv_bwd_padded(plan, x, sh, w, s, r, g, *graph, **k)),
+        (e3j.e3j_conv_vec_bwd_workspace_bytes(plan, n, e), lambda **k: e3j.e3j_conv_vec_bwd(plan, x, vec, w, s, r, g, *graph, **k)),
+        (e3j.e3j_conv_radial_bwd_workspace_bytes(plan, n, e, hidden), lambda **k: e3j.e3j_conv_radial_bwd(plan, x, sh, h, W, s, r, g, *graph, **k)),
+        (e3j.e3j_conv_radial_vec_bwd_workspace_bytes(plan, n, e, hidden), lambda **k: e3j.e3j_conv_radial_vec_bwd(plan, x, vec, h, W, s, r, g, *graph, **k)),
+        (e3j.e3j_conv_bwd_bwd_workspace_bytes(plan, n, e), lambda **k: tuple(e3j.e3j_conv_bwd_bwd(plan, x, sh, w, s, r, g, *graph, x, sh, w, **k)[i] for i in (1, 0, 2, 3))),
+    ]
+    room = e3j.e3j_conv_bwd_shares_bytes(plan, e)
+    assert room >= 4 * e * plan.d_in * plan.n_channels
+    for nbytes, call in calls:
+        full = call()
+        for size in (nbytes, nbytes - room):
+            ws = torch.full((size,), 255, dtype=torch.uint8, device="cuda")
+            grads = call(workspace=ws)
+            assert all(torch.equal(a, b) for a, b in zip(grads[1:], full[1:]))
+            assert torch.equal(grads[0], full[0]) or size < nbytes
+            assert_blockwise_close(grads[0].cpu().numpy(), full[0].cpu().numpy(), blocks_of_paths(cp.paths, "x"), what="x")
+        with pytest.raises(ValueError):
+            call(workspace=ws[:nbytes - room - 256])
