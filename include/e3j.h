@@ -204,8 +204,8 @@ int e3j_noalloc_status(int32_t* status);
  * (then derived into the workspace on every call).  A node that sends nothing gets
  * a zero grad_x row. */
 size_t e3j_conv_bwd_workspace_bytes(const e3j_plan* plan, int64_t n_nodes, int64_t n_edges);
-/* Plans without generated kernels sum grad_x from the edges' shares of it where the workspace has room for them,
- * [n_edges, d, N_q] elements: faster than from the edges' inputs, and in another order, so grad_x has other last bits
+/* Plans without generated kernels sum grad_x from the edges' shares of it where these, [n_edges, d, N_q] elements, take
+ * no more than 2 GiB and the workspace has room for them: faster than from the edges' inputs, and in another order, so grad_x has other last bits
  * (each of the two is the same from run to run; grad_sh and grad_w do not depend on it).  This is what the workspace
  * queries of e3j_conv_bwd, _bwd_padded, _bwd_bwd, _vec_bwd, _radial_bwd and _radial_vec_bwd (element_bytes 4) and
  * e3j_conv_f64_workspace_bytes (8) hold for it: those calls also run with that much less.  0 for other plans. */

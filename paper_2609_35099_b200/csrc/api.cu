@@ -206,10 +206,14 @@ int check_workspace(const void* ws, size_t have, size_t need) {
 
 }  // namespace
 
+// As far as the radial forward's weight array: beyond it a call takes no memory that it can do without, so that a graph
+// which fills the device with its own arrays still runs.
+constexpr size_t kMostSharesBytes = (size_t)2 << 30;
 size_t bwd_shares_bytes(const e3j_plan* plan, int64_t n_edges, int element_bytes) {
     const bool f64 = element_bytes == 8;
     if ((!f64 && fast_lookup(plan)) || !path::covers(plan, f64 ? 2 : 4) || !path::uses_shares(plan)) return 0;
-    return align_up((size_t)element_bytes * n_edges * plan->d * plan->nq, 256);
+    const size_t bytes = align_up((size_t)element_bytes * n_edges * plan->d * plan->nq, 256);
+    return bytes <= kMostSharesBytes ? bytes : 0;
 }
 
 }  // namespace e3j

@@ -74,3 +74,19 @@ def test_the_double_backward_takes_a_workspace_without_the_room(monkeypatch):
     full = e3j.e3j_conv_bwd_bwd_workspace_bytes(plan, N, E)
     asked = _asked_for(monkeypatch, e3j.e3j_conv_bwd_bwd, plan, x, sh, w, snd, rcv, g, None, None, None, x, sh, w)
     assert asked == (full, full - e3j.e3j_conv_bwd_shares_bytes(plan, E)) and asked[1] < asked[0]
+
+
+@pytest.mark.parametrize("element", [4, 8])
+def test_the_room_ends_at_two_gib(element):
+    plan = e3j.e3j_plan_create("120x0e+120x1o+120x2e+120x3o", 3, None, 3)
+    row = element * plan.d_in * plan.n_channels
+    longest = (2 << 30) // row
+    query = e3j._load().e3j_conv_f64_workspace_bytes if element == 8 else e3j._load().e3j_conv_bwd_workspace_bytes
+    full = lambda edges: query(plan.handle, N, edges)
+    room = lambda edges: e3j.e3j_conv_bwd_shares_bytes(plan, edges, element)
+    assert longest * row <= room(longest) <= 2 << 30 and room(longest + 1) == 0
+    assert full(longest + 1) < 24 * longest < full(longest)
+    # what the call needs grows with the list all the same: a workspace for a long one serves every shorter one
+    needs = [full(edges) - room(edges) for edges in (0, 1, longest - 1, longest, longest + 1, 5_000_000)]
+    assert needs == sorted(needs)
+    assert room(0) == 0 and e3j.e3j_conv_bwd_shares_bytes(plan, 10, 2) == 0
