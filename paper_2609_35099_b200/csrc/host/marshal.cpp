@@ -82,19 +82,20 @@ PyObject* empty(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return PyObject_Vectorcall(g_slow_empty, args, 3, nullptr);
 }
 
-// call(address, arguments...) -> status, call_size for functions that return a size.  Every parameter of the C ABI is an
+// call(address, arguments...) -> status, call_size for functions that return a size (of a plan and integers; where an entry
+// point takes pointers and integers, the binding has formed the integers from shapes or computed with them).  Every parameter of the C ABI is an
 // integer or a pointer and has a 64-bit slot of its own in the calling convention, so one signature serves all entry
-// points; slots behind the last are not read.
+// points; slots behind the last are not read.  None is NULL, for the first `pointers` arguments alone.
 constexpr int kMostArgs = 24;
 template <class R>
-bool invoke(PyObject* const* args, Py_ssize_t n, R& result) {
+bool invoke(PyObject* const* args, Py_ssize_t n, Py_ssize_t pointers, R& result) {
     if (n < 1 || n > kMostArgs + 1) {
         PyErr_SetString(PyExc_TypeError, "an address and up to 24 arguments");
         return false;
     }
     uint64_t v[kMostArgs + 1] = {};
     for (Py_ssize_t i = 0; i < n; ++i) {
-        if (args[i] == Py_None) continue;
+        if (args[i] == Py_None && i > 0 && i <= pointers) continue;
         v[i] = PyLong_AsUnsignedLongLongMask(args[i]);
         if (v[i] == (uint64_t)-1 && PyErr_Occurred()) return false;
     }
@@ -109,11 +110,11 @@ bool invoke(PyObject* const* args, Py_ssize_t n, R& result) {
 }
 PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n) {
     int status;
-    return invoke(args, n, status) ? PyLong_FromLong(status) : nullptr;
+    return invoke(args, n, kMostArgs, status) ? PyLong_FromLong(status) : nullptr;
 }
 PyObject* call_size(PyObject*, PyObject* const* args, Py_ssize_t n) {
     size_t bytes;
-    return invoke(args, n, bytes) ? PyLong_FromSize_t(bytes) : nullptr;
+    return invoke(args, n, 1, bytes) ? PyLong_FromSize_t(bytes) : nullptr;
 }
 
 // set_slow(dev_ptr, empty): what the two functions above fall back on

@@ -1,4 +1,5 @@
 """How the binding takes up its native marshalling (csrc/host/marshal.cpp): no device."""
+import ctypes
 import pathlib
 import shutil
 import subprocess
@@ -79,3 +80,18 @@ def test_the_library_is_linked_without_it(missing, tmp_path, monkeypatch, capsys
         monkeypatch.setenv("PATH", str(tmp_path))
     assert build.build().read_text() == "linked"
     assert not stale.exists() and "the binding converts its arguments in Python" in capsys.readouterr().err
+
+
+def test_an_integer_parameter_is_not_null():
+    """A size query without the list's length is refused with the native call as it is without; a plan that is gone has size 0."""
+    import paper_2609_35099_b200 as e3j
+    e3j._torch()
+    plan = e3j.e3j_plan_create("8x0e", 1)
+    for query in (lambda *a: e3j.e3j_conv_bwd_workspace_bytes(plan, *a), lambda *a: e3j.e3j_conv_fwd_workspace_bytes(plan, *a),
+                  lambda *a: e3j.e3j_conv_radial_fwd_workspace_bytes(plan, 10, *a)):
+        for args in ((None, 20), (10, None)):
+            with pytest.raises((TypeError, ctypes.ArgumentError)):
+                query(*args)
+    assert e3j.e3j_conv_bwd_workspace_bytes(plan, 10, 20) > 0
+    e3j.e3j_plan_destroy(plan)
+    assert e3j.e3j_conv_bwd_workspace_bytes(plan, 10, 20) == 0
