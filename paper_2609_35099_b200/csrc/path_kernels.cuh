@@ -329,6 +329,7 @@ template <int l1, int l2, int LA, int LB, class T, int V, bool IDENT>
 __device__ __forceinline__ void pair_group(const PathTable& t, const Args<T>& a, const int p0, const int p1, const unsigned j0,
                                            const unsigned j1, const int step, const int used, const int row, const int q, T* dst) {
     constexpr int NI = 2 * l1 + 1, NY = 2 * l2 + 1, NL = LB - LA + 1, ROWS = (LB + 1) * (LB + 1) - LA * LA;
+    static_assert(NL <= 3, "paths to L = 3 have groups of their own where a pair has others");
     bool has[NL];   // the output filter may have dropped some
     int k[NL], out_off[NL];
     for (int i = 0, p = p0; i < NL; ++i) {
@@ -360,7 +361,6 @@ __device__ __forceinline__ void pair_group(const PathTable& t, const Args<T>& a,
         add_path<Tri<l1, l2, LA>, 0, T, V>(has[0], y, x, w[0], acc);
         if constexpr (NL > 1) add_path<Tri<l1, l2, LA + 1>, (LA + 1) * (LA + 1) - LA * LA, T, V>(has[1], y, x, w[1], acc);
         if constexpr (NL > 2) add_path<Tri<l1, l2, LA + 2>, (LA + 2) * (LA + 2) - LA * LA, T, V>(has[2], y, x, w[2], acc);
-        if constexpr (NL > 3) add_path<Tri<l1, l2, LA + 3>, (LA + 3) * (LA + 3) - LA * LA, T, V>(has[3], y, x, w[3], acc);
     }
 #pragma unroll 1
     for (int off = 32 >> a.split_log2; off < (32 >> a.split_log2) * used; off <<= 1) {
@@ -408,7 +408,7 @@ __device__ __forceinline__ void pair_part(const PathTable& t, const Args<T>& a, 
         case l1 * 4 + l2: { \
             constexpr int lo = l1 > l2 ? l1 - l2 : l2 - l1, hi = l1 + l2 < LM ? l1 + l2 : LM; \
             if constexpr (l1 <= LM && l2 <= LM && lo <= hi) { \
-                constexpr bool split = kTopApart && hi == 3 && lo < 3; \
+                constexpr bool split = hi == 3 && lo < 3; \
                 if constexpr (split) { \
                     if (rec.L == 3) { pair_group<l1, l2, 3, 3, T, V, IDENT>(t, a, p0, p1, j0, j1, step, used, row, q, dst); break; } \
                 } \
@@ -596,15 +596,15 @@ edge_kernel(const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T
 // much for the instruction cache (16x(0e+1o+2e+3o), 35050 edges: 338 to 431 us against 264 us), so grad_x has its own
 // launch; only where all blocks run at once do the parts share one, because there each is a chain of its paths' latencies.
 constexpr bool one_launch(int lm) { return lm < 3; }
-template <class T, int V, int LM, bool IDENT>
+template <class T, int V, int LM>
 __global__ void __launch_bounds__(kThreads, joint_blocks_per_sm(LM))
 joint_kernel(const __grid_constant__ PathTable t, const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     if (blockIdx.x < a.node_blocks) {
-        node_part<T, V, LM, true, IDENT>(t, a, blockIdx.x);
+        node_part<T, V, LM, true, false>(t, a, blockIdx.x);
         return;
     }
-    edge_part<T, V, LM, IDENT, Want::kEdges>(et, a, blockIdx.x - a.node_blocks, smem);
+    edge_part<T, V, LM, false, Want::kEdges>(et, a, blockIdx.x - a.node_blocks, smem);
 }
 
 // grad_x from the edges' shares: one 16-byte unit of a node's row to 2^split_log2 lanes, which take every so manieth

@@ -65,15 +65,17 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     static_assert(smem_bytes<LM>(kThreads) <= 48 * 1024, "more would need the kernel's attribute set");
     if (c.grad_x && !from_shares) {
         a.split_log2 = IDENT ? 0 : split_of(c.n_nodes, a.units, t.n_groups, kBwdWarps);
-        int64_t nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
-        if (tiles > 0 && (one_launch(LM) || nodes + tiles <= (int64_t)sm_count() * joint_blocks_per_sm(LM))) {
-            if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
-            a.group_blocks = (unsigned)(nodes / t.n_groups);
-            a.node_blocks = (unsigned)nodes;
-            joint_kernel<T, V, LM, IDENT><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, et, a);
-            return after_launch();
+        if constexpr (!IDENT) {   // (a tensor product whose edge gradients are wanted has grad_x from the edge part)
+            const int64_t nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, threads);
+            if (tiles > 0 && (one_launch(LM) || nodes + tiles <= (int64_t)sm_count() * joint_blocks_per_sm(LM))) {
+                if (nodes + tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
+                a.group_blocks = (unsigned)(nodes / t.n_groups);
+                a.node_blocks = (unsigned)nodes;
+                joint_kernel<T, V, LM><<<(unsigned)(nodes + tiles), threads, smem_bytes<LM>(threads), c.stream>>>(t, et, a);
+                return after_launch();
+            }
         }
-        nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
+        const int64_t nodes = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
         if (nodes >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
         a.group_blocks = (unsigned)(nodes / t.n_groups);
         node_kernel<T, V, LM, true, IDENT><<<(unsigned)nodes, kThreads, 0, c.stream>>>(t, a);

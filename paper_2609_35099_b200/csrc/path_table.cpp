@@ -35,7 +35,7 @@ void fill_table(const e3j_plan& plan, Group by, int largest_l, PathTable& t) {
         const e3j_path_info_t& pi = plan.paths[k];
         if (by == Group::kOutput) return pi.out_off;
         if (by == Group::kInput) return pi.x_off;
-        return pi.x_off * 64 + pi.l2 * 8 + (kTopApart && largest_l == 3 && pi.L == 3 ? 4 : 0);
+        return pi.x_off * 64 + pi.l2 * 8 + (largest_l == 3 && pi.L == 3 ? 4 : 0);   // paths to L = 3: groups of their own (registers)
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
         return by == Group::kPair && key(a) == key(b) ? plan.paths[a].L < plan.paths[b].L : key(a) < key(b);

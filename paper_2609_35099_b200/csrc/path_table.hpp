@@ -8,7 +8,6 @@ namespace e3j {
 namespace path {
 
 constexpr int tri_id(int l1, int l2, int L) { return l1 * 16 + l2 * 4 + L; }
-constexpr bool kTopApart = true;   // (forward, largest l = 3) paths to L = 3 form groups of their own
 constexpr uint8_t kNoPath = 255;   // a group of input rows that no path reads: nothing to add
 
 // One plan's paths in a processing order, passed by value (kernel parameters: constant-bank reads, nothing to upload).
