@@ -564,6 +564,12 @@ constexpr int fwd_blocks_per_sm(int lm) { return lm == 3 ? 5 : lm == 2 ? 7 : 8; 
 constexpr int grad_x_blocks_per_sm(int lm) { return lm == 3 ? 4 : fwd_blocks_per_sm(lm); }
 constexpr int joint_blocks_per_sm(int lm) { return lm == 3 ? 4 : lm == 2 ? 5 : 8; }
 constexpr int pair_blocks_per_sm(int lm) { return lm == 3 ? 5 : lm == 2 ? 6 : 8; }
+// Where the forward's blocks all run at once with fewer of them per SM, a block is a chain of its edges' latencies, and the
+// spilled values lengthen it: the same kernel with more registers (8 / 4 / 3, float64 8 / 3 / 3).  Six blocks at l = 2 and five
+// at l = 3 against it, 4 nodes of degree 400: 48x(0e+1o+2e), l <= 2, 51 -> 34 us, float64 68 -> 37; 16x(0e+1o+2e+3o), l <= 3, 50 ->
+// 39, float64 64 -> 45.  64 nodes of degree 20, the first: 9.2 -> 6.3.  Large launches want the blocks: 1500 x 50, the first,
+// 143 us against 185 with four; 6000 x 20, the other, 249 against 341 with three.
+template <class T> constexpr int few_pair_blocks_per_sm(int lm) { return lm == 3 || (lm == 2 && sizeof(T) == 8) ? 3 : lm == 2 ? 4 : 8; }
 template <class T> constexpr int edge_blocks_per_sm(int lm) {
     return sizeof(T) == 8 ? (lm == 3 ? 2 : lm == 2 ? 3 : 5) : (lm == 3 ? 3 : lm == 2 ? 4 : 6);
 }
@@ -576,8 +582,8 @@ node_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
     node_part<T, V, LM, TR, IDENT>(t, a, blockIdx.x);
 }
 
-template <class T, int V, int LM, bool IDENT>
-__global__ void __launch_bounds__(kThreads, pair_blocks_per_sm(LM))
+template <class T, int V, int LM, bool IDENT, int BLOCKS>
+__global__ void __launch_bounds__(kThreads, BLOCKS)
 pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
     fast::grid_dependency_wait();
     pair_part<T, V, LM, IDENT>(t, a, blockIdx.x);

@@ -43,7 +43,12 @@ template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, cons
     const int64_t blocks = node_blocks(c.n_nodes, a.units, a.split_log2, t.n_groups, kThreads);
     if (blocks >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
     a.group_blocks = (unsigned)(blocks / t.n_groups);
-    if (pairs) return launch_dependent(pair_kernel<T, V, LM, IDENT>, dim3((unsigned)blocks), dim3(kThreads), 0, c.stream, t, a);
+    if (pairs) {
+        constexpr int few = few_pair_blocks_per_sm<T>(LM);
+        const auto kernel = blocks <= (int64_t)sm_count() * few ? pair_kernel<T, V, LM, IDENT, few>
+                                                                : pair_kernel<T, V, LM, IDENT, pair_blocks_per_sm(LM)>;
+        return launch_dependent(kernel, dim3((unsigned)blocks), dim3(kThreads), 0, c.stream, t, a);
+    }
     node_kernel<T, V, LM, false, IDENT><<<(unsigned)blocks, kThreads, 0, c.stream>>>(t, a);
     return after_launch();
 }
