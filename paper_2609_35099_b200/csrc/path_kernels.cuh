@@ -573,6 +573,12 @@ template <class T> constexpr int few_pair_blocks_per_sm(int lm) { return lm == 3
 template <class T> constexpr int edge_blocks_per_sm(int lm) {
     return sizeof(T) == 8 ? (lm == 3 ? 2 : lm == 2 ? 3 : 5) : (lm == 3 ? 3 : lm == 2 ? 4 : 6);
 }
+// grad_w and grad_sh alone.  In float64 as many blocks as in float32 spill (up to 1100 bytes at l = 3): all three bounds against
+// those, geometric means over 18 to 56 calls, grad_w 0.85 / 0.83 / 0.66, grad_sh 0.92 / 0.92 / 0.78; 120x1o, l <= 1, 120 000 edges: grad_w
+// 295 -> 196 us.  One block less at l = 1 gives grad_w two per cent more and takes up to seven from a grad_sh.
+template <class T> constexpr int edges_alone_blocks_per_sm(int lm) {
+    return sizeof(T) == 8 ? (lm == 3 ? 3 : lm == 2 ? 4 : 7) : joint_blocks_per_sm(lm);
+}
 template <int LM> constexpr int smem_bytes(int threads) { return threads / 32 * ring_bytes<LM>(); }
 
 // TR: the forward's sums, or grad_x on its own.
@@ -590,7 +596,7 @@ pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
 }
 
 template <class T, int V, int LM, bool IDENT, Want WANT>
-__global__ void __launch_bounds__(kThreads, WANT == Want::kEdges ? joint_blocks_per_sm(LM) : edge_blocks_per_sm<T>(LM))
+__global__ void __launch_bounds__(kThreads, WANT == Want::kEdges ? edges_alone_blocks_per_sm<T>(LM) : edge_blocks_per_sm<T>(LM))
 edge_kernel(const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");
