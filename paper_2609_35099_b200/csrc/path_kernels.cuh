@@ -579,6 +579,9 @@ template <class T> constexpr int edge_blocks_per_sm(int lm) {
 template <class T> constexpr int edges_alone_blocks_per_sm(int lm) {
     return sizeof(T) == 8 ? (lm == 3 ? 3 : lm == 2 ? 4 : 7) : joint_blocks_per_sm(lm);
 }
+// grad_x alone in float64: where its blocks do not all run at once, one more per SM.  64x(0e+1o), l <= 3, 5000 edges 37 -> 27 us;
+// 128x(0e+1o), 6000 edges 81 -> 61; in launches that do it costs up to a quarter (4x(0e+1o), l <= 3, 5000 edges 12.4 -> 15.5).
+template <class T> constexpr int only_x_blocks_per_sm(int lm) { return edge_blocks_per_sm<T>(lm) + (sizeof(T) == 8 ? 1 : 0); }
 template <int LM> constexpr int smem_bytes(int threads) { return threads / 32 * ring_bytes<LM>(); }
 
 // TR: the forward's sums, or grad_x on its own.
@@ -595,8 +598,8 @@ pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
     pair_part<T, V, LM, IDENT>(t, a, blockIdx.x);
 }
 
-template <class T, int V, int LM, bool IDENT, Want WANT>
-__global__ void __launch_bounds__(kThreads, WANT == Want::kEdges ? edges_alone_blocks_per_sm<T>(LM) : edge_blocks_per_sm<T>(LM))
+template <class T, int V, int LM, bool IDENT, Want WANT, int BLOCKS>
+__global__ void __launch_bounds__(kThreads, BLOCKS)
 edge_kernel(const __grid_constant__ EdgeTable et, const __grid_constant__ Args<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     static_assert((LM + 1) * (LM + 1) * 32 * (int)sizeof(T) <= ring_bytes<LM>(), "the partials take the rings' place");

@@ -89,8 +89,12 @@ template <class T, int V, int LM, bool IDENT> int bwd(const e3j_plan* plan, cons
     if (tiles > 0) {
         if (tiles >= (int64_t)1 << 31) return E3J_ERR_INVALID_ARG;
         a.dx = !from_shares ? nullptr : IDENT ? c.grad_x : c.shares;
-        const auto kernel = !from_shares ? edge_kernel<T, V, LM, IDENT, Want::kEdges>
-                            : edges || IDENT ? edge_kernel<T, V, LM, IDENT, Want::kAll> : edge_kernel<T, V, LM, false, Want::kX>;
+        constexpr int all = edge_blocks_per_sm<T>(LM);
+        const bool at_once = tiles * threads <= (int64_t)sm_count() * all * kThreads;
+        const auto kernel = !from_shares     ? edge_kernel<T, V, LM, IDENT, Want::kEdges, edges_alone_blocks_per_sm<T>(LM)>
+                            : edges || IDENT ? edge_kernel<T, V, LM, IDENT, Want::kAll, all>
+                            : at_once        ? edge_kernel<T, V, LM, false, Want::kX, all>
+                                             : edge_kernel<T, V, LM, false, Want::kX, only_x_blocks_per_sm<T>(LM)>;
         if (int s = launch_dependent(kernel, dim3((unsigned)tiles), dim3(threads), smem_bytes<LM>(threads), c.stream, et, a)) return s;
     }
     if (!from_shares || IDENT) return E3J_OK;

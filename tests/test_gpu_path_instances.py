@@ -55,3 +55,33 @@ def test_forwards_either_side_of_the_line(irreps, lmax, real):
     assert torch.equal(large[:n], small) and not large[n].any()
     want = oconv.conv_fwd(cp, host[0][:n], *host[1:], snd, rcv)
     assert_blockwise_close(small.cpu().numpy(), want, blocks_of_paths(cp.paths, "out"), tol=1e-12 if real == torch.float64 else 1e-5, what="out")
+
+
+@pytest.mark.parametrize("nodes,degree", [(40, 20), (1500, 40)])   # all blocks at once; several waves of them
+@pytest.mark.parametrize("real", [torch.float32, torch.float64])
+@pytest.mark.parametrize("irreps,lmax", SIGNATURES + [("120x1o", 1)])
+def test_grad_x_alone_has_the_bits_of_the_full_call(irreps, lmax, real, nodes, degree):
+    plan = e3j.e3j_plan_create(irreps, lmax, None, lmax)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=real)
+    e = nodes * degree
+    r = torch.arange(nodes, device="cuda", dtype=torch.int32).repeat_interleave(degree)
+    s = torch.randint(nodes, (e,), generator=gen, device="cuda", dtype=torch.int32)
+    _, perm, colptr = e3j.e3j_graph_prepare(nodes, s, r)
+    x, sh, w, g = draw(nodes, plan.d_in, plan.n_channels), draw(e, plan.d_sh), draw(e, plan.n_paths, plan.n_channels), draw(nodes, plan.d_out, plan.n_channels)
+    lib, f64 = e3j._load(), real == torch.float64
+    nbytes = (lib.e3j_conv_f64_workspace_bytes if f64 else lib.e3j_conv_bwd_workspace_bytes)(plan.handle, nodes, e)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+
+    def call(*wanted):
+        grads = [torch.full_like(t, float("nan")) for t in (x, sh, w)]
+        ptr = lambda t: t.data_ptr()
+        args = [*map(ptr, (x, sh, w, s, r)), *([] if f64 else [None]), *map(ptr, (perm, colptr, g)),
+                *(ptr(t) if want else None for t, want in zip(grads, wanted)), ptr(ws), nbytes, torch.cuda.current_stream().cuda_stream]
+        assert (lib.e3j_conv_bwd_f64 if f64 else lib.e3j_conv_bwd)(plan.handle, nodes, e, *args) == e3j.E3J_OK
+        return grads
+
+    full = call(True, True, True)
+    assert not any(t.isnan().any() for t in full)
+    for wanted in ((True, False, False), (False, True, False), (False, False, True)):
+        assert all(torch.equal(a, b) if want else a.isnan().all() for a, b, want in zip(call(*wanted), full, wanted))
