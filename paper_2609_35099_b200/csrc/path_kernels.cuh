@@ -573,12 +573,11 @@ template <class T> constexpr int few_pair_blocks_per_sm(int lm) { return lm == 3
 template <class T> constexpr int edge_blocks_per_sm(int lm) {
     return sizeof(T) == 8 ? (lm == 3 ? 2 : lm == 2 ? 3 : 5) : (lm == 3 ? 3 : lm == 2 ? 4 : 6);
 }
-// grad_w and grad_sh alone.  In float64 as many blocks as in float32 spill (up to 1100 bytes at l = 3): all three bounds against
-// those, geometric means over 18 to 56 calls, grad_w 0.85 / 0.83 / 0.66, grad_sh 0.92 / 0.92 / 0.78; 120x1o, l <= 1, 120 000 edges: grad_w
-// 295 -> 196 us.  One block less at l = 1 gives grad_w two per cent more and takes up to seven from a grad_sh.
-template <class T> constexpr int edges_alone_blocks_per_sm(int lm) {
-    return sizeof(T) == 8 ? (lm == 3 ? 3 : lm == 2 ? 4 : 7) : joint_blocks_per_sm(lm);
-}
+// grad_w and grad_sh alone.  In float64 the eight and four blocks of l = 1 and 3 spill (1100 bytes at l = 3); one less: geometric
+// means over 18 and 74 calls 0.84 / 0.66 for grad_w, 0.92 / 0.80 for grad_sh (120x1o, l <= 1, 120 000 edges: grad_w 295 -> 195 us).
+// A second one less at l = 1 gives grad_w two per cent more and takes up to seven from a grad_sh.  At l = 2 one less makes grad_w
+// 0.85, and the grad_sh of scalar inputs up to 1.25 where 740 blocks ran at once and 592 do not.
+template <class T> constexpr int edges_alone_blocks_per_sm(int lm) { return joint_blocks_per_sm(lm) - (sizeof(T) == 8 && lm != 2 ? 1 : 0); }
 // grad_x alone in float64: where its blocks do not all run at once, one more per SM.  64x(0e+1o), l <= 3, 5000 edges 37 -> 27 us;
 // 128x(0e+1o), 6000 edges 81 -> 61; in launches that do it costs up to a quarter (4x(0e+1o), l <= 3, 5000 edges 12.4 -> 15.5).
 template <class T> constexpr int only_x_blocks_per_sm(int lm) { return edge_blocks_per_sm<T>(lm) + (sizeof(T) == 8 ? 1 : 0); }
