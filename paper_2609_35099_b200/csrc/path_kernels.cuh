@@ -379,7 +379,7 @@ __device__ __forceinline__ void pair_group(const PathTable& t, const Args<T>& a,
     }
 }
 
-template <class T, int V, int LM, bool IDENT>
+template <class T, int V, int LM, int LX, bool IDENT>   // LX: the largest l of the inputs
 __device__ __forceinline__ void pair_part(const PathTable& t, const Args<T>& a, const unsigned block) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
     const int per_warp = 32 >> a.split_log2, part = lane >> (5 - a.split_log2);
@@ -407,7 +407,7 @@ __device__ __forceinline__ void pair_part(const PathTable& t, const Args<T>& a, 
 #define E3J_CASE(l1, l2) \
         case l1 * 4 + l2: { \
             constexpr int lo = l1 > l2 ? l1 - l2 : l2 - l1, hi = l1 + l2 < LM ? l1 + l2 : LM; \
-            if constexpr (l1 <= LM && l2 <= LM && lo <= hi) { \
+            if constexpr (l1 <= LX && l2 <= LM && lo <= hi) { \
                 constexpr bool split = hi == 3 && lo < 3; \
                 if constexpr (split) { \
                     if (rec.L == 3) { pair_group<l1, l2, 3, 3, T, V, IDENT>(t, a, p0, p1, j0, j1, step, used, row, q, dst); break; } \
@@ -569,6 +569,10 @@ constexpr int pair_blocks_per_sm(int lm) { return lm == 3 ? 5 : lm == 2 ? 6 : 8;
 // at l = 3 against it, 4 nodes of degree 400: 48x(0e+1o+2e), l <= 2, 51 -> 34 us, float64 68 -> 37; 16x(0e+1o+2e+3o), l <= 3, 50 ->
 // 39, float64 64 -> 45.  64 nodes of degree 20, the first: 9.2 -> 6.3.  Large launches want the blocks: 1500 x 50, the first,
 // 143 us against 185 with four; 6000 x 20, the other, 249 against 341 with three.
+// Scalar inputs alone, from l = 2 on: the kernel without the other inputs' cases fits eight blocks per SM in its registers.  96x0e,
+// 75 000 edges, with the six and five blocks of the whole kernel, with this one, and by output blocks: l <= 2 56 / 46 / 48 us, float64 113 /
+// 96 / 93; l <= 3 90 / 65 / 88, float64 167 / 123 / 157.  Where all blocks run at once it is up to 1.6 times as long as the one above.
+constexpr int kScalarPairBlocks = 8;
 template <class T> constexpr int few_pair_blocks_per_sm(int lm) { return lm == 3 || (lm == 2 && sizeof(T) == 8) ? 3 : lm == 2 ? 4 : 8; }
 template <class T> constexpr int edge_blocks_per_sm(int lm) {
     return sizeof(T) == 8 ? (lm == 3 ? 2 : lm == 2 ? 3 : 5) : (lm == 3 ? 3 : lm == 2 ? 4 : 6);
@@ -590,11 +594,11 @@ node_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T>
     node_part<T, V, LM, TR, IDENT>(t, a, blockIdx.x);
 }
 
-template <class T, int V, int LM, bool IDENT, int BLOCKS>
+template <class T, int V, int LM, bool IDENT, int BLOCKS, int LX = LM>
 __global__ void __launch_bounds__(kThreads, BLOCKS)
 pair_kernel(const __grid_constant__ PathTable t, const __grid_constant__ Args<T> a) {
     fast::grid_dependency_wait();
-    pair_part<T, V, LM, IDENT>(t, a, blockIdx.x);
+    pair_part<T, V, LM, LX, IDENT>(t, a, blockIdx.x);
 }
 
 template <class T, int V, int LM, bool IDENT, Want WANT, int BLOCKS>

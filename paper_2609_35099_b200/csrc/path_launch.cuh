@@ -45,7 +45,9 @@ template <class T, int V, int LM, bool IDENT> int fwd(const e3j_plan* plan, cons
     a.group_blocks = (unsigned)(blocks / t.n_groups);
     if (pairs) {
         constexpr int few = few_pair_blocks_per_sm<T>(LM);
+        constexpr int scalar_lx = LM > 1 ? 0 : LM;
         const auto kernel = blocks <= (int64_t)sm_count() * few ? pair_kernel<T, V, LM, IDENT, few>
+                            : plan->path.largest_l1 == 0        ? pair_kernel<T, V, LM, IDENT, kScalarPairBlocks, scalar_lx>
                                                                 : pair_kernel<T, V, LM, IDENT, pair_blocks_per_sm(LM)>;
         return launch_dependent(kernel, dim3((unsigned)blocks), dim3(kThreads), 0, c.stream, t, a);
     }

@@ -10,7 +10,7 @@ from oracle import conv as oconv
 from parity_util import assert_blockwise_close, blocks_of_paths
 
 pytestmark = pytest.mark.gpu
-SIGNATURES = [("8x0e+8x1o", 2), ("12x0e+12x1o+12x2e", 2), ("8x0e+8x1o+8x2e+8x3o", 3)]
+SIGNATURES = [("8x0e+8x1o", 2), ("12x0e+12x1o+12x2e", 2), ("8x0e+8x1o+8x2e+8x3o", 3), ("16x0e", 2), ("8x0e+8x0o", 3)]
 
 
 def _last_small(plan, lmax, real, split):
