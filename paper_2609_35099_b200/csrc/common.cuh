@@ -30,10 +30,11 @@ inline int after_launch() {
     return cuda_status(cudaGetLastError());
 }
 
-// Launch of a kernel that follows another one on the same stream and starts with fast::grid_dependency_wait(): the
+// Launch of a kernel that may follow another one on the same stream and has fast::grid_dependency_wait(): the
 // launch itself (and the scheduling of its first CTAs) overlaps the tail of its predecessor; the wait inside the
 // kernel holds it until the predecessor has finished and its writes are visible (programmatic dependent launch).  128x(0e+1o),
-// 9600 edges: forward 22.6 -> 20.1 us, backward 41.1 -> 38.7; 78 000 edges: 106 -> 104, 278 -> 277.
+// calls back to back, against ordinary launches: 9600 edges, forward 24.6 -> 20.4 us, backward 43.2 -> 39.0; 78 000 edges, 103.4 ->
+// 100.1 and 260 -> 257.
 template <class... KArgs, class... Args>
 inline int launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {
     cudaLaunchConfig_t cfg{};

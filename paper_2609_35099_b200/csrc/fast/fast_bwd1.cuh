@@ -63,7 +63,7 @@ struct Bwd1Smem {
     // room lets have longer tiles, up to where the next warp would take registers away (backward, 78 000 edges of 1500 atoms):
     // 64x(0e+1o+2e+3o) six edges instead of four, with packed arithmetic 857 -> 712 us; 64x(0e+1o) fifteen instead of ten, 154
     // -> 140; 32x(0e+1o) fifteen instead of sixteen, 117 -> 91; 96x(0e+1o) seven instead of six, 256 -> 249.  128 and 256
-    // channels: no gain (128x(0e+1o) 252 -> 259 with eight, 128x(0e+1o+2e) 714 -> 712 with four instead of three).
+    // channels: no gain (128x(0e+1o) 1.03 times as long with eight, 128x(0e+1o+2e) as long with four instead of three).
     static constexpr bool XG = !ROWS && !DBL && S::EXG;
     static constexpr size_t up(size_t v, size_t a) { return (v + a - 1) / a * a; }
     static constexpr size_t off_bar = 0;                                   // full[NS], empty[NS]

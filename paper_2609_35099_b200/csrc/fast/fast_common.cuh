@@ -21,12 +21,16 @@ namespace fast {
 constexpr uint32_t kSpinLimit = 1u << 22;  // polls of mbarrier.try_wait before giving up
 constexpr int kStatusTimeout = 1;          // value stored in the device status word
 
-// First statement of a kernel that is launched with launch_dependent (common.cuh): holds the kernel until the
-// one before it on the stream has finished and its writes are visible; a no-op under an ordinary launch.
+// In a kernel that is launched with launch_dependent (common.cuh): holds the block until the kernel before it on the stream has
+// finished and its writes are visible; a no-op under an ordinary launch.  It comes before every access to memory, with one
+// exception: a kernel that follows one which waits in every block and does not trigger early may before its wait (or
+// in blocks without one, as long as others wait) touch what that kernel does not write, because what came before it is done by
+// then.  bwd_dx_reduce_kernel and share_sum_kernel, which follow sweeps, read the sender order so, and the former zeroes padding rows.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets a dependent kernel's blocks start where there is room for them; they wait for this kernel's end all the same.
 // Always after this kernel's own wait: a block that has started then knows that everything before this kernel is done.
-// Small kernels only: in the sweeps it made the backward slower (128x(0e+1o), 78 000 edges: 268 -> 277 us).
+// Small kernels only: in the sweeps it is slower (128x(0e+1o), 78 000 edges: backward 257 -> 264 us, forward 100.1 -> 100.8; 9600:
+// 39.0 -> 39.9 and 20.4 -> 21.2), and the exception above would not hold.
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------- channel vectors

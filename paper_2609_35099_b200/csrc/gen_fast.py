@@ -162,9 +162,9 @@ class Sig:
     # fast_common.cuh).  Measured on the 128-channel water signature: the forward-shaped bodies and the double
     # backward gain (fewer issue slots).  The first backward's edge body ("ebwd") gains where one warp with two channels per
     # lane does a whole edge, which its instruction supply bounds: 64x(0e+1o+2e), l <= 3, 500 -> 393 us on the 78 000 edges
-    # of 1500 atoms, and with the 255 registers of seven consumer warps instead of eight 330.  With four channels per lane (128x(0e+1o): 255 ->
-    # 274 us) or several warps to an edge (128x(0e+1o+2e+3o), l <= 2: 555 -> 640), which share what they fetch, it loses, and
-    # the body stays scalar.
+    # of 1500 atoms, and with the 255 registers of seven consumer warps instead of eight 330.  With four channels per lane (128x(0e+1o): 1.07 times
+    # as long) or several warps to an edge (128x(0e+1o+2e+3o), l <= 2: 1.15 times), which share what they fetch, it loses, and
+    # the body stays scalar.  A signature without tile parameters of its own has the scalar body: auto_params does not apply this rule.
     PACKED_DEFAULT = ("fwd", "fwd2", "rfwd", "bwd2")
 
     def ops(self, kind):
