@@ -370,8 +370,10 @@ def _workspace(nbytes: int, like, workspace, stream, least=None):
 def _bwd_workspace(nbytes: int, plan, n_edges: int, like, workspace, stream, want_x: bool):
     """_workspace of a call with a backward: nbytes less the room for shares of grad_x where that gradient is not wanted, and a
     caller's workspace may be without that room."""
-    least = lambda: nbytes - e3j_conv_bwd_shares_bytes(plan, n_edges)
-    return _workspace(nbytes if want_x else least(), like, workspace, stream, least)
+    if want_x and workspace is None:
+        return _workspace(nbytes, like, None, stream)
+    least = nbytes - e3j_conv_bwd_shares_bytes(plan, n_edges)
+    return _workspace(nbytes if want_x else least, like, workspace, stream, lambda: least)
 
 
 def e3j_graph_prepare(n_nodes: int, senders, receivers, want_transpose: bool = True, stream=None,
